@@ -78,6 +78,11 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
   }
 }
 
+// The same by a whole warp: true only if every lane's wait succeeded.
+__device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+  return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag, limit));
+}
+
 // ---- tcgen05, cta_group::2 forms ---------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc2(uint32_t* smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(pq::smem_u32(smem_dst)),
@@ -220,12 +225,12 @@ inline bool make_packed_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, 
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tensor map over a dense s8 matrix [rows, K]; box = [128 rows, 128 bytes] landing in the 128-byte-swizzled
+// Tensor map over a dense s8 matrix [rows, K]; box = [box_rows, 128 bytes] landing in the 128-byte-swizzled
 // K-major layout the MMA descriptors read.
-inline bool make_s8_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t K) {
+inline bool make_s8_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t K, int box_rows = BM_CTA) {
   cuuint64_t gdim[2] = {static_cast<cuuint64_t>(K), static_cast<cuuint64_t>(rows)};
   cuuint64_t gstride[1] = {static_cast<cuuint64_t>(K)};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(BM_CTA)};
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(box_rows)};
   cuuint32_t estr[2] = {1, 1};
   return reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
              map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), gdim, gstride, box, estr,

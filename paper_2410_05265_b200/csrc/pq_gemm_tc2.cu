@@ -122,8 +122,8 @@ __global__ void __launch_bounds__(N_THREADS, 1)
 
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");  // operands and output may belong to the previous kernel
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
+  const int warp = pq::warp_index(), lane = threadIdx.x & 31;
+  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int n_tiles = p.tiles_m * p.tiles_n;
   const int n_kb = (p.K + BK - 1) / BK;
@@ -160,23 +160,24 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   __syncthreads();
   cluster_sync_all();  // the peer's barriers exist before anything arrives on them
   pq::tc_fence_after();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   uint32_t loads_issued = 0;  // producer lanes: stages whose copies were started
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-        const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
-        const int n_row = (tile / p.tiles_m) * BN + rank * BN_CTA;
-        for (int kb = 0; kb < n_kb; ++kb, ++it) {
-          const uint32_t s = it % N_PK, ph = (it / N_PK) & 1;
-          if (!wait_bar(&bars->pk_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
-            ok = false;
-            break;
-          }
+    const bool leader = pq::elect_one();
+    uint32_t it = 0;
+    bool ok = true;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
+      const int n_row = (tile / p.tiles_m) * BN + rank * BN_CTA;
+      for (int kb = 0; kb < n_kb; ++kb, ++it) {
+        const uint32_t s = it % N_PK, ph = (it / N_PK) & 1;
+        if (!wait_bar_warp(&bars->pk_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
+        }
+        if (leader) {
           if (A8) {
             pq::mbar_arrive_expect_tx(&bars->pk_full[s], BN_CTA * PK_ROW);
             pq::tma_load_2d(pk_buf + s * PK_STAGE, &tmap_b, kb * PK_ROW, n_row, &bars->pk_full[s]);
@@ -186,50 +187,63 @@ __global__ void __launch_bounds__(N_THREADS, 1)
             pq::tma_load_2d(pk_buf + s * PK_STAGE + BM_CTA * PK_ROW, &tmap_b, kb * PK_ROW, n_row, &bars->pk_full[s]);
           }
         }
+        __syncwarp();
       }
-      loads_issued = it;
-      if (!ok) {
+    }
+    loads_issued = it;
+    if (!ok) {
+      if (leader) {
         bars->abort_flag = 1;
         pq::report(p.status, PQ_ERR_TIMEOUT);
-        // let the copies this thread started land before the CTA can exit
-        const uint32_t first = it > N_PK ? it - N_PK : 0;
-        for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->pk_full[j % N_PK], (j / N_PK) & 1);
       }
+      // let the copies this warp started land before the CTA can exit
+      const uint32_t first = it > N_PK ? it - N_PK : 0;
+      for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->pk_full[j % N_PK], (j / N_PK) & 1);
     }
   } else if (A8 && warp == 2) {
     // ------------------------------------------------------------------ token-operand producer (A8)
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-        const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
-        for (int kb = 0; kb < n_kb; ++kb, ++it) {
-          const uint32_t s = it % N_S8, ph = (it / N_S8) & 1;
-          if (!wait_bar(&bars->s8_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
-            ok = false;
-            break;
-          }
+    const bool leader = pq::elect_one();
+    uint32_t it = 0;
+    bool ok = true;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
+      for (int kb = 0; kb < n_kb; ++kb, ++it) {
+        const uint32_t s = it % N_S8, ph = (it / N_S8) & 1;
+        if (!wait_bar_warp(&bars->s8_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
+        }
+        if (leader) {
           pq::mbar_arrive_expect_tx(&bars->a_full[s], S8_A);
           pq::tma_load_2d(s8_buf + s * S8_STAGE, &tmap_a, kb * BK, m_row, &bars->a_full[s]);
         }
+        __syncwarp();
       }
-      loads_issued = it;
-      if (!ok) {
+    }
+    loads_issued = it;
+    if (!ok) {
+      if (leader) {
         bars->abort_flag = 1;
         pq::report(p.status, PQ_ERR_TIMEOUT);
-        const uint32_t first = it > N_S8 ? it - N_S8 : 0;
-        for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->a_full[j % N_S8], (j / N_S8) & 1);
       }
+      const uint32_t first = it > N_S8 ? it - N_S8 : 0;
+      for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->a_full[j % N_S8], (j / N_S8) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      // The four MMAs of a K block take 512 clocks of the tensor pipe; wait, issue and commit have to stay below that,
+      // or this warp paces the kernel. With the loop in a branch of one lane they took 550-600; kept uniform (see
+      // elect_one) about 350: W4A4 2044 x 28672 x 4096: 165.7 -> 155.8 us, x 6144: 44.1 -> 41.6;
+      // W4A8: 158.4 -> 145.3 and 41.7 -> 36.3.
       constexpr uint32_t idesc = pq::umma_idesc_s8(2 * BM_CTA, BN);
+      const bool leader = pq::elect_one();
+      const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(s8_buf));
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++tcount) {
         const uint32_t ab = tcount & 1, aph = (tcount >> 1) & 1;
-        if (!wait_bar(&bars->acc_empty[ab], aph ^ 1, abort_flag, p.wait_clocks)) {
+        if (!wait_bar_warp(&bars->acc_empty[ab], aph ^ 1, abort_flag, p.wait_clocks)) {
           ok = false;
           break;
         }
@@ -237,30 +251,34 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         const uint32_t d_tmem = tmem_base + ab * BN;
         for (int kb = 0; kb < n_kb; ++kb, ++it) {
           const uint32_t s = it % N_S8, ph = (it / N_S8) & 1;
-          if (!wait_bar(&bars->s8_full[s], ph, abort_flag, p.wait_clocks)) {
+          if (!wait_bar_warp(&bars->s8_full[s], ph, abort_flag, p.wait_clocks)) {
             ok = false;
             break;
           }
           pq::tc_fence_after();
-          const uint32_t a_addr = pq::smem_u32(s8_buf + s * S8_STAGE);
-          const uint32_t b_addr = a_addr + S8_A;
+          if (leader) {
+            const uint64_t a_desc = desc0 + s * (S8_STAGE >> 4), b_desc = a_desc + (S8_A >> 4);
 #pragma unroll
-          for (int kk = 0; kk < BK / 32; ++kk) {
-            mma2_i8_ss(d_tmem, pq::umma_desc_sw128(a_addr + kk * 32), pq::umma_desc_sw128(b_addr + kk * 32), idesc,
-                       (kb | kk) != 0 ? 1u : 0u);
+            for (int kk = 0; kk < BK / 32; ++kk)  // 32 bytes of K further along the 128-byte rows
+              mma2_i8_ss(d_tmem, a_desc + kk * 2, b_desc + kk * 2, idesc, (kb | kk) != 0 ? 1u : 0u);
+            mma2_commit_both(&bars->s8_empty[s]);  // both CTAs may refill the stage once these MMAs have read it
           }
-          mma2_commit_both(&bars->s8_empty[s]);  // both CTAs may refill the stage once these MMAs have read it
+          __syncwarp();
         }
-        if (ok) mma2_commit_both(&bars->acc_full[ab]);
+        if (ok && leader) mma2_commit_both(&bars->acc_full[ab]);
+        __syncwarp();
       }
-      if (!ok) {
-        bars->abort_flag = 1;
-        pq::report(p.status, PQ_ERR_TIMEOUT);
+      if (leader) {
+        if (!ok) {
+          bars->abort_flag = 1;
+          pq::report(p.status, PQ_ERR_TIMEOUT);
+        }
+        // whatever was issued has finished before either CTA releases its tensor memory
+        mma2_commit_both(&bars->drain);
       }
-      // whatever was issued has finished before either CTA releases its tensor memory
-      mma2_commit_both(&bars->drain);
+      __syncwarp();
     }
-    if (lane == 0) pq::mbar_wait(&bars->drain, 0);
+    pq::mbar_wait(&bars->drain, 0);
   } else if (warp >= UNPACK_WARP0) {
     // ------------------------------------------------------------------ unpack warps
     const int group = (warp - UNPACK_WARP0) / GROUP_WARPS;

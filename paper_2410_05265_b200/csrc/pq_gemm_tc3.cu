@@ -101,20 +101,6 @@ __device__ __forceinline__ void mma2_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// 32 lanes x 32 consecutive 32-bit columns: thread i of the warp writes lane (base+i).
-__device__ __forceinline__ void tmem_st_32x32(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
-      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
-      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
 template <bool ZP>
 __global__ void __launch_bounds__(N_THREADS, 1)
     gemm_w4a4_pair_ts_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
@@ -130,8 +116,8 @@ __global__ void __launch_bounds__(N_THREADS, 1)
 
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");  // operands and output may belong to the previous kernel
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
+  const int warp = pq::warp_index(), lane = threadIdx.x & 31;
+  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int n_tiles = p.tiles_m * p.tiles_n;
   const int n_kb = (p.K + BK - 1) / BK;
@@ -165,45 +151,56 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   __syncthreads();
   cluster_sync_all();  // the peer's barriers exist before anything arrives on them
   pq::tc_fence_after();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   uint32_t loads_issued = 0;  // producer lanes: stages whose copies were started
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-        const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
-        const int n_row = (tile / p.tiles_m) * BN + rank * BN_CTA;
-        for (int kb = 0; kb < n_kb; ++kb, ++it) {
-          const uint32_t s = it % N_PK, ph = (it / N_PK) & 1;
-          if (!wait_bar(&bars->pk_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
-            ok = false;
-            break;
-          }
+    const bool leader = pq::elect_one();
+    uint32_t it = 0;
+    bool ok = true;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
+      const int n_row = (tile / p.tiles_m) * BN + rank * BN_CTA;
+      for (int kb = 0; kb < n_kb; ++kb, ++it) {
+        const uint32_t s = it % N_PK, ph = (it / N_PK) & 1;
+        if (!wait_bar_warp(&bars->pk_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
+        }
+        if (leader) {
           pq::mbar_arrive_expect_tx(&bars->pk_full[s], PK_STAGE);
           pq::tma_load_2d(pk_buf + s * PK_STAGE, &tmap_a, kb * PK_ROW, m_row, &bars->pk_full[s]);
           pq::tma_load_2d(pk_buf + s * PK_STAGE + BM_CTA * PK_ROW, &tmap_b, kb * PK_ROW, n_row, &bars->pk_full[s]);
         }
+        __syncwarp();
       }
-      loads_issued = it;
-      if (!ok) {
+    }
+    loads_issued = it;
+    if (!ok) {
+      if (leader) {
         bars->abort_flag = 1;
         pq::report(p.status, PQ_ERR_TIMEOUT);
-        // let the copies this thread started land before the CTA can exit
-        const uint32_t first = it > N_PK ? it - N_PK : 0;
-        for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->pk_full[j % N_PK], (j / N_PK) & 1);
       }
+      // let the copies this warp started land before the CTA can exit
+      const uint32_t first = it > N_PK ? it - N_PK : 0;
+      for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->pk_full[j % N_PK], (j / N_PK) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      // The four MMAs of a K block take 512 clocks of the tensor pipe; wait, issue and commit have to stay below that,
+      // or this warp paces the kernel. With the loop in a branch of one lane they took 550-600; kept uniform (see
+      // elect_one) about 350: 4096 x 57344 x 8192: 1316 -> 1169 us
+      // (3.29 POPS), 4096 x 10240 x 8192: 230 -> 199, 2044 x 4096 x 14336: 89 -> 80.
       constexpr uint32_t idesc = pq::umma_idesc_s8(2 * BM_CTA, BN);
+      const bool leader = pq::elect_one();
+      const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(s8_buf));
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++tcount) {
-        if (!wait_bar(&bars->acc_empty[0], (tcount & 1) ^ 1, abort_flag, p.wait_clocks)) {  // the epilogue has read the last tile
+        // the epilogue has read the last tile
+        if (!wait_bar_warp(&bars->acc_empty[0], (tcount & 1) ^ 1, abort_flag, p.wait_clocks)) {
           ok = false;
           break;
         }
@@ -211,29 +208,35 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         const uint32_t d_tmem = tmem_base;
         for (int kb = 0; kb < n_kb; ++kb, ++it) {
           const uint32_t s = it % N_S8, ph = (it / N_S8) & 1;
-          if (!wait_bar(&bars->s8_full[s], ph, abort_flag, p.wait_clocks)) {
+          if (!wait_bar_warp(&bars->s8_full[s], ph, abort_flag, p.wait_clocks)) {
             ok = false;
             break;
           }
           pq::tc_fence_after();
-          const uint32_t a_tmem = tmem_base + A_COL0 + s * A_SLOT_COLS;
-          const uint32_t b_addr = pq::smem_u32(s8_buf + s * S8_STAGE);
+          if (leader) {
+            const uint32_t a_tmem = tmem_base + A_COL0 + s * A_SLOT_COLS;
+            const uint64_t b_desc = desc0 + s * (S8_STAGE >> 4);
 #pragma unroll
-          for (int kk = 0; kk < BK / 32; ++kk) {
-            mma2_i8_ts(d_tmem, a_tmem + kk * 8, pq::umma_desc_sw128(b_addr + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u);
+            for (int kk = 0; kk < BK / 32; ++kk)  // 32 bytes of K further along the 128-byte rows
+              mma2_i8_ts(d_tmem, a_tmem + kk * 8, b_desc + kk * 2, idesc, (kb | kk) != 0 ? 1u : 0u);
+            mma2_commit_both(&bars->s8_empty[s]);  // both CTAs may refill the stage once these MMAs have read it
           }
-          mma2_commit_both(&bars->s8_empty[s]);  // both CTAs may refill the stage once these MMAs have read it
+          __syncwarp();
         }
-        if (ok) mma2_commit_both(&bars->acc_full[0]);
+        if (ok && leader) mma2_commit_both(&bars->acc_full[0]);
+        __syncwarp();
       }
-      if (!ok) {
-        bars->abort_flag = 1;
-        pq::report(p.status, PQ_ERR_TIMEOUT);
+      if (leader) {
+        if (!ok) {
+          bars->abort_flag = 1;
+          pq::report(p.status, PQ_ERR_TIMEOUT);
+        }
+        // whatever was issued has finished before either CTA releases its tensor memory
+        mma2_commit_both(&bars->drain);
       }
-      // whatever was issued has finished before either CTA releases its tensor memory
-      mma2_commit_both(&bars->drain);
+      __syncwarp();
     }
-    if (lane == 0) pq::mbar_wait(&bars->drain, 0);
+    pq::mbar_wait(&bars->drain, 0);
   } else if (warp >= UNPACK_WARP0) {
     // ------------------------------------------------------------------ unpack warps
     const int group = (warp - UNPACK_WARP0) / GROUP_WARPS;
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
           ar[8 * j + 4] = pq::nib_hi_x16(w.x), ar[8 * j + 5] = pq::nib_hi_x16(w.y);
           ar[8 * j + 6] = pq::nib_hi_x16(w.z), ar[8 * j + 7] = pq::nib_hi_x16(w.w);
         }
-        tmem_st_32x32(tmem_base + A_COL0 + ss * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), ar);
+        pq::tmem_st_32x32(tmem_base + A_COL0 + ss * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), ar);
       }
       // ---- B: the CTA's 128 weight rows into the swizzled operand stage -------------------------------
       const uint8_t* bsrc = src + BM_CTA * PK_ROW;
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         *reinterpret_cast<uint4*>(drow + (((2 * j) ^ sw) << 4)) = lo;
         *reinterpret_cast<uint4*>(drow + (((2 * j + 1) ^ sw) << 4)) = hi;
       }
-      tmem_st_wait();         // the TMEM lane is written ...
+      pq::tmem_st_wait();         // the TMEM lane is written ...
       pq::tc_fence_before();  // ... and ordered before the arrival below
       pq::fence_proxy_async_smem();  // generic-proxy writes -> visible to the tensor core's async proxy
       __syncwarp();
