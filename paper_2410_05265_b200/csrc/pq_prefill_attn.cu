@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
   uint8_t* land = kv_buf + PA_STAGES * 2 * PA_TILE;     // stage s: packed K rows, then packed V rows
   PaBarriers* bars = reinterpret_cast<PaBarriers*>(land + PA_STAGES * PA_LAND);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = pq::warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y, G = p.G;
   const int R = 256 / G;                                   // query tokens of this CTA
   const int t0 = (static_cast<int>(gridDim.x) - 1 - static_cast<int>(blockIdx.x)) * R;  // long tiles first
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
   pq::tc_fence_before();
   __syncthreads();
   pq::tc_fence_after();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   // Bounded wait; also gives up when another role of the CTA has raised the abort flag.
   auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
       if (clock64() - c0 > p.wait_clocks) return false;
     }
   };
+  auto wait_warp = [&](uint64_t* bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, wait(bar, parity)); };
   auto give_up = [&]() {
     bars->abort_flag = 1;
     pq::report(p.status, PQ_ERR_TIMEOUT);
@@ -482,80 +483,99 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
     if (!ok && lane == 0) give_up();
   } else if (warp == PA_WARP_LOAD) {
     // ================================================================== loader
-    if (lane == 0) {
-      bool ok = true;
-      for (int kt = 0; kt < n_kt; ++kt) {
-        const int slot = kt % PA_STAGES;
-        if (!wait(&bars->land_empty[slot], ((kt / PA_STAGES) & 1) ^ 1)) {
-          ok = false;
-          break;
-        }
+    const bool leader = pq::elect_one();
+    bool ok = true;
+    for (int kt = 0; kt < n_kt; ++kt) {
+      const int slot = kt % PA_STAGES;
+      if (!wait_warp(&bars->land_empty[slot], ((kt / PA_STAGES) & 1) ^ 1)) {
+        ok = false;
+        break;
+      }
+      if (leader) {
         const uint32_t bytes = static_cast<uint32_t>(min(PA_KEYS, n_ctx - kt * PA_KEYS)) * 64u;
         const int64_t off = (static_cast<int64_t>(h) * p.Tmax + static_cast<int64_t>(kt) * PA_KEYS) * 64;
         const uint32_t dst = pq::smem_u32(land + slot * PA_LAND);
         pq::mbar_arrive_expect_tx(&bars->land_full[slot], 2 * bytes);
         bulk_load(dst, p.kq + off, bytes, &bars->land_full[slot]);
         bulk_load(dst + PA_KEYS * 64, p.vq + off, bytes, &bars->land_full[slot]);
-        loads_issued = kt + 1;
       }
-      if (!ok) give_up();
+      __syncwarp();
+      loads_issued = kt + 1;
     }
+    if (!ok && leader) give_up();
   } else {
     // ================================================================== MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t IDESC_S = idesc_f16(PA_ROWS, PA_KEYS, false), IDESC_S_PRE = idesc_f16(PA_ROWS, PA_MAX_PREFIX, false);
-      constexpr uint32_t IDESC_O = idesc_f16(PA_ROWS, 128, true);
-      auto issue_s = [&](int i, int jt) {
-        const bool is_pre = has_prefix && jt == 0;
-        const uint32_t q_addr = pq::smem_u32(q_buf + i * PA_TILE), k_addr = pq::smem_u32(kv_buf + (jt % PA_STAGES) * 2 * PA_TILE);
+    // The whole warp runs the loop and the elected lane issues (see elect_one): a group of eight MMAs took 550-850 clocks to
+    // issue from a branch of one lane, which sat in the chain softmax -> P -> MMA -> S of both query tiles. 4096 tokens x 64
+    // heads: 349 -> 316 us (789 -> 870 TFLOP/s), 2048 x 64: 123 -> 112, 515 x 32: 21.3 -> 19.6.
+    constexpr uint32_t IDESC_S = idesc_f16(PA_ROWS, PA_KEYS, false), IDESC_S_PRE = idesc_f16(PA_ROWS, PA_MAX_PREFIX, false);
+    constexpr uint32_t IDESC_O = idesc_f16(PA_ROWS, 128, true);
+    const bool leader = pq::elect_one();
+    const uint64_t q_desc0 = desc_sw128(pq::smem_u32(q_buf), 16), k_desc0 = desc_sw128(pq::smem_u32(kv_buf), 16);
+    const uint64_t v_desc0 = desc_sw128(pq::smem_u32(kv_buf + PA_TILE), PA_HALF);
+    auto issue_s = [&](int i, int jt) {  // by the elected lane
+      const uint32_t idesc = has_prefix && jt == 0 ? IDESC_S_PRE : IDESC_S;
+      const uint64_t q_desc = q_desc0 + i * (PA_TILE >> 4), k_desc = k_desc0 + (jt % PA_STAGES) * (2 * PA_TILE >> 4);
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {  // 16 head dims per instruction
-          const uint32_t off = (kk >> 2) * PA_HALF + (kk & 3) * 32;
-          mma_f16_ss(tmem_base + i * 128, desc_sw128(q_addr + off, 16), desc_sw128(k_addr + off, 16), is_pre ? IDESC_S_PRE : IDESC_S,
-                     kk ? 1u : 0u);
-        }
-        pq::mma_commit(&bars->s_full[i]);
-      };
-      auto issue_pv = [&](int i, int jt) {
-        const bool is_pre = has_prefix && jt == 0;
-        const uint32_t v_addr = pq::smem_u32(kv_buf + (jt % PA_STAGES) * 2 * PA_TILE + PA_TILE);
-        const int n_steps = is_pre ? PA_MAX_PREFIX / 16 : PA_KEYS / 16;  // 16 keys per instruction
-        for (int kk = 0; kk < n_steps; ++kk)
-          mma_f16_ts(tmem_base + 256 + i * 128, tmem_base + i * 128 + kk * 8, desc_sw128(v_addr + kk * 2048, PA_HALF), IDESC_O,
-                     (jt > 0 || kk > 0) ? 1u : 0u);
-      };
-      bool ok = wait(&bars->q_ready, 0) && wait(&bars->kv_full[0], 0);
-      if (ok) {
-        pq::tc_fence_after();
+      for (int kk = 0; kk < 8; ++kk) {  // 16 head dims per instruction
+        const uint32_t off = ((kk >> 2) * PA_HALF + (kk & 3) * 32) >> 4;
+        mma_f16_ss(tmem_base + i * 128, q_desc + off, k_desc + off, idesc, kk ? 1u : 0u);
+      }
+      pq::mma_commit(&bars->s_full[i]);
+    };
+    auto issue_pv = [&](int i, int jt) {
+      const uint32_t o_tm = tmem_base + 256 + i * 128, p_tm = tmem_base + i * 128;
+      const uint64_t v_desc = v_desc0 + (jt % PA_STAGES) * (2 * PA_TILE >> 4);
+#pragma unroll
+      for (int kk = 0; kk < PA_MAX_PREFIX / 16; ++kk)  // 16 keys per instruction
+        mma_f16_ts(o_tm, p_tm + kk * 8, v_desc + kk * (2048 >> 4), IDESC_O, (jt > 0 || kk > 0) ? 1u : 0u);
+      if (!(has_prefix && jt == 0))
+#pragma unroll
+        for (int kk = PA_MAX_PREFIX / 16; kk < PA_KEYS / 16; ++kk) mma_f16_ts(o_tm, p_tm + kk * 8, v_desc + kk * (2048 >> 4), IDESC_O, 1u);
+    };
+    bool ok = wait_warp(&bars->q_ready, 0) && wait_warp(&bars->kv_full[0], 0);
+    if (ok) {
+      pq::tc_fence_after();
+      if (leader) {
         issue_s(0, 0);
         issue_s(1, 0);
       }
-      for (int jt = 0; jt < n_tiles && ok; ++jt) {
-        for (int i = 0; i < 2 && ok; ++i) {
-          if (!wait(&bars->p_full[i], jt & 1)) {
+      __syncwarp();
+    }
+    for (int jt = 0; jt < n_tiles && ok; ++jt) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (!ok) break;
+        if (!wait_warp(&bars->p_full[i], jt & 1)) {
+          ok = false;
+          break;
+        }
+        pq::tc_fence_after();
+        if (leader) {
+          issue_pv(i, jt);
+          if (i == 1) pq::mma_commit(&bars->kv_empty[jt % PA_STAGES]);  // both tiles' S and P V of this stage are issued
+        }
+        __syncwarp();
+        if (jt + 1 < n_tiles) {
+          if (i == 0 && !wait_warp(&bars->kv_full[(jt + 1) % PA_STAGES], ((jt + 1) / PA_STAGES) & 1)) {
             ok = false;
             break;
           }
           pq::tc_fence_after();
-          issue_pv(i, jt);
-          if (i == 1) pq::mma_commit(&bars->kv_empty[jt % PA_STAGES]);  // both tiles' S and P V of this stage are issued
-          if (jt + 1 < n_tiles) {
-            if (i == 0 && !wait(&bars->kv_full[(jt + 1) % PA_STAGES], ((jt + 1) / PA_STAGES) & 1)) {
-              ok = false;
-              break;
-            }
-            pq::tc_fence_after();
-            issue_s(i, jt + 1);
-          } else {
-            pq::mma_commit(&bars->o_final[i]);
-          }
+          if (leader) issue_s(i, jt + 1);
+        } else if (leader) {
+          pq::mma_commit(&bars->o_final[i]);
         }
+        __syncwarp();
       }
+    }
+    if (leader) {
       if (!ok) give_up();
       // whatever was issued has finished before tensor memory is released or shared memory given back
       pq::mma_commit(&bars->drain);
-      pq::mbar_wait(&bars->drain, 0);
     }
+    __syncwarp();
+    pq::mbar_wait(&bars->drain, 0);
   }
 
   pq::tc_fence_before();
