@@ -122,10 +122,10 @@ pq_status pq_rmsnorm_hadamard_quant_act(pq_ctx* ctx, const void* x, int64_t M, i
  *   out  bf16 [M, N], row stride ldo elements
  *   acc_dbg  nullable int32 [M, N] dense: receives the raw accumulators (parity checks)
  *   K % 32 == 0, K <= 65536. Output rows below row_begin are left untouched.
- * Shapes with M - row_begin > 16 run on the tensor-core kernel (TMA + tcgen05, kind::i8);
- * smaller M runs the weight-streaming kernel. No workspace is needed (ws may be NULL).
- * Weights are static (Sec. 3: quantized offline): the weight-streaming kernel starts fetching wq
- * while the kernel before it in the stream is still draining (programmatic dependent launch), and
+ * Shapes with M - row_begin > 16 run on the tensor-core kernels (TMA + tcgen05, kind::i8);
+ * smaller M mostly runs the weight-streaming kernel. No workspace is needed (ws may be NULL).
+ * Weights are static (Sec. 3: quantized offline): below a few hundred rows the kernels start fetching wq
+ * while the kernel before them in the stream is still draining (programmatic dependent launch), and
  * only xq, the scales and out are ordered behind that kernel. wq (and wsum of the _asym call)
  * must therefore be complete before the kernel that precedes this call in the stream starts.
  * Weights written earlier in the same stream by pq_quant_weights / pq_weight_code_sums or by a copy
@@ -143,8 +143,8 @@ pq_status pq_w4a4_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const 
  *     *s_a = max(*s_a, max |y| / 127)                      calibration helper
  *     acc[t, n] = sum_k xq8[t, k] * wq[n, k]   exact, int32;   out[t, n] = bf16(acc * s_a * s_w[n])
  *   xq8  s8 [M, K] dense rows, base 16-byte aligned; every other argument as in the 4-bit calls.
- * Above 16 tokens the GEMM runs on the tensor-core kernel (the token bytes go to the MMA operand
- * buffer untouched, only the weights are expanded), else on the weight-streaming kernel;
+ * Above 16 tokens the GEMM runs on the tensor-core kernels (the token bytes go to the MMA operand
+ * buffer untouched, only the weights are expanded), below mostly on the weight-streaming kernel;
  * K % 32 == 0, K <= 65536. */
 pq_status pq_hadamard_quant_act8(pq_ctx* ctx, const void* x, int64_t M, int64_t K, int64_t ldx, int had_block,
                                  int64_t row_begin, const float* s_a, int8_t* xq8, void* stream);

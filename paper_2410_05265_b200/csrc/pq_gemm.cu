@@ -13,6 +13,43 @@ pq_status pq_gemm_stream_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* w
                                 int32_t* acc_dbg, cudaStream_t st, bool per_token, bool a8, const int32_t* zp,
                                 const int32_t* wsum);
 
+pq_status pq_gemm_split_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w, void* out,
+                               int64_t ldo, int64_t M, int64_t N, int64_t K, int32_t* acc_dbg, cudaStream_t st, bool a8,
+                               const float* s_row, const int32_t* zp, const int32_t* wsum);
+
+// Chooses the kernel for m rows (row_begin already applied). s_row: per-token steps instead of s_a; zp, wsum: Eq. 1's
+// zero point and the weight code sums; a8: one s8 code per activation.
+static pq_status run_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w, void* out, int64_t ldo,
+                          int64_t m, int64_t N, int64_t K, int32_t* dbg, void* stream, bool a8, const float* s_row, const int32_t* zp,
+                          const int32_t* wsum) {
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // Weight-streaming kernel or split-K tensor-core kernel (figures: rotate+quantize and GEMM in a graph, us, streaming against
+  // split). The streaming kernel has the shorter chain, but expands the tokens again for every 16 channels and has no K split:
+  //   up to 8 tokens   it keeps the short layers (1 token, 6144 x 4096: 5.4 / 7.1) and the wide ones (57344 x 8192: 44.4 / 51.2);
+  //                    large layers with long rows and few enough channel tiles for three or more K splits go to the other
+  //                    (8192 x 28672: 29.2 / 24.4, 8192 x 8192: 11.4 / 10.4, 10240 x 8192: 12.2 / 12.1; not 4096 x 14336:
+  //                    9.9 / 9.7 here, but 1.5 us slower inside a decode layer)
+  //   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
+  //                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
+  //   up to 128        always split (the CTA-pair kernels: 33 tokens, 4096 x 4096: 23.1 / 8.5, 28672 x 4096: 40.8 / 18.2)
+  //   above            while the 256-token tiles leave room for two K splits: whole 8B block at 200 tokens 176.5 / 132.1, at 300
+  //                    tokens 201 / 175; with a single split (515 tokens) the o layer gains 2.3 and the down layer loses 8.6.
+  const int64_t ctiles = (N + 127) / 128, weights = N * K;
+  const bool split = m <= 8     ? K >= 8192 && weights >= (int64_t{1} << 26) && 3 * ctiles <= ctx->sm_count * 7 / 4
+                     : m <= 16  ? weights >= (int64_t{20} << 20)
+                     : m <= 128 ? true
+                                : 2 * ((m + 255) / 256) * ctiles <= ctx->sm_count * 7 / 8;
+  if (split) return pq_gemm_split_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, a8, s_row, zp, wsum);
+  if (m <= 16)
+    return pq_gemm_stream_launch(ctx, xq, wq, s_row ? s_row : s_a, s_w, out, ldo, m, N, K, dbg, st, s_row != nullptr, a8, zp, wsum);
+  // Two CTA-pair kernels (every 4-bit setting takes the same choice): with the token operand in shared memory the accumulator is
+  // double-buffered and the epilogue is free, which wins for short K; with the token operand in tensor memory the expansion costs
+  // a third less shared-memory traffic, which wins once a tile's K loop is long enough to hide the single accumulator's epilogue
+  // (measured crossover near K = 8192).
+  if (!a8 && K >= 8192) return pq_gemm_pair_ts_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, s_row, zp, wsum);
+  return pq_gemm_pair_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, a8, s_row, zp, wsum);
+}
+
 extern "C" size_t pq_w4a4_gemm_workspace_bytes(int64_t, int64_t, int64_t) { return 0; }
 
 extern "C" pq_status pq_w4a4_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a,
@@ -31,15 +68,8 @@ extern "C" pq_status pq_w4a4_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t*
   const uint8_t* xq0 = xq + row_begin * (K / 2);
   void* out0 = static_cast<__nv_bfloat16*>(out) + row_begin * ldo;
   int32_t* dbg0 = acc_dbg ? acc_dbg + row_begin * N : nullptr;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (K == 0) return PQ_ERR_SHAPE;
-  if (m <= 16) return pq_gemm_stream_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, false, false, nullptr, nullptr);
-  // Two CTA-pair kernels (every 4-bit setting takes the same choice): with the token operand in shared memory the accumulator is double-buffered
-  // and the epilogue is free, which wins for short K; with the token operand in tensor memory the
-  // expansion costs a third less shared-memory traffic, which wins once a tile's K loop is long enough
-  // to hide the single accumulator's epilogue (measured crossover near K = 8192).
-  if (K >= 8192) return pq_gemm_pair_ts_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, nullptr, nullptr, nullptr);
-  return pq_gemm_pair_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, false, nullptr, nullptr, nullptr);
+  return run_gemm(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, stream, false, nullptr, nullptr, nullptr);
 }
 
 // W4A8 (Sec. 5.1): the token operand is one s8 code per element: the weight-streaming kernel for up to 16
@@ -59,9 +89,7 @@ extern "C" pq_status pq_w4a8_gemm(pq_ctx* ctx, const int8_t* xq8, const uint8_t*
   const uint8_t* xq0 = reinterpret_cast<const uint8_t*>(xq8) + row_begin * K;
   void* out0 = static_cast<__nv_bfloat16*>(out) + row_begin * ldo;
   int32_t* dbg0 = acc_dbg ? acc_dbg + row_begin * N : nullptr;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (m <= 16) return pq_gemm_stream_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, false, true, nullptr, nullptr);
-  return pq_gemm_pair_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, true, nullptr, nullptr, nullptr);
+  return run_gemm(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, stream, true, nullptr, nullptr, nullptr);
 }
 
 // W4A4 with per-token dynamic activation steps (Table 1, O1): out[t,n] = bf16(acc * s_tok[t] * s_w[n]).
@@ -80,10 +108,7 @@ extern "C" pq_status pq_w4a4_gemm_rows(pq_ctx* ctx, const uint8_t* xq, const uin
   const float* s0 = s_tok + row_begin;
   void* out0 = static_cast<__nv_bfloat16*>(out) + row_begin * ldo;
   int32_t* dbg0 = acc_dbg ? acc_dbg + row_begin * N : nullptr;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (m <= 16) return pq_gemm_stream_launch(ctx, xq0, wq, s0, s_w, out0, ldo, m, N, K, dbg0, st, true, false, nullptr, nullptr);
-  if (K >= 8192) return pq_gemm_pair_ts_launch(ctx, xq0, wq, nullptr, s_w, out0, ldo, m, N, K, dbg0, st, s0, nullptr, nullptr);
-  return pq_gemm_pair_launch(ctx, xq0, wq, nullptr, s_w, out0, ldo, m, N, K, dbg0, st, false, s0, nullptr, nullptr);
+  return run_gemm(ctx, xq0, wq, nullptr, s_w, out0, ldo, m, N, K, dbg0, stream, false, s0, nullptr, nullptr);
 }
 
 // W4A4 with the activation quantizer of Eq. 1 as printed (zero point z): the stored token codes are u - 8,
@@ -103,8 +128,5 @@ extern "C" pq_status pq_w4a4_gemm_asym(pq_ctx* ctx, const uint8_t* xq, const uin
   const uint8_t* xq0 = xq + row_begin * (K / 2);
   void* out0 = static_cast<__nv_bfloat16*>(out) + row_begin * ldo;
   int32_t* dbg0 = acc_dbg ? acc_dbg + row_begin * N : nullptr;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (m <= 16) return pq_gemm_stream_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, false, false, z_a, wsum);
-  if (K >= 8192) return pq_gemm_pair_ts_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, nullptr, z_a, wsum);
-  return pq_gemm_pair_launch(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, st, false, nullptr, z_a, wsum);
+  return run_gemm(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, stream, false, nullptr, z_a, wsum);
 }

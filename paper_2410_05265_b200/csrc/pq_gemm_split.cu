@@ -1,0 +1,527 @@
+// W4A4 / W4A8 GEMM for a few tens to a few hundred tokens (batched decode, short prompts):
+//
+//   acc[t,n] = sum_k xq[t,k] * wq[n,k]   (exact int32),   out = bf16(acc * s_a * s_w[n])
+//
+// At these sizes the packed weights are what has to move, and the 256 x 256 tiles of the CTA-pair kernels leave most
+// of the chip idle (16 tiles for a 4096 x 4096 layer). Here the MMA is turned round: 128 output channels are its row
+// side, NT = 16 .. 256 tokens its column side, so a token tile costs what its tokens cost, and the K blocks of a
+// channel tile are split over the CTAs of a cluster (up to 8), whose int32 partial tiles meet in distributed shared
+// memory: exact, no workspace, nothing waits on another cluster.
+//
+// Roles inside a CTA:
+//   warp 0      TMA producer, packed weights: [128 x 64 B] (64-byte swizzle) of a 128-wide K block into a landing ring.
+//               Weights are static: the ring's first copies start before the wait for the previous kernel in the stream.
+//   warp 1      MMA issuer and owner of the tensor memory.
+//   warp 2      TMA producer, tokens: packed rows [NT x 64 B] into a landing ring of their own, or (A8) the s8 bytes
+//               straight into the operand slot (128-byte-swizzled box).
+//   warps 4..   expansion, GROUPS groups of four warps (one per TMEM lane quarter): a thread owns one channel row, reads
+//               its 64 packed bytes, and writes 128 s8 bytes (16 * code) to its lane of an A slot in tensor memory; the
+//               group's threads also expand the token rows into the B slot in shared memory. Even-position codes come
+//               first, then odd-position codes, in both operands (natural order in both with A8).
+// Then every warp takes part in the reduction: a lane owns four channels, a warp one or more tokens at a time, the partial
+// sums of the cluster's CTAs are added, scaled and stored as 256 contiguous bytes per token.
+//
+// What bounds it: up to ~64 tokens the weight stream and the fixed chain launch -> tokens -> expand -> MMA -> two cluster
+// barriers (about 5 us, most of it overlapped with the neighbours under programmatic dependent launch); at 128 and 256 tokens
+// the expansion of the token rows, which every channel tile repeats. Measured (us, calls in a graph over weight copies larger
+// than L2; before: the CTA-pair kernels, for 16 tokens the streaming kernel), layers of the 8B set q|k|v, o, gate|up, down:
+//   M = 16   6.1  3.7 18.2  8.9  ->  6.5  5.6 14.0  9.1 (gate|up at 4.2 TB/s)
+//   M = 32  20.7 20.3 36.0 46.7  ->  7.0  6.1 14.4  9.6
+//   M = 96  20.9 20.5 37.2 46.9  ->  10.1  9.2 20.3 14.6   (W4A8: 18.6 18.4 31.9 46.6 -> 9.5 8.7 17.8 13.5)
+//   M = 256 21.1 20.7   --  47.1  ->  13.2 12.5   --  19.7
+// (In a chain with the rotation kernels the short layers overlap less; the dispatch in pq_gemm.cu was set on such chains.)
+// Tried: the token rows read from L2 into registers instead of a landing ring (gate|up, M = 32: 16.2 us against 14.3); token
+// rows expanded by warps of their own (18.1); three or four expansion groups per CTA (14.9-15.2); a weight stage handed back
+// right after it was read into registers, which pays only where the token part is long (M = 256, gate|up: 46.5 -> 36.4).
+//
+// Every mbarrier wait is bounded; when one runs out the CTA raises an abort flag, its roles drain, and PQ_ERR_TIMEOUT
+// is reported.
+#include "pq_gemm_pair.cuh"
+
+namespace {
+
+using namespace pq_pair;
+
+constexpr int CH = 128;                    // output channels per CTA
+constexpr int W_STAGE = CH * PK_ROW;       // 8 KB of packed weights per K block
+constexpr int A_SLOT_COLS = BK / 4;        // 32 TMEM columns = 128 K bytes per lane
+constexpr int EXPAND_WARP0 = 4;
+constexpr int MAX_SPLIT = 8;               // portable cluster size
+
+// Shapes of the rings. Up to 128 tokens two CTAs share an SM (113 KB and 256 TMEM columns each), so that one loads
+// while the other expands or reduces; 256 tokens take a whole SM.
+template <int NT, bool A8>
+struct Cfg {
+  static constexpr int GROUPS = NT == 256 ? 4 : 2;
+  static constexpr int SLOTS = NT == 48 || NT == 64 || ((NT == 96 || NT == 128) && !A8) ? 2 : 4;
+  static constexpr int STAGES = NT <= 64 ? 8 : 4;    // landing ring, weights
+  static constexpr int X_STAGES = NT <= 32 ? 8 : 4;  // landing ring, tokens
+  static constexpr bool EARLY_W = NT == 256;         // weight stages go back before the (long) token part of the expansion
+  static constexpr int X_STAGE = A8 ? 0 : NT * PK_ROW;
+  static constexpr int SLOT = NT * BK;
+  static constexpr int A_COL0 = NT < 32 ? 32 : NT;  // accumulator columns, then the A slots
+  static constexpr int TMEM_COLS = NT == 256 ? 512 : 256;
+  static constexpr int THREADS = (EXPAND_WARP0 + 4 * GROUPS) * 32;
+  static constexpr int CTAS_PER_SM = NT == 256 ? 1 : 2;
+  static constexpr int RING = SLOTS * SLOT + STAGES * W_STAGE + X_STAGES * X_STAGE;
+  static constexpr int PART = NT * CH * 4;  // the int32 partial tile, laid over the rings at the end
+  static_assert(A_COL0 + SLOTS * A_SLOT_COLS <= TMEM_COLS, "tensor memory budget");
+  static_assert(STAGES % GROUPS == 0 && X_STAGES % GROUPS == 0 && SLOTS % GROUPS == 0, "a ring slot is always served by the same group");
+  static_assert(PART <= RING, "the partial tile fits where the rings were");
+};
+
+struct __align__(8) SplitBarriers {
+  uint64_t w_full[8], w_empty[8];             // landing ring of packed weights
+  uint64_t xp_full[8], xp_empty[8];             // landing ring of packed tokens
+  uint64_t s8_full[4], s8_empty[4], x_full[4];  // operand slots
+  uint64_t acc_full;
+  uint32_t tmem_base;
+  volatile int abort_flag;
+};
+
+// At least 80 KB, so that no more CTAs share an SM than its tensor memory serves: a CTA that waited for columns which
+// another cluster's CTA gives back only behind its cluster barrier could wait for itself.
+template <int NT, bool A8>
+constexpr size_t split_smem() {
+  const size_t need = 1024 /*alignment slack*/ + Cfg<NT, A8>::RING + sizeof(SplitBarriers);
+  return need < 80 * 1024 ? 80 * 1024 : need;
+}
+
+struct SplitParams {
+  const int32_t* zp;
+  const int32_t* wsum;
+  const float* s_row;  // per-token steps or null
+  const float* s_a;
+  const float* s_w;
+  __nv_bfloat16* out;
+  int32_t* acc_dbg;
+  int32_t* status;
+  int64_t ldo;
+  int M, N, n_kb;
+  int t_tiles, splits;
+  int vec_out;  // rows of out take 8-byte stores
+  long long wait_clocks;
+};
+
+// D[tmem] (+)= A[tmem] * B[smem], s8 x s8 -> s32, one thread.
+__device__ __forceinline__ void mma_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n"
+      "}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// 32 lanes x 16 consecutive 32-bit columns.
+__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ int4 ld_cluster_int4(uint32_t addr) {
+  int4 v;
+  asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+// Adds the partial tiles of the cluster's CTAs (at most PEERS), scales and stores: a warp takes tokens first, first + step,
+// ..., U of them at a time so that their shared-memory loads are in flight together; a lane owns four channels.
+template <int PEERS, int U, bool ZP>
+__device__ __forceinline__ void reduce_tile(const SplitParams& p, const uint8_t* part, int t0, int n0, int tokens, int first, int step,
+                                            int lane) {
+  const int n = n0 + 4 * lane;
+  float sw[4];
+  int zw[4];
+  const float s_a = p.s_row ? 1.0f : __ldg(p.s_a);
+  const int zp8 = ZP ? __ldg(p.zp) - 8 : 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    sw[i] = n + i < p.N ? s_a * __ldg(p.s_w + n + i) : 0.0f;
+    zw[i] = ZP && n + i < p.N ? zp8 * __ldg(p.wsum + n + i) : 0;
+  }
+  uint32_t peer[PEERS];
+#pragma unroll
+  for (int r = 0; r < PEERS; ++r) peer[r] = map_to_cta(part, r < p.splits ? r : 0) + lane * 16;
+  for (int tb = first; tb < tokens; tb += U * step) {
+    int4 v[U][PEERS];
+    float rs[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = tb + u * step < tokens ? tb + u * step : tb;
+#pragma unroll
+      for (int r = 0; r < PEERS; ++r) {
+        if (PEERS == 1) v[u][r] = *reinterpret_cast<const int4*>(part + t * (CH * 4) + lane * 16);
+        else v[u][r] = r < p.splits ? ld_cluster_int4(peer[r] + t * (CH * 4)) : make_int4(0, 0, 0, 0);
+      }
+      rs[u] = p.s_row ? __ldg(p.s_row + t0 + t) : 1.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = tb + u * step;
+      if (t >= tokens) break;
+      int sum[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int r = 0; r < PEERS; ++r) sum[0] += v[u][r].x, sum[1] += v[u][r].y, sum[2] += v[u][r].z, sum[3] += v[u][r].w;
+      float f[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (ZP) sum[i] -= zw[i];
+        f[i] = static_cast<float>(sum[i]) * sw[i] * rs[u];
+      }
+      __nv_bfloat16* dst = p.out + static_cast<int64_t>(t0 + t) * p.ldo + n;
+      if (p.vec_out && n + 3 < p.N) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(f[0], f[1]), hi = __floats2bfloat162_rn(f[2], f[3]);
+        *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (n + i < p.N) dst[i] = __float2bfloat16_rn(f[i]);
+      }
+      if (p.acc_dbg) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (n + i < p.N) p.acc_dbg[static_cast<int64_t>(t0 + t) * p.N + n + i] = sum[i];
+      }
+    }
+  }
+}
+
+template <int NT, bool A8, bool ZP>
+__global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM)
+    gemm_w4_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const SplitParams p) {
+  using C = Cfg<NT, A8>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* slot_buf = smem;                                // SLOTS token operands [NT x 128 B], 128-byte swizzle
+  uint8_t* stage_buf = slot_buf + C::SLOTS * C::SLOT;      // STAGES landing buffers of packed weights
+  uint8_t* x_buf = stage_buf + C::STAGES * W_STAGE;        // X_STAGES landing buffers of packed tokens
+  SplitBarriers* bars = reinterpret_cast<SplitBarriers*>(smem + C::RING);
+  volatile int* abort_flag = &bars->abort_flag;
+  const int warp = pq::warp_index(), lane = threadIdx.x & 31;
+  const int rank = __shfl_sync(0xffffffffu, static_cast<int>(cluster_ctarank()), 0);
+  const int tile = static_cast<int>(blockIdx.x) / p.splits;
+  const int t0 = (tile % p.t_tiles) * NT;  // the token tiles of a channel tile are neighbours: its weights are in L2
+  const int n0 = (tile / p.t_tiles) * CH;
+  const int kb0 = static_cast<int>(static_cast<int64_t>(p.n_kb) * rank / p.splits);
+  const int total = static_cast<int>(static_cast<int64_t>(p.n_kb) * (rank + 1) / p.splits) - kb0;  // K blocks of this CTA
+
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const bool leader = pq::elect_one();  // the lane that issues copies and MMAs (each role's loop is warp-uniform)
+  const int first = total < C::STAGES ? total : C::STAGES;
+  if (warp == 0) {
+    if (leader) {
+      pq::tma_prefetch_desc(&tmap_w);
+      pq::tma_prefetch_desc(&tmap_x);
+      for (int i = 0; i < C::STAGES; ++i) {
+        pq::mbar_init(&bars->w_full[i], 1);
+        pq::mbar_init(&bars->w_empty[i], 4);
+      }
+      for (int i = 0; i < C::X_STAGES; ++i) {
+        pq::mbar_init(&bars->xp_full[i], 1);
+        pq::mbar_init(&bars->xp_empty[i], 4);
+      }
+      for (int i = 0; i < C::SLOTS; ++i) {
+        pq::mbar_init(&bars->s8_full[i], 4);
+        pq::mbar_init(&bars->s8_empty[i], 1);
+        pq::mbar_init(&bars->x_full[i], 1);
+      }
+      pq::mbar_init(&bars->acc_full, 1);
+      bars->abort_flag = 0;
+      pq::mbar_fence_init();
+      pq::fence_proxy_async_smem();
+    }
+    __syncwarp();
+    for (int i = 0; i < first; ++i) {  // the first weight copies do not depend on the previous kernel
+      if (leader) {
+        pq::mbar_arrive_expect_tx(&bars->w_full[i], W_STAGE);
+        pq::tma_load_2d(stage_buf + i * W_STAGE, &tmap_w, (kb0 + i) * PK_ROW, n0, &bars->w_full[i]);
+      }
+      __syncwarp();
+    }
+  } else if (warp == 1) {
+    // Ahead of the wait for the previous kernel: every kernel of the library that allocates tensor memory takes so much
+    // shared memory that two of them share an SM only where both find their columns, so nothing waits here for long.
+    pq::tmem_alloc(&bars->tmem_base, C::TMEM_COLS);
+    pq::tmem_relinquish();
+  }
+  pq::tc_fence_before();
+  __syncthreads();
+  pq::tc_fence_after();
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  int loads_issued = 0;  // producer warps: copies started
+  bool ok = true;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ TMA producer
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // room comes back once the tokens are there: the bounded waits start behind them
+    int it = first;
+    for (; it < total; ++it) {
+      const int s = it % C::STAGES;
+      if (!wait_bar_warp(&bars->w_empty[s], ((it / C::STAGES) & 1) ^ 1, abort_flag, p.wait_clocks)) {
+        ok = false;
+        break;
+      }
+      if (leader) {
+        pq::mbar_arrive_expect_tx(&bars->w_full[s], W_STAGE);
+        pq::tma_load_2d(stage_buf + s * W_STAGE, &tmap_w, (kb0 + it) * PK_ROW, n0, &bars->w_full[s]);
+      }
+      __syncwarp();
+    }
+    loads_issued = it;
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // what it waits for needs the tokens
+    constexpr uint32_t idesc = pq::umma_idesc_s8(CH, NT);
+    const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(slot_buf));
+    for (int it = 0; it < total; ++it) {
+      const int s = it % C::SLOTS, ph = (it / C::SLOTS) & 1;
+      if (!wait_bar_warp(&bars->s8_full[s], ph, abort_flag, p.wait_clocks) ||
+          (A8 && !wait_bar_warp(&bars->x_full[s], ph, abort_flag, p.wait_clocks))) {
+        ok = false;
+        break;
+      }
+      pq::tc_fence_after();
+      if (leader) {
+        const uint64_t b_desc = desc0 + s * (C::SLOT >> 4);
+        const uint32_t a_tmem = tmem_base + C::A_COL0 + s * A_SLOT_COLS;
+#pragma unroll
+        for (int kk = 0; kk < BK / 32; ++kk) mma_i8_ts(tmem_base, a_tmem + kk * 8, b_desc + kk * 2, idesc, (it | kk) != 0 ? 1u : 0u);
+        pq::mma_commit(&bars->s8_empty[s]);
+      }
+      __syncwarp();
+    }
+    if (leader) pq::mma_commit(&bars->acc_full);
+    __syncwarp();
+    pq::mbar_wait(&bars->acc_full, 0);  // in every case: tensor memory is released behind the MMAs issued
+  } else if (warp == 2) {
+    // ------------------------------------------------------------------ TMA producer, tokens (A8: into the operand slots)
+    constexpr int RING = A8 ? C::SLOTS : C::X_STAGES, BYTES = A8 ? C::SLOT : C::X_STAGE;
+    uint64_t* full = A8 ? bars->x_full : bars->xp_full;
+    uint64_t* empty = A8 ? bars->s8_empty : bars->xp_empty;
+    uint8_t* buf = A8 ? slot_buf : x_buf;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the tokens may come from the previous kernel
+    int it = 0;
+    for (; it < total; ++it) {
+      const int s = it % RING;
+      if (!wait_bar_warp(&empty[s], ((it / RING) & 1) ^ 1, abort_flag, p.wait_clocks)) {
+        ok = false;
+        break;
+      }
+      if (leader) {
+        pq::mbar_arrive_expect_tx(&full[s], BYTES);
+        pq::tma_load_2d(buf + s * BYTES, &tmap_x, (kb0 + it) * (A8 ? BK : PK_ROW), t0, &full[s]);
+      }
+      __syncwarp();
+    }
+    loads_issued = it;
+  } else if (warp >= EXPAND_WARP0) {
+    // ------------------------------------------------------------------ expansion
+    const int group = (warp - EXPAND_WARP0) >> 2, q = warp & 3;
+    const int gt = q * 32 + lane;  // thread of the group = channel row of the tile = lane of tensor memory
+    for (int it = group; it < total; it += C::GROUPS) {
+      const int ps = it % C::STAGES, xs = it % C::X_STAGES, ss = it % C::SLOTS;
+      if (!wait_bar_warp(&bars->w_full[ps], (it / C::STAGES) & 1, abort_flag, p.wait_clocks)) {
+        ok = false;
+        break;
+      }
+      const uint8_t* src = stage_buf + ps * W_STAGE;
+      uint4 w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)  // 64-byte swizzle of the landing buffer: the row-per-thread reads hit distinct banks
+        w[j] = *reinterpret_cast<const uint4*>(src + gt * PK_ROW + ((j ^ ((gt >> 1) & 3)) << 4));
+      if (it >= C::SLOTS && it < C::SLOTS + C::GROUPS)
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // slots come back once the tokens are there: the bounded wait starts behind them
+      if (!wait_bar_warp(&bars->s8_empty[ss], ((it / C::SLOTS) & 1) ^ 1, abort_flag, p.wait_clocks)) {
+        ok = false;
+        break;
+      }
+      uint32_t a[32];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t in[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t lo = pq::nib_lo_x16(in[i]), hi = pq::nib_hi_x16(in[i]);
+          if (A8) {
+            a[8 * j + 2 * i] = __byte_perm(lo, hi, 0x5140), a[8 * j + 2 * i + 1] = __byte_perm(lo, hi, 0x7362);
+          } else {
+            a[8 * j + i] = lo, a[8 * j + 4 + i] = hi;
+          }
+        }
+      }
+      pq::tmem_st_32x32(tmem_base + C::A_COL0 + ss * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), a);
+      if (C::EARLY_W) {  // behind the store above, for which what was read has arrived in registers
+        __syncwarp();
+        if (lane == 0) pq::mbar_arrive(&bars->w_empty[ps]);
+      }
+      if (!A8) {
+        if (it == group) asm volatile("griddepcontrol.wait;" ::: "memory");  // the tokens' bounded wait starts behind their producer
+        if (!wait_bar_warp(&bars->xp_full[xs], (it / C::X_STAGES) & 1, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
+        }
+        const uint8_t* xsrc = x_buf + xs * C::X_STAGE;
+        uint8_t* dst = slot_buf + ss * C::SLOT;
+        constexpr int UNITS = NT * 4;  // one unit = one 16-byte packed chunk of a token row
+#pragma unroll
+        for (int i = 0; i < (UNITS + 127) / 128; ++i) {
+          const int unit = i * 128 + gt;
+          if (UNITS % 128 != 0 && unit >= UNITS) break;
+          const int row = unit >> 2, j = unit & 3, sw = row & 7;
+          const uint4 v = *reinterpret_cast<const uint4*>(xsrc + unit * 16);
+          uint8_t* drow = dst + row * BK;
+          *reinterpret_cast<uint4*>(drow + (((2 * j) ^ sw) << 4)) =
+              make_uint4(pq::nib_lo_x16(v.x), pq::nib_lo_x16(v.y), pq::nib_lo_x16(v.z), pq::nib_lo_x16(v.w));
+          *reinterpret_cast<uint4*>(drow + (((2 * j + 1) ^ sw) << 4)) =
+              make_uint4(pq::nib_hi_x16(v.x), pq::nib_hi_x16(v.y), pq::nib_hi_x16(v.z), pq::nib_hi_x16(v.w));
+        }
+        pq::fence_proxy_async_smem();  // generic-proxy writes -> visible to the tensor core
+      }
+      pq::tmem_st_wait();
+      pq::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        pq::mbar_arrive(&bars->s8_full[ss]);
+        if (!C::EARLY_W) pq::mbar_arrive(&bars->w_empty[ps]);
+        if (!A8) pq::mbar_arrive(&bars->xp_empty[xs]);
+      }
+    }
+    // ------------------------------------------------------------------ accumulator -> the partial tile [token][channel]
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ok = ok && wait_bar_warp(&bars->acc_full, 0, abort_flag, p.wait_clocks);
+    if (ok) {
+      constexpr int SHIFT = A8 ? 4 : 8;  // the factors 16 the expanded codes carry
+      int* part = reinterpret_cast<int*>(smem);
+      pq::tc_fence_after();
+      for (int c = group; c < NT / 16; c += C::GROUPS) {
+        uint32_t r[16];
+        tmem_ld_32x16(tmem_base + c * 16 + (static_cast<uint32_t>(q * 32) << 16), r);
+        pq::tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) part[(c * 16 + i) * CH + gt] = static_cast<int>(r[i]) >> SHIFT;
+      }
+      pq::tc_fence_before();
+    }
+  }
+  if (!ok && lane == 0) {
+    bars->abort_flag = 1;
+    pq::report(p.status, PQ_ERR_TIMEOUT);
+  }
+  __syncthreads();
+  if (bars->abort_flag) {  // copies that nobody consumed must have landed before the CTA goes on (they only wait for memory)
+    if (warp == 0)
+      for (int j = loads_issued > C::STAGES ? loads_issued - C::STAGES : 0; j < loads_issued; ++j)
+        pq::mbar_wait(&bars->w_full[j % C::STAGES], (j / C::STAGES) & 1);
+    if (warp == 2) {
+      constexpr int RING = A8 ? C::SLOTS : C::X_STAGES;
+      for (int j = loads_issued > RING ? loads_issued - RING : 0; j < loads_issued; ++j)
+        pq::mbar_wait(A8 ? &bars->x_full[j % RING] : &bars->xp_full[j % RING], (j / RING) & 1);
+    }
+    __syncthreads();
+  }
+  cluster_sync_all();  // every CTA's partial tile is in place
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (long past) the scales and the output may belong to the previous kernel
+  if (warp == 1) {
+    pq::tc_fence_after();
+    pq::tmem_dealloc(tmem_base, C::TMEM_COLS);
+  }
+  const int tokens = p.M - t0 < NT ? p.M - t0 : NT;
+  if (p.splits == 1) reduce_tile<1, 4, ZP>(p, smem, t0, n0, tokens, warp, C::THREADS / 32, lane);
+  else if (p.splits <= 4) reduce_tile<4, 2, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane);
+  else reduce_tile<MAX_SPLIT, 1, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane);
+  // no CTA leaves while a peer may still read its partial tile; relaxed: the reads are done, and the output stores need not
+  // have reached memory
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
+template <int NT, bool A8, bool ZP>
+pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw, SplitParams& p, cudaStream_t st) {
+  using C = Cfg<NT, A8>;
+  static bool attr_set[64] = {};  // the attribute belongs to the device's copy of the kernel: once per device
+  if (ctx->device < 0 || ctx->device >= 64) return PQ_ERR_UNSUPPORTED;
+  if (!attr_set[ctx->device]) {
+    if (cudaFuncSetAttribute(gemm_w4_split_kernel<NT, A8, ZP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(split_smem<NT, A8>())) != cudaSuccess)
+      return PQ_ERR_CUDA;
+    attr_set[ctx->device] = true;
+  }
+  p.t_tiles = (p.M + NT - 1) / NT;
+  const int tiles = p.t_tiles * ((p.N + CH - 1) / CH);
+  // As many K splits as leave every CTA resident at once with room for the clusters to be placed (7/8 of the slots: 48 tiles
+  // x 6 = 288 CTAs ran in two waves, 10.7 us against 7.0 with 96), and at least five K blocks per CTA (below that the two
+  // cluster barriers cost more than the shorter loop saves: 4096 x 4096 at 32 tokens 6.1 us with six splits, 6.6 with eight).
+  const int resident = ctx->sm_count * C::CTAS_PER_SM * 7 / 8;
+  int splits = resident / tiles;
+  if (splits > MAX_SPLIT) splits = MAX_SPLIT;
+  if (splits > p.n_kb / 5) splits = p.n_kb / 5;
+  if (splits < 1) splits = 1;
+  p.splits = splits;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles) * splits);
+  cfg.blockDim = dim3(C::THREADS);
+  cfg.dynamicSmemBytes = split_smem<NT, A8>();
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = splits;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, gemm_w4_split_kernel<NT, A8, ZP>, tx, tw, p) != cudaSuccess) return PQ_ERR_CUDA;
+  return pq_launch_status();
+}
+
+template <bool A8, bool ZP>
+pq_status launch_tokens(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, SplitParams& p, int64_t K, cudaStream_t st) {
+  const int nt = p.M <= 16 ? 16 : (p.M <= 32 ? 32 : (p.M <= 48 ? 48 : (p.M <= 64 ? 64 : (p.M <= 96 ? 96 : (p.M <= 128 ? 128 : 256)))));
+  CUtensorMap tx, tw;
+  if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, nt) : make_packed_map(ctx, &tx, xq, p.M, K / 2, nt)) ||
+      !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH, CU_TENSOR_MAP_SWIZZLE_64B))
+    return PQ_ERR_CUDA;
+  switch (nt) {
+    case 16: return launch_split<16, A8, ZP>(ctx, tx, tw, p, st);
+    case 32: return launch_split<32, A8, ZP>(ctx, tx, tw, p, st);
+    case 48: return launch_split<48, A8, ZP>(ctx, tx, tw, p, st);
+    case 64: return launch_split<64, A8, ZP>(ctx, tx, tw, p, st);
+    case 96: return launch_split<96, A8, ZP>(ctx, tx, tw, p, st);
+    case 128: return launch_split<128, A8, ZP>(ctx, tx, tw, p, st);
+    default: return launch_split<256, A8, ZP>(ctx, tx, tw, p, st);
+  }
+}
+
+}  // namespace
+
+// Rows [0, M) of xq/out (the caller has already applied row_begin). s_row: per-token steps (then s_a is ignored), or
+// null. zp, wsum: the zero point of Eq. 1 and the weight code sums, or null.
+pq_status pq_gemm_split_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w, void* out,
+                               int64_t ldo, int64_t M, int64_t N, int64_t K, int32_t* acc_dbg, cudaStream_t st, bool a8,
+                               const float* s_row, const int32_t* zp, const int32_t* wsum) {
+  if (zp && !wsum) return PQ_ERR_INVALID_ARG;
+  SplitParams p;
+  p.zp = zp;
+  p.wsum = wsum;
+  p.s_row = s_row;
+  p.s_a = s_a;
+  p.s_w = s_w;
+  p.out = static_cast<__nv_bfloat16*>(out);
+  p.acc_dbg = acc_dbg;
+  p.status = ctx->d_status;
+  p.ldo = ldo;
+  p.M = static_cast<int>(M);
+  p.N = static_cast<int>(N);
+  p.n_kb = static_cast<int>((K + BK - 1) / BK);
+  p.vec_out = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0;
+  p.wait_clocks = ctx->wait_clocks;
+  if (a8) return launch_tokens<true, false>(ctx, xq, wq, p, K, st);
+  return zp ? launch_tokens<false, true>(ctx, xq, wq, p, K, st) : launch_tokens<false, false>(ctx, xq, wq, p, K, st);
+}

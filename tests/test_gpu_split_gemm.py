@@ -1,0 +1,87 @@
+"""GPU parity of the split-K tensor-core GEMM (a few tens to a few hundred tokens) against the CPU oracle: every token-tile
+width and its edges, ragged channel counts and K tails, the four settings of the call, and the border to the CTA-pair kernels."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import pq_oracle as orc
+from helpers import assert_bf16_close, rand_codes, to_np
+from paper_2410_05265_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2410_05265_b200 import binding
+
+    c = binding.Context()
+    yield c
+    c.check()
+    c.close()
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def check(ctx, mode, M, N, K, ldo_pad=0):
+    rng = np.random.default_rng(M * 1009 + N * 31 + K)
+    wq, s_w = rand_codes(rng, N, K), rng.uniform(0.5, 2.0, N).astype(np.float32) * 1e-3
+    s_a, s_tok = np.float32(0.02), rng.uniform(0.01, 0.03, M).astype(np.float32)
+    out = torch.full((M, N + ldo_pad), 7.0, dtype=torch.bfloat16, device="cuda")
+    view = out[:, :N]
+    acc = torch.zeros((M, N), dtype=torch.int32, device="cuda")
+    kw = dict(out=view, acc_dbg=acc)
+    sa = torch.full((1,), float(s_a), device="cuda")
+    if mode == "w4a8":
+        x8 = rng.integers(-128, 128, (M, K)).astype(np.int8)
+        ref = orc.gemm_i8i4(x8, wq)
+        ctx.w4a8_gemm(dev(x8), dev(wq), sa, dev(s_w), **kw)
+    else:
+        xq = rand_codes(rng, M, K)
+        ref = orc.gemm_i4(xq, wq)
+        if mode == "rows":
+            ctx.w4a4_gemm_rows(dev(xq), dev(wq), dev(s_tok), dev(s_w), **kw)
+        elif mode == "asym":
+            wsum = ctx.weight_code_sums(dev(wq))
+            ref = ref - (5 - 8) * to_np(wsum).astype(ref.dtype)[None]
+            ctx.w4a4_gemm_asym(dev(xq), dev(wq), sa, torch.full((1,), 5, dtype=torch.int32, device="cuda"), dev(s_w), wsum, **kw)
+        else:
+            ctx.w4a4_gemm(dev(xq), dev(wq), sa, dev(s_w), **kw)
+    ctx.check()
+    assert np.array_equal(to_np(acc), ref), "accumulators differ"
+    want = ref.astype(np.float64) * (s_tok.astype(np.float64)[:, None] if mode == "rows" else float(s_a)) * s_w.astype(np.float64)
+    want = torch.from_numpy(want).to(torch.bfloat16)
+    assert_bf16_close(inputs.bits(view), inputs.bits(want), "split GEMM")
+    if ldo_pad:
+        assert bool((out[:, N:] == 7.0).all()), "columns past N must not be written"
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K", [
+    (17, 1, 32), (32, 127, 160), (33, 129, 416), (48, 130, 1152), (49, 257, 640), (64, 128, 2048), (65, 100, 1280),
+    (96, 260, 672), (97, 128, 256), (128, 300, 1280), (129, 128, 4128), (256, 132, 1280), (257, 640, 512), (600, 130, 96), (300, 4000, 640),
+])
+def test_split_gemm_matches_oracle(ctx, mode, M, N, K):
+    check(ctx, mode, M, N, K)
+
+
+@pytest.mark.parametrize("M,N,K,pad", [(40, 131, 1536, 5), (100, 260, 5120, 4), (24, 3000, 10240, 1)])
+def test_split_gemm_with_a_padded_output(ctx, M, N, K, pad):
+    """Row pitches that allow 8-byte stores and that do not; up to eight K splits, two and more K blocks per expansion group."""
+    check(ctx, "w4a4", M, N, K, pad)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8"])
+def test_large_layers_with_few_tokens(ctx, mode):
+    for M, N, K in [(9, 5128, 4128), (16, 5120, 4096), (1, 8200, 8192), (8, 4700, 14336)]:  # just inside the rules for few tokens
+        check(ctx, mode, M, N, K)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K", [(129, 8200, 160), (300, 4104, 416), (130, 8328, 8224)])
+def test_pair_kernels_just_above_the_border(ctx, mode, M, N, K):
+    """Problems just too large for two K splits go to the CTA-pair kernels: ragged edges; K >= 8192 takes the kernel with the
+    token operand in tensor memory."""
+    check(ctx, mode, M, N, K)
