@@ -25,17 +25,16 @@ static pq_status run_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, con
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // Weight-streaming kernel or split-K tensor-core kernel (figures: rotate+quantize and GEMM in a graph, us, streaming against
   // split). The streaming kernel has the shorter chain, but expands the tokens again for every 16 channels and has no K split:
-  //   up to 8 tokens   it keeps the short layers (1 token, 6144 x 4096: 5.4 / 7.1) and the wide ones (57344 x 8192: 44.4 / 51.2);
-  //                    large layers with long rows and few enough channel tiles for three or more K splits go to the other
-  //                    (8192 x 28672: 29.2 / 24.4, 8192 x 8192: 11.4 / 10.4, 10240 x 8192: 12.2 / 12.1; not 4096 x 14336:
-  //                    9.9 / 9.7 here, but 1.5 us slower inside a decode layer)
+  //   up to 8 tokens   always streaming. Alone behind its rotation kernel the other is faster on 8192 x 28672 (1 token: 29.2 / 24.4)
+  //                    and 8192 x 8192 (11.4 / 10.4), but inside a decode layer the streaming kernel's shorter chain and earlier
+  //                    weight requests win: whole 70B layer 124 / 132 us
   //   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
   //                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
   //   up to 128        always split (the CTA-pair kernels: 33 tokens, 4096 x 4096: 23.1 / 8.5, 28672 x 4096: 40.8 / 18.2)
   //   above            while the 256-token tiles leave room for two K splits: whole 8B block at 200 tokens 176.5 / 132.1, at 300
   //                    tokens 201 / 175; with a single split (515 tokens) the o layer gains 2.3 and the down layer loses 8.6.
   const int64_t ctiles = (N + 127) / 128, weights = N * K;
-  const bool split = m <= 8     ? K >= 8192 && weights >= (int64_t{1} << 26) && 3 * ctiles <= ctx->sm_count * 7 / 4
+  const bool split = m <= 8     ? false
                      : m <= 16  ? weights >= (int64_t{20} << 20)
                      : m <= 128 ? true
                                 : 2 * ((m + 255) / 256) * ctiles <= ctx->sm_count * 7 / 8;
