@@ -27,11 +27,13 @@ constexpr int RN_THREADS = 256;
 constexpr int RN_MAX_VEC = 8;  // 8-element vectors per thread kept in registers: K <= 256 * 8 * 8 = 16384
 
 __global__ void __launch_bounds__(RN_THREADS)
-    rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, const __nv_bfloat16* __restrict__ g, float eps,
-                   __nv_bfloat16* __restrict__ y, int64_t ldy, int64_t M, int K) {
+    rmsnorm_kernel(const __nv_bfloat16* x, int64_t ldx, const __nv_bfloat16* __restrict__ g, float eps,
+                   __nv_bfloat16* y, int64_t ldy, int64_t M, int K) {
   __shared__ float red[RN_THREADS / 32];
   __shared__ float s_r;
   const int n_vec = K / 8;
+  pq::pdl_wait();
+  pq::pdl_trigger();
   for (int64_t row = blockIdx.x; row < M; row += gridDim.x) {
     const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
     uint4 v[RN_MAX_VEC];
@@ -39,7 +41,7 @@ __global__ void __launch_bounds__(RN_THREADS)
 #pragma unroll
     for (int i = 0; i < RN_MAX_VEC; ++i) {
       const int j = threadIdx.x + i * RN_THREADS;
-      v[i] = j < n_vec ? __ldg(xr + j) : make_uint4(0, 0, 0, 0);
+      v[i] = j < n_vec ? xr[j] : make_uint4(0, 0, 0, 0);
       const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) ss = fmaf(bf16_lo(w[e]), bf16_lo(w[e]), fmaf(bf16_hi(w[e]), bf16_hi(w[e]), ss));
@@ -78,16 +80,24 @@ __global__ void __launch_bounds__(RN_THREADS)
 // rotates 8-element vectors of the token's heads.
 constexpr int RP_THREADS = 128;
 
+__device__ __forceinline__ void rope_angles(int64_t pos, double log2_theta, float (&cs)[64], float (&sn)[64]) {
+  if (threadIdx.x < 64) {
+    const double inv_freq = exp2(-2.0 * static_cast<double>(threadIdx.x) / 128.0 * log2_theta);
+    double s, c;
+    sincos(static_cast<double>(pos) * inv_freq, &s, &c);
+    cs[threadIdx.x] = static_cast<float>(c), sn[threadIdx.x] = static_cast<float>(s);
+  }
+}
+
 __global__ void __launch_bounds__(RP_THREADS)
     rope_kernel(const __nv_bfloat16* x, __nv_bfloat16* y, int64_t T, int H, int64_t ld, int64_t pos0,
                 double log2_theta) {
   __shared__ float cs[64], sn[64];
   for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
-    if (threadIdx.x < 64) {
-      const double inv_freq = exp2(-2.0 * static_cast<double>(threadIdx.x) / 128.0 * log2_theta);
-      double s, c;
-      sincos(static_cast<double>(pos0 + t) * inv_freq, &s, &c);
-      cs[threadIdx.x] = static_cast<float>(c), sn[threadIdx.x] = static_cast<float>(s);
+    rope_angles(pos0 + t, log2_theta, cs, sn);
+    if (t == blockIdx.x) {  // the angles need nothing from the previous kernel
+      pq::pdl_wait();
+      pq::pdl_trigger();
     }
     __syncthreads();
     // a work item = (head, group of 8 consecutive i in [0, 64)): reads x[i..i+7] and x[64+i..64+i+7]
@@ -150,11 +160,10 @@ __global__ void __launch_bounds__(RP_THREADS)
   __shared__ float cs[64], sn[64];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
-    if (threadIdx.x < 64) {
-      const double inv_freq = exp2(-2.0 * static_cast<double>(threadIdx.x) / 128.0 * log2_theta);
-      double s, c;
-      sincos(static_cast<double>(pos0 + t) * inv_freq, &s, &c);
-      cs[threadIdx.x] = static_cast<float>(c), sn[threadIdx.x] = static_cast<float>(s);
+    rope_angles(pos0 + t, log2_theta, cs, sn);
+    if (t == blockIdx.x) {  // the angles need nothing from the previous kernel
+      pq::pdl_wait();
+      pq::pdl_trigger();
     }
     __syncthreads();
     const float c0 = cs[2 * lane], s0 = sn[2 * lane], c1 = cs[2 * lane + 1], s1 = sn[2 * lane + 1];
@@ -187,15 +196,16 @@ __global__ void __launch_bounds__(RP_THREADS)
   __shared__ float cs[64], sn[64];
   __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int len0 = __ldcg(len);
-  const bool bad = len0 < 0 || len0 + T > Tmax;  // every CTA reaches the same verdict: then nothing is appended
+  int len0 = 0;
+  bool bad = false;
   const int n_heads = Hq + 2 * Hkv;
   for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
-    if (threadIdx.x < 64) {
-      const double inv_freq = exp2(-2.0 * static_cast<double>(threadIdx.x) / 128.0 * log2_theta);
-      double s, c;
-      sincos(static_cast<double>(pos0 + t) * inv_freq, &s, &c);
-      cs[threadIdx.x] = static_cast<float>(c), sn[threadIdx.x] = static_cast<float>(s);
+    rope_angles(pos0 + t, log2_theta, cs, sn);
+    if (t == blockIdx.x) {  // the angles need nothing from the previous kernel
+      pq::pdl_wait();
+      pq::pdl_trigger();
+      len0 = __ldcg(len);
+      bad = len0 < 0 || len0 + T > Tmax;  // every CTA reaches the same verdict: then nothing is appended
     }
     __syncthreads();
     const float c0 = cs[2 * lane], s0 = sn[2 * lane], c1 = cs[2 * lane + 1], s1 = sn[2 * lane + 1];
@@ -245,16 +255,18 @@ __global__ void __launch_bounds__(RP_THREADS)
 constexpr int EW_THREADS = 256;
 
 __global__ void __launch_bounds__(EW_THREADS)
-    silu_mul_kernel(const __nv_bfloat16* __restrict__ gate, const __nv_bfloat16* __restrict__ up, int64_t ld_in,
-                    __nv_bfloat16* __restrict__ y, int64_t ldy, int64_t M, int F) {
+    silu_mul_kernel(const __nv_bfloat16* gate, const __nv_bfloat16* up, int64_t ld_in,
+                    __nv_bfloat16* y, int64_t ldy, int64_t M, int F) {
   const int vec_per_row = F / 8;
   const int64_t n_vec = M * vec_per_row;
+  pq::pdl_wait();
+  pq::pdl_trigger();
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * EW_THREADS + threadIdx.x; i < n_vec;
        i += static_cast<int64_t>(gridDim.x) * EW_THREADS) {
     const int64_t row = i / vec_per_row;
     const int col = static_cast<int>(i % vec_per_row) * 8;
-    const uint4 gv = __ldg(reinterpret_cast<const uint4*>(gate + row * ld_in + col));
-    const uint4 uv = __ldg(reinterpret_cast<const uint4*>(up + row * ld_in + col));
+    const uint4 gv = *reinterpret_cast<const uint4*>(gate + row * ld_in + col);
+    const uint4 uv = *reinterpret_cast<const uint4*>(up + row * ld_in + col);
     const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, uw[4] = {uv.x, uv.y, uv.z, uv.w};
     uint32_t o[4];
 #pragma unroll
@@ -270,6 +282,8 @@ __global__ void __launch_bounds__(EW_THREADS)
 __global__ void __launch_bounds__(EW_THREADS)
     add_kernel(const __nv_bfloat16* a, const __nv_bfloat16* b, __nv_bfloat16* y,
                int64_t n_vec) {
+  pq::pdl_wait();
+  pq::pdl_trigger();
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * EW_THREADS + threadIdx.x; i < n_vec;
        i += static_cast<int64_t>(gridDim.x) * EW_THREADS) {
     const uint4 av = reinterpret_cast<const uint4*>(a)[i], bv = reinterpret_cast<const uint4*>(b)[i];  // y may alias a or b
@@ -320,10 +334,9 @@ extern "C" pq_status pq_rmsnorm(pq_ctx* ctx, const void* x, int64_t M, int64_t K
   // a row that is one transform block of the online rotation takes the first pass of that kernel, so that
   // pq_rmsnorm_hadamard_quant_act equals this call followed by pq_hadamard_quant_act bit for bit
   if ((K & (K - 1)) == 0 && K >= 128 && K <= 8192) return pq_rmsnorm_pow2_launch(ctx, x, M, K, ldx, g, eps, y, ldy, stream);
-  rmsnorm_kernel<<<grid_for(ctx, M, 1), RN_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16*>(x), ldx, static_cast<const __nv_bfloat16*>(g), eps,
-      static_cast<__nv_bfloat16*>(y), ldy, M, static_cast<int>(K));
-  return pq_launch_status();
+  return pq_launch_pdl(rmsnorm_kernel, grid_for(ctx, M, 1), RN_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<const __nv_bfloat16*>(x), ldx, static_cast<const __nv_bfloat16*>(g), eps,
+                       static_cast<__nv_bfloat16*>(y), ldy, M, static_cast<int>(K));
 }
 
 extern "C" pq_status pq_rope(pq_ctx* ctx, const void* x, int64_t T, int32_t H, int32_t D, int64_t ld, int64_t pos0,
@@ -333,9 +346,8 @@ extern "C" pq_status pq_rope(pq_ctx* ctx, const void* x, int64_t T, int32_t H, i
   if (D != 128) return PQ_ERR_SHAPE;
   if (!aligned16(x) || !aligned16(y) || ld % 8 != 0) return PQ_ERR_ALIGN;
   if (T == 0) return PQ_OK;
-  rope_kernel<<<grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(y), T, H, ld, pos0, log2(theta));
-  return pq_launch_status();
+  return pq_launch_pdl(rope_kernel, grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(y), T, H, ld, pos0, log2(theta));
 }
 
 extern "C" pq_status pq_rope_rotate(pq_ctx* ctx, const void* x, int64_t T, int32_t H, int32_t D, int64_t ld,
@@ -345,9 +357,8 @@ extern "C" pq_status pq_rope_rotate(pq_ctx* ctx, const void* x, int64_t T, int32
   if (D != 128) return PQ_ERR_SHAPE;
   if (!aligned16(x) || !aligned16(y) || ld % 8 != 0) return PQ_ERR_ALIGN;
   if (T == 0) return PQ_OK;
-  rope_rotate_kernel<<<grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(y), T, H, ld, pos0, log2(theta));
-  return pq_launch_status();
+  return pq_launch_pdl(rope_rotate_kernel, grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(y), T, H, ld, pos0, log2(theta));
 }
 
 extern "C" pq_status pq_rope_kv4_append(pq_ctx* ctx, const pq_kv4_cache* c, int32_t seq, void* qkv, int64_t T, int64_t ld, int64_t pos0,
@@ -361,10 +372,9 @@ extern "C" pq_status pq_rope_kv4_append(pq_ctx* ctx, const pq_kv4_cache* c, int3
   if (!aligned16(qkv) || ld % 8 != 0 || !aligned16(c->kq) || !aligned16(c->vq)) return PQ_ERR_ALIGN;
   if (T == 0) return PQ_OK;
   const int64_t seq_off = static_cast<int64_t>(seq) * c->Hkv * c->Tmax * 64;
-  rope_kv4_append_kernel<<<grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<__nv_bfloat16*>(qkv), T, c->Hq, c->Hkv, ld, pos0, log2(theta), rotate, c->kq + seq_off, c->vq + seq_off, c->s_k, c->s_v,
-      c->len + seq, c->Tmax, ctx->d_status, ctx->d_tickets + 1);
-  return pq_launch_status();
+  return pq_launch_pdl(rope_kv4_append_kernel, grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<__nv_bfloat16*>(qkv), T, c->Hq, c->Hkv, ld, pos0, log2(theta), rotate, c->kq + seq_off, c->vq + seq_off, c->s_k, c->s_v,
+                       c->len + seq, c->Tmax, ctx->d_status, ctx->d_tickets + 1);
 }
 
 extern "C" pq_status pq_silu_mul(pq_ctx* ctx, const void* gate, const void* up, int64_t M, int64_t F, int64_t ld_in,
@@ -374,10 +384,9 @@ extern "C" pq_status pq_silu_mul(pq_ctx* ctx, const void* gate, const void* up, 
   if (F % 8 != 0 || F > (1 << 30)) return PQ_ERR_SHAPE;
   if (!aligned16(gate) || !aligned16(up) || !aligned16(y) || ld_in % 8 != 0 || ldy % 8 != 0) return PQ_ERR_ALIGN;
   if (M == 0) return PQ_OK;
-  silu_mul_kernel<<<grid_for(ctx, M * (F / 8), EW_THREADS), EW_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16*>(gate), static_cast<const __nv_bfloat16*>(up), ld_in,
-      static_cast<__nv_bfloat16*>(y), ldy, M, static_cast<int>(F));
-  return pq_launch_status();
+  return pq_launch_pdl(silu_mul_kernel, grid_for(ctx, M * (F / 8), EW_THREADS), EW_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<const __nv_bfloat16*>(gate), static_cast<const __nv_bfloat16*>(up), ld_in,
+                       static_cast<__nv_bfloat16*>(y), ldy, M, static_cast<int>(F));
 }
 
 extern "C" pq_status pq_residual_add(pq_ctx* ctx, const void* a, const void* b, void* y, int64_t n, void* stream) {
@@ -385,9 +394,8 @@ extern "C" pq_status pq_residual_add(pq_ctx* ctx, const void* a, const void* b, 
   if (n % 8 != 0) return PQ_ERR_SHAPE;
   if (!aligned16(a) || !aligned16(b) || !aligned16(y)) return PQ_ERR_ALIGN;
   if (n == 0) return PQ_OK;
-  add_kernel<<<grid_for(ctx, n / 8, EW_THREADS), EW_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16*>(a), static_cast<const __nv_bfloat16*>(b), static_cast<__nv_bfloat16*>(y), n / 8);
-  return pq_launch_status();
+  return pq_launch_pdl(add_kernel, grid_for(ctx, n / 8, EW_THREADS), EW_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<const __nv_bfloat16*>(a), static_cast<const __nv_bfloat16*>(b), static_cast<__nv_bfloat16*>(y), n / 8);
 }
 
 extern "C" pq_status pq_calib_kv_scale(pq_ctx* ctx, const void* x, int64_t n_tok, int32_t Hkv, int32_t D, int64_t ld_tok,

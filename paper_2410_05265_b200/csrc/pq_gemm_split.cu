@@ -158,7 +158,7 @@ __device__ __forceinline__ void reduce_tile(const SplitParams& p, const uint8_t*
         if (PEERS == 1) v[u][r] = *reinterpret_cast<const int4*>(part + t * (CH * 4) + lane * 16);
         else v[u][r] = r < p.splits ? ld_cluster_int4(peer[r] + t * (CH * 4)) : make_int4(0, 0, 0, 0);
       }
-      rs[u] = p.s_row ? __ldg(p.s_row + t0 + t) : 1.0f;
+      rs[u] = p.s_row ? p.s_row[t0 + t] : 1.0f;  // may come from the previous kernel: no read-only load
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
   const int kb0 = static_cast<int>(static_cast<int64_t>(p.n_kb) * rank / p.splits);
   const int total = static_cast<int>(static_cast<int64_t>(p.n_kb) * (rank + 1) / p.splits) - kb0;  // K blocks of this CTA
 
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (p.M <= 32) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next kernel is small, too (see pq_launch_pdl)
   const bool leader = pq::elect_one();  // the lane that issues copies and MMAs (each role's loop is warp-uniform)
   const int first = total < C::STAGES ? total : C::STAGES;
   if (warp == 0) {

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   int32_t* zw_buf = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(scale_buf) + SCALE_BYTES);
   Barriers* bars = reinterpret_cast<Barriers*>(reinterpret_cast<uint8_t*>(zw_buf) + ZW_BYTES);
 
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // no early launch of the next kernel: its CTAs would crowd on the SMs whose pair has no tile left (see pq_launch_pdl)
   asm volatile("griddepcontrol.wait;" ::: "memory");  // operands and output may belong to the previous kernel
   const int warp = pq::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);

@@ -229,6 +229,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
     bars->abort_flag = 0;
     pq::mbar_fence_init();
   }
+  pq::pdl_wait();  // queries, cache and output may belong to the previous kernel
+  pq::pdl_trigger();
   if (warp == PA_WARP_MMA) {
     pq::tmem_alloc(&bars->tmem_base, PA_TMEM_COLS);
     pq::tmem_relinquish();
@@ -637,9 +639,6 @@ extern "C" pq_status pq_prefill_attn_kv4_prefix(pq_ctx* ctx, const pq_kv4_cache*
   }
   const int R = 256 / G;
   dim3 grid((T + R - 1) / R, c->Hkv);
-  if (dyn)
-    prefill_attn_kernel<true><<<grid, PA_THREADS, PA_SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(p);
-  else
-    prefill_attn_kernel<false><<<grid, PA_THREADS, PA_SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(p);
-  return pq_launch_status();
+  return pq_launch_pdl(dyn ? prefill_attn_kernel<true> : prefill_attn_kernel<false>, grid, PA_THREADS, PA_SMEM_BYTES,
+                       static_cast<cudaStream_t>(stream), p);
 }
