@@ -1,5 +1,6 @@
 // Offline RTN weight quantization, one symmetric INT4 scale per output channel
-// (Table 1 "per-channel"; Table 6 "RTN"; Eq. 1). One CTA per weight row, two passes over the row.
+// (Table 1 "per-channel"; Table 6 "RTN"; Eq. 1). One CTA per weight row: rows of up to 32768 weights with 16-byte alignment are
+// read once and kept in registers, the others take two passes over the row.
 #include "pq_common.cuh"
 
 namespace {
@@ -39,6 +40,106 @@ __global__ void __launch_bounds__(QW_THREADS) quant_weights_kernel(const __nv_bf
   }
 }
 
+// The same for rows that are read once: VPT 16-byte vectors per thread stay in registers between the maximum and the codes.
+// Bound by HBM (2.5 bytes per weight) once a code costs few instructions. A code is rint(w / s) with an IEEE division; here it is
+// rint(w * r), r ~ 1 / s, from one fused multiply-add into the rounding constant 1.5 * 2^23, checked per row: both are monotone in w
+// and can differ only next to a half-integer, which for bf16 weights means at one of the few bf16 values around (k + 1/2) s,
+// k = 0 .. 6 (bf16 values are 2^-8 apart, the two quotients less than 2^-21). Seven lanes compare the two forms there, for r = 1 / s and
+// its two neighbours; a row where none agrees (about one maximum in nine: a multiple of 7), that holds an infinity or a NaN, or
+// whose step is far from 1 divides element by element.
+// Measured (us, two passes with a division each / now): 28672 x 4096 129 / 60 (4.9 TB/s), 4096 x 14336 64 / 31, 8192 x 28672
+// 256 / 121, 4096 x 4096 20.6 / 13.1.
+__device__ __forceinline__ int code_div(float w, float s) { return max(-8, min(7, __float2int_rn(__fdiv_rn(w, s)))); }
+__device__ __forceinline__ uint32_t code_mul(float w, float r) { return __float_as_uint(fmaf(w, r, 12582912.0f)); }  // code in the low bits
+
+template <int THREADS, int VPT>
+__global__ void __launch_bounds__(THREADS) quant_weights_once_kernel(const __nv_bfloat16* __restrict__ W, int K, int64_t ldw,
+                                                                     uint8_t* __restrict__ wq, float* __restrict__ s_w) {
+  __shared__ uint32_t red[THREADS / 32];
+  const int64_t n = blockIdx.x;
+  const uint4* row = reinterpret_cast<const uint4*>(W + n * ldw);
+  const int n_vec = K / 8;
+  uint4 v[VPT];
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    const int j = threadIdx.x + i * THREADS;
+    v[i] = make_uint4(0, 0, 0, 0);
+    if (j < n_vec)
+      asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w) : "l"(row + j));
+  }
+  uint32_t m2 = 0;  // packed maxima of the patterns without sign
+#pragma unroll
+  for (int i = 0; i < VPT; ++i)
+    m2 = __vmaxu2(__vmaxu2(m2, __vmaxu2(v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu)), __vmaxu2(v[i].z & 0x7FFF7FFFu, v[i].w & 0x7FFF7FFFu));
+  uint32_t m = max(m2 & 0xFFFFu, m2 >> 16);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < THREADS / 32; ++i) m = max(m, red[i]);
+  const bool special = m >= 0x7F80u;
+  if (special) {  // an infinity or a NaN in the row: the maximum that ignores NaN, then the same two steps
+    float mx = 0.0f;
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fmaxf(fabsf(__uint_as_float(w[e] << 16)), fabsf(__uint_as_float(w[e] & 0xFFFF0000u))));
+    }
+    const uint32_t mb = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mb;
+    __syncthreads();
+    m = 0;
+#pragma unroll
+    for (int i = 0; i < THREADS / 32; ++i) m = max(m, red[i]);
+    m >>= 16;
+  }
+  const float mx = __uint_as_float(m << 16);
+  const float s = mx == 0.0f ? 1.0f : __fdiv_rn(mx, 7.0f);
+  if (threadIdx.x == 0) s_w[n] = s;
+  // 1 / s or one of its neighbours: half the maximum is a tie in every row, and which way it falls depends on that last bit
+  float r = __fdiv_rn(1.0f, s);
+  bool same = s > 1e-30f && s < 1e30f && !special;
+  {
+    const int k = min(static_cast<int>(threadIdx.x & 31), 6);
+    const uint32_t h = __float_as_uint((k + 0.5f) * s) >> 16;  // the bf16 value at or below the half-integer, and its neighbours
+    const uint32_t rb = __float_as_uint(r);
+    uint32_t ok = 7;  // bit c: candidate c agrees
+#pragma unroll
+    for (int d = -1; d <= 2; ++d) {
+      const float b = __uint_as_float((h + d) << 16);
+      const uint32_t want = static_cast<uint32_t>(code_div(b, s));
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if ((code_mul(b, __uint_as_float(rb + (c == 2 ? -1 : c))) & 0xFu) != want) ok &= ~(1u << c);
+    }
+    ok = __reduce_and_sync(0xffffffffu, ok);
+    same = same && ok != 0;
+    r = __uint_as_float(rb + ((ok & 1) ? 0 : (ok & 2) ? 1 : -1));
+  }
+  uint32_t* orow = reinterpret_cast<uint32_t*>(wq + n * (K / 2));
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    const int j = threadIdx.x + i * THREADS;
+    if (j >= n_vec) break;
+    const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+    uint32_t o = 0;
+    if (same) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const uint32_t a = code_mul(__uint_as_float(w[e] << 16), r), b = code_mul(__uint_as_float(w[e] & 0xFFFF0000u), r);
+        o |= ((a & 0xFu) | ((b & 0xFu) << 4)) << (8 * e);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        o |= static_cast<uint32_t>((code_div(__uint_as_float(w[e] << 16), s) & 0xF) | ((code_div(__uint_as_float(w[e] & 0xFFFF0000u), s) & 0xF) << 4)) << (8 * e);
+    }
+    orow[j] = o;
+  }
+}
+
 }  // namespace
 
 extern "C" pq_status pq_quant_weights(pq_ctx* ctx, const void* W, int64_t N, int64_t K, int64_t ldw, uint8_t* wq,
@@ -47,8 +148,22 @@ extern "C" pq_status pq_quant_weights(pq_ctx* ctx, const void* W, int64_t N, int
   if (N < 0 || K < 0 || ldw < K) return PQ_ERR_INVALID_ARG;
   if (K % 2 != 0) return PQ_ERR_SHAPE;
   if (N == 0 || K == 0) return PQ_OK;
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // Rows that start on 16 bytes and hold whole vectors are read once; threads and vectors per thread so that four to eight rows'
+  // loads are in flight on an SM.
+  if (K % 8 == 0 && ldw % 8 == 0 && K <= 32768 && N <= 0x7FFFFFFF && (reinterpret_cast<uintptr_t>(W) & 15) == 0 &&
+      (reinterpret_cast<uintptr_t>(wq) & 3) == 0) {
+    const __nv_bfloat16* w = static_cast<const __nv_bfloat16*>(W);
+    const int k = static_cast<int>(K);
+    const unsigned rows = static_cast<unsigned>(N);
+    if (K <= 4096) quant_weights_once_kernel<128, 4><<<rows, 128, 0, st>>>(w, k, ldw, wq, s_w);
+    else if (K <= 8192) quant_weights_once_kernel<256, 4><<<rows, 256, 0, st>>>(w, k, ldw, wq, s_w);
+    else if (K <= 16384) quant_weights_once_kernel<256, 8><<<rows, 256, 0, st>>>(w, k, ldw, wq, s_w);
+    else quant_weights_once_kernel<512, 8><<<rows, 512, 0, st>>>(w, k, ldw, wq, s_w);
+    return pq_launch_status();
+  }
   int grid = static_cast<int>(N < 65535 * 4 ? N : 65535 * 4);
-  quant_weights_kernel<<<grid, QW_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
+  quant_weights_kernel<<<grid, QW_THREADS, 0, st>>>(
       static_cast<const __nv_bfloat16*>(W), N, K, ldw, wq, s_w);
   return pq_launch_status();
 }
