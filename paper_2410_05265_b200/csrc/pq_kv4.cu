@@ -711,12 +711,11 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
   const int csize = S < 8 ? S : 8, n_clusters = MULTI ? S / csize : 1;
   const int n_parts = CLUSTER ? n_clusters : S;  // partials per (sequence, head) that meet in the workspace
   if (CLUSTER) {
-    // every split's partial is in its CTA's shared memory; thread i of the cluster takes (head, four
-    // dims) item i and reads the cluster's partials through distributed shared memory, all loads at once
+    // every split's partial is in its CTA's shared memory; the threads of the cluster take the (head, four
+    // dims) items in turn and read the cluster's partials through distributed shared memory, all loads at once
     cluster_arrive_wait();
     const int rank = split % csize, ci = split / csize;
-    const int item = rank * DA_THREADS + threadIdx.x;
-    if (item < G * 32) {
+    for (int item = rank * DA_THREADS + threadIdx.x; item < G * 32; item += csize * DA_THREADS) {  // one CTA alone has more items than threads
       const int r = item >> 5, c4 = item & 31;
       const uint32_t o_addr = pq::smem_u32(cl_o + r * 128 + 4 * c4), ml_addr = pq::smem_u32(cl_ml + r);
       float4 v[8];
