@@ -122,6 +122,13 @@ __device__ __forceinline__ uint32_t hsub2_u32(uint32_t a, uint32_t b) {
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
+// Two codes of a word as exact fp16 integers: nibbles 0 (even) or 1 (odd) of its 16-bit halves.
+__device__ __forceinline__ uint32_t codes_even(uint32_t w) { return hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(w), 0x64086408u); }
+__device__ __forceinline__ uint32_t codes_odd(uint32_t w) {  // (1152 + 16 code) / 16 - 72
+  uint32_t d;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(and_xor<0x00F000F0u, 0x64806480u>(w)), "r"(0x2C002C00u), "r"(0xD480D480u));
+  return d;
+}
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   __half2 h = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
@@ -185,6 +192,8 @@ struct AttnParams {
   const uint8_t* vq;
   const float* s_k;
   const float* s_v;
+  const float* sk_tok;  // DYN: the steps of the cached vectors [B, Hkv, Tmax]
+  const float* sv_tok;
   const int32_t* len;
   float* ws_o;   // [B*Hkv, S, G, 128] partial outputs, already in value units
   float* ws_ml;  // [B*Hkv, S, G, 2]   running maximum (log2 units) and denominator
@@ -229,8 +238,18 @@ struct AttnParams {
 // the dequantized codes. The last CTA of the grid to finish (every CTA has read the lengths by then) advances
 // every len[b]. As with the two calls, nothing is appended anywhere when any sequence is full.
 // MULTI (with CLUSTER): a (sequence, head) has several clusters of eight splits.
-template <bool CLUSTER, bool FUSED, bool MULTI = false>
-__global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnParams p) {
+// DYN (group-wise dynamic KV, Table 1 O1): every cached vector has its own step. The setting's arithmetic is that of fp32:
+//   scores   codes as exact fp16 integers (one more half2 operation per word pair, no offset to cancel) times the query row
+//            scaled by a power of two into fp16's normal range (a bf16 value is then exact), then the key's step in fp32;
+//   output   the weight of a value row is P * step / R, R a power of two above any value step the warp has seen (it and
+//            the accumulators move together); it enters the MMA as two fp16 terms, hi + lo (22 bits), so twice the MMAs;
+//   the denominator is summed in fp32 on the CUDA cores. P is 2^7 at the row's maximum, which keeps lo above fp16's denormals.
+// A warp reads the steps of its 32 keys one round ahead (one key per lane) and hands them round with shuffles. What bounds it is
+// the per-round chain of the static form, with twice the output MMAs and three CTAs per SM. 8 x 4092 keys, 32 heads: 91.8 us for
+// the CUDA-core fp32 kernel this replaces, 22.9 now; 6 x 1500: 42.9 -> 9.0; one sequence of 30000 keys, 64 heads: 105 -> 20.4
+// (the bf16 outputs differ from the exact result's rounding in 2e-4 to 5e-4 of the elements, as before).
+template <bool CLUSTER, bool FUSED, bool MULTI = false, bool DYN = false>
+__global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(const AttnParams p) {
   extern __shared__ __align__(128) uint8_t da_stage[];  // DA_SLOTS slots of [K rows | V rows] of one round
   // the per-warp partial outputs reuse the staging area once the key loop is over
   // [warp][head][DA_SO_STRIDE]; head dim d = 16a + 2b + c sits at 16b + 2a + c and the rows are padded so
@@ -240,6 +259,7 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
   __shared__ float2 cl_ml[DA_ROWS];
   __shared__ __align__(8) uint64_t full[DA_SLOTS][DA_CHUNKS];
   __shared__ float sm_ml[DA_WARPS][DA_ROWS][2];
+  __shared__ float sm_vref[DYN ? DA_WARPS : 1];         // DYN: what a warp's output accumulators are multiples of
   __shared__ float sm_pre[DA_ROWS][DA_MAX_PREFIX + 1];  // the last column: the key appended by this call
   __shared__ float sm_newv[FUSED ? 128 : 1];             // its dequantized value
   __shared__ float sm_red[DA_WARPS][DA_ROWS];
@@ -275,7 +295,7 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
   if (!FUSED) load_q();
   // the fused kernel writes the lengths at its end: it reads them past the read-only path
   int len_b = FUSED ? __ldcg(p.len + b) : __ldg(p.len + b);
-  const float s_k_h = __ldg(p.s_k + h), s_v_h = __ldg(p.s_v + h);
+  const float s_k_h = DYN ? 1.0f : __ldg(p.s_k + h), s_v_h = DYN ? 1.0f : __ldg(p.s_v + h);
   // prefix values of the four head dims this thread merges after the key loop, so that the merge does
   // not wait for them (keys past the fourth are read there)
   uint2 pv_early[4];
@@ -445,6 +465,19 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
   // 2t, 2t+1 and 2t+8, 2t+9 of score MMA j.
   uint32_t qb[8][2];
   float q_even = 0.0f, q_odd = 0.0f;
+  float q_up = 1.0f, q_down = 1.0f;  // DYN: the row's power of two (largest magnitude near 2^8) and its inverse
+  if (DYN) {
+    uint32_t mx = 0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+      mx = __vmaxu2(mx, __vmaxu2(__vmaxu2(q_raw[w].x & 0x7FFF7FFFu, q_raw[w].y & 0x7FFF7FFFu), __vmaxu2(q_raw[w].z & 0x7FFF7FFFu, q_raw[w].w & 0x7FFF7FFFu)));
+    mx = max(mx & 0xFFFFu, mx >> 16);
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const int ex = min(max(static_cast<int>(mx >> 7), 9), 253);  // biased exponent of the largest magnitude
+    q_up = __uint_as_float(static_cast<uint32_t>(min(254 + 8 - ex, 254)) << 23);
+    q_down = 1.0f / q_up;
+  }
   {
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
@@ -456,8 +489,9 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
 #pragma unroll
       for (int jj = 0; jj < 2; ++jj) {  // score MMA j = 2w + jj uses nibbles 2jj and 2jj + 1
         const int i0 = 2 * jj;
-        const __half2 a0 = __floats2half2_rn(f[i0], f[i0 + 4]);
-        const __half2 a2 = __floats2half2_rn(f[i0 + 1] * 0.0625f, f[i0 + 5] * 0.0625f);
+        const float odd = DYN ? q_up : 0.0625f;
+        const __half2 a0 = DYN ? __floats2half2_rn(f[i0] * q_up, f[i0 + 4] * q_up) : __floats2half2_rn(f[i0], f[i0 + 4]);
+        const __half2 a2 = __floats2half2_rn(f[i0 + 1] * odd, f[i0 + 5] * odd);
         qb[2 * w + jj][0] = *reinterpret_cast<const uint32_t*>(&a0);
         qb[2 * w + jj][1] = *reinterpret_cast<const uint32_t*>(&a2);
         // the offsets are removed with the values the MMA really multiplies
@@ -480,6 +514,21 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
   // exist keeps a huge one: its probabilities are zero and it never asks for a move.
   float m0 = 2 * t < G ? -INFINITY : 1e30f, m1 = 2 * t + 1 < G ? -INFINITY : 1e30f;
   float bm0 = bias0 + m0, bm1 = bias1 + m1;  // what is subtracted from a raw score
+  // DYN: what a score of heads 2t, 2t + 1 is multiplied with beside the key's step
+  const float hs = p.sm_scale * 1.4426950408889634f * q_down;
+  const float hs0 = __shfl_sync(0xffffffffu, hs, 8 * t), hs1 = __shfl_sync(0xffffffffu, hs, 8 * t + 4);
+  constexpr float HEADROOM = DYN ? 14.0f : DA_HEADROOM;
+  float vref = 0.0f;  // DYN: R
+  const float* skb = DYN ? p.sk_tok + static_cast<int64_t>(bh) * p.Tmax : nullptr;
+  const float* svb = DYN ? p.sv_tok + static_cast<int64_t>(bh) * p.Tmax : nullptr;
+  float sk_next = 0.0f, sv_next = 0.0f;
+  auto load_steps = [&](int r) {  // lane i: key i % 16 of block i / 16 of the two blocks this warp takes of round r
+    const int j = round_key0(r) + (lane >> 4) * DA_CHUNK + 16 * warp + (lane & 15);
+    const bool in = r < n_rounds && j < t1;
+    sk_next = in ? __ldg(skb + j) : 0.0f;
+    sv_next = in ? __ldg(svb + j) : 0.0f;
+  };
+  if (DYN) load_steps(0);
 
   // Output accumulators of the transposed product: tile m holds, for this lane, o[m][0], o[m][1] =
   // dim 16g+2m of heads 2t, 2t+1 and o[m][2], o[m][3] = 16 x dim 16g+2m+1 of the same heads.
@@ -514,6 +563,8 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
         if (n >= DA_EARLY * DA_CHUNKS && i < n_rounds && k0 < t1) issue_chunk(i, n % DA_CHUNKS, min(DA_CHUNK, t1 - k0));
       }
     }
+    const float sk_cur = sk_next, sv_cur = sv_next;
+    if (DYN) load_steps(r + 1);
     float c[2][4];  // raw scores: [0], [1] = key g x heads 2t, 2t+1; [2], [3] = key g + 8 x the same heads
     bool dead_lo[2], dead_hi[2];
 #pragma unroll
@@ -528,6 +579,11 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
         const uint32_t wl8 = wl[w] >> 8, wh8 = wh[w] >> 8;
+        if (DYN) {
+          mma_f16_16816_full(ca, codes_even(wl[w]), codes_even(wh[w]), codes_odd(wl[w]), codes_odd(wh[w]), qb[2 * w][0], qb[2 * w][1]);
+          mma_f16_16816_full(cb, codes_even(wl8), codes_even(wh8), codes_odd(wl8), codes_odd(wh8), qb[2 * w + 1][0], qb[2 * w + 1][1]);
+          continue;
+        }
         mma_f16_16816_full(ca, and_xor<0x000F000Fu, 0x64086408u>(wl[w]), and_xor<0x000F000Fu, 0x64086408u>(wh[w]),
                            and_xor<0x00F000F0u, 0x64806480u>(wl[w]), and_xor<0x00F000F0u, 0x64806480u>(wh[w]),
                            qb[2 * w][0], qb[2 * w][1]);
@@ -537,28 +593,32 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) c[u][i] = ca[i] + cb[i];
+      if (DYN) {  // scores in log2 units
+        const float sk_lo = __shfl_sync(0xffffffffu, sk_cur, 16 * u + g), sk_hi = __shfl_sync(0xffffffffu, sk_cur, 16 * u + 8 + g);
+        c[u][0] *= sk_lo * hs0, c[u][1] *= sk_lo * hs1, c[u][2] *= sk_hi * hs0, c[u][3] *= sk_hi * hs1;
+      }
     }
     // ---- softmax against the reference exponents: e = log2 of the probability ----------------------
     float e[2][4];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      e[u][0] = dead_lo[u] ? -INFINITY : fmaf(c[u][0], scale2, -bm0);
-      e[u][1] = dead_lo[u] ? -INFINITY : fmaf(c[u][1], scale2, -bm1);
-      e[u][2] = dead_hi[u] ? -INFINITY : fmaf(c[u][2], scale2, -bm0);
-      e[u][3] = dead_hi[u] ? -INFINITY : fmaf(c[u][3], scale2, -bm1);
+      e[u][0] = dead_lo[u] ? -INFINITY : (DYN ? c[u][0] - m0 : fmaf(c[u][0], scale2, -bm0));
+      e[u][1] = dead_lo[u] ? -INFINITY : (DYN ? c[u][1] - m1 : fmaf(c[u][1], scale2, -bm1));
+      e[u][2] = dead_hi[u] ? -INFINITY : (DYN ? c[u][2] - m0 : fmaf(c[u][2], scale2, -bm0));
+      e[u][3] = dead_hi[u] ? -INFINITY : (DYN ? c[u][3] - m1 : fmaf(c[u][3], scale2, -bm1));
     }
     // A reference moves only when a score exceeds it by more than DA_HEADROOM (probabilities then stay
     // below 2^15, well inside fp16 and fp32 range; the reference is just a common exponent, the
     // merges below rescale by it). The first pass of a warp always takes this path (e = +inf).
     const float e_max = fmaxf(fmaxf(fmaxf(e[0][0], e[0][1]), fmaxf(e[0][2], e[0][3])), fmaxf(fmaxf(e[1][0], e[1][1]), fmaxf(e[1][2], e[1][3])));
-    if (__any_sync(0xffffffffu, e_max > DA_HEADROOM)) {
+    if (__any_sync(0xffffffffu, e_max > HEADROOM)) {
       float s[2][4];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        s[u][0] = dead_lo[u] ? -INFINITY : fmaf(c[u][0], scale2, -bias0);
-        s[u][1] = dead_lo[u] ? -INFINITY : fmaf(c[u][1], scale2, -bias1);
-        s[u][2] = dead_hi[u] ? -INFINITY : fmaf(c[u][2], scale2, -bias0);
-        s[u][3] = dead_hi[u] ? -INFINITY : fmaf(c[u][3], scale2, -bias1);
+        s[u][0] = dead_lo[u] ? -INFINITY : (DYN ? c[u][0] : fmaf(c[u][0], scale2, -bias0));
+        s[u][1] = dead_lo[u] ? -INFINITY : (DYN ? c[u][1] : fmaf(c[u][1], scale2, -bias1));
+        s[u][2] = dead_hi[u] ? -INFINITY : (DYN ? c[u][2] : fmaf(c[u][2], scale2, -bias0));
+        s[u][3] = dead_hi[u] ? -INFINITY : (DYN ? c[u][3] : fmaf(c[u][3], scale2, -bias1));
       }
       // maxima of heads 2t, 2t+1 over the 32 keys of this pass: over the eight lanes of equal t
       float x0 = fmaxf(fmaxf(s[0][0], s[0][2]), fmaxf(s[1][0], s[1][2])), x1 = fmaxf(fmaxf(s[0][1], s[0][3]), fmaxf(s[1][1], s[1][3]));
@@ -568,7 +628,7 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, d));
       }
       // a warp whose 32 keys all lie past the end keeps its reference (-inf - -inf would not be a number)
-      const float n0 = fmaxf(m0, x0), n1 = fmaxf(m1, x1);
+      const float n0 = fmaxf(m0, DYN ? x0 - 7.0f : x0), n1 = fmaxf(m1, DYN ? x1 - 7.0f : x1);
       const float a_lo = n0 == -INFINITY ? 1.0f : ex2(m0 - n0), a_hi = n1 == -INFINITY ? 1.0f : ex2(m1 - n1);
       m0 = n0, m1 = n1;
       bm0 = bias0 + m0, bm1 = bias1 + m1;
@@ -581,6 +641,18 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
         e[u][2] = n0 == -INFINITY ? -INFINITY : s[u][2] - m0, e[u][3] = n1 == -INFINITY ? -INFINITY : s[u][3] - m1;
       }
     }
+    float v_inv = 0.0f;
+    if (DYN) {
+      const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(sv_cur) & 0x7FFFFFFFu);
+      if (top > __float_as_uint(vref)) {
+        const float v_new = __uint_as_float(min((top >> 23) + 1u, 253u) << 23);
+        const float down = vref / v_new;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i][0] *= down, o[i][1] *= down, o[i][2] *= down, o[i][3] *= down;
+        vref = v_new;
+      }
+      v_inv = vref > 0.0f ? 1.0f / vref : 0.0f;
+    }
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int j0 = r0 + u * DA_CHUNK + 16 * warp;
@@ -588,10 +660,26 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
       const uint2 vc0 = lds64(vb + v_off), vc1 = lds64(vb + v_off + 64);
       const uint2 vc2 = lds64(vb + v_off + 8 * 64), vc3 = lds64(vb + v_off + 9 * 64);
       // P in fp16, transposed from (key, head pair) to the (key pair, head) layout of an MMA B operand
-      const uint32_t pb0 = movmatrix_trans(pack_half2(ex2(e[u][0]), ex2(e[u][1])));
-      const uint32_t pb1 = movmatrix_trans(pack_half2(ex2(e[u][2]), ex2(e[u][3])));
-      // the denominator sums the same fp16-rounded probabilities the output MMA multiplies with
-      mma_f16_16816_full(lacc, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u, pb0, pb1);
+      uint32_t pb0, pb1, lb0 = 0, lb1 = 0;
+      if (DYN) {
+        const float v_lo = __shfl_sync(0xffffffffu, sv_cur, 16 * u + g) * v_inv, v_hi = __shfl_sync(0xffffffffu, sv_cur, 16 * u + 8 + g) * v_inv;
+        float w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          w[i] = ex2(e[u][i]);
+          lacc[i & 1] += w[i];
+          w[i] *= i < 2 ? v_lo : v_hi;
+        }
+        const uint32_t h0 = pack_half2(w[0], w[1]), h1 = pack_half2(w[2], w[3]);
+        const float2 b0 = __half22float2(*reinterpret_cast<const __half2*>(&h0)), b1 = __half22float2(*reinterpret_cast<const __half2*>(&h1));
+        pb0 = movmatrix_trans(h0), pb1 = movmatrix_trans(h1);
+        lb0 = movmatrix_trans(pack_half2(w[0] - b0.x, w[1] - b0.y)), lb1 = movmatrix_trans(pack_half2(w[2] - b1.x, w[3] - b1.y));
+      } else {
+        pb0 = movmatrix_trans(pack_half2(ex2(e[u][0]), ex2(e[u][1])));
+        pb1 = movmatrix_trans(pack_half2(ex2(e[u][2]), ex2(e[u][3])));
+        // the denominator sums the same fp16-rounded probabilities the output MMA multiplies with
+        mma_f16_16816_full(lacc, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u, pb0, pb1);
+      }
       // ---- O^T += V^T P^T: rows = head dims, columns = query heads ------------------------------
       // A merged word pairs the same four dims of two neighbouring keys; its nibbles 0 and 2 give
       // exact codes, nibbles 1 and 3 give 16 * code (rows g+8 of the tile, rescaled at the end).
@@ -601,14 +689,14 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
         const uint32_t ya = __byte_perm(q4 < 2 ? vc0.x : vc0.y, q4 < 2 ? vc1.x : vc1.y, sel);
         const uint32_t yb = __byte_perm(q4 < 2 ? vc2.x : vc2.y, q4 < 2 ? vc3.x : vc3.y, sel);
         const uint32_t ya8 = ya >> 8, yb8 = yb >> 8;
-        mma_f16_16816_full(o[2 * q4], hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya), 0x64086408u),
-                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya), 0x64806480u),
-                           hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb), 0x64086408u),
-                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb), 0x64806480u), pb0, pb1);
-        mma_f16_16816_full(o[2 * q4 + 1], hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya8), 0x64086408u),
-                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya8), 0x64806480u),
-                           hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb8), 0x64086408u),
-                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb8), 0x64806480u), pb0, pb1);
+        const uint32_t a0 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya), 0x64086408u), a1 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya), 0x64806480u);
+        const uint32_t a2 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb), 0x64086408u), a3 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb), 0x64806480u);
+        mma_f16_16816_full(o[2 * q4], a0, a1, a2, a3, pb0, pb1);
+        if (DYN) mma_f16_16816_full(o[2 * q4], a0, a1, a2, a3, lb0, lb1);
+        const uint32_t b0 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya8), 0x64086408u), b1 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya8), 0x64806480u);
+        const uint32_t b2 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb8), 0x64086408u), b3 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb8), 0x64806480u);
+        mma_f16_16816_full(o[2 * q4 + 1], b0, b1, b2, b3, pb0, pb1);
+        if (DYN) mma_f16_16816_full(o[2 * q4 + 1], b0, b1, b2, b3, lb0, lb1);
       }
     }
     }  // round_ok
@@ -647,6 +735,14 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
             make_float2(o[m][hh], o[m][2 + hh] * 0.0625f);
     }
   }
+  if (DYN) {  // the lanes' shares of the denominators, and the warp's R
+#pragma unroll
+    for (int d = 4; d < 32; d <<= 1) {
+      lacc[0] += __shfl_xor_sync(0xffffffffu, lacc[0], d);
+      lacc[1] += __shfl_xor_sync(0xffffffffu, lacc[1], d);
+    }
+    if (lane == 0) sm_vref[DYN ? warp : 0] = vref;
+  }
   if (g == 0) {
     if (2 * t < G) sm_ml[warp][2 * t][0] = m0, sm_ml[warp][2 * t][1] = lacc[0];
     if (2 * t + 1 < G) sm_ml[warp][2 * t + 1][0] = m1, sm_ml[warp][2 * t + 1][1] = lacc[1];
@@ -672,7 +768,8 @@ __global__ void __launch_bounds__(DA_THREADS, 4) decode_attn_kernel(const AttnPa
         const float e = mw == -INFINITY ? 0.0f : ex2(mw - m);
         const float* src = sm_o + (w * DA_ROWS + r) * DA_SO_STRIDE + qpos;
         const float2 lo = *reinterpret_cast<const float2*>(src), hi = *reinterpret_cast<const float2*>(src + 16);
-        acc.x = fmaf(lo.x, e, acc.x), acc.y = fmaf(lo.y, e, acc.y), acc.z = fmaf(hi.x, e, acc.z), acc.w = fmaf(hi.y, e, acc.w);
+        const float ev = DYN ? e * sm_vref[DYN ? w : 0] : e;
+        acc.x = fmaf(lo.x, ev, acc.x), acc.y = fmaf(lo.y, ev, acc.y), acc.z = fmaf(hi.x, ev, acc.z), acc.w = fmaf(hi.y, ev, acc.w);
         l = fmaf(sm_ml[w][r][1], e, l);
       }
       // codes -> values; the prefix values below are already in value units
@@ -847,6 +944,12 @@ bool set_attn_smem() {
         cudaFuncSetAttribute(decode_attn_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              DA_SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(decode_attn_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             DA_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(decode_attn_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             DA_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(decode_attn_kernel<true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             DA_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(decode_attn_kernel<true, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              DA_SMEM_BYTES) != cudaSuccess)
       return false;
     done[dev] = true;
@@ -884,8 +987,6 @@ pq_status check_cache(const pq_kv4_cache* c) {
 
 pq_status pq_kv4_append_dyn_launch(pq_ctx* ctx, const pq_kv4_cache* c, const void* k, const void* v, int32_t T_new, int64_t ld_tok,
                                    cudaStream_t st);
-pq_status pq_decode_attn_dyn_launch(pq_ctx* ctx, const pq_kv4_cache* c, const void* q, void* out, float sm_scale, void* ws,
-                                    cudaStream_t st, int ticket0);
 
 extern "C" pq_status pq_kv4_append_strided(pq_ctx* ctx, const pq_kv4_cache* cache, const void* k, const void* v,
                                            int32_t T_new, int64_t ld_tok, void* stream) {
@@ -935,7 +1036,6 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   if (reinterpret_cast<uintptr_t>(ws) & 15) return PQ_ERR_ALIGN;
   if (is_dynamic(cache)) {
     if (k_new) return PQ_ERR_UNSUPPORTED;  // the one-launch decode step serves the static setting
-    return pq_decode_attn_dyn_launch(ctx, cache, q, out, sm_scale, ws, static_cast<cudaStream_t>(stream), DA_TICKET0);
   }
   int S = choose_splits(ctx, cache);
   // With enough (sequence, head) pairs, eight splits already fill the GPU: the splits then form one
@@ -960,6 +1060,8 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   p.vq = cache->vq;
   p.s_k = cache->s_k;
   p.s_v = cache->s_v;
+  p.sk_tok = cache->sk_tok;
+  p.sv_tok = cache->sv_tok;
   p.len = cache->len;
   p.ws_o = static_cast<float*>(ws);
   p.ws_ml = p.ws_o + static_cast<size_t>(cache->B) * cache->Hkv * n_parts * G * 128;
@@ -968,7 +1070,7 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   p.wait_clocks = ctx->wait_clocks;
   p.sm_scale = sm_scale;
   p.B = cache->B, p.Hq = cache->Hq, p.Hkv = cache->Hkv, p.G = G, p.n_prefix = cache->n_prefix, p.Tmax = cache->Tmax;
-  const bool fused = k_new != nullptr;
+  const bool fused = k_new != nullptr, dyn = is_dynamic(cache);
   p.k_new = static_cast<const __nv_bfloat16*>(k_new);
   p.v_new = static_cast<const __nv_bfloat16*>(v_new);
   p.len_rw = cache->len;
@@ -991,7 +1093,10 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
     cfg.attrs = attr;
     cfg.numAttrs = fused ? 2 : 1;  // the plain call gains nothing from an early placement (measured), the one-launch step does
     cudaError_t e;
-    if (multi)
+    if (dyn)
+      e = multi ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true, true>, p)
+                : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, false, true>, p);
+    else if (multi)
       e = fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, true, true>, p)
                 : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true>, p);
     else
@@ -1010,8 +1115,9 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = fused ? 1 : 0;
-  if ((fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, true, false>, p)
-             : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false>, p)) != cudaSuccess)
+  if ((dyn     ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false, true>, p)
+       : fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, true, false>, p)
+               : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false>, p)) != cudaSuccess)
     return PQ_ERR_CUDA;
   return pq_launch_status();
 }

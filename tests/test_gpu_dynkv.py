@@ -115,3 +115,30 @@ def test_dynamic_kv_refuses_overflow_and_the_static_only_calls(ctx):
     with pytest.raises(binding.PQError) as e:
         binding.decode_attn_noalloc(cache, q, 0.1, torch.empty_like(q))
     assert e.value.status == 7
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,P,T,Tmax,qs,vs", [
+    (1, 1, 1, 0, 1, 1, 1.0, 1.0), (2, 6, 2, 3, 127, 130, 2.0**17, 1.0), (1, 8, 1, 64, 129, 300, 2.0**-20, 2.0**-24),
+    (2, 10, 2, 1, 200, 201, 1.0, 2.0**40), (1, 16, 2, 4, 3000, 3001, 1.0, 2.0**-60), (40, 8, 1, 2, 90, 96, 1.0, 1.0),
+])
+def test_dynamic_kv_decode_attention_keeps_fp32_accuracy(ctx, B, Hq, Hkv, P, T, Tmax, qs, vs):
+    """Query and value magnitudes outside fp16's range, any head group, one split to several clusters. The weights enter the
+    output MMA as two fp16 terms (22 bits) and everything else is fp32: 2e-5 of the largest value, plus the bf16 store."""
+    from paper_2410_05265_b200 import binding
+
+    k, v = _scaled_kv(B, T, Hkv, 0, "k"), (_scaled_kv(B, T, Hkv, 0, "v").float() * vs).to(torch.bfloat16)
+    q = (inputs.queries(B, Hq, D, 0).float() * qs).to(torch.bfloat16)
+    pk = inputs.prefix_kv(Hkv, max(P, 1), D, 0, "k", 1.0)[:, :P].contiguous()
+    pv = inputs.prefix_kv(Hkv, max(P, 1), D, 0, "v", 1.0)[:, :P].contiguous()
+    kq = np.zeros((B, Hkv, Tmax, D // 2), np.uint8)
+    vq, sk, sv, length = np.zeros_like(kq), np.zeros((B, Hkv, Tmax), np.float32), np.zeros((B, Hkv, Tmax), np.float32), np.zeros(B, np.int32)
+    assert orc.kv4_append_dyn(inputs.bits(k), inputs.bits(v), kq, vq, sk, sv, length) == 0
+    sm = 1 / math.sqrt(D) / qs
+    _, ref = orc.decode_attn_dyn(inputs.bits(q), inputs.bits(pk), inputs.bits(pv), kq, vq, sk, sv, length, sm)
+    cache = binding.KV4Cache(pk.cuda() if P else None, pv.cuda() if P else None, dev(kq), dev(vq), None, None, dev(length), Hq, sk_tok=dev(sk),
+                             sv_tok=dev(sv))
+    out = ctx.decode_attn(cache, q.cuda(), sm, ctx.decode_attn_workspace(cache))
+    ctx.check()
+    got = out.double().cpu().numpy()
+    half_ulp = np.abs(got) * 2.0**-8
+    assert np.all(np.abs(got - ref) <= 2e-5 * np.abs(ref).max(-1, keepdims=True) + half_ulp)
