@@ -129,11 +129,14 @@ def load_library() -> ctypes.CDLL:
 
 
 def _ptr(t):
-    return c_void_p(t.data_ptr()) if t is not None else c_void_p(0)
+    return t.data_ptr() if t is not None else None  # the argument types turn the address (or None) into a pointer
+
+
+_current_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
 
 
 def _stream():
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(_current_device())  # what torch.cuda.current_stream().cuda_stream is, without building a Stream object
 
 
 def _ok(status: int, where: str):
@@ -283,7 +286,7 @@ class Context:
             _dev(acc_dbg, torch.int32, "acc_dbg")
             assert acc_dbg.shape == (M, N) and acc_dbg.is_contiguous()
         _ok(self.lib.pq_w4a4_gemm(self.h, _ptr(xq), _ptr(wq), _ptr(s_a), _ptr(s_w), _ptr(out), out.stride(0), M, N, K2 * 2,
-                                  row_begin, _ptr(acc_dbg), c_void_p(0), 0, _stream()), "pq_w4a4_gemm")
+                                  row_begin, _ptr(acc_dbg), None, 0, _stream()), "pq_w4a4_gemm")
         return out
 
     def rmsnorm_hadamard_quant_act(self, x: torch.Tensor, g: torch.Tensor, eps: float, s_a: torch.Tensor, row_begin: int = 0,
