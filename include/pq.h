@@ -126,10 +126,10 @@ pq_status pq_rmsnorm_hadamard_quant_act(pq_ctx* ctx, const void* x, int64_t M, i
  * smaller M mostly runs the weight-streaming kernel. No workspace is needed (ws may be NULL).
  * Weights are static (Sec. 3: quantized offline): below a few hundred rows the kernels start fetching wq
  * while the kernel before them in the stream is still draining (programmatic dependent launch), and
- * only xq, the scales and out are ordered behind that kernel. wq (and wsum of the _asym call)
- * must therefore be complete before the kernel that precedes this call in the stream starts.
- * Weights written earlier in the same stream by pq_quant_weights / pq_weight_code_sums or by a copy
- * always are: those never let a successor start early. This holds for pq_w4a4_gemm, pq_w4a8_gemm,
+ * only xq, the activation scales and out are ordered behind that kernel. Whatever writes wq and s_w (and wsum
+ * of the _asym call) in the same stream must therefore be a kernel that does not let its successors start
+ * before it has ended, however far back it is. Weights written by pq_quant_weights / pq_weight_code_sums, by a copy or
+ * by a kernel launched in the ordinary way are safe. This holds for pq_w4a4_gemm, pq_w4a8_gemm,
  * pq_w4a4_gemm_rows and pq_w4a4_gemm_asym alike. */
 size_t pq_w4a4_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K);
 pq_status pq_w4a4_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w,
@@ -245,10 +245,13 @@ pq_status pq_decode_attn_kv4_prefix(pq_ctx* ctx, const pq_kv4_cache* cache, cons
  * len[b] advances by one. If any sequence is full nothing is appended anywhere, the attention runs over the
  * cache as it is and PQ_ERR_SHAPE is reported through the status word. Arguments as in the two calls.
  * The kernel may be placed while its predecessor in the stream still runs (programmatic dependent launch) and
- * requests its first cache rows before it waits for that predecessor; only q, k and v are read after the wait.
- * The cache rows below len[b], the lengths and the steps must therefore not be written by the two kernels that
- * precede this call in the stream (in a decode loop their last writer is the same layer's call of the step
- * before, many kernels back). pq_decode_attn_kv4_prefix has no such condition: it waits before it reads anything. */
+ * requests its first cache rows, and reads the lengths, the steps and the prefix, before it waits for that
+ * predecessor; only q, k and v are read after the wait. Whatever writes those in the same stream must therefore be a
+ * kernel that does not let its successors start before it has ended (no griddepcontrol.launch_dependents, or
+ * cudaTriggerProgrammaticLaunchCompletion, in it), however far back it is. This holds for every call of this library
+ * that writes them (the appends, pq_rope_kv4_append, this call, pq_calib_kv_scale), for copies and for kernels launched
+ * in the ordinary way, so these may stand in any order. pq_decode_attn_kv4_prefix has no such condition: it waits
+ * before it reads anything. */
 pq_status pq_kv4_append_decode_attn(pq_ctx* ctx, const pq_kv4_cache* cache, const void* k, const void* v, const void* q,
                                     void* out, float sm_scale, void* ws, size_t ws_bytes, void* stream);
 

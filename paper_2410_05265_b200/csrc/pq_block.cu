@@ -202,8 +202,7 @@ __global__ void __launch_bounds__(RP_THREADS)
   for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
     rope_angles(pos0 + t, log2_theta, cs, sn);
     if (t == blockIdx.x) {  // the angles need nothing from the previous kernel
-      pq::pdl_wait();
-      pq::pdl_trigger();
+      pq::pdl_wait();       // and no trigger: this kernel writes cache rows and the length (see pq_launch_pdl)
       len0 = __ldcg(len);
       bad = len0 < 0 || len0 + T > Tmax;  // every CTA reaches the same verdict: then nothing is appended
     }

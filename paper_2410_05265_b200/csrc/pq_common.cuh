@@ -44,6 +44,12 @@ static inline pq_status pq_launch_status() { return cudaGetLastError() == cudaSu
 // 395 / 376, per-token set at 1000 253 / 243, W4A8 set at 300 137 / 129; 8B block at 515 tokens 243 / 228, at 1500 418 / 398,
 // at 128 tokens (graph) 115 / 105; decode layer, one sequence at 4000 tokens, 62.2 / 60.0. With every kernel triggering early
 // the 515-token block took 238 us in a graph against 224.
+//
+// Kernels that write KV-cache rows, lengths or steps (the appends and the one-launch decode step), packed weights or code sums
+// never trigger. Some kernels read these ahead of their own wait (the one-launch decode step its first cache rows and lengths,
+// the streaming and split-K GEMMs their weights), and several pass an early start on ahead of their wait (the rotation kernels,
+// those GEMMs): a writer that triggers could then still be running any number of launches further down the stream. One that
+// does not has ended before anything behind it in the stream starts.
 #define PQ_PDL_MAX_CTAS 64
 template <typename... P, typename... A>
 static inline pq_status pq_launch_pdl(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
@@ -65,7 +71,7 @@ namespace pq {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel be placed, from a small grid (see pq_launch_pdl). Issued behind pdl_wait(): whoever starts early then finds
-// everything before this kernel complete.
+// everything before this kernel complete. Not in kernels whose output a later kernel may read ahead of its wait.
 __device__ __forceinline__ void pdl_trigger() {
   if (gridDim.x * gridDim.y <= PQ_PDL_MAX_CTAS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

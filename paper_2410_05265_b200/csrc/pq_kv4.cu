@@ -275,12 +275,14 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   const uint8_t* vbase = p.vq + static_cast<int64_t>(bh) * p.Tmax * 64;
   const uint32_t stage_addr = pq::smem_u32(da_stage);
 
-  // Programmatic dependent launch: the next kernel of the stream may be placed as this one's CTAs retire. What this
-  // kernel reads that its predecessor may have written (everything for the plain call; the query and the new token
-  // for the one-launch decode step, whose cache rows and lengths are older than that by its contract) is read after
-  // griddepcontrol.wait; the one-launch form requests its first cache rows ahead of the wait.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (!FUSED) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // Programmatic dependent launch: the plain call lets the next kernel of the stream be placed as its CTAs retire. The
+  // one-launch decode step does not, because it writes a cache row and the lengths: the step requests its first cache
+  // rows and reads the lengths ahead of griddepcontrol.wait, so whoever writes those may not let a successor start early
+  // (see pq_launch_pdl). The query and the new token are read after the wait; the plain call reads everything after it.
+  if (!FUSED) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+  }
 
   // ---- every small load of the set-up goes out before the first bulk copy: behind the copies of all
   // the CTAs it would wait for megabytes of cache to be served first
