@@ -85,6 +85,7 @@ constexpr int DA_MAX_PREFIX = 64;
 constexpr int DA_ROWS = 8;  // query heads per KV head the MMA tile can carry
 constexpr int DA_TICKET0 = 16;
 constexpr float DA_HEADROOM = 15.0f;  // log2 units a score may exceed the reference exponent before it is moved
+constexpr float DA_HEADROOM_DYN = 4.0f;  // DYN: P * step * code stays within 2^7 of the largest cached value
 constexpr int DA_ROUND = 128;                     // keys staged per round (one half of the staging buffer)
 constexpr int DA_CHUNK = 64;                      // keys per bulk copy and per barrier
 constexpr int DA_CHUNKS = DA_ROUND / DA_CHUNK;
@@ -122,12 +123,25 @@ __device__ __forceinline__ uint32_t hsub2_u32(uint32_t a, uint32_t b) {
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
-// Two codes of a word as exact fp16 integers: nibbles 0 (even) or 1 (odd) of its 16-bit halves.
-__device__ __forceinline__ uint32_t codes_even(uint32_t w) { return hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(w), 0x64086408u); }
-__device__ __forceinline__ uint32_t codes_odd(uint32_t w) {  // (1152 + 16 code) / 16 - 72
+// DYN: the bf16 form of the same MMA, and two codes of a word as exact bf16 integers: nibble I of its 16-bit halves under
+// the exponent of 128 (bf16 has seven fraction bits: 136 + code), less 136.
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                               uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+template <int I>
+__device__ __forceinline__ uint32_t codes_bf16(uint32_t w) {
   uint32_t d;
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(and_xor<0x00F000F0u, 0x64806480u>(w)), "r"(0x2C002C00u), "r"(0xD480D480u));
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(and_xor<0x000F000Fu, 0x43084308u>(w >> (4 * I))), "r"(0x43084308u));
   return d;
+}
+// The upper halves of two fp32 words, their bf16 values rounded towards zero; a and b keep what is missing.
+__device__ __forceinline__ uint32_t take_bf16(float& a, float& b) {
+  const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+  a -= __uint_as_float(ua & 0xFFFF0000u), b -= __uint_as_float(ub & 0xFFFF0000u);
+  return __byte_perm(ua, ub, 0x7632);
 }
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   __half2 h = __floats2half2_rn(lo, hi);
@@ -239,15 +253,16 @@ struct AttnParams {
 // every len[b]. As with the two calls, nothing is appended anywhere when any sequence is full.
 // MULTI (with CLUSTER): a (sequence, head) has several clusters of eight splits.
 // DYN (group-wise dynamic KV, Table 1 O1): every cached vector has its own step. The setting's arithmetic is that of fp32:
-//   scores   codes as exact fp16 integers (one more half2 operation per word pair, no offset to cancel) times the query row
-//            scaled by a power of two into fp16's normal range (a bf16 value is then exact), then the key's step in fp32;
-//   output   the weight of a value row is P * step / R, R a power of two above any value step the warp has seen (it and
-//            the accumulators move together); it enters the MMA as two fp16 terms, hi + lo (22 bits), so twice the MMAs;
-//   the denominator is summed in fp32 on the CUDA cores. P is 2^7 at the row's maximum, which keeps lo above fp16's denormals.
+//   scores   codes as exact bf16 integers (one more operation per word pair, no offset to cancel) times the query as it is
+//            (bf16), then the key's step in fp32;
+//   output   the weight of a value row, P * step in fp32, enters the MMA as three bf16 terms whose sum it is exactly (8 + 8 + 8
+//            significand bits, fp32's exponent range), so thrice the MMAs: nothing depends on how the steps of the cache compare;
+//   the denominator is summed in fp32 on the CUDA cores.
 // A warp reads the steps of its 32 keys one round ahead (one key per lane) and hands them round with shuffles. What bounds it is
-// the per-round chain of the static form, with twice the output MMAs and three CTAs per SM. 8 x 4092 keys, 32 heads: 91.8 us for
-// the CUDA-core fp32 kernel this replaces, 22.9 now; 6 x 1500: 42.9 -> 9.0; one sequence of 30000 keys, 64 heads: 105 -> 20.4
-// (the bf16 outputs differ from the exact result's rounding in 2e-4 to 5e-4 of the elements, as before).
+// the per-round chain of the static form, with thrice the output MMAs and three CTAs per SM (151 registers). us for the CUDA-core
+// fp32 kernel this replaced / now: 8 x 4092 keys, 32 heads: 92 / 24; 6 x 1500: 43 / 9.6; one sequence of 30000 keys, 64 heads:
+// 105 / 24. A form with the weights as two fp16 terms relative to the largest step seen took 25.5, 9.6 and 23.6 us (40 ragged
+// sequences of up to 3000 keys, 64 heads: 50 / 55 now), but lost bits, up to all of them, where one step of the cache was far above the rest.
 template <bool CLUSTER, bool FUSED, bool MULTI = false, bool DYN = false>
 __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(const AttnParams p) {
   extern __shared__ __align__(128) uint8_t da_stage[];  // DA_SLOTS slots of [K rows | V rows] of one round
@@ -259,7 +274,6 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   __shared__ float2 cl_ml[DA_ROWS];
   __shared__ __align__(8) uint64_t full[DA_SLOTS][DA_CHUNKS];
   __shared__ float sm_ml[DA_WARPS][DA_ROWS][2];
-  __shared__ float sm_vref[DYN ? DA_WARPS : 1];         // DYN: what a warp's output accumulators are multiples of
   __shared__ float sm_pre[DA_ROWS][DA_MAX_PREFIX + 1];  // the last column: the key appended by this call
   __shared__ float sm_newv[FUSED ? 128 : 1];             // its dequantized value
   __shared__ float sm_red[DA_WARPS][DA_ROWS];
@@ -460,27 +474,24 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
     }
   }
 
-  // ---- query fragments (fp16 B operand of the score MMA: k = head dims, n = query heads) ----------
+  // ---- query fragments (fp16 or, DYN, bf16 B operand of the score MMA: k = head dims, n = query heads) ----------
   // A 32-bit word of a packed key row holds the codes of dims 8W..8W+7; nibble i of its low half is
   // dim 8W+i, nibble i of its high half dim 8W+4+i. Fragment j of a lane holds (q[D], q[D+4]) in its first and
-  // (q[D+1], q[D+5]) / 16 in its second register with D = 32t + 8(j>>1) + 2(j&1), of head g: the k rows
+  // (q[D+1], q[D+5]) / 16 (DYN: not divided) in its second register with D = 32t + 8(j>>1) + 2(j&1), of head g: the k rows
   // 2t, 2t+1 and 2t+8, 2t+9 of score MMA j.
   uint32_t qb[8][2];
   float q_even = 0.0f, q_odd = 0.0f;
-  float q_up = 1.0f, q_down = 1.0f;  // DYN: the row's power of two (largest magnitude near 2^8) and its inverse
   if (DYN) {
-    uint32_t mx = 0;
 #pragma unroll
-    for (int w = 0; w < 4; ++w)
-      mx = __vmaxu2(mx, __vmaxu2(__vmaxu2(q_raw[w].x & 0x7FFF7FFFu, q_raw[w].y & 0x7FFF7FFFu), __vmaxu2(q_raw[w].z & 0x7FFF7FFFu, q_raw[w].w & 0x7FFF7FFFu)));
-    mx = max(mx & 0xFFFFu, mx >> 16);
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const int ex = min(max(static_cast<int>(mx >> 7), 9), 253);  // biased exponent of the largest magnitude
-    q_up = __uint_as_float(static_cast<uint32_t>(min(254 + 8 - ex, 254)) << 23);
-    q_down = 1.0f / q_up;
-  }
-  {
+    for (int w = 0; w < 4; ++w) {
+      const uint32_t ww[4] = {q_raw[w].x, q_raw[w].y, q_raw[w].z, q_raw[w].w};
+#pragma unroll
+      for (int jj = 0; jj < 2; ++jj) {
+        qb[2 * w + jj][0] = __byte_perm(ww[jj], ww[jj + 2], 0x5410);
+        qb[2 * w + jj][1] = __byte_perm(ww[jj], ww[jj + 2], 0x7632);
+      }
+    }
+  } else {
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       const uint4 v = q_raw[w];  // 8 bf16: d = 32t + 8w + 0..7
@@ -491,9 +502,8 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
 #pragma unroll
       for (int jj = 0; jj < 2; ++jj) {  // score MMA j = 2w + jj uses nibbles 2jj and 2jj + 1
         const int i0 = 2 * jj;
-        const float odd = DYN ? q_up : 0.0625f;
-        const __half2 a0 = DYN ? __floats2half2_rn(f[i0] * q_up, f[i0 + 4] * q_up) : __floats2half2_rn(f[i0], f[i0 + 4]);
-        const __half2 a2 = __floats2half2_rn(f[i0 + 1] * odd, f[i0 + 5] * odd);
+        const __half2 a0 = __floats2half2_rn(f[i0], f[i0 + 4]);
+        const __half2 a2 = __floats2half2_rn(f[i0 + 1] * 0.0625f, f[i0 + 5] * 0.0625f);
         qb[2 * w + jj][0] = *reinterpret_cast<const uint32_t*>(&a0);
         qb[2 * w + jj][1] = *reinterpret_cast<const uint32_t*>(&a2);
         // the offsets are removed with the values the MMA really multiplies
@@ -516,11 +526,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   // exist keeps a huge one: its probabilities are zero and it never asks for a move.
   float m0 = 2 * t < G ? -INFINITY : 1e30f, m1 = 2 * t + 1 < G ? -INFINITY : 1e30f;
   float bm0 = bias0 + m0, bm1 = bias1 + m1;  // what is subtracted from a raw score
-  // DYN: what a score of heads 2t, 2t + 1 is multiplied with beside the key's step
-  const float hs = p.sm_scale * 1.4426950408889634f * q_down;
-  const float hs0 = __shfl_sync(0xffffffffu, hs, 8 * t), hs1 = __shfl_sync(0xffffffffu, hs, 8 * t + 4);
-  constexpr float HEADROOM = DYN ? 14.0f : DA_HEADROOM;
-  float vref = 0.0f;  // DYN: R
+  constexpr float HEADROOM = DYN ? DA_HEADROOM_DYN : DA_HEADROOM;
   const float* skb = DYN ? p.sk_tok + static_cast<int64_t>(bh) * p.Tmax : nullptr;
   const float* svb = DYN ? p.sv_tok + static_cast<int64_t>(bh) * p.Tmax : nullptr;
   float sk_next = 0.0f, sv_next = 0.0f;
@@ -533,7 +539,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   if (DYN) load_steps(0);
 
   // Output accumulators of the transposed product: tile m holds, for this lane, o[m][0], o[m][1] =
-  // dim 16g+2m of heads 2t, 2t+1 and o[m][2], o[m][3] = 16 x dim 16g+2m+1 of the same heads.
+  // dim 16g+2m of heads 2t, 2t+1 and o[m][2], o[m][3] = 16 x (DYN: 1 x) dim 16g+2m+1 of the same heads.
   float o[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.0f;
@@ -582,8 +588,8 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
       for (int w = 0; w < 4; ++w) {
         const uint32_t wl8 = wl[w] >> 8, wh8 = wh[w] >> 8;
         if (DYN) {
-          mma_f16_16816_full(ca, codes_even(wl[w]), codes_even(wh[w]), codes_odd(wl[w]), codes_odd(wh[w]), qb[2 * w][0], qb[2 * w][1]);
-          mma_f16_16816_full(cb, codes_even(wl8), codes_even(wh8), codes_odd(wl8), codes_odd(wh8), qb[2 * w + 1][0], qb[2 * w + 1][1]);
+          mma_bf16_16816(ca, codes_bf16<0>(wl[w]), codes_bf16<0>(wh[w]), codes_bf16<1>(wl[w]), codes_bf16<1>(wh[w]), qb[2 * w][0], qb[2 * w][1]);
+          mma_bf16_16816(cb, codes_bf16<2>(wl[w]), codes_bf16<2>(wh[w]), codes_bf16<3>(wl[w]), codes_bf16<3>(wh[w]), qb[2 * w + 1][0], qb[2 * w + 1][1]);
           continue;
         }
         mma_f16_16816_full(ca, and_xor<0x000F000Fu, 0x64086408u>(wl[w]), and_xor<0x000F000Fu, 0x64086408u>(wh[w]),
@@ -596,8 +602,9 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
 #pragma unroll
       for (int i = 0; i < 4; ++i) c[u][i] = ca[i] + cb[i];
       if (DYN) {  // scores in log2 units
-        const float sk_lo = __shfl_sync(0xffffffffu, sk_cur, 16 * u + g), sk_hi = __shfl_sync(0xffffffffu, sk_cur, 16 * u + 8 + g);
-        c[u][0] *= sk_lo * hs0, c[u][1] *= sk_lo * hs1, c[u][2] *= sk_hi * hs0, c[u][3] *= sk_hi * hs1;
+        const float f = sk_cur * scale2;
+        const float f_lo = __shfl_sync(0xffffffffu, f, 16 * u + g), f_hi = __shfl_sync(0xffffffffu, f, 16 * u + 8 + g);
+        c[u][0] *= f_lo, c[u][1] *= f_lo, c[u][2] *= f_hi, c[u][3] *= f_hi;
       }
     }
     // ---- softmax against the reference exponents: e = log2 of the probability ----------------------
@@ -630,7 +637,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, d));
       }
       // a warp whose 32 keys all lie past the end keeps its reference (-inf - -inf would not be a number)
-      const float n0 = fmaxf(m0, DYN ? x0 - 7.0f : x0), n1 = fmaxf(m1, DYN ? x1 - 7.0f : x1);
+      const float n0 = fmaxf(m0, x0), n1 = fmaxf(m1, x1);
       const float a_lo = n0 == -INFINITY ? 1.0f : ex2(m0 - n0), a_hi = n1 == -INFINITY ? 1.0f : ex2(m1 - n1);
       m0 = n0, m1 = n1;
       bm0 = bias0 + m0, bm1 = bias1 + m1;
@@ -643,18 +650,6 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
         e[u][2] = n0 == -INFINITY ? -INFINITY : s[u][2] - m0, e[u][3] = n1 == -INFINITY ? -INFINITY : s[u][3] - m1;
       }
     }
-    float v_inv = 0.0f;
-    if (DYN) {
-      const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(sv_cur) & 0x7FFFFFFFu);
-      if (top > __float_as_uint(vref)) {
-        const float v_new = __uint_as_float(min((top >> 23) + 1u, 253u) << 23);
-        const float down = vref / v_new;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) o[i][0] *= down, o[i][1] *= down, o[i][2] *= down, o[i][3] *= down;
-        vref = v_new;
-      }
-      v_inv = vref > 0.0f ? 1.0f / vref : 0.0f;
-    }
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int j0 = r0 + u * DA_CHUNK + 16 * warp;
@@ -662,9 +657,9 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
       const uint2 vc0 = lds64(vb + v_off), vc1 = lds64(vb + v_off + 64);
       const uint2 vc2 = lds64(vb + v_off + 8 * 64), vc3 = lds64(vb + v_off + 9 * 64);
       // P in fp16, transposed from (key, head pair) to the (key pair, head) layout of an MMA B operand
-      uint32_t pb0, pb1, lb0 = 0, lb1 = 0;
+      uint32_t pb0, pb1, wb[3][2];  // DYN: wb, the three terms of P * step
       if (DYN) {
-        const float v_lo = __shfl_sync(0xffffffffu, sv_cur, 16 * u + g) * v_inv, v_hi = __shfl_sync(0xffffffffu, sv_cur, 16 * u + 8 + g) * v_inv;
+        const float v_lo = __shfl_sync(0xffffffffu, sv_cur, 16 * u + g), v_hi = __shfl_sync(0xffffffffu, sv_cur, 16 * u + 8 + g);
         float w[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -672,10 +667,8 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
           lacc[i & 1] += w[i];
           w[i] *= i < 2 ? v_lo : v_hi;
         }
-        const uint32_t h0 = pack_half2(w[0], w[1]), h1 = pack_half2(w[2], w[3]);
-        const float2 b0 = __half22float2(*reinterpret_cast<const __half2*>(&h0)), b1 = __half22float2(*reinterpret_cast<const __half2*>(&h1));
-        pb0 = movmatrix_trans(h0), pb1 = movmatrix_trans(h1);
-        lb0 = movmatrix_trans(pack_half2(w[0] - b0.x, w[1] - b0.y)), lb1 = movmatrix_trans(pack_half2(w[2] - b1.x, w[3] - b1.y));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) wb[i][0] = movmatrix_trans(take_bf16(w[0], w[1])), wb[i][1] = movmatrix_trans(take_bf16(w[2], w[3]));
       } else {
         pb0 = movmatrix_trans(pack_half2(ex2(e[u][0]), ex2(e[u][1])));
         pb1 = movmatrix_trans(pack_half2(ex2(e[u][2]), ex2(e[u][3])));
@@ -690,15 +683,25 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
         const uint32_t sel = (q4 & 1) ? 0x7632u : 0x5410u;
         const uint32_t ya = __byte_perm(q4 < 2 ? vc0.x : vc0.y, q4 < 2 ? vc1.x : vc1.y, sel);
         const uint32_t yb = __byte_perm(q4 < 2 ? vc2.x : vc2.y, q4 < 2 ? vc3.x : vc3.y, sel);
+        if (DYN) {
+          const uint32_t a0 = codes_bf16<0>(ya), a1 = codes_bf16<1>(ya), a2 = codes_bf16<0>(yb), a3 = codes_bf16<1>(yb);
+          const uint32_t b0 = codes_bf16<2>(ya), b1 = codes_bf16<3>(ya), b2 = codes_bf16<2>(yb), b3 = codes_bf16<3>(yb);
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            mma_bf16_16816(o[2 * q4], a0, a1, a2, a3, wb[i][0], wb[i][1]);
+            mma_bf16_16816(o[2 * q4 + 1], b0, b1, b2, b3, wb[i][0], wb[i][1]);
+          }
+          continue;
+        }
         const uint32_t ya8 = ya >> 8, yb8 = yb >> 8;
-        const uint32_t a0 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya), 0x64086408u), a1 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya), 0x64806480u);
-        const uint32_t a2 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb), 0x64086408u), a3 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb), 0x64806480u);
-        mma_f16_16816_full(o[2 * q4], a0, a1, a2, a3, pb0, pb1);
-        if (DYN) mma_f16_16816_full(o[2 * q4], a0, a1, a2, a3, lb0, lb1);
-        const uint32_t b0 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya8), 0x64086408u), b1 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya8), 0x64806480u);
-        const uint32_t b2 = hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb8), 0x64086408u), b3 = hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb8), 0x64806480u);
-        mma_f16_16816_full(o[2 * q4 + 1], b0, b1, b2, b3, pb0, pb1);
-        if (DYN) mma_f16_16816_full(o[2 * q4 + 1], b0, b1, b2, b3, lb0, lb1);
+        mma_f16_16816_full(o[2 * q4], hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya), 0x64086408u),
+                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya), 0x64806480u),
+                           hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb), 0x64086408u),
+                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb), 0x64806480u), pb0, pb1);
+        mma_f16_16816_full(o[2 * q4 + 1], hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(ya8), 0x64086408u),
+                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(ya8), 0x64806480u),
+                           hsub2_u32(and_xor<0x000F000Fu, 0x64086408u>(yb8), 0x64086408u),
+                           hsub2_u32(and_xor<0x00F000F0u, 0x64806480u>(yb8), 0x64806480u), pb0, pb1);
       }
     }
     }  // round_ok
@@ -734,16 +737,15 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
 #pragma unroll
       for (int m = 0; m < 8; ++m)
         *reinterpret_cast<float2*>(sm_o + (warp * DA_ROWS + head) * DA_SO_STRIDE + 16 * m + 2 * g) =
-            make_float2(o[m][hh], o[m][2 + hh] * 0.0625f);
+            make_float2(o[m][hh], DYN ? o[m][2 + hh] : o[m][2 + hh] * 0.0625f);
     }
   }
-  if (DYN) {  // the lanes' shares of the denominators, and the warp's R
+  if (DYN) {  // the lanes' shares of the denominators
 #pragma unroll
     for (int d = 4; d < 32; d <<= 1) {
       lacc[0] += __shfl_xor_sync(0xffffffffu, lacc[0], d);
       lacc[1] += __shfl_xor_sync(0xffffffffu, lacc[1], d);
     }
-    if (lane == 0) sm_vref[DYN ? warp : 0] = vref;
   }
   if (g == 0) {
     if (2 * t < G) sm_ml[warp][2 * t][0] = m0, sm_ml[warp][2 * t][1] = lacc[0];
@@ -770,8 +772,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
         const float e = mw == -INFINITY ? 0.0f : ex2(mw - m);
         const float* src = sm_o + (w * DA_ROWS + r) * DA_SO_STRIDE + qpos;
         const float2 lo = *reinterpret_cast<const float2*>(src), hi = *reinterpret_cast<const float2*>(src + 16);
-        const float ev = DYN ? e * sm_vref[DYN ? w : 0] : e;
-        acc.x = fmaf(lo.x, ev, acc.x), acc.y = fmaf(lo.y, ev, acc.y), acc.z = fmaf(hi.x, ev, acc.z), acc.w = fmaf(hi.y, ev, acc.w);
+        acc.x = fmaf(lo.x, e, acc.x), acc.y = fmaf(lo.y, e, acc.y), acc.z = fmaf(hi.x, e, acc.z), acc.w = fmaf(hi.y, e, acc.w);
         l = fmaf(sm_ml[w][r][1], e, l);
       }
       // codes -> values; the prefix values below are already in value units

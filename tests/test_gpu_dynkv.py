@@ -122,8 +122,8 @@ def test_dynamic_kv_refuses_overflow_and_the_static_only_calls(ctx):
     (2, 10, 2, 1, 200, 201, 1.0, 2.0**40), (1, 16, 2, 4, 3000, 3001, 1.0, 2.0**-60), (40, 8, 1, 2, 90, 96, 1.0, 1.0),
 ])
 def test_dynamic_kv_decode_attention_keeps_fp32_accuracy(ctx, B, Hq, Hkv, P, T, Tmax, qs, vs):
-    """Query and value magnitudes outside fp16's range, any head group, one split to several clusters. The weights enter the
-    output MMA as two fp16 terms (22 bits) and everything else is fp32: 2e-5 of the largest value, plus the bf16 store."""
+    """Query and value magnitudes outside fp16's range, any head group, one split to several clusters. Everything is held in
+    fp32 or exactly: 2e-5 of the largest value, plus the bf16 store."""
     from paper_2410_05265_b200 import binding
 
     k, v = _scaled_kv(B, T, Hkv, 0, "k"), (_scaled_kv(B, T, Hkv, 0, "v").float() * vs).to(torch.bfloat16)
@@ -137,6 +137,46 @@ def test_dynamic_kv_decode_attention_keeps_fp32_accuracy(ctx, B, Hq, Hkv, P, T, 
     _, ref = orc.decode_attn_dyn(inputs.bits(q), inputs.bits(pk), inputs.bits(pv), kq, vq, sk, sv, length, sm)
     cache = binding.KV4Cache(pk.cuda() if P else None, pv.cuda() if P else None, dev(kq), dev(vq), None, None, dev(length), Hq, sk_tok=dev(sk),
                              sv_tok=dev(sv))
+    out = ctx.decode_attn(cache, q.cuda(), sm, ctx.decode_attn_workspace(cache))
+    ctx.check()
+    got = out.double().cpu().numpy()
+    half_ulp = np.abs(got) * 2.0**-8
+    assert np.all(np.abs(got - ref) <= 2e-5 * np.abs(ref).max(-1, keepdims=True) + half_ulp)
+
+
+@pytest.mark.parametrize("T,Tmax,Hq,Hkv", [(33, 40, 4, 2), (700, 704, 8, 2), (3000, 3001, 16, 2)])
+@pytest.mark.parametrize("case", ["zero value vector", "large unattended value", "unread query channel"])
+@pytest.mark.parametrize("exponent", [12, 24, 40])
+def test_dynamic_kv_decode_attention_with_magnitudes_far_apart_in_one_cache(ctx, case, exponent, T, Tmax, Hq, Hkv):
+    """A vector or channel that contributes nothing must not cost the others precision, however much larger it is: an all-zero
+    value vector (step 1, codes 0) beside values near 2^-exponent, a value vector 2^exponent times the others whose key no query attends to,
+    a query channel 2^exponent times the others that no key uses. Bound as above."""
+    from paper_2410_05265_b200 import binding
+
+    B, scale = 1, 2.0**exponent
+    k, v = inputs.kv_tensor(B, T, Hkv, D, 0, "k").float(), inputs.kv_tensor(B, T, Hkv, D, 0, "v").float()
+    q = inputs.queries(B, Hq, D, 0).float()
+    at = T // 3
+    if case == "zero value vector":
+        v = v / scale
+        v[0, at] = 0
+    elif case == "large unattended value":  # every query has one sign in the first channel, that key the other: score below -70
+        q[..., 0] = 8.0 + q[..., 0].abs()
+        k[..., 0] *= 0.1
+        k[0, at] = 0
+        k[0, at, :, 0] = -100.0
+        v[0, at] *= scale
+    else:
+        q[..., 5] = scale
+        k[..., 5] = 0
+    k, v, q = k.to(torch.bfloat16), v.to(torch.bfloat16), q.to(torch.bfloat16)
+    kq = np.zeros((B, Hkv, Tmax, D // 2), np.uint8)
+    vq, sk, sv, length = np.zeros_like(kq), np.zeros((B, Hkv, Tmax), np.float32), np.zeros((B, Hkv, Tmax), np.float32), np.zeros(B, np.int32)
+    assert orc.kv4_append_dyn(inputs.bits(k), inputs.bits(v), kq, vq, sk, sv, length) == 0
+    none = np.zeros((Hkv, 0, D), np.uint16)
+    sm = 1 / math.sqrt(D)
+    _, ref = orc.decode_attn_dyn(inputs.bits(q), none, none, kq, vq, sk, sv, length, sm)
+    cache = binding.KV4Cache(None, None, dev(kq), dev(vq), None, None, dev(length), Hq, sk_tok=dev(sk), sv_tok=dev(sv))
     out = ctx.decode_attn(cache, q.cuda(), sm, ctx.decode_attn_workspace(cache))
     ctx.check()
     got = out.double().cpu().numpy()
