@@ -68,6 +68,7 @@ struct Cfg {
   static_assert(A_COL0 + SLOTS * A_SLOT_COLS <= TMEM_COLS, "tensor memory budget");
   static_assert(STAGES % GROUPS == 0 && X_STAGES % GROUPS == 0 && SLOTS % GROUPS == 0, "a ring slot is always served by the same group");
   static_assert(PART <= RING, "the partial tile fits where the rings were");
+  static_assert(SLOTS <= STAGES, "no weight stage is refilled before the first operand slot is");
 };
 
 struct __align__(8) SplitBarriers {
@@ -325,6 +326,8 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
     const int gt = q * 32 + lane;  // thread of the group = channel row of the tile = lane of tensor memory
     for (int it = group; it < total; it += C::GROUPS) {
       const int ps = it % C::STAGES, xs = it % C::X_STAGES, ss = it % C::SLOTS;
+      // A refilled stage or slot (SLOTS <= STAGES) comes back behind the previous kernel only: the bounded waits start there.
+      if (it >= C::SLOTS && it < C::SLOTS + C::GROUPS) asm volatile("griddepcontrol.wait;" ::: "memory");
       if (!wait_bar_warp(&bars->w_full[ps], (it / C::STAGES) & 1, abort_flag, p.wait_clocks)) {
         ok = false;
         break;
@@ -334,8 +337,6 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
 #pragma unroll
       for (int j = 0; j < 4; ++j)  // 64-byte swizzle of the landing buffer: the row-per-thread reads hit distinct banks
         w[j] = *reinterpret_cast<const uint4*>(src + gt * PK_ROW + ((j ^ ((gt >> 1) & 3)) << 4));
-      if (it >= C::SLOTS && it < C::SLOTS + C::GROUPS)
-        asm volatile("griddepcontrol.wait;" ::: "memory");  // slots come back once the tokens are there: the bounded wait starts behind them
       if (!wait_bar_warp(&bars->s8_empty[ss], ((it / C::SLOTS) & 1) ^ 1, abort_flag, p.wait_clocks)) {
         ok = false;
         break;

@@ -91,3 +91,41 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     _, refp = orc.prefill_attn(inputs.bits(qp), inputs.bits(pk), inputs.bits(pv), kq_np[1], vq_np[1], s_k, s_v, sm, want_f64=True)
     assert_attn_close(inputs.bits(outp), refp, "prefill attention after a timed-out call")
     ctx.close()
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8"])
+@pytest.mark.parametrize("M", [16, 40, 96, 128, 200])
+def test_a_slow_predecessor_does_not_count_against_the_bounded_waits(mode, M):
+    """A GEMM placed early (split-K kernel, many K blocks per CTA) behind a kernel that runs several times longer than the wait
+    limit, though each of its own waits is short (causal attention, 128 key tiles in sequence): nothing is stuck, no timeout."""
+    from paper_2410_05265_b200 import binding
+
+    ctx = binding.Context()
+    rng = np.random.default_rng(M)
+    N, K, T, D = 640, 16384, 16384, 128
+    wq = rand_codes(rng, N, K)
+    if M == 16:  # up to 16 tokens only large layers take that kernel
+        wq = np.concatenate([wq, wq, wq])[:1408]
+    if mode == "w4a8":
+        x8 = rng.integers(-128, 128, (M, K)).astype(np.int8)
+        ref, call, xq = orc.gemm_i8i4(x8, wq), ctx.w4a8_gemm, dev(x8)
+    else:
+        x4 = rand_codes(rng, M, K)
+        ref, call, xq = orc.gemm_i4(x4, wq), ctx.w4a4_gemm, dev(x4)
+    kq = torch.randint(0, 256, (1, 1, T, D // 2), dtype=torch.uint8, device="cuda")
+    s = torch.full((1,), 0.3, device="cuda")
+    cache = binding.KV4Cache(None, None, kq, kq.clone(), s, s, torch.full((1,), T, dtype=torch.int32, device="cuda"), 1)
+    q = torch.randn((T, 1, D), device="cuda").to(torch.bfloat16)
+    s_a, s_w = torch.full((1,), 0.02, device="cuda"), torch.full((wq.shape[0],), 0.003, device="cuda")
+    acc, wq = torch.zeros(ref.shape, dtype=torch.int32, device="cuda"), dev(wq)
+    out, attn = torch.empty(ref.shape, dtype=torch.bfloat16, device="cuda"), torch.empty_like(q)
+    for limit in (0, 60_000):                   # the first pass loads the kernels
+        ctx.set_wait_limit(limit)
+        for _ in range(3):
+            acc.zero_()
+            torch.cuda.synchronize()
+            ctx.prefill_attn(cache, 0, q, 1 / math.sqrt(D), out=attn)
+            call(xq, wq, s_a, s_w, out=out, acc_dbg=acc)
+            assert ctx.check_status() == 0
+            assert np.array_equal(to_np(acc), ref)
+    ctx.close()
