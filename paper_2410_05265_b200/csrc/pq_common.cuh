@@ -76,6 +76,23 @@ __device__ __forceinline__ void pdl_trigger() {
   if (gridDim.x * gridDim.y <= PQ_PDL_MAX_CTAS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Loads of what an earlier kernel in the stream may have written, behind pdl_wait(). Not __ldg, nor a plain load through a const
+// __restrict__ pointer: the compiler takes such data for unchanging and may move the load ahead of the wait (the per-token step of the
+// streaming GEMM was read there: in a graph the GEMM behind the two-launch dynamic quantizer saw the zeros the step array starts
+// from, and its outputs were zero). Volatile assembly keeps its order.
+__device__ __forceinline__ uint32_t ld_dep(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_dep(const float* p) { return __uint_as_float(ld_dep(reinterpret_cast<const uint32_t*>(p))); }
+__device__ __forceinline__ int32_t ld_dep(const int32_t* p) { return static_cast<int32_t>(ld_dep(reinterpret_cast<const uint32_t*>(p))); }
+__device__ __forceinline__ uint4 ld_dep(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ void report(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 
 // SiLU(g) * u in fp32 with the hardware exponential and reciprocal (about 2 ulp of fp32, far below the bf16

@@ -138,8 +138,8 @@ __device__ __forceinline__ void reduce_tile(const SplitParams& p, const uint8_t*
   const int n = n0 + 4 * lane;
   float sw[4];
   int zw[4];
-  const float s_a = p.s_row ? 1.0f : __ldg(p.s_a);
-  const int zp8 = ZP ? __ldg(p.zp) - 8 : 0;
+  const float s_a = p.s_row ? 1.0f : pq::ld_dep(p.s_a);
+  const int zp8 = ZP ? pq::ld_dep(p.zp) - 8 : 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     sw[i] = n + i < p.N ? s_a * __ldg(p.s_w + n + i) : 0.0f;
@@ -159,7 +159,7 @@ __device__ __forceinline__ void reduce_tile(const SplitParams& p, const uint8_t*
         if (PEERS == 1) v[u][r] = *reinterpret_cast<const int4*>(part + t * (CH * 4) + lane * 16);
         else v[u][r] = r < p.splits ? ld_cluster_int4(peer[r] + t * (CH * 4)) : make_int4(0, 0, 0, 0);
       }
-      rs[u] = p.s_row ? p.s_row[t0 + t] : 1.0f;  // may come from the previous kernel: no read-only load
+      rs[u] = p.s_row ? pq::ld_dep(p.s_row + t0 + t) : 1.0f;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {

@@ -112,11 +112,11 @@ __global__ void __launch_bounds__(GS_THREADS)
       const int ks = base + u * GS_WARPS;
       const int off = ks * 64;
       const bool in_k = ks < n_steps && off + t * 16 < kbytes;
-      b.xa[u] = (in_k && x0_ok) ? __ldg(reinterpret_cast<const uint4*>(x0p + off * XS)) : zero;
-      if (TWO_GROUPS) b.xb[u] = (in_k && x1_ok) ? __ldg(reinterpret_cast<const uint4*>(x1p + off * XS)) : zero;
+      b.xa[u] = (in_k && x0_ok) ? pq::ld_dep(reinterpret_cast<const uint4*>(x0p + off * XS)) : zero;
+      if (TWO_GROUPS) b.xb[u] = (in_k && x1_ok) ? pq::ld_dep(reinterpret_cast<const uint4*>(x1p + off * XS)) : zero;
       if (A8) {
-        b.xa2[u] = (in_k && x0_ok) ? __ldg(reinterpret_cast<const uint4*>(x0p + off * XS) + 1) : zero;
-        if (TWO_GROUPS) b.xb2[u] = (in_k && x1_ok) ? __ldg(reinterpret_cast<const uint4*>(x1p + off * XS) + 1) : zero;
+        b.xa2[u] = (in_k && x0_ok) ? pq::ld_dep(reinterpret_cast<const uint4*>(x0p + off * XS) + 1) : zero;
+        if (TWO_GROUPS) b.xb2[u] = (in_k && x1_ok) ? pq::ld_dep(reinterpret_cast<const uint4*>(x1p + off * XS) + 1) : zero;
       }
     }
   };
@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(GS_THREADS)
   int base = warp;
   if (base < n_steps) load_w(b0, base);               // static weights: requested ahead of the wait
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the token rows may come from the previous kernel
-  const float e_sa = e_ok ? __ldg(s_a + e_tok * sa_stride) : 0.0f;  // stride 1: one step per token
-  const int e_zp8 = (e_ok && zp) ? __ldg(zp) - 8 : 0;
+  const float e_sa = e_ok ? pq::ld_dep(s_a + e_tok * sa_stride) : 0.0f;  // stride 1: one step per token
+  const int e_zp8 = (e_ok && zp) ? pq::ld_dep(zp) - 8 : 0;
   if (base < n_steps) load_x(b0, base);
   if (DEEP) {
     Batch b1;

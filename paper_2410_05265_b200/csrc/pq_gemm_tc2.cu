@@ -340,11 +340,11 @@ __global__ void __launch_bounds__(N_THREADS, 1)
     // ------------------------------------------------------------------ epilogue warps
     constexpr int SHIFT = A8 ? 4 : 8;  // the factors 16 the expanded codes carry
     const int q = warp & 3;  // TMEM lane quarter this warp may access
-    const float s_a = p.s_row ? 1.0f : __ldg(p.s_a);
+    const float s_a = p.s_row ? 1.0f : pq::ld_dep(p.s_a);
     uint8_t* my_buf = epi_buf + q * EPI_BUFS * EPI_BUF;
     float* my_scale = scale_buf + q * BN;
     int32_t* my_zw = zw_buf + q * BN;
-    const int zp8 = ZP ? __ldg(p.zp) - 8 : 0;
+    const int zp8 = ZP ? pq::ld_dep(p.zp) - 8 : 0;
     uint32_t tcount = 0, n_store = 0;
     bool ok = true;
     for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++tcount) {
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         break;
       }
       pq::tc_fence_after();
-      const float rs = p.s_row ? (m0 + lane < p.M ? __ldg(p.s_row + m0 + lane) : 0.0f) : 1.0f;  // this lane's token step
+      const float rs = p.s_row ? (m0 + lane < p.M ? pq::ld_dep(p.s_row + m0 + lane) : 0.0f) : 1.0f;  // this lane's token step
       const uint32_t taddr = tmem_base + ab * BN + (static_cast<uint32_t>(q * 32) << 16);
       epilogue_tile<SHIFT, ZP, EPI_BUFS>(p, &tmap_out, taddr, m0, n0, lane, rs, my_scale, my_zw, my_buf, n_store,
                                          map_to_cta(&bars->acc_empty[ab], 0));

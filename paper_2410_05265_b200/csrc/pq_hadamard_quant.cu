@@ -86,9 +86,9 @@ __global__ void __launch_bounds__(HQ_THREADS, HQ_CTAS_PER_SM)
 
   const float norm = ROTATE ? __fdiv_rn(1.0f, __fsqrt_rn(static_cast<float>(B))) : 1.0f;
   float inv = norm;
-  if (!CALIB && !PER_TOKEN) inv = __fdiv_rn(norm, __ldg(s_a_in));
+  if (!CALIB && !PER_TOKEN) inv = __fdiv_rn(norm, pq::ld_dep(s_a_in));
   float cal_max = 0.0f, cal_lo = INFINITY, cal_hi = -INFINITY;
-  const int zp = (ZP && !CALIB) ? __ldg(zp_in) - 8 : 0;
+  const int zp = (ZP && !CALIB) ? pq::ld_dep(zp_in) - 8 : 0;
 
   // (row, block inside the row) of this thread's transform block: divided once, then advanced by the grid's stride
   // (a 64-bit division per iteration is a visible share of an instruction-bound kernel)
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(HQ_THREADS, HQ_CTAS_PER_SM)
     row_it += row_step, blk_it += blk_step;
     if (blk_it >= blocks_per_row) blk_it -= blocks_per_row, ++row_it;
     if (!CALIB && PER_TOKEN) {
-      const float s_row = __ldg(s_a_in + row);
+      const float s_row = pq::ld_dep(s_a_in + row);
       inv = __fdiv_rn(norm, s_row == 0.0f ? 1.0f : s_row);  // an all-zero row has no step: any will do
     }
 
@@ -115,12 +115,12 @@ __global__ void __launch_bounds__(HQ_THREADS, HQ_CTAS_PER_SM)
       const uint32_t* src = reinterpret_cast<const uint32_t*>(x + row * ldx + col0) + u;
       uint32_t w[32];
 #pragma unroll
-      for (int r = 0; r < 32; ++r) w[r] = active ? __ldg(src + r * (RSTRIDE / 2)) : 0u;
+      for (int r = 0; r < 32; ++r) w[r] = active ? pq::ld_dep(src + r * (RSTRIDE / 2)) : 0u;
       if (SWIGLU) {
         const uint32_t* src2 = reinterpret_cast<const uint32_t*>(x2 + row * ldx + col0) + u;
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
-          const uint32_t w2 = active ? __ldg(src2 + r * (RSTRIDE / 2)) : 0u;
+          const uint32_t w2 = active ? pq::ld_dep(src2 + r * (RSTRIDE / 2)) : 0u;
           const float a = swiglu_bf16(__uint_as_float(w[r] << 16), __uint_as_float(w2 << 16));
           const float b = swiglu_bf16(__uint_as_float(w[r] & 0xFFFF0000u), __uint_as_float(w2 & 0xFFFF0000u));
           V[r] = ROTATE ? make_float2(a + b, a - b) : make_float2(a, b);
@@ -239,10 +239,10 @@ __global__ void __launch_bounds__(HQ_THREADS, HQ_CTAS_PER_SM)
         for (int c = 0; c < n_cand; ++c) {
           float s, z;
           if (PER_TOKEN) {
-            const float s_row = __ldg(s_a_in + row);
-            s = s_row == 0.0f ? 1.0f : __fmul_rn(__ldg(reinterpret_cast<const float*>(x2) + c), s_row), z = 8.0f;
+            const float s_row = pq::ld_dep(s_a_in + row);
+            s = s_row == 0.0f ? 1.0f : __fmul_rn(pq::ld_dep(reinterpret_cast<const float*>(x2) + c), s_row), z = 8.0f;
           } else {
-            s = __ldg(s_a_in + c), z = static_cast<float>(__ldg(zp_in + c));
+            s = pq::ld_dep(s_a_in + c), z = static_cast<float>(pq::ld_dep(zp_in + c));
           }
           const float inv_s = __fdiv_rn(1.0f, s);
           float acc = 0.0f;
@@ -438,9 +438,9 @@ __global__ void __launch_bounds__(HQ_THREADS, HQW_CTAS_PER_SM)
 
   const float norm = __fdiv_rn(1.0f, __fsqrt_rn(static_cast<float>(B)));
   float inv = norm;
-  if (!CALIB && !PER_TOKEN) inv = __fdiv_rn(norm, __ldg(s_a_in));
+  if (!CALIB && !PER_TOKEN) inv = __fdiv_rn(norm, pq::ld_dep(s_a_in));
   float cal_max = 0.0f, cal_lo = INFINITY, cal_hi = -INFINITY;
-  const int zp = (ZP && !CALIB) ? __ldg(zp_in) - 8 : 0;
+  const int zp = (ZP && !CALIB) ? pq::ld_dep(zp_in) - 8 : 0;
   [[maybe_unused]] const bool out32 = (reinterpret_cast<uintptr_t>(xq) & 31) == 0;
 
   // words of a tensor with the element pitch of x, in the order the MMAs take them: wa[tau][m3 | k3 << 1]
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(HQ_THREADS, HQW_CTAS_PER_SM)
     for (int tau = 0; tau < 8; ++tau)
 #pragma unroll
       for (int v = 0; v < 4; ++v)
-        wa[tau][v] = on ? __ldg(src + ((tau << TAUS) | ((v & 1) << M3S) | ((v >> 1) << K3S)) / 2) : 0u;
+        wa[tau][v] = on ? pq::ld_dep(src + ((tau << TAUS) | ((v & 1) << M3S) | ((v >> 1) << K3S)) / 2) : 0u;
   };
 
   const int64_t gb_step = static_cast<int64_t>(gridDim.x) * G;
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(HQ_THREADS, HQW_CTAS_PER_SM)
     const int64_t row = active ? row_it : 0;
     const int64_t col0 = active ? blk_it * B : 0;
     if (!CALIB && PER_TOKEN && s_a_out == nullptr) {
-      const float s_row = __ldg(s_a_in + row);
+      const float s_row = pq::ld_dep(s_a_in + row);
       inv = __fdiv_rn(norm, s_row == 0.0f ? 1.0f : s_row);
     }
     [[maybe_unused]] uint32_t u[8][4];
@@ -614,10 +614,10 @@ __global__ void __launch_bounds__(HQ_THREADS, HQW_CTAS_PER_SM)
         for (int c = 0; c < n_cand; ++c) {
           float s, z;
           if (PER_TOKEN) {
-            const float s_row = __ldg(s_a_in + row);
-            s = s_row == 0.0f ? 1.0f : __fmul_rn(__ldg(reinterpret_cast<const float*>(x2) + c), s_row), z = 8.0f;
+            const float s_row = pq::ld_dep(s_a_in + row);
+            s = s_row == 0.0f ? 1.0f : __fmul_rn(pq::ld_dep(reinterpret_cast<const float*>(x2) + c), s_row), z = 8.0f;
           } else {
-            s = __ldg(s_a_in + c), z = static_cast<float>(__ldg(zp_in + c));
+            s = pq::ld_dep(s_a_in + c), z = static_cast<float>(pq::ld_dep(zp_in + c));
           }
           const float inv_s = __fdiv_rn(1.0f, s);
           float acc = 0.0f;

@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   auto load_q = [&]() {
     const uint4* q4 = reinterpret_cast<const uint4*>(p.q + (static_cast<int64_t>(b) * p.Hq + h * G + (row_ok ? g : 0)) * 128 + 32 * t);
 #pragma unroll
-    for (int w = 0; w < 4; ++w) q_raw[w] = row_ok ? __ldg(q4 + w) : make_uint4(0, 0, 0, 0);
+    for (int w = 0; w < 4; ++w) q_raw[w] = row_ok ? pq::ld_dep(q4 + w) : make_uint4(0, 0, 0, 0);
   };
   if (!FUSED) load_q();
   // the fused kernel writes the lengths at its end: it reads them past the read-only path
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
     const int r = ok ? pair / p.n_prefix : 0, j = ok ? pair % p.n_prefix : 0;
     const uint4* qr = reinterpret_cast<const uint4*>(p.q + (static_cast<int64_t>(b) * p.Hq + h * G + r) * 128 + 16 * sub);
     const uint4* kr = reinterpret_cast<const uint4*>(p.prefix_k + (static_cast<int64_t>(h) * p.n_prefix + j) * 128 + 16 * sub);
-    if (want_q) pre_q[0] = __ldg(qr), pre_q[1] = __ldg(qr + 1);
+    if (want_q) pre_q[0] = pq::ld_dep(qr), pre_q[1] = pq::ld_dep(qr + 1);
     if (want_k) pre_k[0] = __ldg(kr), pre_k[1] = __ldg(kr + 1);
   };
   load_pre(!FUSED, true);
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
       const uint4* qr = reinterpret_cast<const uint4*>(p.q + (static_cast<int64_t>(b) * p.Hq + h * G + r) * 128 + 16 * sub);
       const uint4* kr = reinterpret_cast<const uint4*>(p.prefix_k + (static_cast<int64_t>(h) * p.n_prefix + j) * 128 + 16 * sub);
       const bool early = pair0 == 0;
-      const uint4 qv[2] = {early ? pre_q[0] : __ldg(qr), early ? pre_q[1] : __ldg(qr + 1)};
+      const uint4 qv[2] = {early ? pre_q[0] : pq::ld_dep(qr), early ? pre_q[1] : pq::ld_dep(qr + 1)};
       const uint4 kv[2] = {early ? pre_k[0] : __ldg(kr), early ? pre_k[1] : __ldg(kr + 1)};
       float acc = 0.0f;
 #pragma unroll

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
         const int rq = i * PA_ROWS + (warp & 3) * 32 + it * 2 + (lane >> 4);
         const int tq = min(t0 + (rq >> lg), p.T - 1), hq = h * G + (rq & (G - 1));  // G is a power of two
         const uint4* src = reinterpret_cast<const uint4*>(p.q + static_cast<int64_t>(tq) * p.ldq + hq * 128) + c16;  // eight bf16: dims 8 c16 .. +7
-        asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"  // volatile: the sixteen requests go out before the first use
+        asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];"  // volatile: the sixteen requests go out before the first use
                      : "=r"(qv[it].x), "=r"(qv[it].y), "=r"(qv[it].z), "=r"(qv[it].w)
                      : "l"(src));
       }

@@ -2,9 +2,12 @@
 calls give with a synchronisation between them."""
 import math
 
+import numpy as np
 import pytest
 import torch
 
+from oracle import pq_oracle as orc
+from helpers import to_np
 from paper_2410_05265_b200 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -76,3 +79,167 @@ def test_cache_written_three_launches_back_is_seen_by_the_decode_step(ctx, T, ro
     for name, a, b in zip(("keys", "values", "lengths", "GEMM", "attention"), want, got):
         assert torch.equal(a, b), f"{name} differ from the synchronised calls"
     assert int(got[2]) == (T + 1 if writer == "rope_kv4_append" else T + 16)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K", [(1, 4096, 4096), (16, 5120, 4096), (24, 4096, 4096), (96, 4096, 4096), (200, 4096, 4096)])
+def test_weights_written_just_before_reach_two_gemms_in_a_row(ctx, mode, M, N, K):
+    """quantize weights (and sum their codes) -> rotate + quantize -> GEMM -> GEMM on other weights of the same quantizer call, back
+    to back: streaming and split-K kernels request weights ahead of the wait for their predecessor and let their successors start early
+    (up to 32 tokens). The buffers are overwritten in every pass: stale weights, sums or tokens would show."""
+    x = [inputs.activations(M, K, seed=s).cuda() for s in range(3)]
+    W = [inputs.weights(2 * N, K, seed=2 + s).cuda() for s in range(3)]
+    wq = torch.zeros((2 * N, K // 2), dtype=torch.uint8, device="cuda")
+    s_w, wsum = torch.zeros(2 * N, device="cuda"), torch.zeros(2 * N, dtype=torch.int32, device="cuda")
+    xq = torch.zeros((M, K if mode == "w4a8" else K // 2), dtype=torch.int8 if mode == "w4a8" else torch.uint8, device="cuda")
+    s_a, s_tok = torch.full((1,), 0.02 if mode == "w4a8" else 0.3, device="cuda"), torch.full((M,), 0.3, device="cuda")
+    z = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+    out = torch.zeros((2, M, N), dtype=torch.bfloat16, device="cuda")
+    acc = torch.zeros((3, 2, M, N), dtype=torch.int32, device="cuda")
+    seen = []
+    torch.cuda.synchronize()
+    for i in range(3):
+        ctx.quant_weights(W[i], out=(wq, s_w))
+        if mode == "asym":
+            assert ctx.lib.pq_weight_code_sums(ctx.h, wq.data_ptr(), 2 * N, K, wsum.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+            ctx.hadamard_quant_act_asym(x[i], K, s_a, z, out=xq)
+        elif mode == "w4a8":
+            ctx.hadamard_quant_act8(x[i], K, s_a, out=xq)
+        elif mode == "rows":
+            ctx.hadamard_quant_act_rows(x[i], K, s_tok, out=xq)
+        else:
+            ctx.hadamard_quant_act(x[i], K, s_a, out=xq)
+        for h in range(2):
+            rows = slice(h * N, (h + 1) * N)
+            kw = dict(out=out[h], acc_dbg=acc[i, h])
+            if mode == "asym":
+                ctx.w4a4_gemm_asym(xq, wq[rows], s_a, z, s_w[rows], wsum[rows], **kw)
+            elif mode == "w4a8":
+                ctx.w4a8_gemm(xq, wq[rows], s_a, s_w[rows], **kw)
+            elif mode == "rows":
+                ctx.w4a4_gemm_rows(xq, wq[rows], s_tok, s_w[rows], **kw)
+            else:
+                ctx.w4a4_gemm(xq, wq[rows], s_a, s_w[rows], **kw)
+        seen.append((xq.clone(), wq.clone(), wsum.clone()))
+    ctx.check()
+    for i, (xc, wc, sums) in enumerate(seen):
+        ref = (orc.gemm_i8i4 if mode == "w4a8" else orc.gemm_i4)(to_np(xc), to_np(wc))
+        if mode == "asym":
+            codes = orc.unpack_int4(to_np(wc)).astype(np.int64).sum(1)
+            assert np.array_equal(to_np(sums), codes)
+            ref = ref - (5 - 8) * codes[None]
+        got = to_np(acc[i])
+        assert np.array_equal(np.concatenate([got[0], got[1]], 1), ref), f"pass {i}"
+
+
+@pytest.mark.parametrize("how", ["dynamic, two launches", "dynamic, one launch", "calibrated", "calibrated, 8 bits", "zero point"])
+@pytest.mark.parametrize("M,N", [(1, 4096), (2, 4096), (3, 4096), (4, 1024), (8, 4096), (12, 1024), (16, 4096), (24, 1024), (96, 4096), (200, 1024), (140, 8264)])
+def test_steps_and_codes_written_just_before_are_the_ones_used(ctx, how, M, N):
+    """step -> codes -> GEMM, every one reading what the launch before it wrote, replayed as one graph and called back to back, against
+    the calls with a synchronisation between them: steps, codes, sums and outputs bit for bit, with other activations every time."""
+    K = 4096 if how == "dynamic, one launch" else 6144          # 6144 = three blocks of 2048: steps and codes are two launches
+    block = K if K == 4096 else 2048
+    bits8 = how == "calibrated, 8 bits"
+    g = torch.Generator(device="cuda").manual_seed(M)
+    wq = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+    s_w, wsum = torch.full((N,), 1e-3, device="cuda"), ctx.weight_code_sums(wq)
+    xs = [(torch.randn((M, K), generator=g, device="cuda") * 3.0**i).to(torch.bfloat16) for i in range(5)]
+    x, s_tok, s_a = torch.zeros_like(xs[0]), torch.zeros(M, device="cuda"), torch.zeros(1, device="cuda")
+    z = torch.full((1,), 6, dtype=torch.int32, device="cuda")
+    xq = torch.zeros((M, K if bits8 else K // 2), dtype=torch.int8 if bits8 else torch.uint8, device="cuda")
+    out, acc = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda"), torch.zeros((M, N), dtype=torch.int32, device="cuda")
+
+    def chain(step):
+        kw = dict(out=out, acc_dbg=acc)
+        if how.startswith("dynamic"):
+            if step is not None and "two" in how:               # the same two launches, apart
+                ctx.dyn_act_scale(x, block, out=s_tok)
+                step()
+                ctx.hadamard_quant_act_rows(x, block, s_tok, out=xq)
+            else:
+                ctx.dyn_hadamard_quant_act(x, block, 1.0, 0, s_tok=s_tok, out=xq)
+            if step is not None:
+                step()
+            ctx.w4a4_gemm_rows(xq, wq, s_tok, s_w, **kw)
+            return
+        s_a.zero_()
+        calib, quant, gemm = ((ctx.calib_act_scale8, ctx.hadamard_quant_act8, ctx.w4a8_gemm) if bits8 else
+                              (ctx.calib_act_scale, ctx.hadamard_quant_act, ctx.w4a4_gemm))
+        calib(x, block, 0, s_a=s_a)
+        if step is not None:
+            step()
+        if how == "zero point":
+            ctx.hadamard_quant_act_asym(x, block, s_a, z, out=xq)
+        else:
+            quant(x, block, s_a, out=xq)
+        if step is not None:
+            step()
+        if how == "zero point":
+            ctx.w4a4_gemm_asym(xq, wq, s_a, z, s_w, wsum, **kw)
+        else:
+            gemm(xq, wq, s_a, s_w, **kw)
+
+    state = lambda: [t.clone() for t in (s_tok, s_a, xq, acc, out)]
+    want = []
+    for v in xs:
+        x.copy_(v)
+        torch.cuda.synchronize()
+        chain(torch.cuda.synchronize)
+        torch.cuda.synchronize()
+        want.append(state())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(None)
+    for name, call in (("graph", graph.replay), ("stream", lambda: chain(None))):
+        for i in (0, 1, 2, 3, 4, 0, 3, 1):
+            x.copy_(xs[i])
+            torch.cuda.synchronize()
+            call()
+            torch.cuda.synchronize()
+            for what, a, b in zip(("per-token steps", "step", "codes", "sums", "outputs"), state(), want[i]):
+                assert torch.equal(a, b), f"{what}, {name}, input {i}"
+    ctx.check()
+
+
+@pytest.mark.parametrize("T", [1, 200])
+def test_query_and_token_written_just_before_reach_the_decode_step(ctx, T):
+    """residual add (writes q, k, v of the step) -> one-launch decode step, in a graph, against the calls apart."""
+    from paper_2410_05265_b200 import binding
+
+    Hq, Hkv, Tmax = 8, 2, 256
+    n = (Hq + 2 * Hkv) * D
+    g = torch.Generator(device="cuda").manual_seed(T)
+    rand = lambda *sh: torch.randn(sh, generator=g, device="cuda").to(torch.bfloat16)
+    kq = torch.randint(0, 256, (1, Hkv, Tmax, D // 2), dtype=torch.uint8, device="cuda", generator=g)
+    s = torch.full((Hkv,), 0.3, device="cuda")
+    cache = binding.KV4Cache(rand(Hkv, 4, D).half(), rand(Hkv, 4, D).half(), kq, kq.clone(), s, s, torch.zeros(1, dtype=torch.int32, device="cuda"), Hq)
+    ws = ctx.decode_attn_workspace(cache)
+    base, a, y, out = rand(n), torch.zeros(n, dtype=torch.bfloat16, device="cuda"), torch.zeros(n, dtype=torch.bfloat16, device="cuda"), rand(1, Hq, D)
+    steps = [rand(n) for _ in range(5)]
+
+    def chain(sync):
+        ctx.residual_add(a, base, out=y)
+        if sync:
+            torch.cuda.synchronize()
+        ctx.kv4_append_decode_attn(cache, y[Hq * D: (Hq + Hkv) * D].view(1, 1, Hkv, D), y[(Hq + Hkv) * D:].view(1, 1, Hkv, D), y[: Hq * D].view(1, Hq, D),
+                                   1 / math.sqrt(D), ws, out=out)
+
+    def run(call):
+        res = []
+        for v in steps:
+            a.copy_(v)
+            cache.length.fill_(T)
+            torch.cuda.synchronize()
+            call()
+            torch.cuda.synchronize()
+            res.append((out.clone(), cache.kq.clone(), cache.vq.clone(), cache.length.clone()))
+        return res
+
+    want = run(lambda: chain(True))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(False)
+    for call in (graph.replay, lambda: chain(False)):
+        for w, r in zip(want, run(call)):
+            assert all(torch.equal(p, q) for p, q in zip(w, r))
+    ctx.check()

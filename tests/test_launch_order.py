@@ -46,3 +46,27 @@ def test_the_one_launch_decode_step_never_triggers():
     plain_only = block_from(body, body.index("if (!FUSED) {"))
     assert TRIGGER.search(plain_only)
     assert not TRIGGER.search(body.replace(plain_only, "")), "a trigger outside the branch of the plain call"
+
+
+@pytest.mark.parametrize("source,name", [
+    ("pq_gemm_stream.cu", "gemm_w4a4_stream_kernel"), ("pq_gemm_split.cu", "gemm_w4_split_kernel"), ("pq_gemm_tc2.cu", "gemm_w4a4_pair_kernel"),
+    ("pq_gemm_tc3.cu", "gemm_w4a4_pair_ts_kernel"), ("pq_hadamard_quant.cu", "hadamard_quant_kernel"),
+    ("pq_hadamard_quant.cu", "hadamard_quant_wide_kernel"), ("pq_kv4.cu", "decode_attn_kernel"), ("pq_prefill_attn.cu", "prefill_attn_kernel"),
+    ("pq_block.cu", "rmsnorm_kernel"), ("pq_block.cu", "rope_kernel"), ("pq_block.cu", "rope_rotate_kernel"), ("pq_block.cu", "silu_mul_kernel"),
+    ("pq_block.cu", "add_kernel"), ("pq_block.cu", "rope_kv4_append_kernel"),
+])
+def test_what_a_predecessor_may_write_is_not_read_through_the_read_only_path(source, name):
+    """The compiler may move a read-only load (__ldg, or one through a const __restrict__ pointer) ahead of the wait for the predecessor.
+    Only data that no early-triggering kernel writes may be read so: weights with their scales and sums, the cache with its steps and
+    prefix, norm weights."""
+    body = kernel_body(source, name)
+    if name == "gemm_w4_split_kernel":
+        with open(os.path.join(CSRC, source)) as f:
+            text = f.read()
+        body += block_from(text, text.index("void reduce_tile("))
+    static = re.compile(r"s_w|wsum|gsrc|\bgr\b|s_k|s_v|p\.len|prefix_|\bkr\b|skb|svb")
+    read_only = re.findall(r"__ldg\(((?:[^()]|\([^()]*\))*)\)", body) + re.findall(r'"ld\.global\.nc[^"]*"[^;]*"l"\((\w+)\)', body)
+    wrong = [a for a in read_only if not static.search(a)]
+    assert not wrong, wrong
+    if name.startswith("hadamard"):  # its parameters are const __restrict__: no plain load through them either
+        assert not re.search(r"\b(?:x|x2|s_a_in|zp_in)\[", body)
