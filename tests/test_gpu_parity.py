@@ -118,14 +118,15 @@ def _gemm_case(ctx, M, N, K, seed, row_begin=0, real_scales=True):
 
 
 @pytest.mark.parametrize("M,N,K", [
-    (128, 256, 128),     # one tile, one K block
-    (128, 256, 512),     # one tile, ring wraps
-    (256, 512, 4096),    # several tiles per CTA pipeline
+    # split-K kernel (the CTA-pair kernels at shapes like these: test_gpu_split_gemm.py, above the border)
+    (128, 256, 128),     # one K block
+    (128, 256, 512),
+    (256, 512, 4096),    # several clusters
     (200, 264, 416),     # ragged M, N and K (K % 128 != 0)
-    (17, 40, 160),       # smallest tensor-core case, mostly padding
+    (17, 40, 160),       # smallest tensor-core case on a small layer, mostly padding
     (333, 1000, 2048),
-    (300, 520, 8192),    # long K: the kernel that keeps the token operand in tensor memory
-    (257, 256, 14336),
+    (300, 520, 8192),
+    (257, 256, 14336),   # long K, eight splits
 ])
 def test_gemm_prefill_shapes_bit_exact(ctx, M, N, K):
     _gemm_case(ctx, M, N, K, seed=M + N + K)

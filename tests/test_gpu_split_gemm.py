@@ -1,5 +1,6 @@
-"""GPU parity of the split-K tensor-core GEMM (a few tens to a few hundred tokens) against the CPU oracle: every token-tile
-width and its edges, ragged channel counts and K tails, the four settings of the call, and the border to the CTA-pair kernels."""
+"""GPU parity of the tensor-core GEMMs against the CPU oracle. Split-K kernel (a few tens to a few hundred tokens): every
+token-tile width and its edges, ragged channel counts and K tails, the four settings of the call, and the border to the CTA-pair
+kernels. CTA-pair kernels at shapes above that border: ragged tiles, both kinds of output store, skipped rows, the ends of int32."""
 import numpy as np
 import pytest
 import torch
@@ -25,14 +26,14 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-def check(ctx, mode, M, N, K, ldo_pad=0):
+def check(ctx, mode, M, N, K, ldo_pad=0, row_begin=0):
     rng = np.random.default_rng(M * 1009 + N * 31 + K)
     wq, s_w = rand_codes(rng, N, K), rng.uniform(0.5, 2.0, N).astype(np.float32) * 1e-3
     s_a, s_tok = np.float32(0.02), rng.uniform(0.01, 0.03, M).astype(np.float32)
     out = torch.full((M, N + ldo_pad), 7.0, dtype=torch.bfloat16, device="cuda")
     view = out[:, :N]
-    acc = torch.zeros((M, N), dtype=torch.int32, device="cuda")
-    kw = dict(out=view, acc_dbg=acc)
+    acc = torch.full((M, N), -77, dtype=torch.int32, device="cuda")
+    kw = dict(out=view, acc_dbg=acc, row_begin=row_begin)
     sa = torch.full((1,), float(s_a), device="cuda")
     if mode == "w4a8":
         x8 = rng.integers(-128, 128, (M, K)).astype(np.int8)
@@ -50,10 +51,11 @@ def check(ctx, mode, M, N, K, ldo_pad=0):
         else:
             ctx.w4a4_gemm(dev(xq), dev(wq), sa, dev(s_w), **kw)
     ctx.check()
-    assert np.array_equal(to_np(acc), ref), "accumulators differ"
+    assert np.array_equal(to_np(acc)[row_begin:], ref[row_begin:]), "accumulators differ"
+    assert np.all(to_np(acc)[:row_begin] == -77) and bool((out[:row_begin] == 7.0).all()), "rows below row_begin must not be written"
     want = ref.astype(np.float64) * (s_tok.astype(np.float64)[:, None] if mode == "rows" else float(s_a)) * s_w.astype(np.float64)
     want = torch.from_numpy(want).to(torch.bfloat16)
-    assert_bf16_close(inputs.bits(view), inputs.bits(want), "split GEMM")
+    assert_bf16_close(inputs.bits(view[row_begin:]), inputs.bits(want[row_begin:]), f"{mode} GEMM {M} x {N} x {K}")
     if ldo_pad:
         assert bool((out[:, N:] == 7.0).all()), "columns past N must not be written"
 
@@ -85,3 +87,37 @@ def test_pair_kernels_just_above_the_border(ctx, mode, M, N, K):
     """Problems just too large for two K splits go to the CTA-pair kernels: ragged edges; K >= 8192 takes the kernel with the
     token operand in tensor memory."""
     check(ctx, mode, M, N, K)
+
+
+# ---- above the border: more than 128 rows and N > 8192 (65 and more channel tiles of 128) always go to the CTA-pair kernels
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K,pad,row_begin", [
+    (200, 8264, 416, 0, 4),        # dense rows, channels a multiple of 8: bulk-tensor stores; skipped rows
+    (141, 8203, 512, 0, 5),        # channels not a multiple of 8: element-wise stores
+    (150, 8264, 1152, 4, 0),       # rows too far apart for the bulk stores' 16-byte pitch
+    (137, 8203, 8224, 3, 1),       # the same with the token operand in tensor memory (K >= 8192; W4A8 keeps shared memory)
+    (290, 10241, 8192, 0, 7),      # more tiles than CTA pairs, element-wise stores
+    (260, 20000, 160, 0, 0),       # more tiles than CTA pairs, two K blocks
+])
+def test_pair_kernels_match_oracle(ctx, mode, M, N, K, pad, row_begin):
+    check(ctx, mode, M, N, K, pad, row_begin)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows"])
+@pytest.mark.parametrize("K", [4096, 28672, 65536])
+def test_pair_kernels_extreme_codes_fit_int32(ctx, mode, K):
+    """Every code at its lowest: the largest sums, and with the factors 16 of the expanded codes 2^30 at K = 65536."""
+    M, N = 130, 8208
+    wq = torch.full((N, K // 2), 0x88, dtype=torch.uint8, device="cuda")
+    one, s_w = torch.ones(1, device="cuda"), torch.ones(N, device="cuda")
+    acc = torch.zeros((M, N), dtype=torch.int32, device="cuda")
+    if mode == "w4a8":
+        ctx.w4a8_gemm(torch.full((M, K), -128, dtype=torch.int8, device="cuda"), wq, one, s_w, acc_dbg=acc)
+    else:
+        xq = torch.full((M, K // 2), 0x88, dtype=torch.uint8, device="cuda")
+        if mode == "rows":
+            ctx.w4a4_gemm_rows(xq, wq, torch.ones(M, device="cuda"), s_w, acc_dbg=acc)
+        else:
+            ctx.w4a4_gemm(xq, wq, one, s_w, acc_dbg=acc)
+    ctx.check()
+    assert int(acc.min()) == int(acc.max()) == 8 * K * (128 if mode == "w4a8" else 8)

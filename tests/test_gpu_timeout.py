@@ -45,12 +45,15 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     ctx = binding.Context()
     rng = np.random.default_rng(0)
     D = 128
-    # operands of a one-tile GEMM with short K (token operand in shared memory) and with long K (in tensor memory)
+    # split-K GEMM with a few and with many K blocks per CTA; CTA-pair GEMMs (more than 128 rows and 64 channel tiles) with short K
+    # (token operand in shared memory), with long K (in tensor memory) and with 8-bit tokens (a producer of their own)
     gemms = []
-    for M, N, K in [(128, 256, 512), (128, 256, 32768)]:
-        xq, wq = rand_codes(rng, M, K), rand_codes(rng, N, K)
-        gemms.append((dev(xq), dev(wq), orc.gemm_i4(xq, wq)))
-    s_a, s_w = torch.full((1,), 0.02, device="cuda"), torch.full((256,), 0.003, device="cuda")
+    for M, N, K, a8 in [(128, 256, 512, False), (128, 256, 32768, False), (96, 256, 32768, True), (129, 8448, 4096, False), (129, 8448, 8192, False),
+                        (129, 8448, 4096, True)]:
+        wq = rand_codes(rng, N, K)
+        xq = rng.integers(-128, 128, (M, K)).astype(np.int8) if a8 else rand_codes(rng, M, K)
+        gemms.append((ctx.w4a8_gemm if a8 else ctx.w4a4_gemm, dev(xq), dev(wq), orc.gemm_i8i4(xq, wq) if a8 else orc.gemm_i4(xq, wq)))
+    s_a, s_w_all = torch.full((1,), 0.02, device="cuda"), torch.full((8448,), 0.003, device="cuda")
     # a small KV4 cache for the decode and the prefill attention
     B, Hq, Hkv, T, Tmax, P = 2, 8, 2, 300, 320, 4
     kq_np, vq_np = rng.integers(0, 256, (B, Hkv, Tmax, D // 2)).astype(np.uint8), rng.integers(0, 256, (B, Hkv, Tmax, D // 2)).astype(np.uint8)
@@ -65,8 +68,8 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
 
     ctx.set_wait_limit(16)                      # a few clocks: no copy from memory is that fast
     seen = []
-    for xq, wq, _ in gemms:
-        ctx.w4a4_gemm(xq, wq, s_a, s_w)
+    for gemm, xq, wq, _ in gemms:
+        gemm(xq, wq, s_a, s_w_all[: wq.shape[0]])
         seen.append(ctx.check_status())
         assert ctx.check_status() == 0          # reading the status word clears it
     ctx.decode_attn(cache, q.cuda(), sm, ws)
@@ -75,12 +78,12 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     seen.append(ctx.check_status())
     torch.cuda.synchronize()                    # the process and the CUDA context are alive
     assert all(st in (0, PQ_ERR_TIMEOUT) for st in seen), seen
-    print("statuses under a 16-clock bound (GEMM short K, GEMM long K, decode attention, prefill attention):", seen)
+    print("statuses under a 16-clock bound (six GEMMs, decode attention, prefill attention):", seen)
 
     ctx.set_wait_limit(0)                       # the default bound again: exact results from the same context
-    for xq, wq, acc_ref in gemms:
+    for gemm, xq, wq, acc_ref in gemms:
         acc = torch.zeros(acc_ref.shape, dtype=torch.int32, device="cuda")
-        ctx.w4a4_gemm(xq, wq, s_a, s_w, acc_dbg=acc)
+        gemm(xq, wq, s_a, s_w_all[: wq.shape[0]], acc_dbg=acc)
         assert ctx.check_status() == 0 and np.array_equal(to_np(acc), acc_ref)
     out = ctx.decode_attn(cache, q.cuda(), sm, ws)
     assert ctx.check_status() == 0
