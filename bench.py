@@ -467,7 +467,7 @@ def section_config0(ctx, device, peaks):
     return {"rotate_quant_us": round(ms_q * 1e3, 3), "gemm_us": round(ms_g * 1e3, 3), "chained_us": round(ms_b * 1e3, 3),
             "gemm_TOPS": round(ops / (ms_g * 1e-3) / 1e12, 1), "chained_TOPS": round(ops / (ms_b * 1e-3) / 1e12, 1),
             "rotate_quant_GBs": round(2.5 * M * K / (ms_q * 1e-3) / 1e9, 1),
-            "note": "launch-bound: 16 tiles of 256 x 256 on 74 CTA pairs, operands resident in L2 across the repeated calls"}
+            "note": "split-K kernel (32 channel tiles, each expanding every token row), operands resident in L2 across the repeated calls"}
 
 
 def section_decode_gemm(ctx, device, peaks):
@@ -588,7 +588,7 @@ def section_decode_attention(ctx, device, peaks):
     return {"attention_us": round(ms_attn * 1e3, 3), "append_us": round(ms_app * 1e3, 3), "append+attention_us": round(ms_both * 1e3, 3),
             "append+attention_one_launch_us": round(ms_fused * 1e3, 3),
             "groupwise_dynamic_kv (Table 1 O1)": {"attention_us": round(ms_dyn_attn * 1e3, 3), "append_us": round(ms_dyn_app * 1e3, 3),
-                                                  "note": "per-vector steps (+2 MB of step reads), plain fp32 kernel: the setting the static path is compared with"},
+                                                  "note": "per-vector steps (+2 MB of step reads), every operand exact or fp32: the setting the static path is compared with"},
             "append+attention_one_launch_frac_measured_hbm": round(by / (ms_fused * 1e-3) / 1e9 / peaks["hbm"], 3),
             "long_context_b1_hq64_t32764": {"attention_us": round(ms_long * 1e3, 3),
                                             "frac_measured_hbm": round(by_long / (ms_long * 1e-3) / 1e9 / peaks["hbm"], 3)},
@@ -891,6 +891,12 @@ def run_case(args):
         out = torch.zeros((M, N), dtype=torch.bfloat16, device=dev)
         fn = lambda: ctx.w4a8_gemm(xq8, wq, s_a, s_w, out=out)
         work = 2.0 * M * N * K
+    elif name == "quant":
+        N, K = dims or [28672, 4096]
+        W = inputs.weights(N, K, seed=2).to(dev)
+        bufs = torch.empty((N, K // 2), dtype=torch.uint8, device=dev), torch.empty((N,), dtype=torch.float32, device=dev)
+        fn = lambda: ctx.quant_weights(W, out=bufs)
+        work = 2.5 * N * K
     elif name == "hadamard8":
         M, K, B = dims or [8192, 14336, 2048]
         x = inputs.activations(M, K, seed=0, device=dev)
@@ -951,7 +957,7 @@ def run_case(args):
 
 def main():
     ap = argparse.ArgumentParser()
-    ap.add_argument("--case", default=None, help="run one kernel on a small case: gemm:M,N,K | hadamard:M,K,B | attn:B,Hq,Hkv,T,layers | prefill:T,Hq,Hkv")
+    ap.add_argument("--case", default=None, help="run one kernel on a small case: gemm:M,N,K | gemm8:M,N,K | quant:N,K | hadamard:M,K,B | attn:B,Hq,Hkv,T,layers | prefill:T,Hq,Hkv")
     ap.add_argument("--gpus", type=int, default=1)
     ap.add_argument("--steps", type=int, default=1000)
     ap.add_argument("--warmup", type=int, default=3)

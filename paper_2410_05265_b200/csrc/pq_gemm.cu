@@ -30,9 +30,13 @@ static pq_status run_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, con
   //                    weight requests win: whole 70B layer 124 / 132 us
   //   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
   //                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
-  //   up to 128        always split (the CTA-pair kernels: 33 tokens, 4096 x 4096: 23.1 / 8.5, 28672 x 4096: 40.8 / 18.2)
+  //   up to 128        always split (the CTA-pair kernels: 33 tokens, 4096 x 4096: 23.1 / 8.5, 28672 x 4096: 40.8 / 18.2; the widest layer,
+  //                    57344 x 8192: 65 tokens 108 / 75, 128 tokens 112 / 85, W4A8 109 / 70)
   //   above            while the 256-token tiles leave room for two K splits: whole 8B block at 200 tokens 176.5 / 132.1, at 300
-  //                    tokens 201 / 175; with a single split (515 tokens) the o layer gains 2.3 and the down layer loses 8.6.
+  //                    tokens 201 / 175 (8192 x 8192 at 256 tokens: 35 / 23, W4A8 34 / 22; 4096 x 14336 at 512: 53 / 33, W4A8 53 / 31).
+  //                    With a single split it goes either way: 57344 x 8192 at 200 tokens 113 / 127, 28672 x 4096 at 300 64 / 71,
+  //                    10240 x 8192 at 200 36 / 32 (W4A8 111 / 113, 56 / 64, 35 / 29); at 515 tokens the o layer gains 2.3 and the
+  //                    down layer loses 8.6.
   const int64_t ctiles = (N + 127) / 128, weights = N * K;
   const bool split = m <= 8     ? false
                      : m <= 16  ? weights >= (int64_t{20} << 20)
@@ -71,8 +75,8 @@ extern "C" pq_status pq_w4a4_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t*
   return run_gemm(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, stream, false, nullptr, nullptr, nullptr);
 }
 
-// W4A8 (Sec. 5.1): the token operand is one s8 code per element: the weight-streaming kernel for up to 16
-// tokens, the CTA-pair tensor-core kernel above that.
+// W4A8 (Sec. 5.1): the token operand is one s8 code per element. The kernels and the rule are those of the 4-bit calls,
+// but for long K: the CTA-pair kernel with the token operand in shared memory serves every K.
 extern "C" pq_status pq_w4a8_gemm(pq_ctx* ctx, const int8_t* xq8, const uint8_t* wq, const float* s_a,
                                   const float* s_w, void* out, int64_t ldo, int64_t M, int64_t N, int64_t K,
                                   int64_t row_begin, int32_t* acc_dbg, void* stream) {
