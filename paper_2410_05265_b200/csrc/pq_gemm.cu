@@ -3,11 +3,10 @@
 #include "pq_common.cuh"
 
 pq_status pq_gemm_pair_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w,
-                              void* out, int64_t ldo, int64_t M, int64_t N, int64_t K, int32_t* acc_dbg, cudaStream_t st,
-                              bool a8, const float* s_row, const int32_t* zp, const int32_t* wsum);
+                              void* out, int64_t ldo, int64_t M, int64_t N, int64_t K, int32_t* acc_dbg, cudaStream_t st);
 pq_status pq_gemm_pair_ts_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w,
                                  void* out, int64_t ldo, int64_t M, int64_t N, int64_t K, int32_t* acc_dbg, cudaStream_t st,
-                                 const float* s_row, const int32_t* zp, const int32_t* wsum);
+                                 bool a8, const float* s_row, const int32_t* zp, const int32_t* wsum);
 pq_status pq_gemm_stream_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a,
                                 const float* s_w, void* out, int64_t ldo, int64_t M, int64_t N, int64_t K,
                                 int32_t* acc_dbg, cudaStream_t st, bool per_token, bool a8, const int32_t* zp,
@@ -30,27 +29,28 @@ static pq_status run_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, con
   //                    weight requests win: whole 70B layer 124 / 132 us
   //   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
   //                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
-  //   up to 128        always split (the CTA-pair kernels: 33 tokens, 4096 x 4096: 23.1 / 8.5, 28672 x 4096: 40.8 / 18.2; the widest layer,
-  //                    57344 x 8192: 65 tokens 108 / 75, 128 tokens 112 / 85, W4A8 109 / 70)
-  //   above            while the 256-token tiles leave room for two K splits: whole 8B block at 200 tokens 176.5 / 132.1, at 300
-  //                    tokens 201 / 175 (8192 x 8192 at 256 tokens: 35 / 23, W4A8 34 / 22; 4096 x 14336 at 512: 53 / 33, W4A8 53 / 31).
-  //                    With a single split it goes either way: 57344 x 8192 at 200 tokens 113 / 127, 28672 x 4096 at 300 64 / 71,
-  //                    10240 x 8192 at 200 36 / 32 (W4A8 111 / 113, 56 / 64, 35 / 29); at 515 tokens the o layer gains 2.3 and the
-  //                    down layer loses 8.6.
+  //   up to 96         always split (CTA pairs: 40 tokens, 28672 x 4096: 23.0 / 19.8; 8192 x 28672: 59.5 / 31.6)
+  //   97 to 128        while every channel tile has its CTAs at once (128 tokens, pairs against split, 57344 x 8192: 74.6 / 85.7,
+  //                    28672 x 4096: 25.1 / 27.0; but 10240 x 8192: 25.3 / 23.5)
+  //   above            while the 256-token tiles leave room for two K splits (pairs against split at 256 tokens: 8192 x 8192 26.0 / 23.5,
+  //                    4096 x 14336 35.7 / 24.2, 6144 x 4096 17.4 / 17.2; at 400, 4096 x 14336 37.8 / 31.9, 4096 x 4096 17.7 / 17.3). With a single
+  //                    split the pairs win: 57344 x 8192 at 200 tokens 91 / 129, 28672 x 4096 30.1 / 39.3, 10240 x 8192 31.5 / 35.8, 6144 x 4096
+  //                    at 300 17.9 / 21.7, 4096 x 14336 at 515 39.2 / 49.4.
   const int64_t ctiles = (N + 127) / 128, weights = N * K;
   const bool split = m <= 8     ? false
                      : m <= 16  ? weights >= (int64_t{20} << 20)
-                     : m <= 128 ? true
+                     : m <= 96  ? true
+                     : m <= 128 ? ctiles <= ctx->sm_count
                                 : 2 * ((m + 255) / 256) * ctiles <= ctx->sm_count * 7 / 8;
   if (split) return pq_gemm_split_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, a8, s_row, zp, wsum);
   if (m <= 16)
     return pq_gemm_stream_launch(ctx, xq, wq, s_row ? s_row : s_a, s_w, out, ldo, m, N, K, dbg, st, s_row != nullptr, a8, zp, wsum);
-  // Two CTA-pair kernels (every 4-bit setting takes the same choice): with the token operand in shared memory the accumulator is
-  // double-buffered and the epilogue is free, which wins for short K; with the token operand in tensor memory the expansion costs
-  // a third less shared-memory traffic, which wins once a tile's K loop is long enough to hide the single accumulator's epilogue
-  // (measured crossover near K = 8192).
-  if (!a8 && K >= 8192) return pq_gemm_pair_ts_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, s_row, zp, wsum);
-  return pq_gemm_pair_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, a8, s_row, zp, wsum);
+  // CTA pairs. Few rounds of 8-bit tiles, and 4-bit tokens always: weights in tensor memory, tiles as wide as fit the chip
+  // (pq_gemm_tc3.cu). More than three rounds of 8-bit tiles at K <= 8192: both operands in shared memory, two whole accumulators
+  // (pq_gemm_tc2.cu, with the figures).
+  const int64_t tiles = ((m + 255) / 256) * ((N + 255) / 256);
+  if (a8 && K <= 8192 && tiles > 3 * (ctx->sm_count / 2)) return pq_gemm_pair_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st);
+  return pq_gemm_pair_ts_launch(ctx, xq, wq, s_a, s_w, out, ldo, m, N, K, dbg, st, a8, s_row, zp, wsum);
 }
 
 extern "C" size_t pq_w4a4_gemm_workspace_bytes(int64_t, int64_t, int64_t) { return 0; }
@@ -75,8 +75,8 @@ extern "C" pq_status pq_w4a4_gemm(pq_ctx* ctx, const uint8_t* xq, const uint8_t*
   return run_gemm(ctx, xq0, wq, s_a, s_w, out0, ldo, m, N, K, dbg0, stream, false, nullptr, nullptr, nullptr);
 }
 
-// W4A8 (Sec. 5.1): the token operand is one s8 code per element. The kernels and the rule are those of the 4-bit calls,
-// but for long K: the CTA-pair kernel with the token operand in shared memory serves every K.
+// W4A8 (Sec. 5.1): the token operand is one s8 code per element. The kernels and the rule are those of the 4-bit calls
+// but for the largest launches (see run_gemm).
 extern "C" pq_status pq_w4a8_gemm(pq_ctx* ctx, const int8_t* xq8, const uint8_t* wq, const float* s_a,
                                   const float* s_w, void* out, int64_t ldo, int64_t M, int64_t N, int64_t K,
                                   int64_t row_begin, int32_t* acc_dbg, void* stream) {

@@ -1,7 +1,6 @@
-// What the two CTA-pair GEMM kernels share: the cluster / tensor-memory / bulk-store wrappers, the launch parameters,
-// the epilogue of a tile (tensor memory -> exact shift -> optional zero-point term -> scale -> bf16 -> swizzled
-// staging -> TMA store) and the host-side tensor maps. The kernels differ in how the token operand reaches the MMA
-// (shared memory in pq_gemm_tc2.cu, tensor memory in pq_gemm_tc3.cu) and in their accumulator buffering.
+// What the tensor-core GEMM kernels share: the cluster / tensor-memory / bulk-store wrappers, the bounded waits, the host-side tensor
+// maps; and the launch parameters and tile epilogue of the kernel in pq_gemm_tc2.cu (tensor memory -> exact shift -> scale -> bf16 ->
+// swizzled staging -> TMA store).
 #pragma once
 
 #include "pq_common.cuh"
@@ -17,9 +16,6 @@ constexpr int EPI_COLS = 64;                // columns per TMA store (128 bytes 
 constexpr int EPI_BUF = 32 * EPI_COLS * 2;  // 4 KB: one warp's 32 rows x 64 columns
 
 struct GemmParams {
-  const int32_t* zp;    // ZP kernels: the activation zero point z (device scalar) ...
-  const int32_t* wsum;  // ... and the sum of every output channel's weight codes [N]
-  const float* s_row;  // per-token steps [M] (dynamic setting) or null: the scalar s_a applies
   const float* s_a;
   const float* s_w;
   __nv_bfloat16* out;
@@ -120,31 +116,24 @@ __device__ __forceinline__ void bulk_wait_read() {
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // ---- epilogue -------------------------------------------------------------------------------------
-// ZP (Eq. 1 as printed): the stored token codes are u - 8 for unsigned codes u with zero point z; what the
-// layer needs is sum_k (u - z) w = sum_k (u - 8) w - (z - 8) sum_k w, so the epilogue subtracts (z - 8) * wsum[n]
-// from the exact integer sum before scaling.
-// This warp's copy of the dequantization factors of a tile's 256 columns (and of those correction terms).
-template <bool ZP>
-__device__ __forceinline__ void fill_tile_scales(const GemmParams& p, int n0, int lane, float s_a, int zp8, float* my_scale,
-                                                 int32_t* my_zw) {
+// This warp's copy of the dequantization factors of a tile's 256 columns.
+__device__ __forceinline__ void fill_tile_scales(const GemmParams& p, int n0, int lane, float s_a, float* my_scale) {
 #pragma unroll
   for (int i = 0; i < BN / 32; ++i) {
     const int col = n0 + i * 32 + lane;
     my_scale[i * 32 + lane] = col < p.N ? s_a * __ldg(p.s_w + col) : 0.0f;
-    if (ZP) my_zw[i * 32 + lane] = col < p.N ? zp8 * __ldg(p.wsum + col) : 0;
   }
   __syncwarp();
 }
 
 // One warp's 32 rows x 256 columns of an accumulator at tensor-memory address taddr: row m0 + lane of the output.
-// SHIFT removes the factors 16 the expanded codes carry (exact). `rs` is the lane's token step (1 in the static
-// setting). After the last column block has been read, lane 0 arrives on `acc_empty` (a cluster address in the
+// SHIFT removes the factors 16 the expanded codes carry (exact). After the last column block has been read, lane 0 arrives on `acc_empty` (a cluster address in the
 // leader CTA), which hands the accumulator back to the MMA warp. n_store counts this warp's TMA stores (rotation of
 // the staging buffers).
-template <int SHIFT, bool ZP, int EPI_BUFS>
+template <int SHIFT, int EPI_BUFS>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, const CUtensorMap* tmap_out, uint32_t taddr, int m0, int n0,
-                                              int lane, float rs, const float* my_scale, const int32_t* my_zw, uint8_t* my_buf,
-                                              uint32_t& n_store, uint32_t acc_empty) {
+                                              int lane, const float* my_scale, uint8_t* my_buf, uint32_t& n_store,
+                                              uint32_t acc_empty) {
   const int row = m0 + lane;
 #pragma unroll 1
   for (int c = 0; c < BN / 32; ++c) {
@@ -157,7 +146,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, const CUtenso
       if (lane == 0) mbar_arrive_cluster(acc_empty);
     }
     const int col0 = n0 + c * 32;
-    auto sum = [&](int i) { return (static_cast<int32_t>(r[i]) >> SHIFT) - (ZP ? my_zw[c * 32 + i] : 0); };
+    auto sum = [&](int i) { return static_cast<int32_t>(r[i]) >> SHIFT; };
     if (p.tma_store) {
       uint8_t* buf = my_buf + (n_store % EPI_BUFS) * EPI_BUF;
       if ((c & 1) == 0) {  // the store that last read this buffer is EPI_BUFS stores back
@@ -169,10 +158,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, const CUtenso
         const float4 sa = *reinterpret_cast<const float4*>(my_scale + c * 32 + g * 8);
         const float4 sb = *reinterpret_cast<const float4*>(my_scale + c * 32 + g * 8 + 4);
         const int b = g * 8;
-        const __nv_bfloat162 p0 = __floats2bfloat162_rn(static_cast<float>(sum(b + 0)) * sa.x * rs, static_cast<float>(sum(b + 1)) * sa.y * rs);
-        const __nv_bfloat162 p1 = __floats2bfloat162_rn(static_cast<float>(sum(b + 2)) * sa.z * rs, static_cast<float>(sum(b + 3)) * sa.w * rs);
-        const __nv_bfloat162 p2 = __floats2bfloat162_rn(static_cast<float>(sum(b + 4)) * sb.x * rs, static_cast<float>(sum(b + 5)) * sb.y * rs);
-        const __nv_bfloat162 p3 = __floats2bfloat162_rn(static_cast<float>(sum(b + 6)) * sb.z * rs, static_cast<float>(sum(b + 7)) * sb.w * rs);
+        const __nv_bfloat162 p0 = __floats2bfloat162_rn(static_cast<float>(sum(b + 0)) * sa.x, static_cast<float>(sum(b + 1)) * sa.y);
+        const __nv_bfloat162 p1 = __floats2bfloat162_rn(static_cast<float>(sum(b + 2)) * sa.z, static_cast<float>(sum(b + 3)) * sa.w);
+        const __nv_bfloat162 p2 = __floats2bfloat162_rn(static_cast<float>(sum(b + 4)) * sb.x, static_cast<float>(sum(b + 5)) * sb.y);
+        const __nv_bfloat162 p3 = __floats2bfloat162_rn(static_cast<float>(sum(b + 6)) * sb.z, static_cast<float>(sum(b + 7)) * sb.w);
         const int chunk = (c & 1) * 4 + g;  // 16-byte chunk inside the 128-byte staging row
         *reinterpret_cast<uint4*>(buf + lane * 128 + ((chunk ^ (lane & 7)) << 4)) =
             make_uint4(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1),
@@ -192,7 +181,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, const CUtenso
       for (int i = 0; i < 32; ++i) {
         const int col = col0 + i;
         if (col < p.N)
-          p.out[static_cast<int64_t>(row) * p.ldo + col] = __float2bfloat16_rn(static_cast<float>(sum(i)) * my_scale[c * 32 + i] * rs);
+          p.out[static_cast<int64_t>(row) * p.ldo + col] = __float2bfloat16_rn(static_cast<float>(sum(i)) * my_scale[c * 32 + i]);
       }
     }
     if (p.acc_dbg && row < p.M) {
@@ -238,15 +227,15 @@ inline bool make_s8_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, int6
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tensor map over the bf16 output [M, N] with row pitch ldo; box = [32 rows, 64 columns], 128-byte swizzle.
-inline bool make_out_map(pq_ctx* ctx, CUtensorMap* map, void* out, int64_t M, int64_t N, int64_t ldo) {
+// Tensor map over the bf16 output [M, N] with row pitch ldo; box = [32 rows, cols columns], swizzled over its whole rows.
+inline bool make_out_map(pq_ctx* ctx, CUtensorMap* map, void* out, int64_t M, int64_t N, int64_t ldo, int cols = EPI_COLS) {
   cuuint64_t gdim[2] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(M)};
   cuuint64_t gstride[1] = {static_cast<cuuint64_t>(ldo) * 2};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(EPI_COLS), 32};
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(cols), 32};
   cuuint32_t estr[2] = {1, 1};
   return reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
              map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, out, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+             cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -1,29 +1,43 @@
-// W4A4 GEMM for prefill-shaped problems: CTA pairs, token operand fed from tensor memory.
+// W4A4 / W4A8 GEMM for prefill-shaped problems: CTA pairs on the 5th-generation tensor cores, weights fed from tensor memory.
 //
 //   acc[t,n] = sum_k xq[t,k] * wq[n,k]   (exact int32),   out = bf16(acc * s_a * s_w[n])
 //
-// Same pair design as pq_gemm_tc2.cu (cta_group::2, 256 x 256 tile, packed nibbles expanded to
-// 16*code as s8 on the way to the MMA), with one change that removes a third of the shared-memory
-// traffic and halves the operand ring: the A operand (token rows) never goes back to shared
-// memory. Each unpack thread owns one token row, reads its 64 packed bytes of a K block from the
-// landing buffer (64-byte-swizzled by TMA, so the row-per-thread reads are conflict-free), expands
-// them in registers and writes the 128 s8 bytes to its lane of tensor memory with tcgen05.st; the
-// MMA takes A from TMEM ([d], [a], b_desc form). Only the weight rows (B) are expanded into the
-// 128-byte-swizzled shared-memory layout.
+// sm_100a has no 4-bit integer MMA, so packed nibbles are expanded to 16*code as s8 on the way to the MMA. Two CTAs of a cluster
+// share a tile of 256 output channels x up to 256 tokens (cta_group::2). The channels are the MMA's row side: each CTA expands its
+// own 128 weight rows in registers (one thread per row, 64-byte-swizzled landing buffer) and writes them to its lanes of tensor
+// memory; the tokens are the column side: each CTA expands half of them into the 128-byte-swizzled shared-memory operand, and the
+// tensor cores of the pair exchange the halves.
 //
-// Tensor memory (512 columns): columns 0..255 the accumulator (one buffer: the epilogue of a tile
-// runs while the unpack warps fill up to eight K blocks of the next tile), columns 256..511 a ring
-// of eight A slots of 32 columns (128 K bytes per lane).
+// The width of a tile is a multiple of 32 tokens, chosen per launch (tile_rule): a token tile costs what its tokens cost, and a
+// launch fills whole rounds of the chip's CTA pairs. A tile is accumulated in two halves of at most 128 columns, each with an MMA
+// issuer and epilogue warps of its own, which go round two to four slots of tensor memory; the rest of it is six to eight A slots of
+// 32 columns (128 K bytes per lane). The half that is ahead is read out while the other still runs.
 //
-// Roles inside each CTA (24 warps):
-//   warp 0        TMA producer: packed A [128 x 64 B, 64-byte swizzle] and packed B half [128 x 64 B].
-//   warps 8..23   unpack, four groups of four warps (one warp per TMEM lane quarter); group g serves
-//                 ring slots g and g+4, so it can work one K block ahead of the MMA's release of its
-//                 other slot. A 16-byte packed chunk (32 codes) becomes 32 s8 bytes: even-position
-//                 codes then odd-position codes, the same order for A (registers -> TMEM columns) and
-//                 B (two 16-byte chunks in shared memory), so the dot product is unchanged.
-//   warp 1        (leader CTA only) MMA issuer; warp 1 of each CTA owns its TMEM allocation.
-//   warps 4..7    epilogue (as in pq_gemm_tc2.cu).
+// What bounds it: on one round of 256-token tiles the MMAs (four of 64 clocks per half and K block, 512 clocks; 578 measured), on narrow
+// tiles the issue and the expansion (450-500 clocks); on many rounds the chip's power limit. Found on the way (clock stamps of each
+// role, then variants; one round of 256-token tiles, K = 4096, weights from HBM, us):
+//   - the former kernels waited for their copies: four landing stages came back (latency, expansion, two barrier hops: 1750 clocks,
+//     2350 from HBM) later than four K blocks of MMAs take. Six to eight stages, their first weights ahead of griddepcontrol.wait:
+//     24.6 -> 19.5; K = 16384 55 -> 45;
+//   - then the issuer: a wait that succeeds at once, four MMAs, a commit and the loop took 500 clocks whatever the width. Two K blocks
+//     per turn (one vote for both waits): 128-token tiles 19.3 -> 16.3; an issuer per half costs the same and needs no ordering of the
+//     halves. mbarrier.try_wait may suspend the warp although another K block could be issued: polls use test_wait;
+//   - then the epilogue: a warp per lane quarter took 2.6 us at the end of a launch and 0.7-1.7 us between tiles. Eight warps, integers
+//     made floats by two additions instead of the conversion unit, fragments transposed by stmatrix: 18.7 -> 18.2, 2044 x 28672 x 4096
+//     158 -> 151.
+// GEMM alone, us, before -> now: 512 x 9472 x 4096 22.3 -> 17.7, 2048 x 9472 x 4096 55.1 -> 49.7, 512 x 9472 x 14336 49.9 -> 41.3.
+//
+// Roles inside each CTA (28 warps):
+//   warp 0        TMA producer: packed weight rows [128 x 64 B] and packed token rows per 128-wide K block into the landing stages.
+//                 Weights are static: the first stages' copies start before the wait for the previous kernel in the stream.
+//   warps 1, 3    (leader CTA only) MMA issuers of the two halves; warp 1 of each CTA owns its TMEM allocation.
+//   warp 2        A8: producer of the s8 token boxes, straight into operand slots (128-byte-swizzled).
+//   warps 4..7    epilogue of the first half, 24..27 of the second: one warp per TMEM lane quarter (32 channels), 32 tokens at a time:
+//                 fragments of 16 lanes x 256 bit, shift, scale, bf16, transposed into token rows by stmatrix, TMA store of
+//                 [32 tokens x 64 B].
+//   warps 8..23   expansion, four groups of four warps (one per TMEM lane quarter), group g serving K blocks g, g + 4, ...
+//                 A 16-byte packed chunk (32 codes) becomes 32 s8 bytes: even-position codes, then odd-position
+//                 codes, the same order in both operands, so the dot product is unchanged (natural order with A8).
 //
 // Every mbarrier wait is bounded; when one runs out the CTA raises an abort flag, every role of
 // the CTA drains, the peer's waits run out in turn, and PQ_ERR_TIMEOUT is reported.
@@ -33,63 +47,81 @@ namespace {
 
 using namespace pq_pair;
 
-constexpr int ROWS = BM_CTA + BN_CTA;       // operand rows per CTA per stage
-#ifndef PQ_GEMM_N_PK
-#define PQ_GEMM_N_PK 4
-#endif
-#ifndef PQ_GEMM_N_S8
-#define PQ_GEMM_N_S8 8
-#endif
-#ifndef PQ_GEMM_EPI_BUFS
-#define PQ_GEMM_EPI_BUFS 1
-#endif
-#ifndef PQ_GEMM_UNPACK_WARPS
-#define PQ_GEMM_UNPACK_WARPS 16
-#endif
-#ifndef PQ_GEMM_GROUPS
-#define PQ_GEMM_GROUPS 4
-#endif
-constexpr int N_PK = PQ_GEMM_N_PK;          // landing-buffer stages
-constexpr int N_S8 = PQ_GEMM_N_S8;          // operand-buffer stages
-constexpr int EPI_BUFS = PQ_GEMM_EPI_BUFS;  // staging buffers per epilogue warp
-constexpr int PK_STAGE = ROWS * PK_ROW;     // 16 KB
-constexpr int S8_STAGE = BN_CTA * BK;       // 16 KB: weight rows only
-constexpr int A_COL0 = 256;                 // first TMEM column of the A ring
+constexpr int UNIT = 32;                    // tokens: granularity of a tile's width (N of a 256-row pair MMA comes in steps of 32)
+constexpr int MAX_UNITS = 8;
+constexpr int CH_CTA = 128;                 // output channels per CTA (256 per pair)
+constexpr int W_STAGE = CH_CTA * PK_ROW;    // 8 KB of packed weights per K block
+constexpr int MAX_LAND = 8, MAX_A = 8, MAX_B = 8, MAX_ACC = 4;  // rings: landing stages, operand slots, accumulator halves
 constexpr int A_SLOT_COLS = BK / 4;         // 32 columns = 128 K bytes per lane
-constexpr int N_UNPACK_WARPS = PQ_GEMM_UNPACK_WARPS;
-constexpr int N_GROUPS = PQ_GEMM_GROUPS;
-constexpr int GROUP_WARPS = N_UNPACK_WARPS / N_GROUPS;
-// A ring slot is always served by the same group, so no group can get a whole phase ahead of a
-// barrier it waits on (a parity wait cannot tell phase k from phase k+2).
-static_assert(N_PK % N_GROUPS == 0 && N_S8 % N_GROUPS == 0, "ring depths must be multiples of the group count");
-static_assert(N_UNPACK_WARPS % N_GROUPS == 0, "equal groups");
-static_assert(N_UNPACK_WARPS / N_GROUPS == 4, "one warp per TMEM lane quarter in every group");
-static_assert(A_COL0 + N_S8 * A_SLOT_COLS <= 512, "tensor memory budget");
-constexpr int GROUP_THREADS = GROUP_WARPS * 32;
-constexpr int UNPACK_WARP0 = 8, EPI_WARP0 = 4;
-constexpr int N_THREADS = (UNPACK_WARP0 + N_UNPACK_WARPS) * 32;
-constexpr int TMEM_COLS = 512;              // one 256-column accumulator + the A ring
-constexpr int EPI_BYTES = 4 * EPI_BUFS * EPI_BUF;
-constexpr int SCALE_BYTES = 4 * BN * 4;     // per-warp copy of s_a * s_w[n0 .. n0+255]
-constexpr int ZW_BYTES = 4 * BN * 4;        // per-warp copy of (z - 8) * wsum[n0 .. n0+255] (zero-point correction)
+constexpr int N_GROUPS = 4, GROUP_THREADS = 128;
+constexpr int EPI_WARP0 = 4, EXPAND_WARP0 = 8, EPI_WARP1 = EXPAND_WARP0 + 4 * N_GROUPS;
+constexpr int N_THREADS = (EPI_WARP1 + 4) * 32;
+constexpr int TMEM_COLS = 512;
+constexpr int ST_BOX = UNIT * 64;           // one store: 32 tokens x 32 channels of bf16
+constexpr int ST_BUFS = 2;                  // staging buffers of an epilogue warp
+constexpr int RING_BYTES = 192 * 1024;      // landing stages and token operands
 
 struct __align__(8) Barriers {
-  uint64_t pk_full[N_PK], pk_empty[N_PK];
-  uint64_t s8_full[N_S8];   // waited on in the leader CTA only: 2 * GROUP_WARPS arrivals
-  uint64_t s8_empty[N_S8];  // one arrival per phase from the multicast tcgen05.commit
-  uint64_t acc_full[1];     // likewise
-  uint64_t acc_empty[1];    // leader CTA only: 4 epilogue warps of each CTA
+  uint64_t land_full[MAX_LAND], land_empty[MAX_LAND];
+  uint64_t s8_full[MAX_A];    // waited on in the leader CTA only: the four warps of a group of each CTA
+  uint64_t s8_empty[MAX_A];   // both issuers' multicast tcgen05.commit
+  uint64_t x_full[MAX_B], x_empty[MAX_B];  // A8 only: token boxes in the operand slots
+  uint64_t acc_full[MAX_ACC];   // multicast tcgen05.commit
+  uint64_t acc_empty[MAX_ACC];  // leader CTA only: 4 epilogue warps of each CTA
   uint64_t drain;
   uint32_t tmem_base;
   volatile int abort_flag;
 };
 
-constexpr size_t SMEM_BYTES =
-    1024 /*alignment slack*/ + N_S8 * S8_STAGE + N_PK * PK_STAGE + EPI_BYTES + SCALE_BYTES + ZW_BYTES + sizeof(Barriers);
-static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+constexpr size_t PAIR_SMEM = 1024 /*alignment slack*/ + RING_BYTES + 8 * ST_BUFS * ST_BOX + sizeof(Barriers);
+static_assert(PAIR_SMEM <= 227 * 1024, "shared memory budget");
 
-// D[tmem of both CTAs] (+)= A[tmem of both CTAs] * B[smem halves of both CTAs], issued by one thread
-// of the leader CTA.
+// A position in a ring of n slots and the parity of its current round.
+struct Pos {
+  int i = 0, ph = 0;
+  __device__ __forceinline__ void advance(int k, int n) {  // k <= n
+    i += k;
+    if (i >= n) i -= n, ph ^= 1;
+  }
+};
+
+struct PairParams {
+  const int32_t* zp;    // ZP: the activation zero point z (device scalar) ...
+  const int32_t* wsum;  // ... and the sum of every output channel's weight codes [N]
+  const float* s_row;   // ROWS: per-token steps [M]; else the scalar s_a applies
+  const float* s_a;
+  const float* s_w;
+  __nv_bfloat16* out;
+  int32_t* acc_dbg;
+  int32_t* status;
+  int64_t ldo;
+  int M, N, n_kb;
+  int c_tiles, t_tiles;    // tiles along the channels and along the tokens
+  int base_units, rem_units;  // token tile i is base_units + (i < rem_units) units wide
+  int half_units;          // units of a tile's first half (as far as it has so many): half of the widest tile's
+  int box;                 // token rows per TMA box and of a CTA's share of a first half
+  int n_land, n_a, n_b, n_acc;  // ring lengths (4-bit tokens: n_b = n_a, the two operand rings turn together)
+  int stage, slot, acc_cols;    // bytes of a landing stage and of a token operand slot, columns of an accumulator half
+  int tma_store;           // out can be written with TMA stores (16-byte aligned base and row pitch)
+  long long wait_clocks;   // bound of every device-side wait, in SM clocks
+};
+
+struct Tile {
+  int n0, t0;  // first channel, first token
+  int u0, u1;  // units of the two halves (u1 = 0: one half)
+};
+__device__ __forceinline__ Tile tile_at(const PairParams& p, int idx) {
+  const int c = idx / p.t_tiles, i = idx - c * p.t_tiles;  // the token tiles of a channel tile are neighbours: its weights are in L2
+  const int units = p.base_units + (i < p.rem_units ? 1 : 0);
+  Tile t;
+  t.n0 = c * 2 * CH_CTA;
+  t.t0 = (i * p.base_units + (i < p.rem_units ? i : p.rem_units)) * UNIT;
+  t.u0 = units < p.half_units ? units : p.half_units;
+  t.u1 = units - t.u0;
+  return t;
+}
+
+// D[tmem of both CTAs] (+)= A[tmem of both CTAs] * B[smem halves of both CTAs], issued by one thread of the leader CTA.
 __device__ __forceinline__ void mma2_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                            uint32_t accumulate) {
   asm volatile(
@@ -101,46 +133,77 @@ __device__ __forceinline__ void mma2_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-template <bool ZP>
+// Has the phase completed? Unlike try_wait this never suspends the thread, which has MMAs to issue meanwhile.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(pq::smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// 16 lanes x 32 columns as 8 x 8 fragments: register 4j + 2h + e holds lane i/4 + 8h, column 8j + 2(i%4) + e (thread i of the warp).
+__device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// Four 8 x 8 matrices of 16-bit elements, each stored transposed: thread i gives the address of stored row i % 8 of matrix i / 8.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+               : "memory");
+}
+
+template <bool A8, bool ZP, bool ROWS, bool SMALL>
 __global__ void __launch_bounds__(N_THREADS, 1)
-    gemm_w4a4_pair_ts_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                          const __grid_constant__ CUtensorMap tmap_out, const GemmParams p) {
+    gemm_w4a4_pair_ts_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
+                             const __grid_constant__ CUtensorMap tmap_out, const PairParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* s8_buf = smem;                                   // N_S8 stages of expanded weight rows, 1024-aligned
-  uint8_t* pk_buf = s8_buf + N_S8 * S8_STAGE;               // N_PK stages: packed A rows then packed B rows
-  uint8_t* epi_buf = pk_buf + N_PK * PK_STAGE;              // 4 warps x 2 buffers, 1024-aligned
-  float* scale_buf = reinterpret_cast<float*>(epi_buf + EPI_BYTES);
-  int32_t* zw_buf = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(scale_buf) + SCALE_BYTES);
-  Barriers* bars = reinterpret_cast<Barriers*>(reinterpret_cast<uint8_t*>(zw_buf) + ZW_BYTES);
+  uint8_t* b_buf = smem;                          // n_b token operands, 1024-aligned
+  uint8_t* land_buf = b_buf + p.n_b * p.slot;     // n_land stages: packed weight rows, then packed token rows
+  uint8_t* st_buf = smem + RING_BYTES;            // 8 warps x ST_BUFS buffers
+  Barriers* bars = reinterpret_cast<Barriers*>(st_buf + 8 * ST_BUFS * ST_BOX);
+  volatile int* abort_flag = &bars->abort_flag;
 
-  // no early launch of the next kernel: its CTAs would crowd on the SMs whose pair has no tile left (see pq_launch_pdl)
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // operands and output may belong to the previous kernel
   const int warp = pq::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int n_tiles = p.tiles_m * p.tiles_n;
-  const int n_kb = (p.K + BK - 1) / BK;
+  const int n_tiles = p.c_tiles * p.t_tiles;
   const int my_tiles = pair < n_tiles ? (n_tiles - pair + n_pairs - 1) / n_pairs : 0;
-  volatile int* abort_flag = &bars->abort_flag;
+  const uint32_t total = static_cast<uint32_t>(my_tiles) * p.n_kb;  // K blocks of this pair
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < N_PK; ++i) {
-      pq::mbar_init(&bars->pk_full[i], 1);
-      pq::mbar_init(&bars->pk_empty[i], GROUP_WARPS);
+    for (int i = 0; i < MAX_LAND; ++i) {
+      pq::mbar_init(&bars->land_full[i], 1);
+      pq::mbar_init(&bars->land_empty[i], 4);
     }
-    for (int i = 0; i < N_S8; ++i) {
-      pq::mbar_init(&bars->s8_full[i], 2 * GROUP_WARPS);
-      pq::mbar_init(&bars->s8_empty[i], 1);
+    for (int i = 0; i < MAX_A; ++i) {
+      pq::mbar_init(&bars->s8_full[i], 8);
+      pq::mbar_init(&bars->s8_empty[i], 2);
     }
-    pq::mbar_init(&bars->acc_full[0], 1);
-    pq::mbar_init(&bars->acc_empty[0], 8);
-    pq::mbar_init(&bars->drain, 1);
+    for (int i = 0; i < MAX_B; ++i) {
+      pq::mbar_init(&bars->x_full[i], 1);
+      pq::mbar_init(&bars->x_empty[i], 2);
+    }
+    for (int i = 0; i < MAX_ACC; ++i) {
+      pq::mbar_init(&bars->acc_full[i], 1);
+      pq::mbar_init(&bars->acc_empty[i], 8);
+    }
+    pq::mbar_init(&bars->drain, 2);
     bars->abort_flag = 0;
     pq::mbar_fence_init();
     pq::fence_proxy_async_smem();
-    pq::tma_prefetch_desc(&tmap_a);
-    pq::tma_prefetch_desc(&tmap_b);
+    pq::tma_prefetch_desc(&tmap_x);
+    pq::tma_prefetch_desc(&tmap_w);
     pq::tma_prefetch_desc(&tmap_out);
   }
   if (warp == 1) {
@@ -152,193 +215,342 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   cluster_sync_all();  // the peer's barriers exist before anything arrives on them
   pq::tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
-  uint32_t loads_issued = 0;  // producer lanes: stages whose copies were started
+  const uint32_t a_ring = tmem_base + p.n_acc * p.acc_cols;  // A slots behind the accumulator halves
+  uint32_t loads_issued = 0;  // producer warps: stages whose copies were started
+  bool ok = true;
 
+  // no early launch of the next kernel: its CTAs would crowd on the SMs whose pair has no tile left (see pq_launch_pdl)
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     const bool leader = pq::elect_one();
+    auto begin_stage = [&](int s, const Tile& t, int kb) {  // the stage's bytes are announced, its weights requested
+      const int boxes = A8 ? 0 : (t.u1 > 0 ? 2 : 1);
+      pq::mbar_arrive_expect_tx(&bars->land_full[s], W_STAGE + boxes * p.box * PK_ROW);
+      pq::tma_load_2d(land_buf + s * p.stage, &tmap_w, kb * PK_ROW, t.n0 + rank * CH_CTA, &bars->land_full[s]);
+    };
+    const uint32_t early = total < static_cast<uint32_t>(p.n_land) ? total : p.n_land;
+    for (uint32_t i = 0; i < early; ++i) {  // the first weight copies do not depend on the previous kernel
+      const Tile t = tile_at(p, pair + static_cast<int>(i / p.n_kb) * n_pairs);
+      if (leader) begin_stage(i, t, i % p.n_kb);
+      __syncwarp();
+    }
+    loads_issued = early;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the tokens may come from the previous kernel
     uint32_t it = 0;
-    bool ok = true;
+    Pos ls;
     for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-      const int m_row = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA;
-      const int n_row = (tile / p.tiles_m) * BN + rank * BN_CTA;
-      for (int kb = 0; kb < n_kb; ++kb, ++it) {
-        const uint32_t s = it % N_PK, ph = (it / N_PK) & 1;
-        if (!wait_bar_warp(&bars->pk_empty[s], ph ^ 1, abort_flag, p.wait_clocks)) {
+      const Tile t = tile_at(p, tile);
+      for (int kb = 0; kb < p.n_kb; ++kb, ++it, ls.advance(1, p.n_land)) {
+        if (it >= early) {
+          if (!wait_bar_warp(&bars->land_empty[ls.i], ls.ph ^ 1, abort_flag, p.wait_clocks)) {
+            ok = false;
+            break;
+          }
+          if (leader) begin_stage(ls.i, t, kb);
+          loads_issued = it + 1;
+        }
+        if (!A8 && leader) {
+          uint8_t* dst = land_buf + ls.i * p.stage + W_STAGE;
+          pq::tma_load_2d(dst, &tmap_x, kb * PK_ROW, t.t0 + rank * t.u0 * (UNIT / 2), &bars->land_full[ls.i]);
+          if (t.u1 > 0)
+            pq::tma_load_2d(dst + p.box * PK_ROW, &tmap_x, kb * PK_ROW, t.t0 + t.u0 * UNIT + rank * t.u1 * (UNIT / 2), &bars->land_full[ls.i]);
+        }
+        __syncwarp();
+      }
+    }
+  } else if (A8 && warp == 2) {
+    // ------------------------------------------------------------------ token producer (A8)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const bool leader = pq::elect_one();
+    uint32_t it = 0;
+    Pos xs;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const Tile t = tile_at(p, tile);
+      for (int kb = 0; kb < p.n_kb; ++kb, ++it, xs.advance(1, p.n_b)) {
+        if (!wait_bar_warp(&bars->x_empty[xs.i], xs.ph ^ 1, abort_flag, p.wait_clocks)) {
           ok = false;
           break;
         }
         if (leader) {
-          pq::mbar_arrive_expect_tx(&bars->pk_full[s], PK_STAGE);
-          pq::tma_load_2d(pk_buf + s * PK_STAGE, &tmap_a, kb * PK_ROW, m_row, &bars->pk_full[s]);
-          pq::tma_load_2d(pk_buf + s * PK_STAGE + BM_CTA * PK_ROW, &tmap_b, kb * PK_ROW, n_row, &bars->pk_full[s]);
+          uint8_t* dst = b_buf + xs.i * p.slot;
+          pq::mbar_arrive_expect_tx(&bars->x_full[xs.i], (t.u1 > 0 ? 2 : 1) * p.box * BK);
+          pq::tma_load_2d(dst, &tmap_x, kb * BK, t.t0 + rank * t.u0 * (UNIT / 2), &bars->x_full[xs.i]);
+          if (t.u1 > 0)
+            pq::tma_load_2d(dst + p.box * BK, &tmap_x, kb * BK, t.t0 + t.u0 * UNIT + rank * t.u1 * (UNIT / 2), &bars->x_full[xs.i]);
         }
         __syncwarp();
       }
     }
     loads_issued = it;
-    if (!ok) {
-      if (leader) {
-        bars->abort_flag = 1;
-        pq::report(p.status, PQ_ERR_TIMEOUT);
-      }
-      // let the copies this warp started land before the CTA can exit
-      const uint32_t first = it > N_PK ? it - N_PK : 0;
-      for (uint32_t j = first; j < it; ++j) pq::mbar_wait(&bars->pk_full[j % N_PK], (j / N_PK) & 1);
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer (leader CTA)
+  } else if (warp == 1 || warp == 3) {
+    // ------------------------------------------------------------------ MMA issuers (leader CTA): one per accumulator half
     if (rank == 0) {
-      // The four MMAs of a K block take 512 clocks of the tensor pipe; wait, issue and commit have to stay below that,
-      // or this warp paces the kernel. With the loop in a branch of one lane they took 550-600; kept uniform (see
-      // elect_one) about 350: 4096 x 57344 x 8192: 1316 -> 1169 us
-      // (3.29 POPS), 4096 x 10240 x 8192: 230 -> 199, 2044 x 4096 x 14336: 89 -> 80.
-      constexpr uint32_t idesc = pq::umma_idesc_s8(2 * BM_CTA, BN);
+      asm volatile("griddepcontrol.wait;" ::: "memory");  // what they wait for needs the tokens
       const bool leader = pq::elect_one();
-      const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(s8_buf));
-      uint32_t it = 0, tcount = 0;
-      bool ok = true;
-      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++tcount) {
-        // the epilogue has read the last tile
-        if (!wait_bar_warp(&bars->acc_empty[0], (tcount & 1) ^ 1, abort_flag, p.wait_clocks)) {
+      const int h = warp >> 1;
+      const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(b_buf) + h * p.box * BK);
+      const uint32_t slot_desc = p.slot >> 4;
+      Pos as, bs, u;  // operand slots (8-bit tokens: of their own), accumulator halves
+      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+        const Tile t = tile_at(p, tile);
+        const int units = h ? t.u1 : t.u0;  // none: only the slots are handed on
+        Pos mine = u;
+        mine.advance(h, p.n_acc);
+        const uint32_t d_tmem = tmem_base + mine.i * p.acc_cols, idesc = pq::umma_idesc_s8(2 * CH_CTA, units * UNIT);
+        if (units > 0 && !wait_bar_warp(&bars->acc_empty[mine.i], mine.ph ^ 1, abort_flag, p.wait_clocks)) {
           ok = false;
           break;
         }
         pq::tc_fence_after();
-        const uint32_t d_tmem = tmem_base;
-        for (int kb = 0; kb < n_kb; ++kb, ++it) {
-          const uint32_t s = it % N_S8, ph = (it / N_S8) & 1;
-          if (!wait_bar_warp(&bars->s8_full[s], ph, abort_flag, p.wait_clocks)) {
+        auto k_block = [&](bool first) {  // with the operands in slots as, bs; both CTAs may refill them once both halves' MMAs have read them
+          if (leader) {
+            if (units > 0) {
+              const uint32_t a_tmem = a_ring + as.i * A_SLOT_COLS;
+              const uint64_t b_desc = desc0 + bs.i * slot_desc;
+              mma2_i8_ts(d_tmem, a_tmem, b_desc, idesc, first ? 0u : 1u);
+#pragma unroll
+              for (int kk = 1; kk < BK / 32; ++kk) mma2_i8_ts(d_tmem, a_tmem + kk * 8, b_desc + kk * 2, idesc, 1u);  // 32 bytes of K further
+            }
+            mma2_commit_both(&bars->s8_empty[as.i]);
+            if (A8) mma2_commit_both(&bars->x_empty[bs.i]);
+          }
+          __syncwarp();
+          as.advance(1, p.n_a), bs.advance(1, p.n_b);
+        };
+        int kb = 0;
+        for (; kb + 1 < p.n_kb; kb += 2) {  // two K blocks per turn: one vote and one branch for both waits
+          Pos next = as;
+          next.advance(1, p.n_a);
+          const bool r0 = mbar_test(&bars->s8_full[as.i], as.ph), r1 = mbar_test(&bars->s8_full[next.i], next.ph);
+          const bool both = __all_sync(0xffffffffu, r0 && r1);
+          if (!both && !wait_bar_warp(&bars->s8_full[as.i], as.ph, abort_flag, p.wait_clocks)) {
             ok = false;
             break;
           }
           pq::tc_fence_after();
-          if (leader) {
-            const uint32_t a_tmem = tmem_base + A_COL0 + s * A_SLOT_COLS;
-            const uint64_t b_desc = desc0 + s * (S8_STAGE >> 4);
-#pragma unroll
-            for (int kk = 0; kk < BK / 32; ++kk)  // 32 bytes of K further along the 128-byte rows
-              mma2_i8_ts(d_tmem, a_tmem + kk * 8, b_desc + kk * 2, idesc, (kb | kk) != 0 ? 1u : 0u);
-            mma2_commit_both(&bars->s8_empty[s]);  // both CTAs may refill the stage once these MMAs have read it
+          k_block(kb == 0);
+          if (!both && !wait_bar_warp(&bars->s8_full[as.i], as.ph, abort_flag, p.wait_clocks)) {
+            ok = false;
+            break;
           }
-          __syncwarp();
+          pq::tc_fence_after();
+          k_block(false);
         }
-        if (ok && leader) mma2_commit_both(&bars->acc_full[0]);
+        if (ok && kb < p.n_kb) {
+          ok = wait_bar_warp(&bars->s8_full[as.i], as.ph, abort_flag, p.wait_clocks);
+          pq::tc_fence_after();
+          if (ok) k_block(kb == 0);
+        }
+        if (!ok) break;
+        if (leader && units > 0) mma2_commit_both(&bars->acc_full[mine.i]);
         __syncwarp();
+        u.advance(t.u1 > 0 ? 2 : 1, p.n_acc);
       }
-      if (leader) {
-        if (!ok) {
-          bars->abort_flag = 1;
-          pq::report(p.status, PQ_ERR_TIMEOUT);
-        }
-        // whatever was issued has finished before either CTA releases its tensor memory
-        mma2_commit_both(&bars->drain);
-      }
+      if (leader) mma2_commit_both(&bars->drain);  // whatever was issued has finished before either CTA releases its tensor memory
       __syncwarp();
     }
     pq::mbar_wait(&bars->drain, 0);
-  } else if (warp >= UNPACK_WARP0) {
-    // ------------------------------------------------------------------ unpack warps
-    const int group = (warp - UNPACK_WARP0) / GROUP_WARPS;
-    const int gt = (warp - UNPACK_WARP0) % GROUP_WARPS * 32 + lane;
-    const uint32_t total = static_cast<uint32_t>(my_tiles) * n_kb;
-    bool ok = true;
-    for (uint32_t it = group; it < total; it += N_GROUPS) {
-      const uint32_t ps = it % N_PK, pph = (it / N_PK) & 1;
-      const uint32_t ss = it % N_S8, sph = (it / N_S8) & 1;
-      const bool stuck =
-          !wait_bar(&bars->pk_full[ps], pph, abort_flag, p.wait_clocks) || !wait_bar(&bars->s8_empty[ss], sph ^ 1, abort_flag, p.wait_clocks);
-      if (__any_sync(0xffffffffu, stuck)) {  // warp-uniform decision
+  } else if (warp >= EXPAND_WARP0 && warp < EPI_WARP1) {
+    // ------------------------------------------------------------------ expansion
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the landing stages' tokens come behind it
+    const int group = (warp - EXPAND_WARP0) >> 2, q = warp & 3;
+    const int gt = q * 32 + lane;  // thread of the group = channel row of the CTA = lane of tensor memory
+    int tile = pair, kb = group;
+    Tile t = tile_at(p, tile);
+    Pos ls, as, xs;
+    ls.advance(group, p.n_land), as.advance(group, p.n_a), xs.advance(group, p.n_b);
+    for (uint32_t it = group; it < total;
+         it += N_GROUPS, kb += N_GROUPS, ls.advance(N_GROUPS, p.n_land), as.advance(N_GROUPS, p.n_a), xs.advance(N_GROUPS, p.n_b)) {
+      if (kb >= p.n_kb) {
+        do kb -= p.n_kb, tile += n_pairs;
+        while (kb >= p.n_kb);
+        t = tile_at(p, tile);
+      }
+      // The operand slot first: once it is free, the MMAs of K block it - n_a and of all before it have run, so the copies of those K
+      // blocks have landed, and with n_land >= n_a (and n_b >= n_a) the parities below cannot be mistaken for those of two rounds back.
+      if (!wait_bar_warp(&bars->s8_empty[as.i], as.ph ^ 1, abort_flag, p.wait_clocks) ||
+          !wait_bar_warp(&bars->land_full[ls.i], ls.ph, abort_flag, p.wait_clocks)) {
         ok = false;
         break;
       }
-      const uint8_t* src = pk_buf + ps * PK_STAGE;
-      // ---- A: this thread's token row, 64 packed bytes -> 128 s8 bytes -> its TMEM lane ------------
-      {
-        const int q = warp & 3, arow = q * 32 + lane;
-        const uint8_t* arow_p = src + arow * PK_ROW;
-        const int sx = (arow >> 1) & 3;  // 64-byte swizzle of the landing buffer
-        uint32_t ar[32];
+      const uint8_t* src = land_buf + ls.i * p.stage;
+      const int chunks = (t.u0 + t.u1) * (UNIT / 2) * 4;  // 16-byte chunks of this CTA's token rows (the second box's follow the first's)
+      uint4 w[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint4 w = *reinterpret_cast<const uint4*>(arow_p + ((j ^ sx) << 4));
-          ar[8 * j + 0] = pq::nib_lo_x16(w.x), ar[8 * j + 1] = pq::nib_lo_x16(w.y);
-          ar[8 * j + 2] = pq::nib_lo_x16(w.z), ar[8 * j + 3] = pq::nib_lo_x16(w.w);
-          ar[8 * j + 4] = pq::nib_hi_x16(w.x), ar[8 * j + 5] = pq::nib_hi_x16(w.y);
-          ar[8 * j + 6] = pq::nib_hi_x16(w.z), ar[8 * j + 7] = pq::nib_hi_x16(w.w);
+      for (int j = 0; j < 4; ++j)  // 64-byte swizzle of the landing buffer: the row-per-thread reads hit distinct banks
+        w[j] = *reinterpret_cast<const uint4*>(src + gt * PK_ROW + ((j ^ ((gt >> 1) & 3)) << 4));
+      uint4 x[4];
+      if (!A8) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i * GROUP_THREADS + gt < chunks) x[i] = *reinterpret_cast<const uint4*>(src + W_STAGE + (i * GROUP_THREADS + gt) * 16);
+      }
+      uint32_t a[32];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t in[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t lo = pq::nib_lo_x16(in[i]), hi = pq::nib_hi_x16(in[i]);
+          if (A8) {
+            a[8 * j + 2 * i] = __byte_perm(lo, hi, 0x5140), a[8 * j + 2 * i + 1] = __byte_perm(lo, hi, 0x7362);
+          } else {
+            a[8 * j + i] = lo, a[8 * j + 4 + i] = hi;
+          }
         }
-        pq::tmem_st_32x32(tmem_base + A_COL0 + ss * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), ar);
       }
-      // ---- B: the CTA's 128 weight rows into the swizzled operand stage -------------------------------
-      const uint8_t* bsrc = src + BM_CTA * PK_ROW;
-      uint8_t* dst = s8_buf + ss * S8_STAGE;
-      constexpr int UNITS = BN_CTA * 4;  // one unit = one 16-byte packed chunk
+      pq::tmem_st_32x32(a_ring + as.i * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), a);
+      if (!A8) {
+        const int row = gt >> 2, j = gt & 3, sw = row & 7;  // the thread's rows are 32 apart: one swizzle
+        uint8_t* lo = b_buf + as.i * p.slot + row * BK + (((2 * j) ^ sw) << 4);
+        uint8_t* hi = b_buf + as.i * p.slot + row * BK + (((2 * j + 1) ^ sw) << 4);
 #pragma unroll
-      for (int i = 0; i < UNITS / GROUP_THREADS; ++i) {
-        const int unit = i * GROUP_THREADS + gt;
-        const int row = unit >> 2, j = unit & 3;
-        const uint4 w = *reinterpret_cast<const uint4*>(bsrc + row * PK_ROW + j * 16);
-        uint4 lo, hi;
-        lo.x = pq::nib_lo_x16(w.x), lo.y = pq::nib_lo_x16(w.y), lo.z = pq::nib_lo_x16(w.z), lo.w = pq::nib_lo_x16(w.w);
-        hi.x = pq::nib_hi_x16(w.x), hi.y = pq::nib_hi_x16(w.y), hi.z = pq::nib_hi_x16(w.z), hi.w = pq::nib_hi_x16(w.w);
-        uint8_t* drow = dst + row * BK;
-        const int sw = row & 7;
-        *reinterpret_cast<uint4*>(drow + (((2 * j) ^ sw) << 4)) = lo;
-        *reinterpret_cast<uint4*>(drow + (((2 * j + 1) ^ sw) << 4)) = hi;
+        for (int i = 0; i < 4; ++i) {
+          if (i * GROUP_THREADS + gt < chunks) {
+            *reinterpret_cast<uint4*>(lo + i * 32 * BK) =
+                make_uint4(pq::nib_lo_x16(x[i].x), pq::nib_lo_x16(x[i].y), pq::nib_lo_x16(x[i].z), pq::nib_lo_x16(x[i].w));
+            *reinterpret_cast<uint4*>(hi + i * 32 * BK) =
+                make_uint4(pq::nib_hi_x16(x[i].x), pq::nib_hi_x16(x[i].y), pq::nib_hi_x16(x[i].z), pq::nib_hi_x16(x[i].w));
+          }
+        }
       }
-      pq::tmem_st_wait();         // the TMEM lane is written ...
+      if (A8) {  // the slot is complete only with this CTA's token boxes in place
+        if (!wait_bar_warp(&bars->x_full[xs.i], xs.ph, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
+        }
+      }
+      pq::tmem_st_wait();     // the TMEM lane is written ...
       pq::tc_fence_before();  // ... and ordered before the arrival below
-      pq::fence_proxy_async_smem();  // generic-proxy writes -> visible to the tensor core's async proxy
+      if (!A8) pq::fence_proxy_async_smem();  // generic-proxy writes -> visible to the tensor core's async proxy
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive_cluster(map_to_cta(&bars->s8_full[ss], 0));
-        pq::mbar_arrive(&bars->pk_empty[ps]);
+        mbar_arrive_cluster(map_to_cta(&bars->s8_full[as.i], 0));
+        pq::mbar_arrive(&bars->land_empty[ls.i]);  // behind the stores, for which what was read has arrived in registers
       }
-    }
-    if (!ok && lane == 0) {
-      bars->abort_flag = 1;
-      pq::report(p.status, PQ_ERR_TIMEOUT);
     }
   } else if (warp >= EPI_WARP0) {
-    // ------------------------------------------------------------------ epilogue warps
-    const int q = warp & 3;  // TMEM lane quarter this warp may access
-    const float s_a = p.s_row ? 1.0f : pq::ld_dep(p.s_a);
-    uint8_t* my_buf = epi_buf + q * EPI_BUFS * EPI_BUF;
-    float* my_scale = scale_buf + q * BN;
-    int32_t* my_zw = zw_buf + q * BN;
+    // ------------------------------------------------------------------ epilogue
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the scales and the output may belong to the previous kernel
+    constexpr int SHIFT = A8 ? 4 : 8;  // the factors 16 the expanded codes carry
+    const int q = warp & 3;            // TMEM lane quarter this warp may access
+    const float s_a = ROWS ? 1.0f : pq::ld_dep(p.s_a);
     const int zp8 = ZP ? pq::ld_dep(p.zp) - 8 : 0;
-    uint32_t tcount = 0, n_store = 0;
-    bool ok = true;
-    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++tcount) {
-      const int m0 = (tile % p.tiles_m) * (2 * BM_CTA) + rank * BM_CTA + q * 32;
-      const int n0 = (tile / p.tiles_m) * BN;
-      const uint32_t aph = tcount & 1;
-      fill_tile_scales<ZP>(p, n0, lane, s_a, zp8, my_scale, my_zw);
-      const bool stuck = !wait_bar(&bars->acc_full[0], aph, abort_flag, p.wait_clocks);
-      if (__any_sync(0xffffffffu, stuck)) {  // warp-uniform: the TMEM loads below are warp-collective
-        ok = false;
-        break;
+    const int h = warp >= EPI_WARP1 ? 1 : 0;  // the accumulator half this warp reads
+    uint8_t* my_buf = st_buf + (4 * h + q) * ST_BUFS * ST_BOX;
+    const uint32_t st_row = pq::smem_u32(my_buf) + (lane & 7) * 64;  // stmatrix: this lane addresses token row lane % 8 of a group of eight ...
+    const int st_chunk = lane >> 3;                                  // ... and the 16-byte chunk (eight channels) of matrix lane / 8
+    uint32_t n_store = 0;
+    Pos u;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const Tile t = tile_at(p, tile);
+      const int n0 = t.n0 + static_cast<int>(rank) * CH_CTA + q * 32;  // the warp's channels
+      float sw[4];
+      int zw[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {  // this lane's channels: lane / 4 of each group of eight
+        const int n = n0 + i * 8 + (lane >> 2);
+        sw[i] = n < p.N ? s_a * __ldg(p.s_w + n) : 0.0f;
+        zw[i] = ZP && n < p.N ? zp8 * __ldg(p.wsum + n) : 0;
       }
-      pq::tc_fence_after();
-      const float rs = p.s_row ? (m0 + lane < p.M ? pq::ld_dep(p.s_row + m0 + lane) : 0.0f) : 1.0f;  // this lane's token step
-      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-      epilogue_tile<8, ZP, EPI_BUFS>(p, &tmap_out, taddr, m0, n0, lane, rs, my_scale, my_zw, my_buf, n_store,
-                                     map_to_cta(&bars->acc_empty[0], 0));
+      Pos mine = u;
+      mine.advance(h, p.n_acc);
+      u.advance(t.u1 > 0 ? 2 : 1, p.n_acc);
+      const int units = h ? t.u1 : t.u0, th = t.t0 + (h ? t.u0 * UNIT : 0);
+      if (units > 0) {
+        if (!wait_bar_warp(&bars->acc_full[mine.i], mine.ph, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
+        }
+        pq::tc_fence_after();
+        const uint32_t taddr = tmem_base + mine.i * p.acc_cols + (static_cast<uint32_t>(q * 32) << 16);
+#pragma unroll 1
+        for (int c = 0; c < units; ++c) {
+          const int t0 = th + c * UNIT;
+          uint32_t r[2][16];  // lanes (channels) 0..15 and 16..31 of the quarter
+          tmem_ld_16x32(taddr + c * UNIT, r[0]);
+          tmem_ld_16x32(taddr + c * UNIT + (16u << 16), r[1]);
+          float rs[8];  // the steps of this lane's tokens
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int tok = t0 + (i >> 1) * 8 + (lane & 3) * 2 + (i & 1);
+            rs[i] = ROWS && tok < p.M ? pq::ld_dep(p.s_row + tok) : 1.0f;
+          }
+          pq::tmem_ld_wait();
+          if (c == units - 1) {  // the half is read: its MMA warp may overwrite it
+            pq::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_to_cta(&bars->acc_empty[mine.i], 0));
+          }
+          auto sum = [&](int g, int j, int e) { return (static_cast<int32_t>(r[g >> 1][4 * j + 2 * (g & 1) + e]) >> SHIFT) - (ZP ? zw[g] : 0); };
+          auto val = [&](int g, int j, int e) {
+            const int v = sum(g, j, e);
+            // SMALL: |v| <= 2^22, so v + 1.5 * 2^23 is exact and its bits are those of the integer sum; the conversion instruction runs
+            // at an eighth of the rate of the two additions.
+            const float f = (SMALL ? __int_as_float(0x4B400000 + v) - 12582912.0f : static_cast<float>(v)) * sw[g];
+            return ROWS ? f * rs[2 * j + e] : f;
+          };
+          const uint32_t buf = (n_store % ST_BUFS) * ST_BOX;
+          if (lane == 0) bulk_wait_read<ST_BUFS - 1>();  // the store that last read this buffer is ST_BUFS stores back
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {  // eight tokens: four matrices of eight channels
+            uint32_t v[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              const __nv_bfloat162 b = __floats2bfloat162_rn(val(g, j, 0), val(g, j, 1));
+              v[g] = *reinterpret_cast<const uint32_t*>(&b);
+            }
+            // 64-byte rows under the 64-byte swizzle: chunk XOR (row / 2) % 4
+            stmatrix_x4_trans(st_row + buf + j * 512 + ((st_chunk ^ ((lane >> 1) & 3)) << 4), v[0], v[1], v[2], v[3]);
+          }
+          if (p.acc_dbg) {
+            int32_t* d = p.acc_dbg + static_cast<int64_t>(t0 + (lane & 3) * 2) * p.N + n0 + (lane >> 2);
+#pragma unroll
+            for (int i = 0; i < 8; ++i, d += i & 1 ? p.N : 7 * static_cast<int64_t>(p.N))
+#pragma unroll
+              for (int g = 0; g < 4; ++g)
+                if (t0 + (i >> 1) * 8 + (lane & 3) * 2 + (i & 1) < p.M && n0 + g * 8 + (lane >> 2) < p.N) d[g * 8] = sum(g, i >> 1, i & 1);
+          }
+          if (p.tma_store) {
+            pq::fence_proxy_async_smem();
+            __syncwarp();
+            if (n0 < p.N) {  // counted only when stored: the wait above is in stores
+              if (lane == 0) {
+                tma_store_2d(&tmap_out, my_buf + buf, n0, t0);
+                bulk_commit();
+              }
+              ++n_store;
+            }
+          } else {
+            __syncwarp();
+            for (int row = 0; row < UNIT && t0 + row < p.M; ++row)
+              if (n0 + lane < p.N)
+                p.out[static_cast<int64_t>(t0 + row) * p.ldo + n0 + lane] =
+                    *reinterpret_cast<const __nv_bfloat16*>(my_buf + buf + row * 64 + (((lane >> 3) ^ ((row >> 1) & 3)) << 4) + (lane & 7) * 2);
+            __syncwarp();
+          }
+        }
+      }
     }
-    if (lane == 0) bulk_wait_all();
-    if (!ok && lane == 0) {
-      bars->abort_flag = 1;
-      pq::report(p.status, PQ_ERR_TIMEOUT);
-    }
+    if (lane == 0) bulk_wait_read<0>();  // the staging buffers have been read: the CTA may end
   }
 
+  if (!ok && lane == 0) {
+    bars->abort_flag = 1;
+    pq::report(p.status, PQ_ERR_TIMEOUT);
+  }
   pq::tc_fence_before();
   __syncthreads();
   if (bars->abort_flag) {
-    // a role gave up: copies that nobody consumed must still have landed before the CTA may exit (they only wait
-    // for memory, hence the generous bound)
+    // a role gave up: copies that nobody consumed must still have landed before the CTA may exit (they only wait for memory,
+    // hence the generous bound; a stage whose weights were requested got its tokens, too)
     if (warp == 0 && lane == 0)
-      for (uint32_t j = loads_issued > N_PK ? loads_issued - N_PK : 0; j < loads_issued; ++j) pq::mbar_wait(&bars->pk_full[j % N_PK], (j / N_PK) & 1);
+      for (uint32_t j = loads_issued > static_cast<uint32_t>(p.n_land) ? loads_issued - p.n_land : 0; j < loads_issued; ++j)
+        pq::mbar_wait(&bars->land_full[j % p.n_land], (j / p.n_land) & 1);
+    if (A8 && warp == 2 && lane == 0)
+      for (uint32_t j = loads_issued > static_cast<uint32_t>(p.n_b) ? loads_issued - p.n_b : 0; j < loads_issued; ++j)
+        pq::mbar_wait(&bars->x_full[j % p.n_b], (j / p.n_b) & 1);
     __syncthreads();
   }
   cluster_sync_all();  // neither CTA frees tensor memory or exits while the pair may still touch it
@@ -348,26 +560,105 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   }
 }
 
+// The number of token tiles per channel tile: the one with the shortest estimate for the launch, in whole rounds of the chip's pairs.
+// Clocks of a K block, measured on one round of tiles of 64, 128, 192 and 256 tokens (K = 4096 and 8192): 458, 472, 497, 578 (8-bit tokens
+// 397, 416, 452, 578): wide tiles take their MMAs' time (64 clocks per unit) and a little, narrow ones that of the expansion and of
+// the issue, which hardly depend on the width. A tile adds about 1800 clocks of its own. Gains, narrower tiles against the widest (us,
+// with the rotation): 1000 x 6144 x 4096 34.2 / 41, 1000 x 4096 x 4096 21.5 / 24.6, 1500 x 4096 x 14336 76 / 86.
+// With more than three rounds of the widest tiles those stay: the ragged round weighs less there, the chip runs at its power limit, and
+// narrower tiles expand the weights more often (2044 x 28672 x 4096: 169 with nine tiles, 156 with eight).
+int tile_rule(int units, int c_tiles, int n_pairs, int n_kb) {
+  int best = 0;
+  double best_clocks = 0.0;
+  const int t_min = (units + MAX_UNITS - 1) / MAX_UNITS;
+  if (c_tiles * t_min > 3 * n_pairs) return t_min;
+  for (int t = t_min; t <= units && t <= t_min + 8; ++t) {
+    const int rounds = (c_tiles * t + n_pairs - 1) / n_pairs;
+    auto tile = [n_kb](double w) { return n_kb * fmax(72.0 * w, 440.0 + 9.0 * w) + 1800.0; };
+    const double mean = static_cast<double>(units) / t, widest = (units + t - 1) / t;
+    const double clocks = (rounds - 1) * tile(mean) + tile(widest);
+    if (best == 0 || clocks < best_clocks) best = t, best_clocks = clocks;
+  }
+  return best;
+}
+
+template <bool A8, bool ZP, bool ROWS, bool SMALL>
+pq_status launch_pair(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, void* out, int64_t K, PairParams& p, cudaStream_t st) {
+  static bool attr_set[64] = {};  // the attribute belongs to the device's copy of the kernel: once per device
+  if (ctx->device < 0 || ctx->device >= 64) return PQ_ERR_UNSUPPORTED;
+  if (!attr_set[ctx->device]) {
+    if (cudaFuncSetAttribute(gemm_w4a4_pair_ts_kernel<A8, ZP, ROWS, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(PAIR_SMEM)) != cudaSuccess)
+      return PQ_ERR_CUDA;
+    attr_set[ctx->device] = true;
+  }
+  const int max_pairs = ctx->sm_count / 2;
+  const int units = (p.M + UNIT - 1) / UNIT;
+  p.c_tiles = (p.N + 2 * CH_CTA - 1) / (2 * CH_CTA);
+  p.t_tiles = tile_rule(units, p.c_tiles, max_pairs, p.n_kb);
+  p.base_units = units / p.t_tiles;
+  p.rem_units = units % p.t_tiles;
+  const int widest = p.base_units + (p.rem_units > 0 ? 1 : 0);
+  p.half_units = (widest + 1) / 2;
+  p.box = p.half_units * (UNIT / 2);
+  const bool two = widest > p.half_units;
+  p.acc_cols = p.half_units * UNIT;
+  p.n_acc = (TMEM_COLS - 7 * A_SLOT_COLS) / p.acc_cols;  // what seven A slots leave
+  if (p.n_acc > MAX_ACC) p.n_acc = MAX_ACC;
+  p.n_a = (TMEM_COLS - p.n_acc * p.acc_cols) / A_SLOT_COLS;
+  if (p.n_a > MAX_A) p.n_a = MAX_A;
+  p.slot = (two ? 2 : 1) * p.box * BK;
+  p.stage = W_STAGE + (A8 ? 0 : (two ? 2 : 1) * p.box * PK_ROW);
+  p.n_b = MAX_B;
+  if (!A8) {
+    while (p.n_a > 6 && p.n_a * p.slot + 7 * p.stage > RING_BYTES) --p.n_a;
+    p.n_b = p.n_a;
+  }
+  p.n_land = (RING_BYTES - p.n_b * p.slot) / p.stage;
+  if (p.n_land > MAX_LAND) p.n_land = MAX_LAND;
+  if (p.n_land < p.n_a || p.n_b < p.n_a || p.n_a < N_GROUPS) return PQ_ERR_UNSUPPORTED;  // the kernel's parities rely on it
+  CUtensorMap tx, tw, to;
+  if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, p.box) : make_packed_map(ctx, &tx, xq, p.M, K / 2, p.box)) ||
+      !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH_CTA, CU_TENSOR_MAP_SWIZZLE_64B))
+    return PQ_ERR_CUDA;
+  p.tma_store = (p.ldo % 8 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
+  if (p.tma_store) {
+    if (!make_out_map(ctx, &to, out, p.M, p.N, p.ldo, 32)) return PQ_ERR_CUDA;
+  } else {
+    to = tx;  // never dereferenced
+  }
+  const int n_tiles = p.c_tiles * p.t_tiles;
+  const int pairs = n_tiles < max_pairs ? n_tiles : max_pairs;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * pairs);
+  cfg.blockDim = dim3(N_THREADS);
+  cfg.dynamicSmemBytes = PAIR_SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  // the kernel may be launched while its predecessor drains; it waits for it on the device before it reads or writes anything
+  // but the (static) weights, which hides the launch itself
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, gemm_w4a4_pair_ts_kernel<A8, ZP, ROWS, SMALL>, tx, tw, to, p) != cudaSuccess) return PQ_ERR_CUDA;
+  return pq_launch_status();
+}
+
 }  // namespace
 
-// Launches the CTA-pair kernel with the token operand in tensor memory on rows [0, M) of xq/out (the caller has already
-// applied row_begin). s_row: per-token steps (then s_a is ignored), or null. zp, wsum: the zero point of Eq. 1 and the
-// weight code sums, or null.
+// Rows [0, M) of xq/out (the caller has already applied row_begin). a8: xq holds one s8 code per element. s_row: per-token steps
+// (then s_a is ignored), or null. zp, wsum: the zero point of Eq. 1 and the weight code sums, or null.
 pq_status pq_gemm_pair_ts_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, const float* s_a, const float* s_w,
                                  void* out, int64_t ldo, int64_t M, int64_t N, int64_t K, int32_t* acc_dbg,
-                                 cudaStream_t st, const float* s_row, const int32_t* zp, const int32_t* wsum) {
-  if (zp && !wsum) return PQ_ERR_INVALID_ARG;
-  CUtensorMap ta, tb, to;
-  if (!make_packed_map(ctx, &ta, xq, M, K / 2, BM_CTA, CU_TENSOR_MAP_SWIZZLE_64B) ||
-      !make_packed_map(ctx, &tb, wq, N, K / 2, BN_CTA, CU_TENSOR_MAP_SWIZZLE_NONE))
-    return PQ_ERR_CUDA;
-  GemmParams p;
-  p.tma_store = (ldo % 8 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
-  if (p.tma_store) {
-    if (!make_out_map(ctx, &to, out, M, N, ldo)) return PQ_ERR_CUDA;
-  } else {
-    to = ta;  // never dereferenced
-  }
+                                 cudaStream_t st, bool a8, const float* s_row, const int32_t* zp, const int32_t* wsum) {
+  if (zp && (a8 || !wsum || s_row)) return PQ_ERR_INVALID_ARG;
+  if (a8 && s_row) return PQ_ERR_INVALID_ARG;
+  PairParams p;
   p.s_a = s_a;
   p.s_w = s_w;
   p.s_row = s_row;
@@ -380,40 +671,9 @@ pq_status pq_gemm_pair_ts_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* 
   p.ldo = ldo;
   p.M = static_cast<int>(M);
   p.N = static_cast<int>(N);
-  p.K = static_cast<int>(K);
-  p.tiles_m = static_cast<int>((M + 2 * BM_CTA - 1) / (2 * BM_CTA));
-  p.tiles_n = static_cast<int>((N + BN - 1) / BN);
-  static bool attr_set[64] = {};  // the attribute belongs to the device's copy of the kernel: once per device
-  if (ctx->device < 0 || ctx->device >= 64) return PQ_ERR_UNSUPPORTED;
-  if (!attr_set[ctx->device]) {
-    if (cudaFuncSetAttribute(gemm_w4a4_pair_ts_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(SMEM_BYTES)) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w4a4_pair_ts_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(SMEM_BYTES)) != cudaSuccess)
-      return PQ_ERR_CUDA;
-    attr_set[ctx->device] = true;
-  }
-  const int n_tiles = p.tiles_m * p.tiles_n;
-  const int max_pairs = ctx->sm_count / 2;
-  const int pairs = n_tiles < max_pairs ? n_tiles : max_pairs;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(N_THREADS);
-  cfg.dynamicSmemBytes = SMEM_BYTES;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  // the kernel may be launched while its predecessor drains; it waits for it on the device before it
-  // reads or writes anything (griddepcontrol.wait at its top), which hides the launch itself
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  if ((zp ? cudaLaunchKernelEx(&cfg, gemm_w4a4_pair_ts_kernel<true>, ta, tb, to, p)
-          : cudaLaunchKernelEx(&cfg, gemm_w4a4_pair_ts_kernel<false>, ta, tb, to, p)) != cudaSuccess)
-    return PQ_ERR_CUDA;
-  return pq_launch_status();
+  p.n_kb = static_cast<int>((K + BK - 1) / BK);
+  const bool small = K <= 4096;  // 8-bit tokens: |sum| <= 128 * 8 * K <= 2^22; 4-bit tokens: 8 * 8 * K for every K
+  if (a8) return small ? launch_pair<true, false, false, true>(ctx, xq, wq, out, K, p, st) : launch_pair<true, false, false, false>(ctx, xq, wq, out, K, p, st);
+  if (zp) return launch_pair<false, true, false, false>(ctx, xq, wq, out, K, p, st);
+  return s_row ? launch_pair<false, false, true, true>(ctx, xq, wq, out, K, p, st) : launch_pair<false, false, false, true>(ctx, xq, wq, out, K, p, st);
 }

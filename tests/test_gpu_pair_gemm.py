@@ -1,0 +1,24 @@
+"""GPU parity of the CTA-pair GEMMs against the CPU oracle where their tiles can go wrong: every width of a token tile, tiles of two
+widths in one launch, a second half narrower than the first, one K block and K tails, more K blocks than any ring holds, several tiles
+per pair, ragged channels, both kinds of output store; and 8-bit tokens on more than three rounds of tiles (the kernel with both
+operands in shared memory)."""
+import pytest
+
+from test_gpu_split_gemm import check, ctx  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K,ldo_pad", [
+    (129, 8448, 32, 0), (161, 8300, 416, 0), (193, 8448, 1152, 3), (256, 8300, 160, 0), (100, 19000, 96, 0),  # one tile per channel tile, or two
+    (257, 4250, 1312, 5), (300, 6144, 1152, 0), (515, 2250, 640, 0), (700, 1500, 2080, 8), (1000, 770, 128, 0), (1500, 264, 992, 0),
+    (333, 9500, 256, 0),                                                                                     # several tiles per pair
+])
+def test_pair_gemm_matches_oracle(ctx, mode, M, N, K, ldo_pad):  # noqa: F811
+    check(ctx, mode, M, N, K, ldo_pad)
+
+
+@pytest.mark.parametrize("M,N,K,row_begin", [(130, 57100, 32, 0), (300, 28700, 416, 4)])
+def test_many_tiles_of_8bit_tokens_match_oracle(ctx, M, N, K, row_begin):  # noqa: F811
+    check(ctx, "w4a8", M, N, K, row_begin=row_begin)
