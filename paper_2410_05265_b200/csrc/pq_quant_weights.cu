@@ -44,13 +44,17 @@ __global__ void __launch_bounds__(QW_THREADS) quant_weights_kernel(const __nv_bf
 // Bound by HBM (2.5 bytes per weight) once a code costs few instructions. A code is rint(w / s) with an IEEE division; here it is
 // rint(w * r), r ~ 1 / s, from one fused multiply-add into the rounding constant 1.5 * 2^23, checked per row: both are monotone in w
 // and can differ only next to a half-integer, which for bf16 weights means at one of the few bf16 values around (k + 1/2) s,
-// k = 0 .. 6 (bf16 values are 2^-8 apart, the two quotients less than 2^-21). Seven lanes compare the two forms there, for r = 1 / s and
+// k = 0 .. 6 (bf16 values are 2^-8 apart, the two quotients less than 2^-21). A lane each compares the two forms there, for r = 1 / s and
 // its two neighbours; a row where none agrees (about one maximum in nine: a multiple of 7), that holds an infinity or a NaN, or
 // whose step is far from 1 divides element by element.
-// Measured (us, two passes with a division each / now): 28672 x 4096 129 / 60 (4.9 TB/s), 4096 x 14336 64 / 31, 8192 x 28672
-// 256 / 121, 4096 x 4096 20.6 / 13.1.
+// Eight codes are packed by multiply-adds (a digit each), and each lane checks one of the 28 values, for all of its four vectors: with
+// masks and shifts, and four checked values per lane, instruction issue (82 %) was the bound.
+// Measured (us, two passes with a division each / masks, four values a lane / now): 28672 x 4096 129 / 58.7 / 48.9 (6.0 TB/s),
+// 4096 x 14336 64 / 31.5 / 29.0, 8192 x 28672 256 / 118 / 106, 4096 x 4096 20.6 / 12.2 / 10.6. Half the threads with twice the
+// vectors: 47.7, 32.6 (512 threads), 106, 12.0.
 __device__ __forceinline__ int code_div(float w, float s) { return max(-8, min(7, __float2int_rn(__fdiv_rn(w, s)))); }
-__device__ __forceinline__ uint32_t code_mul(float w, float r) { return __float_as_uint(fmaf(w, r, 12582912.0f)); }  // code in the low bits
+// code + 8 in the low bits; what stands above them is constant
+__device__ __forceinline__ uint32_t code_mul(float w, float r) { return __float_as_uint(fmaf(w, r, 12582920.0f)); }
 
 template <int THREADS, int VPT>
 __global__ void __launch_bounds__(THREADS) quant_weights_once_kernel(const __nv_bfloat16* __restrict__ W, int K, int64_t ldw,
@@ -102,18 +106,15 @@ __global__ void __launch_bounds__(THREADS) quant_weights_once_kernel(const __nv_
   float r = __fdiv_rn(1.0f, s);
   bool same = s > 1e-30f && s < 1e30f && !special;
   {
-    const int k = min(static_cast<int>(threadIdx.x & 31), 6);
-    const uint32_t h = __float_as_uint((k + 0.5f) * s) >> 16;  // the bf16 value at or below the half-integer, and its neighbours
+    const int k = min(static_cast<int>(threadIdx.x & 7), 6), d = static_cast<int>((threadIdx.x & 31) >> 3) - 1;
+    const uint32_t h = __float_as_uint((k + 0.5f) * s) >> 16;  // the bf16 value at or below the half-integer; its neighbours: one a lane
     const uint32_t rb = __float_as_uint(r);
     uint32_t ok = 7;  // bit c: candidate c agrees
+    const float b = __uint_as_float((h + d) << 16);
+    const uint32_t want = static_cast<uint32_t>(code_div(b, s) + 8);
 #pragma unroll
-    for (int d = -1; d <= 2; ++d) {
-      const float b = __uint_as_float((h + d) << 16);
-      const uint32_t want = static_cast<uint32_t>(code_div(b, s));
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        if ((code_mul(b, __uint_as_float(rb + (c == 2 ? -1 : c))) & 0xFu) != want) ok &= ~(1u << c);
-    }
+    for (int c = 0; c < 3; ++c)
+      if ((code_mul(b, __uint_as_float(rb + (c == 2 ? -1 : c))) & 0xFu) != want) ok &= ~(1u << c);
     ok = __reduce_and_sync(0xffffffffu, ok);
     same = same && ok != 0;
     r = __uint_as_float(rb + ((ok & 1) ? 0 : (ok & 2) ? 1 : -1));
@@ -126,11 +127,12 @@ __global__ void __launch_bounds__(THREADS) quant_weights_once_kernel(const __nv_
     const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
     uint32_t o = 0;
     if (same) {
+      // the sum of (constant + code + 8) * 16^i: no digit carries into the next, the constants' part is subtracted, and flipping
+      // every digit's top bit turns code + 8 into the two's-complement code
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t a = code_mul(__uint_as_float(w[e] << 16), r), b = code_mul(__uint_as_float(w[e] & 0xFFFF0000u), r);
-        o |= ((a & 0xFu) | ((b & 0xFu) << 4)) << (8 * e);
-      }
+      for (int e = 3; e >= 0; --e)
+        o = (o * 16u + code_mul(__uint_as_float(w[e] & 0xFFFF0000u), r)) * 16u + code_mul(__uint_as_float(w[e] << 16), r);
+      o = (o - 0x4B400000u * 0x11111111u) ^ 0x88888888u;
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e)
