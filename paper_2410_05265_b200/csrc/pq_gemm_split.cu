@@ -49,12 +49,15 @@ constexpr int EXPAND_WARP0 = 4;
 constexpr int MAX_SPLIT = 8;               // portable cluster size
 
 // Shapes of the rings. Up to 128 tokens two CTAs share an SM (113 KB and 256 TMEM columns each), so that one loads
-// while the other expands or reduces; 256 tokens take a whole SM.
+// while the other expands or reduces; 256 tokens take a whole SM. Four operand slots where they fit: with two, a slot came back later
+// (commit, expansion, fence, arrival) than the other's MMAs took. us, rotation and GEMM in a graph, two slots -> four: 33 x 28672 x 4096
+// 19.9 -> 19.5, 64 x 28672 x 4096 21.2 -> 20.3 (for two of its eight weight stages), 64 x 4096 x 14336 16.2 -> 15.7; linear set of the 70B layer at
+// 64 tokens, W4A8, 150.4 -> 128.4, 8B layer at 64 65.2 -> 63.1.
 template <int NT, bool A8>
 struct Cfg {
   static constexpr int GROUPS = NT == 256 ? 4 : 2;
-  static constexpr int SLOTS = NT == 48 || NT == 64 || ((NT == 96 || NT == 128) && !A8) ? 2 : 4;
-  static constexpr int STAGES = NT <= 64 ? 8 : 4;    // landing ring, weights
+  static constexpr int SLOTS = NT == 128 && !A8 ? 2 : 4;
+  static constexpr int STAGES = NT <= 48 ? 8 : (NT == 64 ? 6 : 4);  // landing ring, weights
   static constexpr int X_STAGES = NT <= 32 ? 8 : 4;  // landing ring, tokens
   static constexpr bool EARLY_W = NT == 256;         // weight stages go back before the (long) token part of the expansion
   static constexpr int X_STAGE = A8 ? 0 : NT * PK_ROW;
