@@ -312,7 +312,7 @@ def run_gpu(args):
         attainable = {"error": repr(e)}
     traffic, traffic_note = recorded_traffic()
     roofline = {
-        "kernel": "gemm_w4a4_pair_kernel (the four GEMM launches of the step)", "bound": "tensor", "achieved": round(achieved, 1),
+        "kernel": "gemm_w4a4_pair_ts_kernel (the four GEMM launches of the step)", "bound": "tensor", "achieved": round(achieved, 1),
         "peak": round(int8_peak, 1), "unit": "TOPS", "frac": round(achieved / int8_peak, 4), "traffic": traffic, "traffic_note": traffic_note,
         "peak_source": f"2 x bf16 {peak_kind} GEMM of {peaks['src']} (timed region {timed_s:.2f} s)",
         "frac_of_nominal_4500": round(achieved / NOMINAL_INT8_TOPS, 4), "attainable_int8": attainable,

@@ -55,17 +55,17 @@ constexpr int MAX_SPLIT = 8;               // portable cluster size
 // 64 tokens, W4A8, 150.4 -> 128.4, 8B layer at 64 65.2 -> 63.1.
 template <int NT, bool A8>
 struct Cfg {
-  static constexpr int GROUPS = NT == 256 ? 4 : 2;
+  static constexpr int GROUPS = NT > 128 ? 4 : 2;
   static constexpr int SLOTS = NT == 128 && !A8 ? 2 : 4;
   static constexpr int STAGES = NT <= 48 ? 8 : (NT == 64 ? 6 : 4);  // landing ring, weights
   static constexpr int X_STAGES = NT <= 32 ? 8 : 4;  // landing ring, tokens
-  static constexpr bool EARLY_W = NT == 256;         // weight stages go back before the (long) token part of the expansion
+  static constexpr bool EARLY_W = NT > 128;          // weight stages go back before the (long) token part of the expansion
   static constexpr int X_STAGE = A8 ? 0 : NT * PK_ROW;
   static constexpr int SLOT = NT * BK;
   static constexpr int A_COL0 = NT < 32 ? 32 : NT;  // accumulator columns, then the A slots
-  static constexpr int TMEM_COLS = NT == 256 ? 512 : 256;
+  static constexpr int TMEM_COLS = NT > 128 ? 512 : 256;
   static constexpr int THREADS = (EXPAND_WARP0 + 4 * GROUPS) * 32;
-  static constexpr int CTAS_PER_SM = NT == 256 ? 1 : 2;
+  static constexpr int CTAS_PER_SM = NT > 128 ? 1 : 2;
   static constexpr int RING = SLOTS * SLOT + STAGES * W_STAGE + X_STAGES * X_STAGE;
   static constexpr int PART = NT * CH * 4;  // the int32 partial tile, laid over the rings at the end
   static_assert(A_COL0 + SLOTS * A_SLOT_COLS <= TMEM_COLS, "tensor memory budget");
@@ -487,7 +487,8 @@ pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw
 
 template <bool A8, bool ZP>
 pq_status launch_tokens(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, SplitParams& p, int64_t K, cudaStream_t st) {
-  const int nt = p.M <= 16 ? 16 : (p.M <= 32 ? 32 : (p.M <= 48 ? 48 : (p.M <= 64 ? 64 : (p.M <= 96 ? 96 : (p.M <= 128 ? 128 : 256)))));
+  const int per_tile = (p.M + (p.M + 255) / 256 - 1) / ((p.M + 255) / 256);  // above 128 tokens: spread over as few tiles as hold them
+  const int nt = p.M <= 16 ? 16 : (p.M <= 32 ? 32 : (p.M <= 48 ? 48 : (p.M <= 64 ? 64 : (p.M <= 96 ? 96 : (p.M <= 128 ? 128 : (per_tile <= 192 ? 192 : 256))))));
   CUtensorMap tx, tw;
   if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, nt) : make_packed_map(ctx, &tx, xq, p.M, K / 2, nt)) ||
       !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH, CU_TENSOR_MAP_SWIZZLE_64B))
@@ -499,6 +500,7 @@ pq_status launch_tokens(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, Split
     case 64: return launch_split<64, A8, ZP>(ctx, tx, tw, p, st);
     case 96: return launch_split<96, A8, ZP>(ctx, tx, tw, p, st);
     case 128: return launch_split<128, A8, ZP>(ctx, tx, tw, p, st);
+    case 192: return launch_split<192, A8, ZP>(ctx, tx, tw, p, st);
     default: return launch_split<256, A8, ZP>(ctx, tx, tw, p, st);
   }
 }

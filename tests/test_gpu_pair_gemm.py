@@ -22,3 +22,9 @@ def test_pair_gemm_matches_oracle(ctx, mode, M, N, K, ldo_pad):  # noqa: F811
 @pytest.mark.parametrize("M,N,K,row_begin", [(130, 57100, 32, 0), (300, 28700, 416, 4)])
 def test_many_tiles_of_8bit_tokens_match_oracle(ctx, M, N, K, row_begin):  # noqa: F811
     check(ctx, "w4a8", M, N, K, row_begin=row_begin)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M", [129, 192, 193, 257, 384, 385])
+def test_split_gemm_at_the_edges_of_its_192_token_tiles(ctx, mode, M):  # noqa: F811
+    check(ctx, mode, M, 300, 1312)
