@@ -710,8 +710,7 @@ def section_dynamic(ctx, device, peaks, acts, wqs, sws):
     ctx.check()
     ms = t0.elapsed_time(t1) / steps
     return {"ms_per_step": round(ms, 4), "TOPS": round(step_ops(m_rows) / (ms * 1e-3) / 1e12, 1),
-            "launches_per_step": "3 x (dyn_hadamard_quant_act in one pass + w4a4_gemm_rows) for the 4096-wide inputs, "
-                                 "1 x (step pass + memset + code pass + w4a4_gemm_rows) for the down projection (7 blocks per row)"}
+            "launches_per_step": "4 x (dyn_hadamard_quant_act in one pass + w4a4_gemm_rows)"}
 
 
 def section_block(ctx, device, peaks):
