@@ -4,14 +4,15 @@
 #pragma once
 
 #include "pq_common.cuh"
+#include "pq_gemm_plan.cuh"
 
 namespace pq_pair {
 
 constexpr int BM_CTA = 128;                 // token rows per CTA (256 per pair)
 constexpr int BN = 256;                     // output channels per pair tile
 constexpr int BN_CTA = 128;                 // weight rows expanded by each CTA
-constexpr int BK = 128;                     // K elements per stage
-constexpr int PK_ROW = BK / 2;              // packed bytes per row per stage
+using pq_plan::BK;
+using pq_plan::PK_ROW;
 constexpr int EPI_COLS = 64;                // columns per TMA store (128 bytes of bf16)
 constexpr int EPI_BUF = 32 * EPI_COLS * 2;  // 4 KB: one warp's 32 rows x 64 columns
 

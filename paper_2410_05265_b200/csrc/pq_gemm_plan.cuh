@@ -1,0 +1,202 @@
+// What a GEMM call runs and in which shape: the kernel, its tiles, its rings and what they take of shared and tensor memory. Plain C++
+// without a CUDA header, so that the rules are compiled for the host, too, and walked over all sizes by tests/test_gemm_plan.py.
+#pragma once
+
+#include <math.h>
+#include <stddef.h>
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define PQ_HD __host__ __device__ __forceinline__
+#else
+#define PQ_HD inline
+#endif
+
+namespace pq_plan {
+
+constexpr int BK = 128;                     // K elements per stage
+constexpr int PK_ROW = BK / 2;              // packed bytes per row per stage
+constexpr int A_SLOT_COLS = BK / 4;         // 32 columns of tensor memory = 128 K bytes per lane
+
+// ---- which kernel ---------------------------------------------------------------------------------
+enum Route { STREAM, SPLIT, PAIR_TS, PAIR };
+
+// The kernel for m rows.
+// Weight-streaming kernel or split-K tensor-core kernel (figures: rotate+quantize and GEMM in a graph, us, streaming against
+// split). The streaming kernel has the shorter chain, but expands the tokens again for every 16 channels and has no K split:
+//   up to 8 tokens   always streaming. Alone behind its rotation kernel the other is faster on 8192 x 28672 (1 token: 29.2 / 24.4)
+//                    and 8192 x 8192 (11.4 / 10.4), but inside a decode layer the streaming kernel's shorter chain and earlier
+//                    weight requests win: whole 70B layer 124 / 132 us
+//   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
+//                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
+//   up to 96         always split (CTA pairs: 40 tokens, 28672 x 4096: 23.0 / 19.8; 8192 x 28672: 59.5 / 31.6)
+//   97 to 128        while every channel tile has its CTAs at once (128 tokens, pairs against split, 57344 x 8192: 74.6 / 85.7,
+//                    28672 x 4096: 25.1 / 27.0; but 10240 x 8192: 25.3 / 23.5)
+//   above            while the 256-token tiles leave room for two K splits (pairs against split at 256 tokens: 8192 x 8192 26.0 / 23.5,
+//                    4096 x 14336 35.7 / 24.2, 6144 x 4096 17.4 / 17.2; at 400, 4096 x 14336 37.8 / 31.9, 4096 x 4096 17.7 / 17.3). With a single
+//                    split the pairs win: 57344 x 8192 at 200 tokens 91 / 129, 28672 x 4096 30.1 / 39.3, 10240 x 8192 31.5 / 35.8, 6144 x 4096
+//                    at 300 17.9 / 21.7, 4096 x 14336 at 515 39.2 / 49.4.
+// CTA pairs. Few rounds of 8-bit tiles, and 4-bit tokens always: weights in tensor memory, tiles as wide as fit the chip
+// (pq_gemm_tc3.cu). More than three rounds of 8-bit tiles at K <= 8192: both operands in shared memory, two whole accumulators
+// (pq_gemm_tc2.cu, with the figures).
+inline Route gemm_route(int64_t m, int64_t N, int64_t K, bool a8, int sm_count) {
+  const int64_t ctiles = (N + 127) / 128, weights = N * K;
+  const bool split = m <= 8     ? false
+                     : m <= 16  ? weights >= (int64_t{20} << 20)
+                     : m <= 96  ? true
+                     : m <= 128 ? ctiles <= sm_count
+                                : 2 * ((m + 255) / 256) * ctiles <= sm_count * 7 / 8;
+  if (split) return SPLIT;
+  if (m <= 16) return STREAM;
+  const int64_t tiles = ((m + 255) / 256) * ((N + 255) / 256);
+  return a8 && K <= 8192 && tiles > 3 * (sm_count / 2) ? PAIR : PAIR_TS;
+}
+
+// A position in a ring of n slots and the parity of its current round.
+struct Pos {
+  int i = 0, ph = 0;
+  PQ_HD void advance(int k, int n) {  // k <= n
+    i += k;
+    if (i >= n) i -= n, ph ^= 1;
+  }
+};
+
+// ---- CTA pairs, weights in tensor memory (pq_gemm_tc3.cu) --------------------------------------------
+constexpr int UNIT = 32;                    // tokens: granularity of a tile's width (N of a 256-row pair MMA comes in steps of 32)
+constexpr int MAX_UNITS = 8;
+constexpr int CH_CTA = 128;                 // output channels per CTA (256 per pair)
+constexpr int W_STAGE = CH_CTA * PK_ROW;    // 8 KB of packed weights per K block
+constexpr int MAX_LAND = 8, MAX_A = 8, MAX_B = 8, MAX_ACC = 4;  // rings: landing stages, operand slots, accumulator halves
+constexpr int N_GROUPS = 4;                 // expansion groups
+constexpr int PAIR_TMEM_COLS = 512;
+constexpr int RING_BYTES = 192 * 1024;      // landing stages and token operands
+
+struct PairPlan {
+  int c_tiles, t_tiles;    // tiles along the channels and along the tokens
+  int base_units, rem_units;  // token tile i is base_units + (i < rem_units) units wide
+  int half_units;          // units of a tile's first half (as far as it has so many): half of the widest tile's
+  int box;                 // token rows per TMA box and of a CTA's share of a first half
+  int n_land, n_a, n_b, n_acc;  // ring lengths (4-bit tokens: n_b = n_a, the two operand rings turn together)
+  int stage, slot, acc_cols;    // bytes of a landing stage and of a token operand slot, columns of an accumulator half
+};
+
+struct Tile {
+  int n0, t0;  // first channel, first token
+  int u0, u1;  // units of the two halves (u1 = 0: one half)
+};
+PQ_HD Tile tile_at(const PairPlan& p, int idx) {
+  const int c = idx / p.t_tiles, i = idx - c * p.t_tiles;  // the token tiles of a channel tile are neighbours: its weights are in L2
+  const int units = p.base_units + (i < p.rem_units ? 1 : 0);
+  Tile t;
+  t.n0 = c * 2 * CH_CTA;
+  t.t0 = (i * p.base_units + (i < p.rem_units ? i : p.rem_units)) * UNIT;
+  t.u0 = units < p.half_units ? units : p.half_units;
+  t.u1 = units - t.u0;
+  return t;
+}
+
+// The accumulator slots a tile's halves take in turn.
+struct AccRing {
+  Pos u;
+  PQ_HD Pos slot(int h, const PairPlan& p) const {
+    Pos mine = u;
+    mine.advance(h, p.n_acc);
+    return mine;
+  }
+  PQ_HD void advance(int, const Tile& t, const PairPlan& p) { u.advance(t.u1 > 0 ? 2 : 1, p.n_acc); }
+};
+
+// The number of token tiles per channel tile: the one with the shortest estimate for the launch, in whole rounds of the chip's pairs.
+// Clocks of a K block, measured on one round of tiles of 64, 128, 192 and 256 tokens (K = 4096 and 8192): 458, 472, 497, 578 (8-bit tokens
+// 397, 416, 452, 578): wide tiles take their MMAs' time (64 clocks per unit) and a little, narrow ones that of the expansion and of
+// the issue, which hardly depend on the width. A tile adds about 1800 clocks of its own. Gains, narrower tiles against the widest (us,
+// with the rotation): 1000 x 6144 x 4096 34.2 / 41, 1000 x 4096 x 4096 21.5 / 24.6, 1500 x 4096 x 14336 76 / 86.
+// With more than three rounds of the widest tiles those stay: the ragged round weighs less there, the chip runs at its power limit, and
+// narrower tiles expand the weights more often (2044 x 28672 x 4096: 169 with nine tiles, 156 with eight).
+inline int tile_rule(int units, int c_tiles, int n_pairs, int n_kb) {
+  int best = 0;
+  double best_clocks = 0.0;
+  const int t_min = (units + MAX_UNITS - 1) / MAX_UNITS;
+  if (c_tiles * t_min > 3 * n_pairs) return t_min;
+  for (int t = t_min; t <= units && t <= t_min + 8; ++t) {
+    const int rounds = (c_tiles * t + n_pairs - 1) / n_pairs;
+    auto tile = [n_kb](double w) { return n_kb * fmax(72.0 * w, 440.0 + 9.0 * w) + 1800.0; };
+    const double mean = static_cast<double>(units) / t, widest = (units + t - 1) / t;
+    const double clocks = (rounds - 1) * tile(mean) + tile(widest);
+    if (best == 0 || clocks < best_clocks) best = t, best_clocks = clocks;
+  }
+  return best;
+}
+
+// False when the rings do not fit (no size known).
+inline bool pair_plan(PairPlan& p, int M, int N, int n_kb, bool a8, int sm_count) {
+  const int units = (M + UNIT - 1) / UNIT;
+  p.c_tiles = (N + 2 * CH_CTA - 1) / (2 * CH_CTA);
+  p.t_tiles = tile_rule(units, p.c_tiles, sm_count / 2, n_kb);
+  p.base_units = units / p.t_tiles;
+  p.rem_units = units % p.t_tiles;
+  const int widest = p.base_units + (p.rem_units > 0 ? 1 : 0);
+  p.half_units = (widest + 1) / 2;
+  p.box = p.half_units * (UNIT / 2);
+  const bool two = widest > p.half_units;
+  p.acc_cols = p.half_units * UNIT;
+  p.n_acc = (PAIR_TMEM_COLS - 7 * A_SLOT_COLS) / p.acc_cols;  // what seven A slots leave
+  if (p.n_acc > MAX_ACC) p.n_acc = MAX_ACC;
+  p.n_a = (PAIR_TMEM_COLS - p.n_acc * p.acc_cols) / A_SLOT_COLS;
+  if (p.n_a > MAX_A) p.n_a = MAX_A;
+  p.slot = (two ? 2 : 1) * p.box * BK;
+  p.stage = W_STAGE + (a8 ? 0 : (two ? 2 : 1) * p.box * PK_ROW);
+  p.n_b = MAX_B;
+  if (!a8) {
+    while (p.n_a > 6 && p.n_a * p.slot + 7 * p.stage > RING_BYTES) --p.n_a;
+    p.n_b = p.n_a;
+  }
+  p.n_land = (RING_BYTES - p.n_b * p.slot) / p.stage;
+  if (p.n_land > MAX_LAND) p.n_land = MAX_LAND;
+  return p.n_land >= p.n_a && p.n_b >= p.n_a && p.n_a >= N_GROUPS;  // the kernel's parities rely on it
+}
+
+// ---- split K (pq_gemm_split.cu) -----------------------------------------------------------------------
+constexpr int CH = 128;                    // output channels per CTA
+constexpr int SPLIT_BAR_BYTES = 512;       // no less than the kernel's barriers take
+
+// Shapes of the rings. Up to 128 tokens two CTAs share an SM (113 KB and 256 TMEM columns each), so that one loads
+// while the other expands or reduces; 256 tokens take a whole SM. Four operand slots where they fit: with two, a slot came back later
+// (commit, expansion, fence, arrival) than the other's MMAs took. us, rotation and GEMM in a graph, two slots -> four: 33 x 28672 x 4096
+// 19.9 -> 19.5, 64 x 28672 x 4096 21.2 -> 20.3 (for two of its eight weight stages), 64 x 4096 x 14336 16.2 -> 15.7; linear set of the 70B layer at
+// 64 tokens, W4A8, 150.4 -> 128.4, 8B layer at 64 65.2 -> 63.1.
+template <int NT, bool A8>
+struct SplitCfg {
+  static constexpr int GROUPS = NT > 128 ? 4 : 2;
+  static constexpr int SLOTS = NT == 128 && !A8 ? 2 : 4;
+  static constexpr int STAGES = NT <= 48 ? 8 : (NT == 64 ? 6 : 4);  // landing ring, weights
+  static constexpr int X_STAGES = NT <= 32 ? 8 : 4;  // landing ring, tokens
+  static constexpr bool EARLY_W = NT > 128;          // weight stages go back before the (long) token part of the expansion
+  static constexpr int X_STAGE = A8 ? 0 : NT * PK_ROW;
+  static constexpr int SLOT = NT * BK;
+  static constexpr int A_COL0 = NT < 32 ? 32 : NT;  // accumulator columns, then the A slots
+  static constexpr int TMEM_COLS = NT > 128 ? 512 : 256;
+  static constexpr int CTAS_PER_SM = NT > 128 ? 1 : 2;
+  static constexpr int RING = SLOTS * SLOT + STAGES * (CH * PK_ROW) + X_STAGES * X_STAGE;
+  static constexpr int PART = NT * CH * 4;  // the int32 partial tile, laid over the rings at the end
+  static_assert(A_COL0 + SLOTS * A_SLOT_COLS <= TMEM_COLS, "tensor memory budget");
+  static_assert(STAGES % GROUPS == 0 && X_STAGES % GROUPS == 0 && SLOTS % GROUPS == 0, "a ring slot is always served by the same group");
+  static_assert(PART <= RING, "the partial tile fits where the rings were");
+  static_assert(SLOTS <= STAGES, "no weight stage is refilled before the first operand slot is");
+};
+
+// At least 80 KB, so that no more CTAs share an SM than its tensor memory serves: a CTA that waited for columns which
+// another cluster's CTA gives back only behind its cluster barrier could wait for itself.
+template <int NT, bool A8>
+constexpr size_t split_smem() {
+  const size_t need = 1024 /*alignment slack*/ + SplitCfg<NT, A8>::RING + SPLIT_BAR_BYTES;
+  return need < 80 * 1024 ? 80 * 1024 : need;
+}
+
+// The width of the token tiles: above 128 tokens they are spread over as few tiles as hold them.
+inline int split_width(int M) {
+  const int per_tile = (M + (M + 255) / 256 - 1) / ((M + 255) / 256);
+  return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 48 ? 48 : (M <= 64 ? 64 : (M <= 96 ? 96 : (M <= 128 ? 128 : (per_tile <= 192 ? 192 : 256))))));
+}
+
+}  // namespace pq_plan

@@ -41,37 +41,14 @@
 namespace {
 
 using namespace pq_pair;
+using namespace pq_plan;
 
-constexpr int CH = 128;                    // output channels per CTA
-constexpr int W_STAGE = CH * PK_ROW;       // 8 KB of packed weights per K block
-constexpr int A_SLOT_COLS = BK / 4;        // 32 TMEM columns = 128 K bytes per lane
 constexpr int EXPAND_WARP0 = 4;
 constexpr int MAX_SPLIT = 8;               // portable cluster size
 
-// Shapes of the rings. Up to 128 tokens two CTAs share an SM (113 KB and 256 TMEM columns each), so that one loads
-// while the other expands or reduces; 256 tokens take a whole SM. Four operand slots where they fit: with two, a slot came back later
-// (commit, expansion, fence, arrival) than the other's MMAs took. us, rotation and GEMM in a graph, two slots -> four: 33 x 28672 x 4096
-// 19.9 -> 19.5, 64 x 28672 x 4096 21.2 -> 20.3 (for two of its eight weight stages), 64 x 4096 x 14336 16.2 -> 15.7; linear set of the 70B layer at
-// 64 tokens, W4A8, 150.4 -> 128.4, 8B layer at 64 65.2 -> 63.1.
 template <int NT, bool A8>
-struct Cfg {
-  static constexpr int GROUPS = NT > 128 ? 4 : 2;
-  static constexpr int SLOTS = NT == 128 && !A8 ? 2 : 4;
-  static constexpr int STAGES = NT <= 48 ? 8 : (NT == 64 ? 6 : 4);  // landing ring, weights
-  static constexpr int X_STAGES = NT <= 32 ? 8 : 4;  // landing ring, tokens
-  static constexpr bool EARLY_W = NT > 128;          // weight stages go back before the (long) token part of the expansion
-  static constexpr int X_STAGE = A8 ? 0 : NT * PK_ROW;
-  static constexpr int SLOT = NT * BK;
-  static constexpr int A_COL0 = NT < 32 ? 32 : NT;  // accumulator columns, then the A slots
-  static constexpr int TMEM_COLS = NT > 128 ? 512 : 256;
-  static constexpr int THREADS = (EXPAND_WARP0 + 4 * GROUPS) * 32;
-  static constexpr int CTAS_PER_SM = NT > 128 ? 1 : 2;
-  static constexpr int RING = SLOTS * SLOT + STAGES * W_STAGE + X_STAGES * X_STAGE;
-  static constexpr int PART = NT * CH * 4;  // the int32 partial tile, laid over the rings at the end
-  static_assert(A_COL0 + SLOTS * A_SLOT_COLS <= TMEM_COLS, "tensor memory budget");
-  static_assert(STAGES % GROUPS == 0 && X_STAGES % GROUPS == 0 && SLOTS % GROUPS == 0, "a ring slot is always served by the same group");
-  static_assert(PART <= RING, "the partial tile fits where the rings were");
-  static_assert(SLOTS <= STAGES, "no weight stage is refilled before the first operand slot is");
+struct Cfg : SplitCfg<NT, A8> {
+  static constexpr int THREADS = (EXPAND_WARP0 + 4 * Cfg::GROUPS) * 32;
 };
 
 struct __align__(8) SplitBarriers {
@@ -83,13 +60,7 @@ struct __align__(8) SplitBarriers {
   volatile int abort_flag;
 };
 
-// At least 80 KB, so that no more CTAs share an SM than its tensor memory serves: a CTA that waited for columns which
-// another cluster's CTA gives back only behind its cluster barrier could wait for itself.
-template <int NT, bool A8>
-constexpr size_t split_smem() {
-  const size_t need = 1024 /*alignment slack*/ + Cfg<NT, A8>::RING + sizeof(SplitBarriers);
-  return need < 80 * 1024 ? 80 * 1024 : need;
-}
+static_assert(sizeof(SplitBarriers) <= SPLIT_BAR_BYTES, "shared memory budget");
 
 struct SplitParams {
   const int32_t* zp;
@@ -487,8 +458,7 @@ pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw
 
 template <bool A8, bool ZP>
 pq_status launch_tokens(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, SplitParams& p, int64_t K, cudaStream_t st) {
-  const int per_tile = (p.M + (p.M + 255) / 256 - 1) / ((p.M + 255) / 256);  // above 128 tokens: spread over as few tiles as hold them
-  const int nt = p.M <= 16 ? 16 : (p.M <= 32 ? 32 : (p.M <= 48 ? 48 : (p.M <= 64 ? 64 : (p.M <= 96 ? 96 : (p.M <= 128 ? 128 : (per_tile <= 192 ? 192 : 256))))));
+  const int nt = split_width(p.M);
   CUtensorMap tx, tw;
   if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, nt) : make_packed_map(ctx, &tx, xq, p.M, K / 2, nt)) ||
       !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH, CU_TENSOR_MAP_SWIZZLE_64B))

@@ -8,7 +8,7 @@
 // memory; the tokens are the column side: each CTA expands half of them into the 128-byte-swizzled shared-memory operand, and the
 // tensor cores of the pair exchange the halves.
 //
-// The width of a tile is a multiple of 32 tokens, chosen per launch (tile_rule): a token tile costs what its tokens cost, and a
+// The width of a tile is a multiple of 32 tokens, chosen per launch (tile_rule in pq_gemm_plan.cuh): a token tile costs what its tokens cost, and a
 // launch fills whole rounds of the chip's CTA pairs. A tile is accumulated in two halves of at most 128 columns, each with an MMA
 // issuer and epilogue warps of its own, which go round two to four slots of tensor memory; the rest of it is six to eight A slots of
 // 32 columns (128 K bytes per lane). The half that is ahead is read out while the other still runs.
@@ -46,20 +46,13 @@
 namespace {
 
 using namespace pq_pair;
+using namespace pq_plan;
 
-constexpr int UNIT = 32;                    // tokens: granularity of a tile's width (N of a 256-row pair MMA comes in steps of 32)
-constexpr int MAX_UNITS = 8;
-constexpr int CH_CTA = 128;                 // output channels per CTA (256 per pair)
-constexpr int W_STAGE = CH_CTA * PK_ROW;    // 8 KB of packed weights per K block
-constexpr int MAX_LAND = 8, MAX_A = 8, MAX_B = 8, MAX_ACC = 4;  // rings: landing stages, operand slots, accumulator halves
-constexpr int A_SLOT_COLS = BK / 4;         // 32 columns = 128 K bytes per lane
-constexpr int N_GROUPS = 4, GROUP_THREADS = 128;
+constexpr int GROUP_THREADS = 128;
 constexpr int EPI_WARP0 = 4, EXPAND_WARP0 = 8, EPI_WARP1 = EXPAND_WARP0 + 4 * N_GROUPS;
 constexpr int N_THREADS = (EPI_WARP1 + 4) * 32;
-constexpr int TMEM_COLS = 512;
 constexpr int ST_BOX = UNIT * 64;           // one store: 32 tokens x 32 channels of bf16
 constexpr int ST_BUFS = 2;                  // staging buffers of an epilogue warp
-constexpr int RING_BYTES = 192 * 1024;      // landing stages and token operands
 
 struct __align__(8) Barriers {
   uint64_t land_full[MAX_LAND], land_empty[MAX_LAND];
@@ -76,16 +69,7 @@ struct __align__(8) Barriers {
 constexpr size_t PAIR_SMEM = 1024 /*alignment slack*/ + RING_BYTES + 8 * ST_BUFS * ST_BOX + sizeof(Barriers);
 static_assert(PAIR_SMEM <= 227 * 1024, "shared memory budget");
 
-// A position in a ring of n slots and the parity of its current round.
-struct Pos {
-  int i = 0, ph = 0;
-  __device__ __forceinline__ void advance(int k, int n) {  // k <= n
-    i += k;
-    if (i >= n) i -= n, ph ^= 1;
-  }
-};
-
-struct PairParams {
+struct PairParams : PairPlan {
   const int32_t* zp;    // ZP: the activation zero point z (device scalar) ...
   const int32_t* wsum;  // ... and the sum of every output channel's weight codes [N]
   const float* s_row;   // ROWS: per-token steps [M]; else the scalar s_a applies
@@ -96,30 +80,9 @@ struct PairParams {
   int32_t* status;
   int64_t ldo;
   int M, N, n_kb;
-  int c_tiles, t_tiles;    // tiles along the channels and along the tokens
-  int base_units, rem_units;  // token tile i is base_units + (i < rem_units) units wide
-  int half_units;          // units of a tile's first half (as far as it has so many): half of the widest tile's
-  int box;                 // token rows per TMA box and of a CTA's share of a first half
-  int n_land, n_a, n_b, n_acc;  // ring lengths (4-bit tokens: n_b = n_a, the two operand rings turn together)
-  int stage, slot, acc_cols;    // bytes of a landing stage and of a token operand slot, columns of an accumulator half
   int tma_store;           // out can be written with TMA stores (16-byte aligned base and row pitch)
   long long wait_clocks;   // bound of every device-side wait, in SM clocks
 };
-
-struct Tile {
-  int n0, t0;  // first channel, first token
-  int u0, u1;  // units of the two halves (u1 = 0: one half)
-};
-__device__ __forceinline__ Tile tile_at(const PairParams& p, int idx) {
-  const int c = idx / p.t_tiles, i = idx - c * p.t_tiles;  // the token tiles of a channel tile are neighbours: its weights are in L2
-  const int units = p.base_units + (i < p.rem_units ? 1 : 0);
-  Tile t;
-  t.n0 = c * 2 * CH_CTA;
-  t.t0 = (i * p.base_units + (i < p.rem_units ? i : p.rem_units)) * UNIT;
-  t.u0 = units < p.half_units ? units : p.half_units;
-  t.u1 = units - t.u0;
-  return t;
-}
 
 // D[tmem of both CTAs] (+)= A[tmem of both CTAs] * B[smem halves of both CTAs], issued by one thread of the leader CTA.
 __device__ __forceinline__ void mma2_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
@@ -207,7 +170,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
     pq::tma_prefetch_desc(&tmap_out);
   }
   if (warp == 1) {
-    tmem_alloc2(&bars->tmem_base, TMEM_COLS);
+    tmem_alloc2(&bars->tmem_base, PAIR_TMEM_COLS);
     tmem_relinquish2();
   }
   pq::tc_fence_before();
@@ -290,12 +253,12 @@ __global__ void __launch_bounds__(N_THREADS, 1)
       const int h = warp >> 1;
       const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(b_buf) + h * p.box * BK);
       const uint32_t slot_desc = p.slot >> 4;
-      Pos as, bs, u;  // operand slots (8-bit tokens: of their own), accumulator halves
+      Pos as, bs;  // operand slots (8-bit tokens: of their own)
+      AccRing u;
       for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
         const Tile t = tile_at(p, tile);
         const int units = h ? t.u1 : t.u0;  // none: only the slots are handed on
-        Pos mine = u;
-        mine.advance(h, p.n_acc);
+        const Pos mine = u.slot(h, p);
         const uint32_t d_tmem = tmem_base + mine.i * p.acc_cols, idesc = pq::umma_idesc_s8(2 * CH_CTA, units * UNIT);
         if (units > 0 && !wait_bar_warp(&bars->acc_empty[mine.i], mine.ph ^ 1, abort_flag, p.wait_clocks)) {
           ok = false;
@@ -344,7 +307,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         if (!ok) break;
         if (leader && units > 0) mma2_commit_both(&bars->acc_full[mine.i]);
         __syncwarp();
-        u.advance(t.u1 > 0 ? 2 : 1, p.n_acc);
+        u.advance(h, t, p);
       }
       if (leader) mma2_commit_both(&bars->drain);  // whatever was issued has finished before either CTA releases its tensor memory
       __syncwarp();
@@ -441,7 +404,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
     const uint32_t st_row = pq::smem_u32(my_buf) + (lane & 7) * 64;  // stmatrix: this lane addresses token row lane % 8 of a group of eight ...
     const int st_chunk = lane >> 3;                                  // ... and the 16-byte chunk (eight channels) of matrix lane / 8
     uint32_t n_store = 0;
-    Pos u;
+    AccRing u;
     for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
       const Tile t = tile_at(p, tile);
       const int n0 = t.n0 + static_cast<int>(rank) * CH_CTA + q * 32;  // the warp's channels
@@ -453,9 +416,8 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         sw[i] = n < p.N ? s_a * __ldg(p.s_w + n) : 0.0f;
         zw[i] = ZP && n < p.N ? zp8 * __ldg(p.wsum + n) : 0;
       }
-      Pos mine = u;
-      mine.advance(h, p.n_acc);
-      u.advance(t.u1 > 0 ? 2 : 1, p.n_acc);
+      const Pos mine = u.slot(h, p);
+      u.advance(h, t, p);
       const int units = h ? t.u1 : t.u0, th = t.t0 + (h ? t.u0 * UNIT : 0);
       if (units > 0) {
         if (!wait_bar_warp(&bars->acc_full[mine.i], mine.ph, abort_flag, p.wait_clocks)) {
@@ -556,30 +518,8 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   cluster_sync_all();  // neither CTA frees tensor memory or exits while the pair may still touch it
   if (warp == 1) {
     pq::tc_fence_after();
-    tmem_dealloc2(tmem_base, TMEM_COLS);
+    tmem_dealloc2(tmem_base, PAIR_TMEM_COLS);
   }
-}
-
-// The number of token tiles per channel tile: the one with the shortest estimate for the launch, in whole rounds of the chip's pairs.
-// Clocks of a K block, measured on one round of tiles of 64, 128, 192 and 256 tokens (K = 4096 and 8192): 458, 472, 497, 578 (8-bit tokens
-// 397, 416, 452, 578): wide tiles take their MMAs' time (64 clocks per unit) and a little, narrow ones that of the expansion and of
-// the issue, which hardly depend on the width. A tile adds about 1800 clocks of its own. Gains, narrower tiles against the widest (us,
-// with the rotation): 1000 x 6144 x 4096 34.2 / 41, 1000 x 4096 x 4096 21.5 / 24.6, 1500 x 4096 x 14336 76 / 86.
-// With more than three rounds of the widest tiles those stay: the ragged round weighs less there, the chip runs at its power limit, and
-// narrower tiles expand the weights more often (2044 x 28672 x 4096: 169 with nine tiles, 156 with eight).
-int tile_rule(int units, int c_tiles, int n_pairs, int n_kb) {
-  int best = 0;
-  double best_clocks = 0.0;
-  const int t_min = (units + MAX_UNITS - 1) / MAX_UNITS;
-  if (c_tiles * t_min > 3 * n_pairs) return t_min;
-  for (int t = t_min; t <= units && t <= t_min + 8; ++t) {
-    const int rounds = (c_tiles * t + n_pairs - 1) / n_pairs;
-    auto tile = [n_kb](double w) { return n_kb * fmax(72.0 * w, 440.0 + 9.0 * w) + 1800.0; };
-    const double mean = static_cast<double>(units) / t, widest = (units + t - 1) / t;
-    const double clocks = (rounds - 1) * tile(mean) + tile(widest);
-    if (best == 0 || clocks < best_clocks) best = t, best_clocks = clocks;
-  }
-  return best;
 }
 
 template <bool A8, bool ZP, bool ROWS, bool SMALL>
@@ -592,31 +532,7 @@ pq_status launch_pair(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, void* o
       return PQ_ERR_CUDA;
     attr_set[ctx->device] = true;
   }
-  const int max_pairs = ctx->sm_count / 2;
-  const int units = (p.M + UNIT - 1) / UNIT;
-  p.c_tiles = (p.N + 2 * CH_CTA - 1) / (2 * CH_CTA);
-  p.t_tiles = tile_rule(units, p.c_tiles, max_pairs, p.n_kb);
-  p.base_units = units / p.t_tiles;
-  p.rem_units = units % p.t_tiles;
-  const int widest = p.base_units + (p.rem_units > 0 ? 1 : 0);
-  p.half_units = (widest + 1) / 2;
-  p.box = p.half_units * (UNIT / 2);
-  const bool two = widest > p.half_units;
-  p.acc_cols = p.half_units * UNIT;
-  p.n_acc = (TMEM_COLS - 7 * A_SLOT_COLS) / p.acc_cols;  // what seven A slots leave
-  if (p.n_acc > MAX_ACC) p.n_acc = MAX_ACC;
-  p.n_a = (TMEM_COLS - p.n_acc * p.acc_cols) / A_SLOT_COLS;
-  if (p.n_a > MAX_A) p.n_a = MAX_A;
-  p.slot = (two ? 2 : 1) * p.box * BK;
-  p.stage = W_STAGE + (A8 ? 0 : (two ? 2 : 1) * p.box * PK_ROW);
-  p.n_b = MAX_B;
-  if (!A8) {
-    while (p.n_a > 6 && p.n_a * p.slot + 7 * p.stage > RING_BYTES) --p.n_a;
-    p.n_b = p.n_a;
-  }
-  p.n_land = (RING_BYTES - p.n_b * p.slot) / p.stage;
-  if (p.n_land > MAX_LAND) p.n_land = MAX_LAND;
-  if (p.n_land < p.n_a || p.n_b < p.n_a || p.n_a < N_GROUPS) return PQ_ERR_UNSUPPORTED;  // the kernel's parities rely on it
+  if (!pair_plan(p, p.M, p.N, p.n_kb, A8, ctx->sm_count)) return PQ_ERR_UNSUPPORTED;
   CUtensorMap tx, tw, to;
   if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, p.box) : make_packed_map(ctx, &tx, xq, p.M, K / 2, p.box)) ||
       !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH_CTA, CU_TENSOR_MAP_SWIZZLE_64B))
@@ -627,7 +543,7 @@ pq_status launch_pair(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, void* o
   } else {
     to = tx;  // never dereferenced
   }
-  const int n_tiles = p.c_tiles * p.t_tiles;
+  const int n_tiles = p.c_tiles * p.t_tiles, max_pairs = ctx->sm_count / 2;
   const int pairs = n_tiles < max_pairs ? n_tiles : max_pairs;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
