@@ -95,15 +95,22 @@ PQ_HD Tile tile_at(const PairPlan& p, int idx) {
   return t;
 }
 
-// The accumulator slots a tile's halves take in turn.
+// The accumulator slots one half of a pair's tiles takes in turn: half 0 the even ones, half 1 the odd ones. A slot has one issuer and
+// one group of epilogue warps, which wait for every phase of its barriers in order, so that the parity they wait for cannot be
+// that of two rounds back. (Slots that both halves took in turn, as three did, were waited on by warps that had not seen the phase
+// before: a half could be read before it was written, in principle.) Three slots of up to 96 columns, two for the first half and one for the
+// second, against one each and against two each with four A slots (us, with the rotation): 300 x 28672 x 4096 42.9 / 44.1 / 45.8,
+// 515 x 28672 x 4096 54.1 / 54.8 / 56.7, 515 x 57344 x 8192 179 / 179 / 189.
 struct AccRing {
   Pos u;
-  PQ_HD Pos slot(int h, const PairPlan& p) const {
-    Pos mine = u;
-    mine.advance(h, p.n_acc);
-    return mine;
+  PQ_HD Pos slot(int h, const PairPlan&) const {
+    Pos s = u;
+    s.i = 2 * u.i + h;
+    return s;
   }
-  PQ_HD void advance(int, const Tile& t, const PairPlan& p) { u.advance(t.u1 > 0 ? 2 : 1, p.n_acc); }
+  PQ_HD void advance(int h, const Tile& t, const PairPlan& p) {
+    if ((h ? t.u1 : t.u0) > 0) u.advance(1, (p.n_acc + 1 - h) / 2);
+  }
 };
 
 // The number of token tiles per channel tile: the one with the shortest estimate for the launch, in whole rounds of the chip's pairs.
@@ -153,7 +160,7 @@ inline bool pair_plan(PairPlan& p, int M, int N, int n_kb, bool a8, int sm_count
   }
   p.n_land = (RING_BYTES - p.n_b * p.slot) / p.stage;
   if (p.n_land > MAX_LAND) p.n_land = MAX_LAND;
-  return p.n_land >= p.n_a && p.n_b >= p.n_a && p.n_a >= N_GROUPS;  // the kernel's parities rely on it
+  return p.n_land >= p.n_a && p.n_b >= p.n_a && p.n_a >= N_GROUPS && p.n_acc >= 2;  // the kernel's parities rely on it
 }
 
 // ---- split K (pq_gemm_split.cu) -----------------------------------------------------------------------

@@ -10,7 +10,7 @@
 //
 // The width of a tile is a multiple of 32 tokens, chosen per launch (tile_rule in pq_gemm_plan.cuh): a token tile costs what its tokens cost, and a
 // launch fills whole rounds of the chip's CTA pairs. A tile is accumulated in two halves of at most 128 columns, each with an MMA
-// issuer and epilogue warps of its own, which go round two to four slots of tensor memory; the rest of it is six to eight A slots of
+// issuer, epilogue warps and one or two slots of tensor memory of its own; the rest of it is six to eight A slots of
 // 32 columns (128 K bytes per lane). The half that is ahead is read out while the other still runs.
 //
 // What bounds it: on one round of 256-token tiles the MMAs (four of 64 clocks per half and K block, 512 clocks; 578 measured), on narrow

@@ -1,6 +1,7 @@
-"""The launch rules of the tensor-core GEMMs, compiled for the host: tiles that cover every token once, rings that fit, the kernel
-a call takes."""
+"""The launch rules of the tensor-core GEMMs, compiled for the host: tiles that cover every token once, rings that fit, and waits of the
+accumulator ring that can only return for the phase they mean."""
 import functools
+import random
 
 import pytest
 
@@ -35,6 +36,122 @@ def test_tiles_cover_the_tokens_and_rings_fit():
             assert (t.n0, t.t0) == (0, done) and 1 <= t.u0 <= 4 and 0 <= t.u1 <= t.u0 and (t.u1 == 0 or t.u0 == p.half_units)
             done += 32 * (t.u0 + t.u1)
         assert done - 32 < M <= done
+
+
+def test_an_accumulator_slot_belongs_to_one_half():
+    """Issuer and epilogue of a half wait for every phase of their slots in turn; a parity cannot be mistaken then. A slot that
+    both halves took in turn would be waited on by warps that have not seen its phase before."""
+    for M, N, K, a8 in plans():
+        _, slots = gp.pair_tiles(gp.pair_plan(M, N, K, a8))
+        owner, uses = {}, {}
+        for h in range(2):
+            for s, ph in slots[h]:
+                if s >= 0:
+                    assert owner.setdefault(s, h) == h, f"{M} x {N} x {K}: slot {s} serves both halves"
+                    assert ph == uses.get(s, 0) % 2
+                    uses[s] = uses.get(s, 0) + 1
+
+
+class Walk:
+    """The waits and arrivals of one CTA pair as the kernel makes them, one step of a randomly chosen role at a time. Barriers count
+    completed phases; a wait sees their parity only, and the walk checks that it returned for the phase that was meant."""
+
+    def __init__(self, p, n_kb, rng, count):
+        tiles, slots = gp.pair_tiles(p)
+        self.p, self.n_kb, self.rng = p, n_kb, rng
+        self.tiles, self.slots = tiles[:count], [s[:count] for s in slots]
+        used, self.nth = {}, [[], []]  # which use of its slot a half is
+        for i in range(len(self.tiles)):
+            for h in range(2):
+                s = self.slots[h][i][0]
+                self.nth[h].append(used.get(s, 0))
+                if s >= 0:
+                    used[s] = used.get(s, 0) + 1
+        self.full, self.empty = [0] * 4, [0] * 4
+        total = len(self.tiles) * n_kb
+        self.s8_full, self.s8_done = [False] * total, [0] * total
+        self.queue = [[], []]  # arrivals of the issuers' commits: in order, some time after the commit
+
+    def parity(self, phases, parity, meant):
+        if phases % 2 == parity:
+            return False
+        assert phases == meant + 1, f"a wait for phase {meant} returned in phase {phases}"
+        return True
+
+    def issuer(self, h):
+        for i in range(len(self.tiles)):
+            slot, ph = self.slots[h][i]
+            if slot >= 0:
+                while self.nth[h][i] > 0 and not self.parity(self.empty[slot], ph ^ 1, self.nth[h][i] - 1):
+                    yield False
+            for kb in range(self.n_kb):
+                b = i * self.n_kb + kb
+                while not self.s8_full[b]:
+                    yield False
+                self.queue[h].append(("s8", b))
+                yield True
+            if slot >= 0:
+                self.queue[h].append(("acc", slot))
+            yield True
+
+    def commits(self, h):
+        while True:
+            if self.queue[h]:
+                what, i = self.queue[h].pop(0)
+                if what == "s8":
+                    self.s8_done[i] += 1
+                else:
+                    self.full[i] += 1
+                yield True
+            else:
+                yield False
+
+    def group(self, g):
+        for b in range(g, len(self.s8_full), 4):
+            while b >= self.p.n_a and self.s8_done[b - self.p.n_a] < 2:
+                yield False
+            self.s8_full[b] = True
+            yield True
+
+    def epilogue(self, h):
+        for i, t in enumerate(self.tiles):
+            slot, ph = self.slots[h][i]
+            if slot < 0:
+                continue
+            while not self.parity(self.full[slot], ph, self.nth[h][i]):
+                yield False
+            for _ in range(t.u1 if h else t.u0):
+                yield True
+            self.empty[slot] += 1
+            yield True
+
+    def run(self):
+        roles = {("issuer", h): self.issuer(h) for h in range(2)} | {("epilogue", h): self.epilogue(h) for h in range(2)}
+        roles |= {("group", g): self.group(g) for g in range(4)}
+        commits = {("commits", h): self.commits(h) for h in range(2)}
+        weight = {k: self.rng.choice((1, 1, 4, 20)) for k in roles | commits}
+        idle = 0
+        while roles:
+            names = list(roles) + list(commits)
+            if self.rng.random() < 0.02:
+                weight[self.rng.choice(names)] = self.rng.choice((0.1, 1, 4, 20))
+            k = self.rng.choices(names, [weight[n] for n in names])[0]
+            try:
+                idle = 0 if next((roles | commits)[k]) else idle + 1
+            except StopIteration:
+                del roles[k]
+                idle = 0
+            assert idle < 20000, "no role gets on"
+
+
+def test_waits_return_for_the_phase_they_mean_under_any_interleaving():
+    for n, (M, N, K, a8) in enumerate(plans()):
+        p = gp.pair_plan(M, N, K, a8)
+        if p.c_tiles * p.t_tiles <= gp.SMS // 2:
+            continue  # one tile a pair: no slot comes round again
+        for n_kb in (1, 2, 3, 5, 8):
+            for seed in range(3):
+                Walk(p, n_kb, random.Random(n * 100 + n_kb * 10 + seed), 6).run()
 
 
 @pytest.mark.parametrize("M,N,K,a8,want", [
