@@ -192,12 +192,13 @@ struct SplitCfg {
   static_assert(SLOTS <= STAGES, "no weight stage is refilled before the first operand slot is");
 };
 
-// At least 80 KB, so that no more CTAs share an SM than its tensor memory serves: a CTA that waited for columns which
-// another cluster's CTA gives back only behind its cluster barrier could wait for itself.
+// At least 80 KB for 256 columns of tensor memory and 160 KB for 512, so that no more CTAs share an SM (228 KB) than its tensor memory
+// serves, those of other launches included: a CTA that waited for columns which another cluster's CTA gives back only behind its
+// cluster barrier could wait for itself. (8-bit tokens 192 wide need 130 KB, which leave room for a CTA of a narrow form.)
 template <int NT, bool A8>
 constexpr size_t split_smem() {
-  const size_t need = 1024 /*alignment slack*/ + SplitCfg<NT, A8>::RING + SPLIT_BAR_BYTES;
-  return need < 80 * 1024 ? 80 * 1024 : need;
+  const size_t need = 1024 /*alignment slack*/ + SplitCfg<NT, A8>::RING + SPLIT_BAR_BYTES, least = SplitCfg<NT, A8>::TMEM_COLS / 256 * (80 * 1024);
+  return need < least ? least : need;
 }
 
 // The width of the token tiles: above 128 tokens they are spread over as few tiles as hold them.

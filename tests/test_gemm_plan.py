@@ -161,3 +161,15 @@ def test_waits_return_for_the_phase_they_mean_under_any_interleaving():
 ])
 def test_route(M, N, K, a8, want):
     assert gp.route(M, N, K, a8) == want
+
+
+def test_ctas_that_fit_one_sm_find_their_tensor_memory():
+    """The split kernel's clusters hold their columns until all their CTAs have met, and an allocation waits without a bound: two launches
+    whose CTAs share SMs by shared memory, but not by tensor memory, could each hold what the other waits for."""
+    forms = gp.split_shapes()
+    for a in forms:
+        for b in forms:
+            for c in forms + [(0, 0, 0, 0)]:
+                group = [f for f in (a, b, c) if f[0]]
+                if sum(smem + 1024 for *_, smem in group) <= 228 * 1024:
+                    assert sum(cols for _, _, cols, _ in group) <= 512, group
