@@ -81,9 +81,13 @@ struct __align__(8) Barriers {
   volatile int abort_flag;
 };
 
-constexpr size_t SMEM_BYTES =
+constexpr size_t NEED_BYTES =
     1024 /*alignment slack*/ + N_S8 * S8_STAGE + N_PK * PK_STAGE + EPI_BYTES + SCALE_BYTES + sizeof(Barriers);
-static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+// The whole SM, although 191 KB are used: placed beside CTAs of the rotation kernel that still run, this kernel would take the L1 cache
+// from them, on which blocks up to 1024 rely (rotation and GEMM, us, 191 / 226 KB: 1604 x 11040 x 1920 in blocks of 128 41.8 / 39.4,
+// 1997 x 7096 x 2560 40.0 / 37.3, 1902 x 9728 x 4992 88.1 / 84.3; blocks of 2048 and more leave no room for it: 2044 x 28672 x 4096 150.6).
+constexpr size_t SMEM_BYTES = 226 * 1024;
+static_assert(NEED_BYTES <= SMEM_BYTES, "shared memory budget");
 
 // D[tmem of both CTAs] (+)= A[smem of both CTAs] * B[smem halves of both CTAs], issued by one thread
 // of the leader CTA.
