@@ -30,26 +30,32 @@ enum Route { STREAM, SPLIT, PAIR_TS, PAIR };
 //   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
 //                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
 //   up to 96         always split (CTA pairs: 40 tokens, 28672 x 4096: 23.0 / 19.8; 8192 x 28672: 59.5 / 31.6)
-//   97 to 128        while every channel tile has its CTAs at once (128 tokens, pairs against split, 57344 x 8192: 74.6 / 85.7,
-//                    28672 x 4096: 25.1 / 27.0; but 10240 x 8192: 25.3 / 23.5)
+//   97 to 128        while every channel tile has an SM at once (128 tokens, pairs against split, 57344 x 8192: 74.6 / 85.7,
+//                    28672 x 4096: 25.1 / 27.0; but 10240 x 8192: 25.3 / 23.5); 8-bit tokens, whose expansion is shorter, while every
+//                    channel tile has one of the two CTAs of an SM (28672 x 4096 22.8 / 23.0, 28672 x 8192 39.6 / 38.1, 20480 x 4096
+//                    21.8 / 21.0; but 38912 x 4096 30.6 / 36.2, 45056 x 8192 54 / 64, 57344 x 8192 66.0 / 68.8, 128256 x 8192 122 / 136)
 //   above            while the 256-token tiles leave room for two K splits (pairs against split at 256 tokens: 8192 x 8192 26.0 / 23.5,
 //                    4096 x 14336 35.7 / 24.2, 6144 x 4096 17.4 / 17.2; at 400, 4096 x 14336 37.8 / 31.9, 4096 x 4096 17.7 / 17.3). With a single
 //                    split the pairs win: 57344 x 8192 at 200 tokens 91 / 129, 28672 x 4096 30.1 / 39.3, 10240 x 8192 31.5 / 35.8, 6144 x 4096
 //                    at 300 17.9 / 21.7, 4096 x 14336 at 515 39.2 / 49.4.
-// CTA pairs. Few rounds of 8-bit tiles, and 4-bit tokens always: weights in tensor memory, tiles as wide as fit the chip
-// (pq_gemm_tc3.cu). More than three rounds of 8-bit tiles at K <= 8192: both operands in shared memory, two whole accumulators
-// (pq_gemm_tc2.cu, with the figures).
+// CTA pairs: weights in tensor memory, tiles as wide as fit the chip (pq_gemm_tc3.cu), or for 8-bit tokens both operands in shared
+// memory, whole tiles of 256 tokens and two whole accumulators (pq_gemm_tc2.cu). The second takes launches of more than three rounds, 2048 <= K <= 8192
+// and 1024 tokens and more, of which its whole tiles pad at most a twentieth: it is up to a tenth faster per padded token, and as much
+// slower where it pads more or where its longer start-up shows. With the rotation, us, first / second kernel: 28672 x 4096 at 300 tokens 39.5 / 57,
+// 515 52 / 67, 800 75 / 85, 1024 89 / 89, 1100 92 / 101, 1500 126 / 121, 1664 131 / 137, 2044 164 / 154, 2100 165 / 170, 3000 231 / 223,
+// 4096 315 / 296; 57344 x 8192 at 129 82 / 108, 515 180 / 224, 1024 305 / 308, 1100 330 / 368, 1280 380 / 372, 2044 619 / 564, 2100 601 / 621,
+// 4096 1204 / 1083; 28672 x 1024 at 4096 109 / 127, 28672 x 2048 181 / 166; 10240 x 8192 at 1500 98 / 101, 3000 173 / 170, 4096 229 / 222; 128256 x 4096 at 1024 357 / 340.
 inline Route gemm_route(int64_t m, int64_t N, int64_t K, bool a8, int sm_count) {
   const int64_t ctiles = (N + 127) / 128, weights = N * K;
   const bool split = m <= 8     ? false
                      : m <= 16  ? weights >= (int64_t{20} << 20)
                      : m <= 96  ? true
-                     : m <= 128 ? ctiles <= sm_count
+                     : m <= 128 ? ctiles <= (a8 ? 2 : 1) * sm_count
                                 : 2 * ((m + 255) / 256) * ctiles <= sm_count * 7 / 8;
   if (split) return SPLIT;
   if (m <= 16) return STREAM;
-  const int64_t tiles = ((m + 255) / 256) * ((N + 255) / 256);
-  return a8 && K <= 8192 && tiles > 3 * (sm_count / 2) ? PAIR : PAIR_TS;
+  const int64_t t_tiles = (m + 255) / 256, tiles = t_tiles * ((N + 255) / 256);
+  return a8 && K >= 2048 && K <= 8192 && m >= 1024 && 20 * m >= 19 * 256 * t_tiles && tiles > 3 * (sm_count / 2) ? PAIR : PAIR_TS;
 }
 
 // A position in a ring of n slots and the parity of its current round.

@@ -5,10 +5,8 @@
 // Two CTAs of a cluster share one 256 x 256 tile (cta_group::2): each CTA holds its own 128 token rows (A), whose s8 codes TMA copies
 // straight into the operand stage, and expands half of the 256 weight rows (B); the tensor cores of the pair exchange the B halves
 // themselves. Two 256-column accumulators, so a tile's epilogue runs wholly beside the next tile's MMAs. The kernel with the weights in
-// tensor memory (pq_gemm_tc3.cu) hides the latency of the copies better and wins on few rounds of tiles; with more than three, and K up
-// to 8192, this one does (with the rotation, us, that one / this one: 2044 x 28672 x 4096 171 / 157, 4096 x 6144 x 4096 93 / 87,
-// 2044 x 8192 x 8192 111 / 106, 4096 x 57344 x 8192 1240 / 1200; the other way round: 2044 x 4096 x 4096 33.6 / 35.4,
-// 2044 x 8192 x 28672 367 / 380).
+// tensor memory (pq_gemm_tc3.cu) hides the latency of the copies better, fits its tiles to the tokens and wins on few rounds of
+// tiles; on many rounds of full tiles this one does (gemm_route in pq_gemm_plan.cuh, with the figures).
 //
 // Roles inside each CTA (24 warps):
 //   warp 0        TMA producer: packed weight rows [128 x 64 B] of a 128-wide K block into a ring of landing buffers.

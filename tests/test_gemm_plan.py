@@ -158,6 +158,12 @@ def test_waits_return_for_the_phase_they_mean_under_any_interleaving():
     (8, 57344, 8192, False, "stream"), (16, 4096, 4096, False, "stream"), (9, 5120, 4096, False, "split"), (96, 57344, 8192, True, "split"),
     (128, 18944, 4096, False, "split"), (128, 18945, 4096, False, "pair_ts"), (256, 8192, 8192, False, "split"), (257, 8192, 8192, False, "pair_ts"),
     (4096, 57344, 8192, True, "pair"), (4096, 57344, 8192, False, "pair_ts"), (2044, 28672, 16384, True, "pair_ts"),
+    # 8-bit tokens: up to 128 the split kernel while its channel tiles are resident at once; the kernel of whole 256-token tiles only
+    # for many tokens that fill them
+    (128, 37888, 4096, True, "split"), (97, 37889, 4096, True, "pair_ts"), (97, 57344, 8192, True, "pair_ts"), (128, 128256, 4096, True, "pair_ts"),
+    (129, 57344, 8192, True, "pair_ts"), (515, 57344, 8192, True, "pair_ts"), (1023, 57344, 8192, True, "pair_ts"), (1024, 57344, 8192, True, "pair"), (1100, 57344, 8192, True, "pair_ts"),
+    (1215, 28672, 4096, True, "pair_ts"), (1216, 28672, 4096, True, "pair"), (2044, 28672, 4096, True, "pair"), (2044, 28672, 1920, True, "pair_ts"),
+    (2044, 4096, 4096, True, "pair_ts"),
 ])
 def test_route(M, N, K, a8, want):
     assert gp.route(M, N, K, a8) == want

@@ -4,6 +4,7 @@ per pair, ragged channels, both kinds of output store; and 8-bit tokens on more 
 operands in shared memory)."""
 import pytest
 
+import gemm_plan
 from test_gpu_split_gemm import check, ctx  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -22,6 +23,15 @@ def test_pair_gemm_matches_oracle(ctx, mode, M, N, K, ldo_pad):  # noqa: F811
 @pytest.mark.parametrize("M,N,K,row_begin", [(130, 57100, 32, 0), (300, 28700, 416, 4)])
 def test_many_tiles_of_8bit_tokens_match_oracle(ctx, M, N, K, row_begin):  # noqa: F811
     check(ctx, "w4a8", M, N, K, row_begin=row_begin)
+
+
+@pytest.mark.parametrize("M,N,K,ldo_pad,row_begin", [
+    (1216, 11304, 2048, 8, 0), (1280, 11521, 2080, 3, 0), (1250, 11400, 2176, 0, 5), (2033, 7424, 4128, 0, 0), (1500, 9600, 8192, 0, 0),
+])
+def test_8bit_tokens_on_whole_tiles_match_oracle(ctx, M, N, K, ldo_pad, row_begin):  # noqa: F811
+    """The kernel with both operands in shared memory: three rounds of tiles and more, token, channel and K tails, both kinds of store."""
+    assert gemm_plan.route(M - row_begin, N, K, True) == "pair"
+    check(ctx, "w4a8", M, N, K, ldo_pad, row_begin)
 
 
 @pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
