@@ -25,7 +25,7 @@ struct GemmParams {
   int64_t ldo;
   int M, N, K;
   int tiles_m, tiles_n;
-  int tma_store;  // out can be written with TMA stores (16-byte aligned base and row pitch)
+  int tma_store;  // out can be written with TMA stores (tma_store_fits)
   long long wait_clocks;  // bound of every device-side wait, in SM clocks
 };
 
@@ -226,6 +226,12 @@ inline bool make_s8_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, int6
              map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), gdim, gstride, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Can bulk-tensor stores write the output? Base and row pitch on 16-byte boundaries, and a width of whole 16-byte chunks: a box is cut
+// at the chunk that holds the last channel, so that up to seven columns past a ragged width were overwritten with zeros.
+inline bool tma_store_fits(const void* out, int64_t N, int64_t ldo) {
+  return N % 8 == 0 && ldo % 8 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
 }
 
 // Tensor map over the bf16 output [M, N] with row pitch ldo; box = [32 rows, cols columns], swizzled over its whole rows.

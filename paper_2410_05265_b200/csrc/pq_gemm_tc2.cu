@@ -373,7 +373,7 @@ pq_status pq_gemm_pair_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq,
   if (!make_s8_map(ctx, &ta, xq, M, K, BM_CTA) || !make_packed_map(ctx, &tb, wq, N, K / 2, BN_CTA))
     return PQ_ERR_CUDA;
   GemmParams p;
-  p.tma_store = (ldo % 8 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
+  p.tma_store = tma_store_fits(out, N, ldo);
   if (p.tma_store) {
     if (!make_out_map(ctx, &to, out, M, N, ldo)) return PQ_ERR_CUDA;
   } else {

@@ -80,7 +80,7 @@ struct PairParams : PairPlan {
   int32_t* status;
   int64_t ldo;
   int M, N, n_kb;
-  int tma_store;           // out can be written with TMA stores (16-byte aligned base and row pitch)
+  int tma_store;           // out can be written with TMA stores (tma_store_fits)
   long long wait_clocks;   // bound of every device-side wait, in SM clocks
 };
 
@@ -537,7 +537,7 @@ pq_status launch_pair(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, void* o
   if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, p.box) : make_packed_map(ctx, &tx, xq, p.M, K / 2, p.box)) ||
       !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH_CTA, CU_TENSOR_MAP_SWIZZLE_64B))
     return PQ_ERR_CUDA;
-  p.tma_store = (p.ldo % 8 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
+  p.tma_store = tma_store_fits(out, p.N, p.ldo);
   if (p.tma_store) {
     if (!make_out_map(ctx, &to, out, p.M, p.N, p.ldo, 32)) return PQ_ERR_CUDA;
   } else {

@@ -38,3 +38,17 @@ def test_8bit_tokens_on_whole_tiles_match_oracle(ctx, M, N, K, ldo_pad, row_begi
 @pytest.mark.parametrize("M", [129, 192, 193, 257, 384, 385])
 def test_split_gemm_at_the_edges_of_its_192_token_tiles(ctx, mode, M):  # noqa: F811
     check(ctx, mode, M, 300, 1312)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K,ldo_pad", [(129, 8444, 160, 4), (257, 8301, 96, 3), (150, 8266, 416, 14), (129, 19007, 64, 1)])
+def test_columns_past_a_ragged_width_stay_as_they_are(ctx, mode, M, N, K, ldo_pad):  # noqa: F811
+    """A width that is no multiple of eight inside rows whose pitch is one: bulk stores are cut at 16 bytes, not at the last channel."""
+    assert (N + ldo_pad) % 8 == 0 and N % 8 and gemm_plan.route(M, N, K, mode == "w4a8") == "pair_ts"
+    check(ctx, mode, M, N, K, ldo_pad)
+
+
+def test_columns_past_a_ragged_width_stay_as_they_are_on_whole_tiles(ctx):  # noqa: F811
+    M, N, K, ldo_pad = 1216, 11300, 2048, 4
+    assert gemm_plan.route(M, N, K, True) == "pair"
+    check(ctx, "w4a8", M, N, K, ldo_pad)
