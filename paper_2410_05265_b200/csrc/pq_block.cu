@@ -139,11 +139,11 @@ __device__ __forceinline__ void rope_rotate_head(float a0, float a1, float b0, f
   u = v1, v1 = u + v3, v3 = u - v3;
 #pragma unroll
   for (int m = 1; m < 32; m <<= 1) {  // index bits 1..5: the upper partner holds the difference
-    const bool up = lane & m;
+    const float sg = lane & m ? -1.0f : 1.0f;  // one multiply-add each: o - v or o + v, exact product
     const float o0 = __shfl_xor_sync(0xffffffffu, v0, m), o1 = __shfl_xor_sync(0xffffffffu, v1, m);
     const float o2 = __shfl_xor_sync(0xffffffffu, v2, m), o3 = __shfl_xor_sync(0xffffffffu, v3, m);
-    v0 = up ? o0 - v0 : v0 + o0, v1 = up ? o1 - v1 : v1 + o1;
-    v2 = up ? o2 - v2 : v2 + o2, v3 = up ? o3 - v3 : v3 + o3;
+    v0 = fmaf(v0, sg, o0), v1 = fmaf(v1, sg, o1);
+    v2 = fmaf(v2, sg, o2), v3 = fmaf(v3, sg, o3);
   }
   const float norm = 0.08838834764831845f;  // 1 / sqrt(128)
   pa = pack_bf16(v0 * norm, v1 * norm);
@@ -190,8 +190,9 @@ __global__ void __launch_bounds__(RP_THREADS)
 constexpr int RP_AHEAD = 6;
 __device__ __forceinline__ int kv_code(float x, float s) { return max(-8, min(7, __float2int_rn(__fdiv_rn(x, s)))); }
 
-__global__ void __launch_bounds__(RP_THREADS, 12)
-    rope_kv4_append_kernel(__nv_bfloat16* qkv, int64_t T, int Hq, int Hkv, int64_t ld, int64_t pos0, double log2_theta, int rotate,
+template <bool ROTATE, int CTAS>
+__global__ void __launch_bounds__(RP_THREADS, CTAS)
+    rope_kv4_append_kernel(__nv_bfloat16* qkv, int64_t T, int Hq, int Hkv, int64_t ld, int64_t pos0, double log2_theta,
                            uint8_t* __restrict__ kq, uint8_t* __restrict__ vq, const float* __restrict__ s_k,
                            const float* __restrict__ s_v, int32_t* len, int Tmax, int32_t* status, uint32_t* ticket) {
   __shared__ float cs[64], sn[64];
@@ -202,8 +203,10 @@ __global__ void __launch_bounds__(RP_THREADS, 12)
   const int n_heads = Hq + 2 * Hkv;
   // A warp's heads are requested RP_AHEAD at a time (with one after the other a token waited for memory once per head of a warp), and
   // from the second token on before the angles are computed; twelve CTAs to an SM (40 registers) keep 1500 tokens one wave. us, before ->
-  // now: 4096 tokens x 80 heads 49.7 -> 36.3 (with R3 58.5 -> 56.6), 1500 x 48 15.3 -> 13.1, 515 x 48 8.3 -> 7.6; five at a time, 56 registers:
-  // 40.4, 55.8, 15.8, 7.9.
+  // now: 4096 tokens x 80 heads 49.7 -> 36.3, 1500 x 48 15.3 -> 13.1, 515 x 48 8.3 -> 7.6; five at a time, 56 registers: 40.4, 15.8, 7.9.
+  // With R3 its instructions are the bound, and 40 registers cost some: as long as eight CTAs to an SM hold the tokens, 56 are taken. With R3
+  // and the clearing of the length, before -> 40 / 56 registers: 40 x 48 8.3 -> 7.3 / 6.8, 515 x 48 9.9 -> 9.3 / 8.8, 800 x 48 10.9 -> 11.4 / 10.9,
+  // 1500 x 48 17.0 -> 16.5 / 16.5, 4096 x 80 58.8 -> 52.4 / 51.8, 1500 x 12 8.0 -> 8.0 / 8.8.
   uint32_t wa[RP_AHEAD], wb[RP_AHEAD];
   auto request = [&](int64_t t, int first) {
 #pragma unroll
@@ -236,7 +239,7 @@ __global__ void __launch_bounds__(RP_THREADS, 12)
         uint32_t pa = wa[u], pb = wb[u];
         if (hd < Hq + Hkv) {  // q and k heads are rotated; v passes through
           const float a0 = bf16_lo(pa), a1 = bf16_hi(pa), b0 = bf16_lo(pb), b1 = bf16_hi(pb);
-          if (rotate) {
+          if (ROTATE) {
             rope_rotate_head(a0, a1, b0, b1, c0, s0, c1, s1, lane, pa, pb);
           } else {
             float l0, h0, l1, h1;
@@ -395,8 +398,9 @@ extern "C" pq_status pq_rope_kv4_append(pq_ctx* ctx, const pq_kv4_cache* c, int3
   if (!aligned16(qkv) || ld % 8 != 0 || !aligned16(c->kq) || !aligned16(c->vq)) return PQ_ERR_ALIGN;
   if (T == 0) return PQ_OK;
   const int64_t seq_off = static_cast<int64_t>(seq) * c->Hkv * c->Tmax * 64;
-  return pq_launch_pdl(rope_kv4_append_kernel, grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream),
-                       static_cast<__nv_bfloat16*>(qkv), T, c->Hq, c->Hkv, ld, pos0, log2(theta), rotate, c->kq + seq_off, c->vq + seq_off, c->s_k, c->s_v,
+  const auto kern = !rotate ? rope_kv4_append_kernel<false, 12> : T <= 8 * ctx->sm_count ? rope_kv4_append_kernel<true, 8> : rope_kv4_append_kernel<true, 12>;
+  return pq_launch_pdl(kern, grid_for(ctx, T, 1), RP_THREADS, 0, static_cast<cudaStream_t>(stream),
+                       static_cast<__nv_bfloat16*>(qkv), T, c->Hq, c->Hkv, ld, pos0, log2(theta), c->kq + seq_off, c->vq + seq_off, c->s_k, c->s_v,
                        c->len + seq, c->Tmax, ctx->d_status, ctx->d_tickets + 1);
 }
 

@@ -523,7 +523,8 @@ def test_rope_rotate_matches_oracle(ctx, T, H, pos0):
     assert float((s_plain - s_rot).abs().max()) <= 2.0**-6 * float(s_plain.abs().max())
 
 
-@pytest.mark.parametrize("T,Hq,Hkv,rotate,start", [(1, 4, 1, False, 0), (37, 8, 2, False, 5), (300, 8, 2, True, 11), (64, 64, 8, True, 0)])
+@pytest.mark.parametrize("T,Hq,Hkv,rotate,start", [(1, 4, 1, False, 0), (37, 8, 2, False, 5), (300, 8, 2, True, 11), (64, 64, 8, True, 0),
+                                                    (1184, 8, 1, True, 2), (1185, 8, 2, True, 0), (2400, 16, 2, True, 0), (2400, 16, 2, False, 0)])
 def test_rope_fused_with_kv4_append_equals_the_two_calls(ctx, T, Hq, Hkv, rotate, start):
     """pq_rope_kv4_append against pq_rope (or pq_rope_rotate) followed by pq_kv4_append_strided: the q|k|v buffer, the
     appended codes and the length bit for bit (each of those calls is checked against the oracle on its own)."""
