@@ -134,7 +134,7 @@ def test_prefill_attention_llama70b_4096_sampled_queries(ctx):
 
 
 def test_gemm_llama70b_prefill_4096_sampled_rows(ctx):
-    """The long-K kernel (token operand in tensor memory) at the configs[4] down-projection shape."""
+    """The pair kernel with weights in tensor memory at the configs[4] down-projection shape."""
     M, N, K = 4096, 8192, 28672
     g = torch.Generator(device="cuda").manual_seed(5)
     xq = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device="cuda", generator=g)

@@ -82,11 +82,12 @@ def test_cache_written_three_launches_back_is_seen_by_the_decode_step(ctx, T, ro
 
 
 @pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
-@pytest.mark.parametrize("M,N,K", [(1, 4096, 4096), (16, 5120, 4096), (24, 4096, 4096), (96, 4096, 4096), (200, 4096, 4096)])
+@pytest.mark.parametrize("M,N,K", [(1, 4096, 4096), (16, 5120, 4096), (24, 4096, 4096), (96, 4096, 4096), (200, 4096, 4096),
+                                   (140, 8448, 1024), (300, 4200, 1024)])
 def test_weights_written_just_before_reach_two_gemms_in_a_row(ctx, mode, M, N, K):
     """quantize weights (and sum their codes) -> rotate + quantize -> GEMM -> GEMM on other weights of the same quantizer call, back
-    to back: streaming and split-K kernels request weights ahead of the wait for their predecessor and let their successors start early
-    (up to 32 tokens). The buffers are overwritten in every pass: stale weights, sums or tokens would show."""
+    to back: the streaming, split-K and tensor-memory pair kernels request weights ahead of the wait for their predecessor, the first two let
+    their successors start early (up to 32 tokens). The buffers are overwritten in every pass: stale weights, sums or tokens would show."""
     x = [inputs.activations(M, K, seed=s).cuda() for s in range(3)]
     W = [inputs.weights(2 * N, K, seed=2 + s).cuda() for s in range(3)]
     wq = torch.zeros((2 * N, K // 2), dtype=torch.uint8, device="cuda")
@@ -132,13 +133,14 @@ def test_weights_written_just_before_reach_two_gemms_in_a_row(ctx, mode, M, N, K
         assert np.array_equal(np.concatenate([got[0], got[1]], 1), ref), f"pass {i}"
 
 
-@pytest.mark.parametrize("how", ["dynamic, two launches", "dynamic, one launch", "calibrated", "calibrated, 8 bits", "zero point"])
+@pytest.mark.parametrize("how", ["dynamic, two launches", "dynamic, one launch", "dynamic, a row per CTA", "calibrated", "calibrated, 8 bits", "zero point"])
 @pytest.mark.parametrize("M,N", [(1, 4096), (2, 4096), (3, 4096), (4, 1024), (8, 4096), (12, 1024), (16, 4096), (24, 1024), (96, 4096), (200, 1024), (140, 8264)])
 def test_steps_and_codes_written_just_before_are_the_ones_used(ctx, how, M, N):
     """step -> codes -> GEMM, every one reading what the launch before it wrote, replayed as one graph and called back to back, against
     the calls with a synchronisation between them: steps, codes, sums and outputs bit for bit, with other activations every time."""
-    K = 4096 if how == "dynamic, one launch" else 6144          # 6144 = three blocks of 2048: steps and codes are two launches
-    block = K if K == 4096 else 2048
+    K = 4096 if how == "dynamic, one launch" else 6144
+    # one block of 4096 or three of 2048: steps and codes from one launch; blocks of 1024: from two
+    block = K if K == 4096 else 1024 if how == "dynamic, two launches" else 2048
     bits8 = how == "calibrated, 8 bits"
     g = torch.Generator(device="cuda").manual_seed(M)
     wq = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
@@ -152,7 +154,7 @@ def test_steps_and_codes_written_just_before_are_the_ones_used(ctx, how, M, N):
     def chain(step):
         kw = dict(out=out, acc_dbg=acc)
         if how.startswith("dynamic"):
-            if step is not None and "two" in how:               # the same two launches, apart
+            if step is not None and how != "dynamic, one launch":  # two launches, apart
                 ctx.dyn_act_scale(x, block, out=s_tok)
                 step()
                 ctx.hadamard_quant_act_rows(x, block, s_tok, out=xq)

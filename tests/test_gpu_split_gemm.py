@@ -84,8 +84,7 @@ def test_large_layers_with_nine_to_sixteen_tokens(ctx, mode):
 @pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
 @pytest.mark.parametrize("M,N,K", [(129, 8200, 160), (300, 4104, 416), (130, 8328, 8224)])
 def test_pair_kernels_just_above_the_border(ctx, mode, M, N, K):
-    """Problems just too large for two K splits go to the CTA-pair kernels: ragged edges; K >= 8192 takes the kernel with the
-    token operand in tensor memory."""
+    """Problems just too large for two K splits go to the CTA-pair kernel: ragged edges, short and long K."""
     check(ctx, mode, M, N, K)
 
 
@@ -95,7 +94,7 @@ def test_pair_kernels_just_above_the_border(ctx, mode, M, N, K):
     (200, 8264, 416, 0, 4),        # dense rows, channels a multiple of 8: bulk-tensor stores; skipped rows
     (141, 8203, 512, 0, 5),        # channels not a multiple of 8: element-wise stores
     (150, 8264, 1152, 4, 0),       # rows too far apart for the bulk stores' 16-byte pitch
-    (137, 8203, 8224, 3, 1),       # the same with the token operand in tensor memory (K >= 8192; W4A8 keeps shared memory)
+    (137, 8203, 8224, 3, 1),       # the same with a long K
     (290, 10241, 8192, 0, 7),      # more tiles than CTA pairs, element-wise stores
     (260, 20000, 160, 0, 0),       # more tiles than CTA pairs, two K blocks
 ])

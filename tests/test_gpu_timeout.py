@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 import torch
 
+import gemm_plan
 from oracle import pq_oracle as orc
 from paper_2410_05265_b200 import inputs
 from helpers import assert_attn_close, rand_codes, to_np
@@ -45,15 +46,15 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     ctx = binding.Context()
     rng = np.random.default_rng(0)
     D = 128
-    # split-K GEMM with a few and with many K blocks per CTA; CTA-pair GEMMs (more than 128 rows and 64 channel tiles) with short K
-    # (token operand in shared memory), with long K (in tensor memory) and with 8-bit tokens (a producer of their own)
+    # split-K GEMM with a few and with many K blocks per CTA; CTA-pair GEMM with weights in tensor memory (more than 128 rows and 64
+    # channel tiles), short and long K and with 8-bit tokens (a producer of their own); the one with both operands in shared memory
     gemms = []
     for M, N, K, a8 in [(128, 256, 512, False), (128, 256, 32768, False), (96, 256, 32768, True), (129, 8448, 4096, False), (129, 8448, 8192, False),
-                        (129, 8448, 4096, True)]:
+                        (129, 8448, 4096, True), (1216, 11304, 2048, True)]:
         wq = rand_codes(rng, N, K)
         xq = rng.integers(-128, 128, (M, K)).astype(np.int8) if a8 else rand_codes(rng, M, K)
         gemms.append((ctx.w4a8_gemm if a8 else ctx.w4a4_gemm, dev(xq), dev(wq), orc.gemm_i8i4(xq, wq) if a8 else orc.gemm_i4(xq, wq)))
-    s_a, s_w_all = torch.full((1,), 0.02, device="cuda"), torch.full((8448,), 0.003, device="cuda")
+    s_a, s_w_all = torch.full((1,), 0.02, device="cuda"), torch.full((11304,), 0.003, device="cuda")
     # a small KV4 cache for the decode and the prefill attention
     B, Hq, Hkv, T, Tmax, P = 2, 8, 2, 300, 320, 4
     kq_np, vq_np = rng.integers(0, 256, (B, Hkv, Tmax, D // 2)).astype(np.uint8), rng.integers(0, 256, (B, Hkv, Tmax, D // 2)).astype(np.uint8)
@@ -78,7 +79,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     seen.append(ctx.check_status())
     torch.cuda.synchronize()                    # the process and the CUDA context are alive
     assert all(st in (0, PQ_ERR_TIMEOUT) for st in seen), seen
-    print("statuses under a 16-clock bound (six GEMMs, decode attention, prefill attention):", seen)
+    print("statuses under a 16-clock bound (seven GEMMs, decode attention, prefill attention):", seen)
 
     ctx.set_wait_limit(0)                       # the default bound again: exact results from the same context
     for gemm, xq, wq, acc_ref in gemms:
@@ -97,16 +98,19 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
 
 
 @pytest.mark.parametrize("mode", ["w4a4", "w4a8"])
-@pytest.mark.parametrize("M", [16, 40, 96, 128, 200])
+@pytest.mark.parametrize("M", [16, 40, 96, 128, 200, 130])
 def test_a_slow_predecessor_does_not_count_against_the_bounded_waits(mode, M):
-    """A GEMM placed early (split-K kernel, many K blocks per CTA) behind a kernel that runs several times longer than the wait
+    """A GEMM placed early (split-K kernel, many K blocks per CTA; CTA-pair kernel) behind a kernel that runs several times longer than the wait
     limit, though each of its own waits is short (causal attention, 128 key tiles in sequence): nothing is stuck, no timeout."""
     from paper_2410_05265_b200 import binding
 
     ctx = binding.Context()
     rng = np.random.default_rng(M)
-    N, K, T, D = 640, 16384, 16384, 128
+    N, K, T, D = 640, 4096 if M == 130 else 16384, 16384, 128
     wq = rand_codes(rng, N, K)
+    if M == 130:  # a layer wide enough for the CTA-pair kernel, which requests its first weights early, too
+        wq = np.tile(wq, (14, 1))[:8448]
+        assert gemm_plan.route(M, len(wq), K, mode == "w4a8") == "pair_ts"
     if M == 16:  # up to 16 tokens only large layers take that kernel
         wq = np.concatenate([wq, wq, wq])[:1408]
     if mode == "w4a8":
