@@ -17,8 +17,7 @@
 // tiles the issue and the expansion (450-500 clocks); on many rounds the chip's power limit. Found on the way (clock stamps of each
 // role, then variants; one round of 256-token tiles, K = 4096, weights from HBM, us):
 //   - the former kernels waited for their copies: four landing stages came back (latency, expansion, two barrier hops: 1750 clocks,
-//     2350 from HBM) later than four K blocks of MMAs take. Six to eight stages, their first weights ahead of griddepcontrol.wait:
-//     24.6 -> 19.5; K = 16384 55 -> 45;
+//     2350 from HBM) later than four K blocks of MMAs take. Six to eight stages: 24.6 -> 19.5; K = 16384 55 -> 45;
 //   - then the issuer: a wait that succeeds at once, four MMAs, a commit and the loop took 500 clocks whatever the width. Two K blocks
 //     per turn (one vote for both waits): 128-token tiles 19.3 -> 16.3; an issuer per half costs the same and needs no ordering of the
 //     halves. mbarrier.try_wait may suspend the warp although another K block could be issued: polls use test_wait;
@@ -28,8 +27,11 @@
 // GEMM alone, us, before -> now: 512 x 9472 x 4096 22.3 -> 17.7, 2048 x 9472 x 4096 55.1 -> 49.7, 512 x 9472 x 14336 49.9 -> 41.3.
 //
 // Roles inside each CTA (28 warps):
-//   warp 0        TMA producer: packed weight rows [128 x 64 B] and packed token rows per 128-wide K block into the landing stages.
-//                 Weights are static: the first stages' copies start before the wait for the previous kernel in the stream.
+//   warp 0        TMA producer: packed weight rows [128 x 64 B] and packed token rows per 128-wide K block into the landing stages,
+//                 all behind the wait for the previous kernel in the stream. First weights requested ahead of it would ask of every
+//                 writer of weights what the header asks for small calls only, and the tokens of the first K block would queue behind
+//                 them (us, ahead of the wait / behind it: 8B block at 515 tokens 173.2 / 169.5, 300 x 6144 x 4096 with the rotation 17.8 / 16.2,
+//                 515 x 8192 x 28672 125.3 / 120.9, 2044 x 28672 x 4096 153.3 / 152.5).
 //   warps 1, 3    (leader CTA only) MMA issuers of the two halves; warp 1 of each CTA owns its TMEM allocation.
 //   warp 2        A8: producer of the s8 token boxes, straight into operand slots (128-byte-swizzled).
 //   warps 4..7    epilogue of the first half, 24..27 of the second: one warp per TMEM lane quarter (32 channels), 32 tokens at a time:
@@ -186,41 +188,29 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     const bool leader = pq::elect_one();
-    auto begin_stage = [&](int s, const Tile& t, int kb) {  // the stage's bytes are announced, its weights requested
-      const int boxes = A8 ? 0 : (t.u1 > 0 ? 2 : 1);
-      pq::mbar_arrive_expect_tx(&bars->land_full[s], W_STAGE + boxes * p.box * PK_ROW);
-      pq::tma_load_2d(land_buf + s * p.stage, &tmap_w, kb * PK_ROW, t.n0 + rank * CH_CTA, &bars->land_full[s]);
-    };
-    const uint32_t early = total < static_cast<uint32_t>(p.n_land) ? total : p.n_land;
-    for (uint32_t i = 0; i < early; ++i) {  // the first weight copies do not depend on the previous kernel
-      const Tile t = tile_at(p, pair + static_cast<int>(i / p.n_kb) * n_pairs);
-      if (leader) begin_stage(i, t, i % p.n_kb);
-      __syncwarp();
-    }
-    loads_issued = early;
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the tokens may come from the previous kernel
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the operands may come from the previous kernel
     uint32_t it = 0;
     Pos ls;
     for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
       const Tile t = tile_at(p, tile);
       for (int kb = 0; kb < p.n_kb; ++kb, ++it, ls.advance(1, p.n_land)) {
-        if (it >= early) {
-          if (!wait_bar_warp(&bars->land_empty[ls.i], ls.ph ^ 1, abort_flag, p.wait_clocks)) {
-            ok = false;
-            break;
-          }
-          if (leader) begin_stage(ls.i, t, kb);
-          loads_issued = it + 1;
+        if (!wait_bar_warp(&bars->land_empty[ls.i], ls.ph ^ 1, abort_flag, p.wait_clocks)) {
+          ok = false;
+          break;
         }
-        if (!A8 && leader) {
-          uint8_t* dst = land_buf + ls.i * p.stage + W_STAGE;
-          pq::tma_load_2d(dst, &tmap_x, kb * PK_ROW, t.t0 + rank * t.u0 * (UNIT / 2), &bars->land_full[ls.i]);
-          if (t.u1 > 0)
-            pq::tma_load_2d(dst + p.box * PK_ROW, &tmap_x, kb * PK_ROW, t.t0 + t.u0 * UNIT + rank * t.u1 * (UNIT / 2), &bars->land_full[ls.i]);
+        if (leader) {
+          const int boxes = A8 ? 0 : (t.u1 > 0 ? 2 : 1);
+          uint8_t* dst = land_buf + ls.i * p.stage;
+          pq::mbar_arrive_expect_tx(&bars->land_full[ls.i], W_STAGE + boxes * p.box * PK_ROW);
+          pq::tma_load_2d(dst, &tmap_w, kb * PK_ROW, t.n0 + rank * CH_CTA, &bars->land_full[ls.i]);
+          if (boxes > 0) pq::tma_load_2d(dst + W_STAGE, &tmap_x, kb * PK_ROW, t.t0 + rank * t.u0 * (UNIT / 2), &bars->land_full[ls.i]);
+          if (boxes > 1)
+            pq::tma_load_2d(dst + W_STAGE + p.box * PK_ROW, &tmap_x, kb * PK_ROW, t.t0 + t.u0 * UNIT + rank * t.u1 * (UNIT / 2), &bars->land_full[ls.i]);
         }
         __syncwarp();
       }
     }
+    loads_issued = it;
   } else if (A8 && warp == 2) {
     // ------------------------------------------------------------------ token producer (A8)
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -506,7 +496,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   __syncthreads();
   if (bars->abort_flag) {
     // a role gave up: copies that nobody consumed must still have landed before the CTA may exit (they only wait for memory,
-    // hence the generous bound; a stage whose weights were requested got its tokens, too)
+    // hence the generous bound)
     if (warp == 0 && lane == 0)
       for (uint32_t j = loads_issued > static_cast<uint32_t>(p.n_land) ? loads_issued - p.n_land : 0; j < loads_issued; ++j)
         pq::mbar_wait(&bars->land_full[j % p.n_land], (j / p.n_land) & 1);
@@ -555,8 +545,8 @@ pq_status launch_pair(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, void* o
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  // the kernel may be launched while its predecessor drains; it waits for it on the device before it reads or writes anything
-  // but the (static) weights, which hides the launch itself
+  // the kernel may be launched while its predecessor drains; it waits for it on the device before it reads or writes anything,
+  // which hides the launch itself
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;

@@ -70,3 +70,10 @@ def test_what_a_predecessor_may_write_is_not_read_through_the_read_only_path(sou
     assert not wrong, wrong
     if name.startswith("hadamard"):  # its parameters are const __restrict__: no plain load through them either
         assert not re.search(r"\b(?:x|x2|s_a_in|zp_in)\[", body)
+
+
+@pytest.mark.parametrize("source,name", [("pq_gemm_tc2.cu", "gemm_w4a4_pair_kernel"), ("pq_gemm_tc3.cu", "gemm_w4a4_pair_ts_kernel")])
+def test_the_kernels_for_any_number_of_tokens_request_nothing_ahead_of_their_wait(source, name):
+    """The header asks of a writer of weights that it does not let its successors start early for calls of few rows only."""
+    body = kernel_body(source, name)
+    assert body.index("griddepcontrol.wait") < body.index("tma_load_2d")
