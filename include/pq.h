@@ -124,10 +124,11 @@ pq_status pq_rmsnorm_hadamard_quant_act(pq_ctx* ctx, const void* x, int64_t M, i
  *   K % 32 == 0, K <= 65536. Output rows below row_begin are left untouched.
  * Shapes with M - row_begin > 16 run on the tensor-core kernels (TMA + tcgen05, kind::i8);
  * smaller M mostly runs the weight-streaming kernel. No workspace is needed (ws may be NULL).
- * Weights are static (Sec. 3: quantized offline): below a few hundred rows the kernels start fetching wq
+ * Weights are static (Sec. 3: quantized offline): below a few hundred rows (of layers of few output channels also
+ * above, while ceil(rows / 256) * ceil(N / 128) is at most 7/16 of the SMs) the kernels start fetching wq
  * while the kernel before them in the stream is still draining (programmatic dependent launch), and
  * only xq, the activation scales and out are ordered behind that kernel. Whatever writes wq and s_w (and wsum
- * of the _asym call) in the same stream must therefore be a kernel that does not let its successors start
+ * of the _asym call) in the same stream for such a call must therefore be a kernel that does not let its successors start
  * before it has ended, however far back it is. Weights written by pq_quant_weights / pq_weight_code_sums, by a copy or
  * by a kernel launched in the ordinary way are safe. This holds for pq_w4a4_gemm, pq_w4a8_gemm,
  * pq_w4a4_gemm_rows and pq_w4a4_gemm_asym alike. */
@@ -172,8 +173,8 @@ pq_status pq_w4a8_gemm(pq_ctx* ctx, const int8_t* xq8, const uint8_t* wq, const 
 pq_status pq_dyn_act_scale(pq_ctx* ctx, const void* x, int64_t M, int64_t K, int64_t ldx, int had_block,
                            int64_t row_begin, float clip, float* s_tok, void* stream);
 /* The first and the second pass in one call (same passage): s_tok [M] and xq [M, K/2] are both outputs, with the bits
- * the two calls give. When a row is a single transform block of 2048 or more elements (had_block == K) the activations
- * are read once and the call is one launch; otherwise it runs the two passes. */
+ * the two calls give. When a row is a single transform block of 2048 or more elements (had_block == K), or 2 to 16 blocks
+ * of 2048, the activations are read once and the call is one launch; otherwise it runs the two passes. */
 pq_status pq_dyn_hadamard_quant_act(pq_ctx* ctx, const void* x, int64_t M, int64_t K, int64_t ldx, int had_block,
                                     int64_t row_begin, float clip, float* s_tok, uint8_t* xq, void* stream);
 pq_status pq_hadamard_quant_act_rows(pq_ctx* ctx, const void* x, int64_t M, int64_t K, int64_t ldx, int had_block,

@@ -6,7 +6,8 @@
 // straight into the operand stage, and expands half of the 256 weight rows (B); the tensor cores of the pair exchange the B halves
 // themselves. Two 256-column accumulators, so a tile's epilogue runs wholly beside the next tile's MMAs. The kernel with the weights in
 // tensor memory (pq_gemm_tc3.cu) hides the latency of the copies better, fits its tiles to the tokens and wins on few rounds of
-// tiles; on many rounds of full tiles this one does (gemm_route in pq_gemm_plan.cuh, with the figures).
+// tiles; on many rounds of full tiles this one does (gemm_route in pq_gemm_plan.cuh, with the figures). 8-bit tokens only, whatever the name
+// of the kernel function says.
 //
 // Roles inside each CTA (24 warps):
 //   warp 0        TMA producer: packed weight rows [128 x 64 B] of a 128-wide K block into a ring of landing buffers.
@@ -107,7 +108,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* s8_buf = smem;                                   // N_S8 stages: A rows then B rows, 1024-aligned
   uint8_t* pk_buf = s8_buf + N_S8 * S8_STAGE;               // N_PK stages: packed weight rows
-  uint8_t* epi_buf = pk_buf + N_PK * PK_STAGE;              // 4 warps x 2 buffers, 1024-aligned
+  uint8_t* epi_buf = pk_buf + N_PK * PK_STAGE;              // 4 warps x EPI_BUFS buffers, 1024-aligned
   float* scale_buf = reinterpret_cast<float*>(epi_buf + EPI_BYTES);
   Barriers* bars = reinterpret_cast<Barriers*>(reinterpret_cast<uint8_t*>(scale_buf) + SCALE_BYTES);
 
@@ -218,8 +219,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
     if (rank == 0) {
       // The four MMAs of a K block take 512 clocks of the tensor pipe; wait, issue and commit have to stay below that,
       // or this warp paces the kernel. With the loop in a branch of one lane they took 550-600; kept uniform (see
-      // elect_one) about 350: W4A4 2044 x 28672 x 4096: 165.7 -> 155.8 us, x 6144: 44.1 -> 41.6;
-      // W4A8: 158.4 -> 145.3 and 41.7 -> 36.3.
+      // elect_one) about 350: 2044 x 28672 x 4096 158.4 -> 145.3 us.
       constexpr uint32_t idesc = pq::umma_idesc_s8(2 * BM_CTA, BN);
       const bool leader = pq::elect_one();
       const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(s8_buf));
