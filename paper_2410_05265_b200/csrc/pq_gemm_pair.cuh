@@ -64,6 +64,20 @@ __device__ __forceinline__ bool mbar_try_wait_local(uint64_t* bar, uint32_t pari
       : "memory");
   return ok != 0;
 }
+// Has the phase completed? Unlike try_wait this never suspends the thread, which has other work meanwhile.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(pq::smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait (`limit` SM clocks); also gives up when the CTA's abort flag is raised.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
   if (mbar_try_wait_local(bar, parity)) return true;
@@ -200,14 +214,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor map over a dense packed matrix [rows, kbytes] of bytes; box = [box_rows, 64 bytes]. The kernel that reads
+// Tensor map over a dense packed matrix [rows, kbytes] of bytes; box = [box_rows, box_bytes]. The kernel that reads
 // the landing buffer one row per thread asks for the 64-byte swizzle (16-byte chunk index XOR (row >> 1) & 3) so that
 // those reads hit distinct banks; the other reads it chunk by chunk and takes it unswizzled.
 inline bool make_packed_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t kbytes, int box_rows,
-                            CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE) {
+                            CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE, int box_bytes = PK_ROW) {
   cuuint64_t gdim[2] = {static_cast<cuuint64_t>(kbytes), static_cast<cuuint64_t>(rows)};
   cuuint64_t gstride[1] = {static_cast<cuuint64_t>(kbytes)};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(PK_ROW), static_cast<cuuint32_t>(box_rows)};
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(box_bytes), static_cast<cuuint32_t>(box_rows)};
   cuuint32_t estr[2] = {1, 1};
   return reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
              map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), gdim, gstride, box, estr,

@@ -24,9 +24,9 @@ enum Route { STREAM, SPLIT, PAIR_TS, PAIR };
 // The kernel for m rows.
 // Weight-streaming kernel or split-K tensor-core kernel (figures: rotate+quantize and GEMM in a graph, us, streaming against
 // split). The streaming kernel has the shorter chain, but expands the tokens again for every 16 channels and has no K split:
-//   up to 8 tokens   always streaming. Alone behind its rotation kernel the other is faster on 8192 x 28672 (1 token: 29.2 / 24.4)
-//                    and 8192 x 8192 (11.4 / 10.4), but inside a decode layer the streaming kernel's shorter chain and earlier
-//                    weight requests win: whole 70B layer 124 / 132 us
+//   up to 8 tokens   streaming; the other one for a long K, where a CTA of the streaming kernel walks rows alone (8192 x 28672, 1 token: 29 / 24;
+//                    whole 70B decode layer 117.8 / 114.1). On 8192 x 8192 it is faster alone (11.4 / 10.4), but inside a decode layer the streaming
+//                    kernel's shorter chain and earlier weight requests win (124 / 132 with every layer on the other)
 //   9 to 16 tokens   only layers below 20 M weights (16 tokens, 4096 x 4096: 5.6 / 7.1; 6144 x 4096: 8.1 / 7.8,
 //                    28672 x 4096: 21.3 / 15.7, 8192 x 28672: 33.9 / 26.0)
 //   up to 96         always split (CTA pairs: 40 tokens, 28672 x 4096: 23.0 / 19.8; 8192 x 28672: 59.5 / 31.6)
@@ -47,7 +47,7 @@ enum Route { STREAM, SPLIT, PAIR_TS, PAIR };
 // 4096 1204 / 1083; 28672 x 1024 at 4096 109 / 127, 28672 x 2048 181 / 166; 10240 x 8192 at 1500 98 / 101, 3000 173 / 170, 4096 229 / 222; 128256 x 4096 at 1024 357 / 340.
 inline Route gemm_route(int64_t m, int64_t N, int64_t K, bool a8, int sm_count) {
   const int64_t ctiles = (N + 127) / 128, weights = N * K;
-  const bool split = m <= 8     ? false
+  const bool split = m <= 8     ? K > 16384
                      : m <= 16  ? weights >= (int64_t{20} << 20)
                      : m <= 96  ? true
                      : m <= 128 ? ctiles <= (a8 ? 2 : 1) * sm_count
@@ -173,29 +173,40 @@ inline bool pair_plan(PairPlan& p, int M, int N, int n_kb, bool a8, int sm_count
 constexpr int CH = 128;                    // output channels per CTA
 constexpr int SPLIT_BAR_BYTES = 512;       // no less than the kernel's barriers take
 
-// Shapes of the rings. Up to 128 tokens two CTAs share an SM (113 KB and 256 TMEM columns each), so that one loads
-// while the other expands or reduces; 256 tokens take a whole SM. Four operand slots where they fit: with two, a slot came back later
-// (commit, expansion, fence, arrival) than the other's MMAs took. us, rotation and GEMM in a graph, two slots -> four: 33 x 28672 x 4096
-// 19.9 -> 19.5, 64 x 28672 x 4096 21.2 -> 20.3 (for two of its eight weight stages), 64 x 4096 x 14336 16.2 -> 15.7; linear set of the 70B layer at
-// 64 tokens, W4A8, 150.4 -> 128.4, 8B layer at 64 65.2 -> 63.1.
+// Shapes of the rings. Up to 128 tokens two CTAs share an SM (112 KB and 256 TMEM columns each), so that one loads
+// while the other expands or reduces; 256 tokens take a whole SM. K blocks of 256 elements, whose weight rows are 128 bytes (why: pq_gemm_split.cu),
+// where the rings hold enough of them: two operand slots, one per expansion group, and as many landing stages as fit beside them. us, rotation and
+// GEMM in a graph: 64 x 57344 x 8192 62.9 (128 elements) / 62.5 (256, four weight stages and two of tokens) / 59.5 (three and three);
+// 8-bit tokens, 128 x 28672 x 4096 22.6 / 23.0 (two stages) / 20.2 (three). At 96 and 128 packed tokens the landing stages of the tokens leave no room.
+constexpr int split_kb(int nt, bool a8) { return nt <= (a8 ? 128 : 64) ? 256 : 128; }
+
 template <int NT, bool A8>
 struct SplitCfg {
+  static constexpr int KB = split_kb(NT, A8), SUBS = KB / BK;  // elements of a K block
+  static constexpr int ROWB = KB / 2;                          // packed bytes of a row in it
   static constexpr int GROUPS = NT > 128 ? 4 : 2;
-  static constexpr int SLOTS = NT == 128 && !A8 ? 2 : 4;
-  static constexpr int STAGES = NT <= 48 ? 8 : (NT == 64 ? 6 : 4);  // landing ring, weights
-  static constexpr int X_STAGES = NT <= 32 ? 8 : 4;  // landing ring, tokens
+  static constexpr int SLOTS = KB == 256 || (NT == 128 && !A8) ? 2 : 4;
+  static constexpr int W_STAGE = CH * ROWB;
+  static constexpr int STAGES = KB == 128 ? 4 : (NT <= (A8 ? 32 : 16) ? 6 : (NT <= (A8 ? 96 : 48) ? 4 : 3));  // landing ring, weights
+  static constexpr int X_STAGES = KB == 256 && NT > 48 ? 3 : 4;                                               // landing ring, tokens
+  static constexpr bool TOGETHER = KB == 256;  // weights and tokens of a K block are waited for together
+  static constexpr bool SLOT_FIRST = STAGES % GROUPS != 0 || (!A8 && X_STAGES % GROUPS != 0);
   static constexpr bool EARLY_W = NT > 128;          // weight stages go back before the (long) token part of the expansion
-  static constexpr int X_STAGE = A8 ? 0 : NT * PK_ROW;
-  static constexpr int SLOT = NT * BK;
+  static constexpr int X_STAGE = A8 ? 0 : NT * ROWB;
+  static constexpr int SUB_SLOT = NT * BK;           // token operand of 128 elements
+  static constexpr int SLOT = SUBS * SUB_SLOT;
+  static constexpr int A_COLS = SUBS * A_SLOT_COLS;
   static constexpr int A_COL0 = NT < 32 ? 32 : NT;  // accumulator columns, then the A slots
   static constexpr int TMEM_COLS = NT > 128 ? 512 : 256;
   static constexpr int CTAS_PER_SM = NT > 128 ? 1 : 2;
-  static constexpr int RING = SLOTS * SLOT + STAGES * (CH * PK_ROW) + X_STAGES * X_STAGE;
+  static constexpr int RING = SLOTS * SLOT + STAGES * W_STAGE + X_STAGES * X_STAGE;
   static constexpr int PART = NT * CH * 4;  // the int32 partial tile, laid over the rings at the end
-  static_assert(A_COL0 + SLOTS * A_SLOT_COLS <= TMEM_COLS, "tensor memory budget");
-  static_assert(STAGES % GROUPS == 0 && X_STAGES % GROUPS == 0 && SLOTS % GROUPS == 0, "a ring slot is always served by the same group");
+  static_assert(A_COL0 + SLOTS * A_COLS <= TMEM_COLS, "tensor memory budget");
+  static_assert(SLOTS % GROUPS == 0, "an operand slot is always served by the same group");
+  static_assert(SLOTS <= X_STAGES, "what frees an operand slot has landed in both rings");
   static_assert(PART <= RING, "the partial tile fits where the rings were");
   static_assert(SLOTS <= STAGES, "no weight stage is refilled before the first operand slot is");
+  static_assert((RING + SPLIT_BAR_BYTES + 1024) * CTAS_PER_SM <= 228 * 1024, "shared memory budget");
 };
 
 // At least 80 KB for 256 columns of tensor memory and 160 KB for 512, so that no more CTAs share an SM (228 KB) than its tensor memory
@@ -203,7 +214,7 @@ struct SplitCfg {
 // cluster barrier could wait for itself. (8-bit tokens 192 wide need 130 KB, which leave room for a CTA of a narrow form.)
 template <int NT, bool A8>
 constexpr size_t split_smem() {
-  const size_t need = 1024 /*alignment slack*/ + SplitCfg<NT, A8>::RING + SPLIT_BAR_BYTES, least = SplitCfg<NT, A8>::TMEM_COLS / 256 * (80 * 1024);
+  const size_t need = SplitCfg<NT, A8>::RING + SPLIT_BAR_BYTES, least = SplitCfg<NT, A8>::TMEM_COLS / 256 * (80 * 1024);
   return need < least ? least : need;
 }
 

@@ -9,30 +9,37 @@
 // memory: exact, no workspace, nothing waits on another cluster.
 //
 // Roles inside a CTA:
-//   warp 0      TMA producer, packed weights: [128 x 64 B] (64-byte swizzle) of a 128-wide K block into a landing ring.
+//   warp 0      TMA producer, packed weights: a K block of 256 elements [128 x 128 B] (128 at the widest token tiles) into a landing ring.
 //               Weights are static: the ring's first copies start before the wait for the previous kernel in the stream.
 //   warp 1      MMA issuer and owner of the tensor memory.
-//   warp 2      TMA producer, tokens: packed rows [NT x 64 B] into a landing ring of their own, or (A8) the s8 bytes
+//   warp 2      TMA producer, tokens: packed rows [NT x 64 B per 128 elements] into a landing ring of their own, or (A8) the s8 bytes
 //               straight into the operand slot (128-byte-swizzled box).
 //   warps 4..   expansion, GROUPS groups of four warps (one per TMEM lane quarter): a thread owns one channel row, reads
-//               its 64 packed bytes, and writes 128 s8 bytes (16 * code) to its lane of an A slot in tensor memory; the
-//               group's threads also expand the token rows into the B slot in shared memory. Even-position codes come
-//               first, then odd-position codes, in both operands (natural order in both with A8).
+//               its packed bytes, and writes the s8 bytes (16 * code) to its lane of an A slot in tensor memory; the
+//               group's threads also expand the token rows into the B slot in shared memory. Of every 32 codes the even-position ones come
+//               first, then the odd-position ones, in both operands (natural order in both with A8).
 // Then every warp takes part in the reduction: a lane owns four channels, a warp one or more tokens at a time, the partial
 // sums of the cluster's CTAs are added, scaled and stored as 256 contiguous bytes per token.
 //
 // What bounds it: up to ~64 tokens the weight stream and the fixed chain launch -> tokens -> expand -> MMA -> two cluster
 // barriers (about 5 us, most of it overlapped with the neighbours under programmatic dependent launch); at 128 and 256 tokens
-// the expansion of the token rows, which every channel tile repeats. Measured (us, calls in a graph over weight copies larger
-// than L2; before: the CTA-pair kernels, for 16 tokens the streaming kernel), layers of the 8B set q|k|v, o, gate|up, down:
-//   M = 16   6.1  3.7 18.2  8.9  ->  6.5  5.6 14.0  9.1 (gate|up at 4.2 TB/s)
-//   M = 32  20.7 20.3 36.0 46.7  ->  7.0  6.1 14.4  9.6
-//   M = 96  20.9 20.5 37.2 46.9  ->  10.1  9.2 20.3 14.6   (W4A8: 18.6 18.4 31.9 46.6 -> 9.5 8.7 17.8 13.5)
-//   M = 256 21.1 20.7   --  47.1  ->  13.2 12.5   --  19.7
-// (In a chain with the rotation kernels the short layers overlap less; the dispatch in pq_gemm.cu was set on such chains.)
+// the expansion of the token rows, which every channel tile repeats.
+//
+// Why a K block has 256 elements: copies of 64 bytes a row do not reach the memory's rate. Copies alone, without any arithmetic (TB/s, the
+// same CTAs and bytes in flight): 57344 x 4096 bytes 64-byte rows 4.9, 128-byte rows 5.8-6.3; 28672 x 2048 bytes 4.0 / 4.7. A K block also has a fixed
+// price, three waits, three arrivals and a proxy fence, about half of its 1200 clocks, and an mbarrier arrival is the dearest of
+// them (it waits for the thread's stores): those that come together are one instruction with a lane each. us, GEMM alone over
+// weight copies larger than L2, 64-byte rows / now:
+//   4-bit, 33 tokens: 6144 x 4096 8.9 / 8.0, 4096 x 4096 8.4 / 7.5, 28672 x 4096 19.0 / 16.9, 4096 x 14336 13.0 / 11.7, 57344 x 8192 58.9 / 51.2
+//   4-bit, 16 tokens: 28672 x 4096 14.8 / 14.2, 57344 x 8192 50.8 / 46.3, 8192 x 28672 24.0 / 22.7, 10240 x 8192 11.5 / 10.4
+//   8-bit, 96 tokens: 6144 x 4096 11.1 / 10.1, 4096 x 4096 10.6 / 9.5, 28672 x 4096 20.2 / 17.5, 4096 x 14336 15.8 / 14.5, 57344 x 8192 63.1 / 58.5
+//   8-bit, 128 tokens: 28672 x 4096 21.0 / 19.0, 8192 x 28672 34.1 / 32.2
 // Tried: the token rows read from L2 into registers instead of a landing ring (gate|up, M = 32: 16.2 us against 14.3); token
 // rows expanded by warps of their own (18.1); three or four expansion groups per CTA (14.9-15.2); a weight stage handed back
-// right after it was read into registers, which pays only where the token part is long (M = 256, gate|up: 46.5 -> 36.4).
+// right after it was read into registers, which pays only where the token part is long (M = 256, gate|up: 46.5 -> 36.4); with 64-byte rows,
+// one vote for the three waits (33 x 28672 x 4096 19.1 -> 21.0: the weights are no longer expanded while the tokens are on their way); tokens
+// before weights, or their stage handed back at once (64 x 28672 x 4096 19.2 -> 21.9); the K blocks of several tiles dealt evenly over a cluster
+// (five CTAs for four tiles of 28672 x 4096, so that all SMs have the same share: 17.0 -> 20.9; the memory, not the fullest SM, sets the time).
 //
 // Every mbarrier wait is bounded; when one runs out the CTA raises an abort flag, its roles drain, and PQ_ERR_TIMEOUT
 // is reported.
@@ -72,7 +79,7 @@ struct SplitParams {
   int32_t* acc_dbg;
   int32_t* status;
   int64_t ldo;
-  int M, N, n_kb;
+  int M, N, K, n_kb;
   int t_tiles, splits;
   int vec_out;  // rows of out take 8-byte stores
   long long wait_clocks;
@@ -108,17 +115,8 @@ __device__ __forceinline__ int4 ld_cluster_int4(uint32_t addr) {
 // ..., U of them at a time so that their shared-memory loads are in flight together; a lane owns four channels.
 template <int PEERS, int U, bool ZP>
 __device__ __forceinline__ void reduce_tile(const SplitParams& p, const uint8_t* part, int t0, int n0, int tokens, int first, int step,
-                                            int lane) {
+                                            int lane, const float (&sw)[4], const int (&zw)[4]) {
   const int n = n0 + 4 * lane;
-  float sw[4];
-  int zw[4];
-  const float s_a = p.s_row ? 1.0f : pq::ld_dep(p.s_a);
-  const int zp8 = ZP ? pq::ld_dep(p.zp) - 8 : 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    sw[i] = n + i < p.N ? s_a * __ldg(p.s_w + n + i) : 0.0f;
-    zw[i] = ZP && n + i < p.N ? zp8 * __ldg(p.wsum + n + i) : 0;
-  }
   uint32_t peer[PEERS];
 #pragma unroll
   for (int r = 0; r < PEERS; ++r) peer[r] = map_to_cta(part, r < p.splits ? r : 0) + lane * 16;
@@ -170,13 +168,17 @@ template <int NT, bool A8, bool ZP>
 __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM)
     gemm_w4_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const SplitParams p) {
   using C = Cfg<NT, A8>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw;
   uint8_t* slot_buf = smem;                                // SLOTS token operands [NT x 128 B], 128-byte swizzle
   uint8_t* stage_buf = slot_buf + C::SLOTS * C::SLOT;      // STAGES landing buffers of packed weights
-  uint8_t* x_buf = stage_buf + C::STAGES * W_STAGE;        // X_STAGES landing buffers of packed tokens
+  uint8_t* x_buf = stage_buf + C::STAGES * C::W_STAGE;     // X_STAGES landing buffers of packed tokens
   SplitBarriers* bars = reinterpret_cast<SplitBarriers*>(smem + C::RING);
   volatile int* abort_flag = &bars->abort_flag;
+  if (pq::smem_u32(smem_raw) & 1023) {  // the swizzled buffers need it (no slack is kept: two CTAs share the SM to the last kilobyte)
+    if (threadIdx.x == 0) pq::report(p.status, PQ_ERR_ALIGN);
+    return;
+  }
   const int warp = pq::warp_index(), lane = threadIdx.x & 31;
   const int rank = __shfl_sync(0xffffffffu, static_cast<int>(cluster_ctarank()), 0);
   const int tile = static_cast<int>(blockIdx.x) / p.splits;
@@ -213,8 +215,8 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
     __syncwarp();
     for (int i = 0; i < first; ++i) {  // the first weight copies do not depend on the previous kernel
       if (leader) {
-        pq::mbar_arrive_expect_tx(&bars->w_full[i], W_STAGE);
-        pq::tma_load_2d(stage_buf + i * W_STAGE, &tmap_w, (kb0 + i) * PK_ROW, n0, &bars->w_full[i]);
+        pq::mbar_arrive_expect_tx(&bars->w_full[i], C::W_STAGE);
+        pq::tma_load_2d(stage_buf + i * C::W_STAGE, &tmap_w, (kb0 + i) * C::ROWB, n0, &bars->w_full[i]);
       }
       __syncwarp();
     }
@@ -230,10 +232,27 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   int loads_issued = 0;  // producer warps: copies started
   bool ok = true;
+  // The steps and code sums of this lane's channels in the reduction are static, like the weights: they are requested here, not behind
+  // the cluster barrier, where their trip to memory would stand in the chain.
+  float sw[4];
+  int zw[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int n = n0 + 4 * lane + i;
+    sw[i] = n < p.N ? __ldg(p.s_w + n) : 0.0f;
+    zw[i] = ZP && n < p.N ? __ldg(p.wsum + n) : 0;
+  }
+  float s_a = 1.0f;  // behind the wait for the previous kernel: the token step and the zero point
+  int zp8 = 0;
+  auto load_steps = [&]() {
+    if (!p.s_row) s_a = pq::ld_dep(p.s_a);
+    if (ZP) zp8 = pq::ld_dep(p.zp) - 8;
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     asm volatile("griddepcontrol.wait;" ::: "memory");  // room comes back once the tokens are there: the bounded waits start behind them
+    load_steps();
     int it = first;
     for (; it < total; ++it) {
       const int s = it % C::STAGES;
@@ -242,8 +261,8 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
         break;
       }
       if (leader) {
-        pq::mbar_arrive_expect_tx(&bars->w_full[s], W_STAGE);
-        pq::tma_load_2d(stage_buf + s * W_STAGE, &tmap_w, (kb0 + it) * PK_ROW, n0, &bars->w_full[s]);
+        pq::mbar_arrive_expect_tx(&bars->w_full[s], C::W_STAGE);
+        pq::tma_load_2d(stage_buf + s * C::W_STAGE, &tmap_w, (kb0 + it) * C::ROWB, n0, &bars->w_full[s]);
       }
       __syncwarp();
     }
@@ -251,24 +270,46 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     asm volatile("griddepcontrol.wait;" ::: "memory");  // what it waits for needs the tokens
+    load_steps();
     constexpr uint32_t idesc = pq::umma_idesc_s8(CH, NT);
     const uint64_t desc0 = pq::umma_desc_sw128(pq::smem_u32(slot_buf));
-    for (int it = 0; it < total; ++it) {
-      const int s = it % C::SLOTS, ph = (it / C::SLOTS) & 1;
-      if (!wait_bar_warp(&bars->s8_full[s], ph, abort_flag, p.wait_clocks) ||
-          (A8 && !wait_bar_warp(&bars->x_full[s], ph, abort_flag, p.wait_clocks))) {
-        ok = false;
-        break;
-      }
+    auto there = [&](int i) {
+      const int s = i % C::SLOTS, ph = (i / C::SLOTS) & 1;
+      return mbar_test(&bars->s8_full[s], ph) && (!A8 || mbar_test(&bars->x_full[s], ph));
+    };
+    auto wait_for = [&](int i) {
+      const int s = i % C::SLOTS, ph = (i / C::SLOTS) & 1;
+      return wait_bar_warp(&bars->s8_full[s], ph, abort_flag, p.wait_clocks) &&
+             (!A8 || wait_bar_warp(&bars->x_full[s], ph, abort_flag, p.wait_clocks));
+    };
+    auto issue = [&](int i) {
       pq::tc_fence_after();
       if (leader) {
+        const int s = i % C::SLOTS;
         const uint64_t b_desc = desc0 + s * (C::SLOT >> 4);
-        const uint32_t a_tmem = tmem_base + C::A_COL0 + s * A_SLOT_COLS;
+        const uint32_t a_tmem = tmem_base + C::A_COL0 + s * C::A_COLS;
 #pragma unroll
-        for (int kk = 0; kk < BK / 32; ++kk) mma_i8_ts(tmem_base, a_tmem + kk * 8, b_desc + kk * 2, idesc, (it | kk) != 0 ? 1u : 0u);
+        for (int kk = 0; kk < C::KB / 32; ++kk)
+          mma_i8_ts(tmem_base, a_tmem + kk * 8, b_desc + (kk >> 2) * (C::SUB_SLOT >> 4) + (kk & 3) * 2, idesc, (i | kk) != 0 ? 1u : 0u);
         pq::mma_commit(&bars->s8_empty[s]);
       }
       __syncwarp();
+    };
+    for (int it = 0; it < total; it += 2) {  // two K blocks per turn: one vote and one branch for both waits
+      const bool second = it + 1 < total;
+      const bool r0 = there(it), r1 = second && there(it + 1);
+      const bool both = __all_sync(0xffffffffu, r0 && r1);
+      if (!both && !wait_for(it)) {
+        ok = false;
+        break;
+      }
+      issue(it);
+      if (!second) break;
+      if (!both && !wait_for(it + 1)) {
+        ok = false;
+        break;
+      }
+      issue(it + 1);
     }
     if (leader) pq::mma_commit(&bars->acc_full);
     __syncwarp();
@@ -280,6 +321,7 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
     uint64_t* empty = A8 ? bars->s8_empty : bars->xp_empty;
     uint8_t* buf = A8 ? slot_buf : x_buf;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the tokens may come from the previous kernel
+    load_steps();
     int it = 0;
     for (; it < total; ++it) {
       const int s = it % RING;
@@ -289,7 +331,9 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
       }
       if (leader) {
         pq::mbar_arrive_expect_tx(&full[s], BYTES);
-        pq::tma_load_2d(buf + s * BYTES, &tmap_x, (kb0 + it) * (A8 ? BK : PK_ROW), t0, &full[s]);
+#pragma unroll
+        for (int h = 0; h < C::SUBS; ++h)  // 128 elements of every token row per box
+          pq::tma_load_2d(buf + s * BYTES + h * (BYTES / C::SUBS), &tmap_x, (kb0 + it) * (A8 ? C::KB : C::ROWB) + h * (A8 ? BK : PK_ROW), t0, &full[s]);
       }
       __syncwarp();
     }
@@ -298,23 +342,14 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
     // ------------------------------------------------------------------ expansion
     const int group = (warp - EXPAND_WARP0) >> 2, q = warp & 3;
     const int gt = q * 32 + lane;  // thread of the group = channel row of the tile = lane of tensor memory
-    for (int it = group; it < total; it += C::GROUPS) {
-      const int ps = it % C::STAGES, xs = it % C::X_STAGES, ss = it % C::SLOTS;
-      // A refilled stage or slot (SLOTS <= STAGES) comes back behind the previous kernel only: the bounded waits start there.
-      if (it >= C::SLOTS && it < C::SLOTS + C::GROUPS) asm volatile("griddepcontrol.wait;" ::: "memory");
-      if (!wait_bar_warp(&bars->w_full[ps], (it / C::STAGES) & 1, abort_flag, p.wait_clocks)) {
-        ok = false;
-        break;
-      }
-      const uint8_t* src = stage_buf + ps * W_STAGE;
-      uint4 w[4];
+    uint4 w[4];
+    auto load_w = [&](int ps, int h) {  // 128 elements of this thread's row; swizzled landing buffer: the row-per-thread reads hit distinct banks
+      const uint8_t* src = stage_buf + ps * C::W_STAGE + gt * C::ROWB;
+      const int sw = C::ROWB == 64 ? (gt >> 1) & 3 : gt & 7;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)  // 64-byte swizzle of the landing buffer: the row-per-thread reads hit distinct banks
-        w[j] = *reinterpret_cast<const uint4*>(src + gt * PK_ROW + ((j ^ ((gt >> 1) & 3)) << 4));
-      if (!wait_bar_warp(&bars->s8_empty[ss], ((it / C::SLOTS) & 1) ^ 1, abort_flag, p.wait_clocks)) {
-        ok = false;
-        break;
-      }
+      for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint4*>(src + (((4 * h + j) ^ sw) << 4));
+    };
+    auto put_w = [&](int ss, int h) {
       uint32_t a[32];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -329,45 +364,116 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
           }
         }
       }
-      pq::tmem_st_32x32(tmem_base + C::A_COL0 + ss * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), a);
+      pq::tmem_st_32x32(tmem_base + C::A_COL0 + ss * C::A_COLS + h * A_SLOT_COLS + (static_cast<uint32_t>(q * 32) << 16), a);
+    };
+    auto rest_w = [&](int ps, int ss) {  // what follows the first 128 elements
+#pragma unroll
+      for (int h = 1; h < C::SUBS; ++h) load_w(ps, h), put_w(ss, h);
       if (C::EARLY_W) {  // behind the store above, for which what was read has arrived in registers
         __syncwarp();
         if (lane == 0) pq::mbar_arrive(&bars->w_empty[ps]);
       }
-      if (!A8) {
-        if (it == group) asm volatile("griddepcontrol.wait;" ::: "memory");  // the tokens' bounded wait starts behind their producer
-        if (!wait_bar_warp(&bars->xp_full[xs], (it / C::X_STAGES) & 1, abort_flag, p.wait_clocks)) {
+    };
+    // The weights of the first operand slots, ahead of the tokens (and of the wait for the kernel that writes those).
+    for (int it = group; it < C::SLOTS && it < total; it += C::GROUPS) {
+      if (!wait_bar_warp(&bars->w_full[it], 0, abort_flag, p.wait_clocks)) {
+        ok = false;
+        break;
+      }
+      load_w(it, 0);
+      put_w(it, 0);
+      rest_w(it, it);
+    }
+    // Tokens, and refilled stages and slots (SLOTS <= STAGES), come behind the previous kernel only: the bounded waits start there.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    load_steps();
+    // Of a K block's three waits and three arrivals, those that come together are one instruction, a lane each: lane 0 has the landing ring
+    // of the weights, lane 1 that of the tokens, lane 2 the operand slots.
+    const int role = lane == 1 && !A8 ? 1 : (lane == 2 ? 2 : 0);
+    uint64_t* const r_full = role == 1 ? bars->xp_full : bars->w_full;
+    uint64_t* const r_arrive = role == 1 ? bars->xp_empty : (role == 2 ? bars->s8_full : bars->w_empty);
+    const int r_len = role == 1 ? C::X_STAGES : (role == 2 ? C::SLOTS : C::STAGES);
+    const bool arrives = lane == 2 || (lane == 0 && !C::EARLY_W) || (lane == 1 && !A8);
+    int r_pos = group, r_ph = 0, w_ph = 0;  // group < every ring's length
+    int ps = group, xs = group, x_ph = 0, ss = group, s_ph = 1;
+    for (int it = group; ok && it < total; it += C::GROUPS) {
+      const bool first_slots = it < C::SLOTS;  // the weights are expanded already
+      {
+        const int pos = role == 1 ? r_pos : ps, ph = role == 1 ? r_ph : w_ph;
+        const bool skip = role == 1 ? !C::TOGETHER : first_slots;
+        // A landing ring that is no multiple of the groups is served by all of them in turn, and a group has not seen every round of a stage. The
+        // operand slot is asked for first there: once it is free, K block it - SLOTS and all before it have landed, so that the parity
+        // below cannot be that of two rounds back (SLOTS <= STAGES, X_STAGES).
+        const bool r0 = !C::SLOT_FIRST || first_slots || mbar_test(&bars->s8_empty[ss], s_ph);
+        const bool r1 = skip || mbar_test(r_full + pos, ph);
+        if (!__all_sync(0xffffffffu, r0 && r1)) {
+          if ((C::SLOT_FIRST && !first_slots && !wait_bar_warp(&bars->s8_empty[ss], s_ph, abort_flag, p.wait_clocks)) ||
+              !__all_sync(0xffffffffu, skip || wait_bar(r_full + pos, ph, abort_flag, p.wait_clocks))) {
+            ok = false;
+            break;
+          }
+        }
+        __syncwarp();  // what one lane waited for is there for all
+      }
+      if (!first_slots) {
+        load_w(ps, 0);
+        if (!C::SLOT_FIRST && !__all_sync(0xffffffffu, mbar_test(&bars->s8_empty[ss], s_ph)) &&
+            !wait_bar_warp(&bars->s8_empty[ss], s_ph, abort_flag, p.wait_clocks)) {
           ok = false;
           break;
         }
+        put_w(ss, 0);
+        rest_w(ps, ss);
+      }
+      if (!A8 && !C::TOGETHER && !wait_bar_warp(&bars->xp_full[xs], x_ph, abort_flag, p.wait_clocks)) {
+        ok = false;
+        break;
+      }
+      if (!A8) {
         const uint8_t* xsrc = x_buf + xs * C::X_STAGE;
         uint8_t* dst = slot_buf + ss * C::SLOT;
-        constexpr int UNITS = NT * 4;  // one unit = one 16-byte packed chunk of a token row
+        constexpr int UNITS = NT * 4, PER_THREAD = (UNITS + 127) / 128;       // per 128 elements; one unit = one 16-byte packed chunk of a token row
+        constexpr int BATCH = PER_THREAD <= 4 ? PER_THREAD : PER_THREAD / 2;  // chunks read together
+        static_assert(PER_THREAD % BATCH == 0, "whole batches");
 #pragma unroll
-        for (int i = 0; i < (UNITS + 127) / 128; ++i) {
-          const int unit = i * 128 + gt;
-          if (UNITS % 128 != 0 && unit >= UNITS) break;
-          const int row = unit >> 2, j = unit & 3, sw = row & 7;
-          const uint4 v = *reinterpret_cast<const uint4*>(xsrc + unit * 16);
-          uint8_t* drow = dst + row * BK;
-          *reinterpret_cast<uint4*>(drow + (((2 * j) ^ sw) << 4)) =
-              make_uint4(pq::nib_lo_x16(v.x), pq::nib_lo_x16(v.y), pq::nib_lo_x16(v.z), pq::nib_lo_x16(v.w));
-          *reinterpret_cast<uint4*>(drow + (((2 * j + 1) ^ sw) << 4)) =
-              make_uint4(pq::nib_hi_x16(v.x), pq::nib_hi_x16(v.y), pq::nib_hi_x16(v.z), pq::nib_hi_x16(v.w));
+        for (int h = 0; h < C::SUBS; ++h) {
+#pragma unroll
+          for (int i0 = 0; i0 < PER_THREAD; i0 += BATCH) {
+            uint4 x[BATCH];
+#pragma unroll
+            for (int i = 0; i < BATCH; ++i) {
+              const int unit = (i0 + i) * 128 + gt;
+              if (UNITS % 128 == 0 || unit < UNITS) x[i] = *reinterpret_cast<const uint4*>(xsrc + h * (NT * PK_ROW) + unit * 16);
+            }
+#pragma unroll
+            for (int i = 0; i < BATCH; ++i) {
+              const int unit = (i0 + i) * 128 + gt;
+              if (UNITS % 128 != 0 && unit >= UNITS) break;
+              const int row = unit >> 2, j = unit & 3, sw = row & 7;
+              uint8_t* drow = dst + h * C::SUB_SLOT + row * BK;
+              *reinterpret_cast<uint4*>(drow + (((2 * j) ^ sw) << 4)) =
+                  make_uint4(pq::nib_lo_x16(x[i].x), pq::nib_lo_x16(x[i].y), pq::nib_lo_x16(x[i].z), pq::nib_lo_x16(x[i].w));
+              *reinterpret_cast<uint4*>(drow + (((2 * j + 1) ^ sw) << 4)) =
+                  make_uint4(pq::nib_hi_x16(x[i].x), pq::nib_hi_x16(x[i].y), pq::nib_hi_x16(x[i].z), pq::nib_hi_x16(x[i].w));
+            }
+          }
         }
         pq::fence_proxy_async_smem();  // generic-proxy writes -> visible to the tensor core
       }
       pq::tmem_st_wait();
       pq::tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        pq::mbar_arrive(&bars->s8_full[ss]);
-        if (!C::EARLY_W) pq::mbar_arrive(&bars->w_empty[ps]);
-        if (!A8) pq::mbar_arrive(&bars->xp_empty[xs]);
-      }
+      if (arrives) pq::mbar_arrive(r_arrive + (role == 0 ? ps : r_pos));
+      r_pos += C::GROUPS;
+      if (r_pos >= r_len) r_pos -= r_len, r_ph ^= 1;
+      ps += C::GROUPS;
+      if (ps >= C::STAGES) ps -= C::STAGES, w_ph ^= 1;
+      xs += C::GROUPS;
+      if (xs >= C::X_STAGES) xs -= C::X_STAGES, x_ph ^= 1;
+      ss += C::GROUPS;
+      if (ss >= C::SLOTS) ss -= C::SLOTS, s_ph ^= 1;
     }
     // ------------------------------------------------------------------ accumulator -> the partial tile [token][channel]
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     ok = ok && wait_bar_warp(&bars->acc_full, 0, abort_flag, p.wait_clocks);
     if (ok) {
       constexpr int SHIFT = A8 ? 4 : 8;  // the factors 16 the expanded codes carry
@@ -382,6 +488,9 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
       }
       pq::tc_fence_before();
     }
+  } else {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    load_steps();
   }
   if (!ok && lane == 0) {
     bars->abort_flag = 1;
@@ -400,15 +509,16 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
     __syncthreads();
   }
   cluster_sync_all();  // every CTA's partial tile is in place
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // (long past) the scales and the output may belong to the previous kernel
   if (warp == 1) {
     pq::tc_fence_after();
     pq::tmem_dealloc(tmem_base, C::TMEM_COLS);
   }
   const int tokens = p.M - t0 < NT ? p.M - t0 : NT;
-  if (p.splits == 1) reduce_tile<1, 4, ZP>(p, smem, t0, n0, tokens, warp, C::THREADS / 32, lane);
-  else if (p.splits <= 4) reduce_tile<4, 2, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane);
-  else reduce_tile<MAX_SPLIT, 1, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) sw[i] *= s_a, zw[i] *= zp8;
+  if (p.splits == 1) reduce_tile<1, 4, ZP>(p, smem, t0, n0, tokens, warp, C::THREADS / 32, lane, sw, zw);
+  else if (p.splits <= 4) reduce_tile<4, 2, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane, sw, zw);
+  else reduce_tile<MAX_SPLIT, 1, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane, sw, zw);
   // no CTA leaves while a peer may still read its partial tile; relaxed: the reads are done, and the output stores need not
   // have reached memory
   __syncwarp();
@@ -435,7 +545,8 @@ pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw
   const int resident = ctx->sm_count * C::CTAS_PER_SM * 7 / 8;
   int splits = resident / tiles;
   if (splits > MAX_SPLIT) splits = MAX_SPLIT;
-  if (splits > p.n_kb / 5) splits = p.n_kb / 5;
+  p.n_kb = (p.K + C::KB - 1) / C::KB;
+  if (splits > p.K / (5 * BK)) splits = p.K / (5 * BK);
   if (splits < 1) splits = 1;
   p.splits = splits;
   cudaLaunchConfig_t cfg = {};
@@ -458,10 +569,10 @@ pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw
 
 template <bool A8, bool ZP>
 pq_status launch_tokens(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, SplitParams& p, int64_t K, cudaStream_t st) {
-  const int nt = split_width(p.M);
+  const int nt = split_width(p.M), kb = split_kb(nt, A8);
   CUtensorMap tx, tw;
   if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, nt) : make_packed_map(ctx, &tx, xq, p.M, K / 2, nt)) ||
-      !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH, CU_TENSOR_MAP_SWIZZLE_64B))
+      !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH, kb == BK ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, kb / 2))
     return PQ_ERR_CUDA;
   switch (nt) {
     case 16: return launch_split<16, A8, ZP>(ctx, tx, tw, p, st);
@@ -495,7 +606,7 @@ pq_status pq_gemm_split_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq
   p.ldo = ldo;
   p.M = static_cast<int>(M);
   p.N = static_cast<int>(N);
-  p.n_kb = static_cast<int>((K + BK - 1) / BK);
+  p.K = static_cast<int>(K);
   p.vec_out = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0;
   p.wait_clocks = ctx->wait_clocks;
   if (a8) return launch_tokens<true, false>(ctx, xq, wq, p, K, st);

@@ -98,20 +98,6 @@ __device__ __forceinline__ void mma2_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Has the phase completed? Unlike try_wait this never suspends the thread, which has MMAs to issue meanwhile.
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(pq::smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 // 16 lanes x 32 columns as 8 x 8 fragments: register 4j + 2h + e holds lane i/4 + 8h, column 8j + 2(i%4) + e (thread i of the warp).
 __device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(

@@ -69,6 +69,20 @@ def test_split_gemm_matches_oracle(ctx, mode, M, N, K):
     check(ctx, mode, M, N, K)
 
 
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M", [17, 33, 49, 64, 96, 128])
+def test_split_gemm_ends_of_the_k_blocks_and_rings(ctx, mode, M):
+    """K around whole K blocks of 128 and 256 elements (a part of one, one and a half, a ring's length and one more, with and without a K split),
+    at each width of the token tiles."""
+    for N, K in [(130, 96), (128, 224), (129, 256), (64, 288), (130, 1536), (130, 1664), (70, 1824), (200, 7168 + 160)]:
+        check(ctx, mode, M, N, K)
+
+
+def test_few_tokens_of_a_long_k(ctx):
+    for mode, M, N, K in [("w4a4", 1, 136, 16416), ("w4a8", 8, 130, 20480), ("rows", 3, 264, 28672), ("asym", 5, 100, 16512)]:
+        check(ctx, mode, M, N, K)
+
+
 @pytest.mark.parametrize("M,N,K,pad", [(40, 131, 1536, 5), (100, 260, 5120, 4), (24, 3000, 10240, 1)])
 def test_split_gemm_with_a_padded_output(ctx, M, N, K, pad):
     """Row pitches that allow 8-byte stores and that do not; up to eight K splits, two and more K blocks per expansion group."""
