@@ -178,17 +178,18 @@ constexpr int SPLIT_BAR_BYTES = 512;       // no less than the kernel's barriers
 // where the rings hold enough of them: two operand slots, one per expansion group, and as many landing stages as fit beside them. us, rotation and
 // GEMM in a graph: 64 x 57344 x 8192 62.9 (128 elements) / 62.5 (256, four weight stages and two of tokens) / 59.5 (three and three);
 // 8-bit tokens, 128 x 28672 x 4096 22.6 / 23.0 (two stages) / 20.2 (three). At 96 and 128 packed tokens the landing stages of the tokens leave no room.
-constexpr int split_kb(int nt, bool a8) { return nt <= (a8 ? 128 : 64) ? 256 : 128; }
+constexpr int split_kb(int nt, bool a8, bool whole) { return nt <= (a8 && !whole ? 128 : 64) ? 256 : 128; }
 
-template <int NT, bool A8>
+// WHOLE: one CTA to an SM, four expansion groups (above 128 tokens).
+template <int NT, bool A8, bool WHOLE = (NT > 128)>
 struct SplitCfg {
-  static constexpr int KB = split_kb(NT, A8), SUBS = KB / BK;  // elements of a K block
+  static constexpr int KB = split_kb(NT, A8, WHOLE), SUBS = KB / BK;  // elements of a K block
   static constexpr int ROWB = KB / 2;                          // packed bytes of a row in it
-  static constexpr int GROUPS = NT > 128 ? 4 : 2;
-  static constexpr int SLOTS = KB == 256 || (NT == 128 && !A8) ? 2 : 4;
+  static constexpr int GROUPS = WHOLE ? 4 : 2;
+  static constexpr int SLOTS = !WHOLE && (KB == 256 || (NT == 128 && !A8)) ? 2 : 4;
   static constexpr int W_STAGE = CH * ROWB;
-  static constexpr int STAGES = KB == 128 ? 4 : (NT <= (A8 ? 32 : 16) ? 6 : (NT <= (A8 ? 96 : 48) ? 4 : 3));  // landing ring, weights
-  static constexpr int X_STAGES = KB == 256 && NT > 48 ? 3 : 4;                                               // landing ring, tokens
+  static constexpr int STAGES = WHOLE ? (NT <= 128 ? 8 : 4) : KB == 128 ? 4 : (NT <= (A8 ? 32 : 16) ? 6 : (NT <= (A8 ? 96 : 48) ? 4 : 3));  // landing ring, weights
+  static constexpr int X_STAGES = !WHOLE && KB == 256 && NT > 48 ? 3 : 4;                                               // landing ring, tokens
   static constexpr bool TOGETHER = KB == 256;  // weights and tokens of a K block are waited for together
   static constexpr bool SLOT_FIRST = STAGES % GROUPS != 0 || (!A8 && X_STAGES % GROUPS != 0);
   static constexpr bool EARLY_W = NT > 128;          // weight stages go back before the (long) token part of the expansion
@@ -197,8 +198,8 @@ struct SplitCfg {
   static constexpr int SLOT = SUBS * SUB_SLOT;
   static constexpr int A_COLS = SUBS * A_SLOT_COLS;
   static constexpr int A_COL0 = NT < 32 ? 32 : NT;  // accumulator columns, then the A slots
-  static constexpr int TMEM_COLS = NT > 128 ? 512 : 256;
-  static constexpr int CTAS_PER_SM = NT > 128 ? 1 : 2;
+  static constexpr int TMEM_COLS = WHOLE ? 512 : 256;
+  static constexpr int CTAS_PER_SM = WHOLE ? 1 : 2;
   static constexpr int RING = SLOTS * SLOT + STAGES * W_STAGE + X_STAGES * X_STAGE;
   static constexpr int PART = NT * CH * 4;  // the int32 partial tile, laid over the rings at the end
   static_assert(A_COL0 + SLOTS * A_COLS <= TMEM_COLS, "tensor memory budget");
@@ -212,16 +213,46 @@ struct SplitCfg {
 // At least 80 KB for 256 columns of tensor memory and 160 KB for 512, so that no more CTAs share an SM (228 KB) than its tensor memory
 // serves, those of other launches included: a CTA that waited for columns which another cluster's CTA gives back only behind its
 // cluster barrier could wait for itself. (8-bit tokens 192 wide need 130 KB, which leave room for a CTA of a narrow form.)
-template <int NT, bool A8>
+template <int NT, bool A8, bool WHOLE = (NT > 128)>
 constexpr size_t split_smem() {
-  const size_t need = SplitCfg<NT, A8>::RING + SPLIT_BAR_BYTES, least = SplitCfg<NT, A8>::TMEM_COLS / 256 * (80 * 1024);
+  const size_t need = SplitCfg<NT, A8, WHOLE>::RING + SPLIT_BAR_BYTES, least = SplitCfg<NT, A8, WHOLE>::TMEM_COLS / 256 * (80 * 1024);
   return need < least ? least : need;
 }
 
-// The width of the token tiles: above 128 tokens they are spread over as few tiles as hold them.
-inline int split_width(int M) {
-  const int per_tile = (M + (M + 255) / 256 - 1) / ((M + 255) / 256);
-  return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 48 ? 48 : (M <= 64 ? 64 : (M <= 96 ? 96 : (M <= 128 ? 128 : (per_tile <= 192 ? 192 : 256))))));
+constexpr int MAX_SPLIT = 8;  // portable cluster size
+
+// As many K splits as leave every CTA resident at once with room for the clusters to be placed (7/8 of the slots: 48 tiles
+// x 6 = 288 CTAs ran in two waves, 10.7 us against 7.0 with 96), and at least 640 elements of K per CTA (below that the two
+// cluster barriers cost more than the shorter loop saves: 4096 x 4096 at 32 tokens 6.1 us with six splits, 6.6 with eight).
+inline int split_count(int tiles, int K, int slots) {
+  int splits = slots * 7 / 8 / tiles;
+  if (splits > MAX_SPLIT) splits = MAX_SPLIT;
+  if (splits > K / (5 * BK)) splits = K / (5 * BK);
+  return splits < 1 ? 1 : splits;
+}
+
+// The width of the token tiles up to 128 tokens.
+inline int split_width(int M) { return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 48 ? 48 : (M <= 64 ? 64 : (M <= 96 ? 96 : 128)))); }
+
+// The width above 128 tokens, by the estimate of a launch (one CTA to an SM): K blocks per CTA times what 128 elements of one take at that
+// width, and what the partial tiles cost that cross the cluster. Their sums move at some 25 bytes per ns and SM (four splits of 256 tokens: 96 KB per
+// CTA, 4 us), so a launch that leaves SMs idle at 256 tokens takes narrower tiles rather than more splits, although the weights are then
+// expanded more often. us per 128 elements at 64, 128, 192, 256 tokens: 0.164, 0.275, 0.36, 0.385, with 8-bit tokens 0.13, 0.21, 0.31, 0.33.
+// us with the rotation, 192 or 256 tokens wide -> by this rule: 256 x 4096 x 4096 15.2 -> 12.8 (two splits of 128), 192 x 6144 x 4096 14.9 -> 13.1 (64),
+// W4A8 256 x 4096 x 4096 14.9 -> 12.1, 256 x 4096 x 14336 23.1 -> 21.7, 512 x 4096 x 4096 15.6 -> 15.2.
+inline int split_width_whole(int M, int N, int K, bool a8, int sm_count) {
+  const int widths[] = {64, 128, 192, 256};
+  const double us4[] = {0.164, 0.275, 0.36, 0.385}, us8[] = {0.13, 0.21, 0.31, 0.33};
+  int best = 0;
+  double best_us = 0.0;
+  for (int i = 0; i < 4; ++i) {
+    const int t_tiles = (M + widths[i] - 1) / widths[i], tiles = t_tiles * ((N + CH - 1) / CH), splits = split_count(tiles, K, sm_count);
+    const int rounds = (tiles * splits + sm_count - 1) / sm_count, blocks = ((K + BK - 1) / BK + splits - 1) / splits;
+    const double tokens = (M + t_tiles - 1) / t_tiles;
+    const double us = rounds * blocks * (a8 ? us8 : us4)[i] + tokens * tokens * (splits - 1) / splits * (4.5 / 65536);
+    if (best == 0 || us < best_us) best = widths[i], best_us = us;
+  }
+  return best;
 }
 
 }  // namespace pq_plan

@@ -53,8 +53,8 @@ using namespace pq_plan;
 constexpr int EXPAND_WARP0 = 4;
 constexpr int MAX_SPLIT = 8;               // portable cluster size
 
-template <int NT, bool A8>
-struct Cfg : SplitCfg<NT, A8> {
+template <int NT, bool A8, bool WHOLE>
+struct Cfg : SplitCfg<NT, A8, WHOLE> {
   static constexpr int THREADS = (EXPAND_WARP0 + 4 * Cfg::GROUPS) * 32;
 };
 
@@ -164,10 +164,10 @@ __device__ __forceinline__ void reduce_tile(const SplitParams& p, const uint8_t*
   }
 }
 
-template <int NT, bool A8, bool ZP>
-__global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM)
+template <int NT, bool A8, bool ZP, bool WHOLE>
+__global__ void __launch_bounds__(Cfg<NT, A8, WHOLE>::THREADS, Cfg<NT, A8, WHOLE>::CTAS_PER_SM)
     gemm_w4_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const SplitParams p) {
-  using C = Cfg<NT, A8>;
+  using C = Cfg<NT, A8, WHOLE>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
   uint8_t* slot_buf = smem;                                // SLOTS token operands [NT x 128 B], 128-byte swizzle
@@ -526,63 +526,62 @@ __global__ void __launch_bounds__(Cfg<NT, A8>::THREADS, Cfg<NT, A8>::CTAS_PER_SM
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
-template <int NT, bool A8, bool ZP>
+template <int NT, bool A8, bool ZP, bool WHOLE>
 pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw, SplitParams& p, cudaStream_t st) {
-  using C = Cfg<NT, A8>;
+  using C = Cfg<NT, A8, WHOLE>;
+  constexpr size_t smem = split_smem<NT, A8, WHOLE>();
   static bool attr_set[64] = {};  // the attribute belongs to the device's copy of the kernel: once per device
   if (ctx->device < 0 || ctx->device >= 64) return PQ_ERR_UNSUPPORTED;
   if (!attr_set[ctx->device]) {
-    if (cudaFuncSetAttribute(gemm_w4_split_kernel<NT, A8, ZP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(split_smem<NT, A8>())) != cudaSuccess)
+    if (cudaFuncSetAttribute(gemm_w4_split_kernel<NT, A8, ZP, WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
       return PQ_ERR_CUDA;
     attr_set[ctx->device] = true;
   }
   p.t_tiles = (p.M + NT - 1) / NT;
-  const int tiles = p.t_tiles * ((p.N + CH - 1) / CH);
-  // As many K splits as leave every CTA resident at once with room for the clusters to be placed (7/8 of the slots: 48 tiles
-  // x 6 = 288 CTAs ran in two waves, 10.7 us against 7.0 with 96), and at least five K blocks per CTA (below that the two
-  // cluster barriers cost more than the shorter loop saves: 4096 x 4096 at 32 tokens 6.1 us with six splits, 6.6 with eight).
-  const int resident = ctx->sm_count * C::CTAS_PER_SM * 7 / 8;
-  int splits = resident / tiles;
-  if (splits > MAX_SPLIT) splits = MAX_SPLIT;
   p.n_kb = (p.K + C::KB - 1) / C::KB;
-  if (splits > p.K / (5 * BK)) splits = p.K / (5 * BK);
-  if (splits < 1) splits = 1;
-  p.splits = splits;
+  const int tiles = p.t_tiles * ((p.N + CH - 1) / CH);
+  p.splits = split_count(tiles, p.K, ctx->sm_count * C::CTAS_PER_SM);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(tiles) * splits);
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles) * p.splits);
   cfg.blockDim = dim3(C::THREADS);
-  cfg.dynamicSmemBytes = split_smem<NT, A8>();
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = splits;
+  attr[0].val.clusterDim.x = p.splits;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, gemm_w4_split_kernel<NT, A8, ZP>, tx, tw, p) != cudaSuccess) return PQ_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, gemm_w4_split_kernel<NT, A8, ZP, WHOLE>, tx, tw, p) != cudaSuccess) return PQ_ERR_CUDA;
   return pq_launch_status();
 }
 
 template <bool A8, bool ZP>
 pq_status launch_tokens(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq, SplitParams& p, int64_t K, cudaStream_t st) {
-  const int nt = split_width(p.M), kb = split_kb(nt, A8);
+  const bool whole = p.M > 128;
+  const int nt = whole ? split_width_whole(p.M, p.N, p.K, A8, ctx->sm_count) : split_width(p.M), kb = split_kb(nt, A8, whole);
   CUtensorMap tx, tw;
   if (!(A8 ? make_s8_map(ctx, &tx, xq, p.M, K, nt) : make_packed_map(ctx, &tx, xq, p.M, K / 2, nt)) ||
       !make_packed_map(ctx, &tw, wq, p.N, K / 2, CH, kb == BK ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, kb / 2))
     return PQ_ERR_CUDA;
+  if (whole) {
+    switch (nt) {
+      case 64: return launch_split<64, A8, ZP, true>(ctx, tx, tw, p, st);
+      case 128: return launch_split<128, A8, ZP, true>(ctx, tx, tw, p, st);
+      case 192: return launch_split<192, A8, ZP, true>(ctx, tx, tw, p, st);
+      default: return launch_split<256, A8, ZP, true>(ctx, tx, tw, p, st);
+    }
+  }
   switch (nt) {
-    case 16: return launch_split<16, A8, ZP>(ctx, tx, tw, p, st);
-    case 32: return launch_split<32, A8, ZP>(ctx, tx, tw, p, st);
-    case 48: return launch_split<48, A8, ZP>(ctx, tx, tw, p, st);
-    case 64: return launch_split<64, A8, ZP>(ctx, tx, tw, p, st);
-    case 96: return launch_split<96, A8, ZP>(ctx, tx, tw, p, st);
-    case 128: return launch_split<128, A8, ZP>(ctx, tx, tw, p, st);
-    case 192: return launch_split<192, A8, ZP>(ctx, tx, tw, p, st);
-    default: return launch_split<256, A8, ZP>(ctx, tx, tw, p, st);
+    case 16: return launch_split<16, A8, ZP, false>(ctx, tx, tw, p, st);
+    case 32: return launch_split<32, A8, ZP, false>(ctx, tx, tw, p, st);
+    case 48: return launch_split<48, A8, ZP, false>(ctx, tx, tw, p, st);
+    case 64: return launch_split<64, A8, ZP, false>(ctx, tx, tw, p, st);
+    case 96: return launch_split<96, A8, ZP, false>(ctx, tx, tw, p, st);
+    default: return launch_split<128, A8, ZP, false>(ctx, tx, tw, p, st);
   }
 }
 

@@ -31,6 +31,7 @@ void acc_slots(const PairPlan* p, int h, int first, int step, int count, int* ou
   }
 }
 int width(int m) { return split_width(m); }
+int width_whole(int m, int n, int k, int a8) { return split_width_whole(m, n, k, a8 != 0, 148); }
 #define ROW(NT, A8) {NT, A8, SplitCfg<NT, A8>::TMEM_COLS, (int)split_smem<NT, A8>()}
 int split_rows(int (*out)[4]) {
   const int rows[][4] = {ROW(16, 0), ROW(32, 0), ROW(48, 0), ROW(64, 0), ROW(96, 0), ROW(128, 0), ROW(192, 0), ROW(256, 0),
@@ -38,6 +39,13 @@ int split_rows(int (*out)[4]) {
   for (int i = 0; i < 16; ++i)
     for (int j = 0; j < 4; ++j) out[i][j] = rows[i][j];
   return 16;
+}
+#define WHOLE_ROW(NT, A8) {NT, A8, SplitCfg<NT, A8, true>::TMEM_COLS, (int)split_smem<NT, A8, true>()}
+int whole_rows(int (*out)[4]) {
+  const int rows[][4] = {WHOLE_ROW(64, 0), WHOLE_ROW(128, 0), WHOLE_ROW(64, 1), WHOLE_ROW(128, 1)};
+  for (int i = 0; i < 4; ++i)
+    for (int j = 0; j < 4; ++j) out[i][j] = rows[i][j];
+  return 4;
 }
 }
 """
@@ -100,3 +108,15 @@ def split_shapes():
     out = ((ctypes.c_int * 4) * 16)()
     n = lib().split_rows(out)
     return [tuple(out[i]) for i in range(n)]
+
+
+def whole_shapes():
+    """The same of the narrow forms that take an SM alone."""
+    out = ((ctypes.c_int * 4) * 4)()
+    n = lib().whole_rows(out)
+    return [tuple(out[i]) for i in range(n)]
+
+
+def width_whole(M, N, K, a8):
+    """Width of the split-K kernel's token tiles above 128 tokens."""
+    return lib().width_whole(M, N, K, int(a8))

@@ -179,3 +179,17 @@ def test_ctas_that_fit_one_sm_find_their_tensor_memory():
                 group = [f for f in (a, b, c) if f[0]]
                 if sum(smem + 1024 for *_, smem in group) <= 228 * 1024:
                     assert sum(cols for _, _, cols, _ in group) <= 512, group
+
+
+def test_narrow_forms_that_take_an_sm_alone_share_it_with_no_other():
+    for a in gp.whole_shapes():
+        for b in gp.whole_shapes() + gp.split_shapes():
+            assert a[3] + b[3] + 2048 > 228 * 1024 or a[2] + b[2] <= 512, (a, b)
+
+
+@pytest.mark.parametrize("M,N,K,a8,want", [
+    (256, 4096, 4096, False, 128), (192, 6144, 4096, False, 64), (130, 4096, 4096, False, 192), (512, 4096, 4096, False, 256),
+    (256, 8192, 28672, False, 256), (256, 4096, 14336, True, 128), (130, 6144, 4096, True, 64), (512, 4096, 14336, True, 256),
+])
+def test_width_above_128_tokens(M, N, K, a8, want):
+    assert gp.width_whole(M, N, K, a8) == want

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import gemm_plan
 from oracle import pq_oracle as orc
 from helpers import assert_bf16_close, rand_codes, to_np
 from paper_2410_05265_b200 import inputs
@@ -76,6 +77,17 @@ def test_split_gemm_ends_of_the_k_blocks_and_rings(ctx, mode, M):
     at each width of the token tiles."""
     for N, K in [(130, 96), (128, 224), (129, 256), (64, 288), (130, 1536), (130, 1664), (70, 1824), (200, 7168 + 160)]:
         check(ctx, mode, M, N, K)
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M,N,K,width", [
+    (129, 5000, 1280, 64), (192, 6001, 1536, 64), (191, 6144, 96, 64), (136, 6100, 4128, 64), (250, 3000, 416, 64),
+    (210, 3900, 2592, 128), (255, 2600, 2080, 128), (256, 3000, 3232, 128),
+])
+def test_narrow_tiles_above_128_tokens(ctx, mode, M, N, K, width):
+    """The forms that take an SM alone, 64 and 128 tokens wide: ragged last tiles, one K block to more than the rings hold, one K split and two."""
+    assert gemm_plan.width_whole(M, N, K, mode == "w4a8") == width
+    check(ctx, mode, M, N, K)
 
 
 def test_few_tokens_of_a_long_k(ctx):
