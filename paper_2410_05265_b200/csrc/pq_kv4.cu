@@ -84,6 +84,11 @@ constexpr int DA_MAX_SPLITS = 32;
 constexpr int DA_MAX_PREFIX = 64;
 constexpr int DA_ROWS = 8;  // query heads per KV head the MMA tile can carry
 constexpr int DA_TICKET0 = 16;
+// Few (sequence, head) pairs: up to this many rounds of keys the (at most eight) splits of a pair are one cluster, which merges on chip; beyond,
+// more splits pay for their second merge through the workspace. us, one cluster / more splits, plain call in a graph: 1 x 1021 keys (8 pairs)
+// 5.4 / 9.1, 1 x 2000 6.2 / 8.5, 1 x 4092 8.0 / 8.9, 3 x 3000 7.8 / 13.6, steps per vector 2 x 4000 10.4 / 15.5; the one-launch step inside a
+// decode layer: 1021 keys 55.4 / 55.7, 4000 keys 58.5 / 58.0 (its first rounds are on their way before it starts).
+constexpr int DA_ONE_CLUSTER_ROUNDS = 32, DA_ONE_CLUSTER_ROUNDS_FUSED = 24;
 constexpr float DA_HEADROOM = 15.0f;  // log2 units a score may exceed the reference exponent before it is moved
 constexpr float DA_HEADROOM_DYN = 4.0f;  // DYN: P * step * code stays within 2^7 of the largest cached value
 constexpr int DA_ROUND = 128;                     // keys staged per round (one half of the staging buffer)
@@ -289,12 +294,14 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   const uint8_t* vbase = p.vq + static_cast<int64_t>(bh) * p.Tmax * 64;
   const uint32_t stage_addr = pq::smem_u32(da_stage);
 
-  // Programmatic dependent launch: the plain call lets the next kernel of the stream be placed as its CTAs retire. The
-  // one-launch decode step does not, because it writes a cache row and the lengths: the step requests its first cache
+  // Programmatic dependent launch: the plain call is placed without a launch gap (in a stream, us: 8 x 4092 keys 15.3 -> 14.0, 6 x 1500 with
+  // steps per vector 10.5 -> 9.3, 1 x 1021 8.2 -> 5.5), and a small one lets its successor be placed at once; with the trigger in every grid back-to-back
+  // calls crowded on the SMs that had room (1 x 16000 keys, 64 heads, 13.6 -> 16.2 us). The
+  // one-launch decode step never triggers, because it writes a cache row and the lengths: the step requests its first cache
   // rows and reads the lengths ahead of griddepcontrol.wait, so whoever writes those may not let a successor start early
   // (see pq_launch_pdl). The query and the new token are read after the wait; the plain call reads everything after it.
   if (!FUSED) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (gridDim.x * gridDim.y * gridDim.z <= PQ_PDL_MAX_CTAS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
   }
 
@@ -323,6 +330,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
 
   const bool has_extra = FUSED && split == S - 1;
   float k_new_d = 0.0f, v_new_d = 0.0f;  // this thread's head dim of the token being appended
+  float q_new[FUSED ? DA_ROWS : 1];      // and of the group's queries, for the new key's scores
   if (FUSED && threadIdx.x == 0) sm_full = 0;
   if (threadIdx.x == 0) sm_abort = 0;
   // the operands of the first 16 (head, prefix key) pairs (all of them for a 4-token prefix under 4 heads)
@@ -372,6 +380,9 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
     if (has_extra) {
       const int64_t off = (static_cast<int64_t>(b) * p.Hkv + h) * 128 + threadIdx.x;
       k_new_d = __bfloat162float(p.k_new[off]), v_new_d = __bfloat162float(p.v_new[off]);
+#pragma unroll
+      for (int r = 0; r < DA_ROWS; ++r)  // requested together: one after the other in the loop over the heads, each waited for its own trip
+        if (FUSED) q_new[FUSED ? r : 0] = r < G ? __bfloat162float(p.q[(static_cast<int64_t>(b) * p.Hq + h * G + r) * 128 + threadIdx.x]) : 0.0f;
     }
   }
   __syncthreads();  // every barrier is initialised (all warps are still together here: this costs nothing)
@@ -380,29 +391,26 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
       const int l = __ldcg(p.len + i);
       if (l < 0 || l + 1 > p.Tmax) sm_full = 1;
     }
+    if (len_b < 0 || len_b + 1 > p.Tmax) sm_full = 1;  // also: this thread's length is in its register before the ticket below
     __syncthreads();
   }
   const bool append_ok = FUSED && !sm_full;
   const int len_raw = len_b;
-  // Called by every thread of every CTA when the CTA is done. The last CTA of the whole grid advances every length:
-  // by then each CTA has read the lengths it needs (its own sequence's, and all of them for the verdict above),
-  // so no CTA can ever see a length this launch has already moved.
-  auto finish_append = [&]() {
+  // This CTA has read every length it needs (its own sequence's, and all of them for the verdict above): it takes its ticket here and looks
+  // at it when it is done, so that the counter's trip is hidden. Whoever draws the last one advances every length: no CTA can
+  // ever see a length this launch has already moved.
+  uint32_t ticket = 0;
+  if (FUSED && append_ok && threadIdx.x == DA_THREADS - 32) ticket = atomicAdd(p.len_tickets, 1u);
+  auto finish_append = [&]() {  // by every thread of every CTA when the CTA is done
     if (!FUSED) return;
     if (!append_ok) {
       if (threadIdx.x == 0 && p.status && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) pq::report(p.status, PQ_ERR_SHAPE);
       return;
     }
-    __syncthreads();  // is_last is free again, and this CTA's cache writes precede the ticket
-    if (threadIdx.x == 0) {
-      __threadfence();
-      const uint32_t n_ctas = gridDim.x * gridDim.y * gridDim.z;
-      is_last = atomicAdd(p.len_tickets, 1u) == n_ctas - 1;
-    }
-    __syncthreads();
-    if (is_last) {
-      for (int i = threadIdx.x; i < p.B; i += DA_THREADS) p.len_rw[i] = __ldcg(p.len_rw + i) + 1;
-      if (threadIdx.x == 0) *p.len_tickets = 0;
+    if (warp != DA_WARPS - 1) return;
+    if (__shfl_sync(0xffffffffu, ticket, 0) == gridDim.x * gridDim.y * gridDim.z - 1) {
+      for (int i = lane; i < p.B; i += 32) p.len_rw[i] = __ldcg(p.len_rw + i) + 1;
+      if (lane == 0) *p.len_tickets = 0;
     }
   };
   len_b = len_b < 0 ? 0 : (len_b > p.Tmax ? p.Tmax : len_b);
@@ -459,8 +467,10 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
       const_cast<uint8_t*>(p.vq)[row] = static_cast<uint8_t>((vc & 0xF) | ((vc_hi & 0xF) << 4));
     }
     sm_newv[FUSED ? threadIdx.x : 0] = static_cast<float>(vc) * s_v_h;
-    for (int r = 0; r < G; ++r) {  // q[r] . k_code over the 128 threads
-      float part = __bfloat162float(p.q[(static_cast<int64_t>(b) * p.Hq + h * G + r) * 128 + threadIdx.x]) * static_cast<float>(kc);
+#pragma unroll
+    for (int r = 0; r < DA_ROWS; ++r) {  // q[r] . k_code over the 128 threads
+      if (r >= G) break;
+      float part = q_new[FUSED ? r : 0] * static_cast<float>(kc);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
       if (lane == 0) sm_red[warp][r] = part;
@@ -1041,12 +1051,18 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
     if (k_new) return PQ_ERR_UNSUPPORTED;  // the one-launch decode step serves the static setting
   }
   int S = choose_splits(ctx, cache);
+  const int rounds = (cache->Tmax + DA_ROUND - 1) / DA_ROUND;  // a split without a round would only take part in the merge
   // With enough (sequence, head) pairs, eight splits already fill the GPU: the splits then form one
   // cluster and merge through distributed shared memory (the workspace and the tickets stay unused).
   bool cluster = static_cast<int64_t>(cache->B) * cache->Hkv * 8 >= 2LL * ctx->sm_count;
   if (cluster && S > 8) S = 8;
+  if (S > rounds && rounds > 0) S = rounds;
   // Few (sequence, head) pairs with long caches: several clusters of eight splits per pair; each merges its eight
   // partials on chip, the workspace sees one partial per cluster.
+  if (!cluster && rounds <= (k_new ? DA_ONE_CLUSTER_ROUNDS_FUSED : DA_ONE_CLUSTER_ROUNDS)) {
+    if (S > 8) S = 8;
+    cluster = true;
+  }
   if (!cluster && S >= 16) {
     S = S / 8 * 8;
     cluster = true;
@@ -1094,7 +1110,7 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = fused ? 2 : 1;  // the plain call gains nothing from an early placement (measured), the one-launch step does
+    cfg.numAttrs = 2;
     cudaError_t e;
     if (dyn)
       e = multi ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true, true>, p)
@@ -1117,7 +1133,7 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = fused ? 1 : 0;
+  cfg.numAttrs = 1;
   if ((dyn     ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false, true>, p)
        : fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, true, false>, p)
                : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false>, p)) != cudaSuccess)
