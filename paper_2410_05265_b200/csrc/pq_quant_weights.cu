@@ -63,13 +63,14 @@ __global__ void __launch_bounds__(THREADS) quant_weights_once_kernel(const __nv_
   const int64_t n = blockIdx.x;
   const uint4* row = reinterpret_cast<const uint4*>(W + n * ldw);
   const int n_vec = K / 8;
+  pq::pdl_wait();  // placed while the kernel before it drains; it never lets its own successor start early (see pq_launch_pdl)
   uint4 v[VPT];
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
     const int j = threadIdx.x + i * THREADS;
     v[i] = make_uint4(0, 0, 0, 0);
     if (j < n_vec)
-      asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w) : "l"(row + j));
+      asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w) : "l"(row + j));
   }
   uint32_t m2 = 0;  // packed maxima of the patterns without sign
 #pragma unroll
@@ -158,11 +159,10 @@ extern "C" pq_status pq_quant_weights(pq_ctx* ctx, const void* W, int64_t N, int
     const __nv_bfloat16* w = static_cast<const __nv_bfloat16*>(W);
     const int k = static_cast<int>(K);
     const unsigned rows = static_cast<unsigned>(N);
-    if (K <= 4096) quant_weights_once_kernel<128, 4><<<rows, 128, 0, st>>>(w, k, ldw, wq, s_w);
-    else if (K <= 8192) quant_weights_once_kernel<256, 4><<<rows, 256, 0, st>>>(w, k, ldw, wq, s_w);
-    else if (K <= 16384) quant_weights_once_kernel<256, 8><<<rows, 256, 0, st>>>(w, k, ldw, wq, s_w);
-    else quant_weights_once_kernel<512, 8><<<rows, 512, 0, st>>>(w, k, ldw, wq, s_w);
-    return pq_launch_status();
+    if (K <= 4096) return pq_launch_pdl(quant_weights_once_kernel<128, 4>, dim3(rows), 128, 0, st, w, k, ldw, wq, s_w);
+    if (K <= 8192) return pq_launch_pdl(quant_weights_once_kernel<256, 4>, dim3(rows), 256, 0, st, w, k, ldw, wq, s_w);
+    if (K <= 16384) return pq_launch_pdl(quant_weights_once_kernel<256, 8>, dim3(rows), 256, 0, st, w, k, ldw, wq, s_w);
+    return pq_launch_pdl(quant_weights_once_kernel<512, 8>, dim3(rows), 512, 0, st, w, k, ldw, wq, s_w);
   }
   int grid = static_cast<int>(N < 65535 * 4 ? N : 65535 * 4);
   quant_weights_kernel<<<grid, QW_THREADS, 0, st>>>(
