@@ -492,6 +492,8 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
           w[tau][v] = pack_bf16x2(pq::silu_mul_f32(__uint_as_float(w[tau][v] << 16), __uint_as_float(u[tau][v] << 16)),
                                   pq::silu_mul_f32(__uint_as_float(w[tau][v] & 0xFFFF0000u), __uint_as_float(u[tau][v] & 0xFFFF0000u)));
     } else if (NORM) {
+      uint32_t g_w[8][4];  // requested ahead of the sum: behind it their trip stood in the chain of every row
+      load_words(x2 + col0, true, g_w);
       // sum of squares of the row in a fixed order: the thread's values, the warp's lanes, the block's warps
       float ss = 0.0f;
 #pragma unroll
@@ -512,8 +514,6 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
         __syncthreads();
       }
       const float rr = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(ss, static_cast<float>(B)), clip)));
-      uint32_t g_w[8][4];
-      load_words(x2 + col0, true, g_w);
 #pragma unroll
       for (int tau = 0; tau < 8; ++tau)
 #pragma unroll
