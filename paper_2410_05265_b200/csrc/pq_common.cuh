@@ -95,10 +95,27 @@ __device__ __forceinline__ uint4 ld_dep(const uint4* p) {
 
 __device__ __forceinline__ void report(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 
-// SiLU(g) * u in fp32 with the hardware exponential and reciprocal (about 2 ulp of fp32, far below the bf16
-// rounding that follows); the stand-alone kernel and the one fused into the rotation share it, so they agree
-// bit for bit.
-__device__ __forceinline__ float silu_mul_f32(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
+// SiLU(g) * u = g / (1 + 2^(-g log2 e)) * u in fp32 with the hardware's 2^x and reciprocal (about 2 ulp of fp32, far below the bf16
+// rounding that follows). The form for two elements does the same operations on packed pairs: the stand-alone kernel and the one fused
+// into the rotation agree bit for bit.
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float silu_mul_f32(float g, float u) {
+  return __fmul_rn(__fmul_rn(g, rcp_approx(__fadd_rn(1.0f, ex2_approx(__fmul_rn(g, -1.4426950408889634f))))), u);
+}
+__device__ __forceinline__ float2 silu_mul_f32(float2 g, float2 u) {
+  const float2 t = __fmul2_rn(g, make_float2(-1.4426950408889634f, -1.4426950408889634f));
+  const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(ex2_approx(t.x), ex2_approx(t.y)));
+  return __fmul2_rn(__fmul2_rn(g, make_float2(rcp_approx(d.x), rcp_approx(d.y))), u);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 

@@ -377,10 +377,11 @@ __device__ __forceinline__ void mma_bf16_m16n8k16(float (&d)[4], const uint32_t 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+__device__ __forceinline__ uint32_t pack_bf16x2(float2 v) {
+  __nv_bfloat162 p = __floats2bfloat162_rn(v.x, v.y);
   return *reinterpret_cast<uint32_t*>(&p);
 }
+__device__ __forceinline__ float2 bf16_pair(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
 
 //
 // ROW (the one-call dynamic quantizer of rows of several 2048-element blocks): a CTA has a warp for every block of a row, up to 16, so
@@ -489,8 +490,7 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
       for (int tau = 0; tau < 8; ++tau)
 #pragma unroll
         for (int v = 0; v < 4; ++v)
-          w[tau][v] = pack_bf16x2(pq::silu_mul_f32(__uint_as_float(w[tau][v] << 16), __uint_as_float(u[tau][v] << 16)),
-                                  pq::silu_mul_f32(__uint_as_float(w[tau][v] & 0xFFFF0000u), __uint_as_float(u[tau][v] & 0xFFFF0000u)));
+          w[tau][v] = pack_bf16x2(pq::silu_mul_f32(bf16_pair(w[tau][v]), bf16_pair(u[tau][v])));
     } else if (NORM) {
       uint32_t g_w[8][4];  // requested ahead of the sum: behind it their trip stood in the chain of every row
       load_words(x2 + col0, true, g_w);
@@ -518,8 +518,7 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
       for (int tau = 0; tau < 8; ++tau)
 #pragma unroll
         for (int v = 0; v < 4; ++v)
-          w[tau][v] = pack_bf16x2(__fmul_rn(__fmul_rn(__uint_as_float(w[tau][v] << 16), rr), __uint_as_float(g_w[tau][v] << 16)),
-                                  __fmul_rn(__fmul_rn(__uint_as_float(w[tau][v] & 0xFFFF0000u), rr), __uint_as_float(g_w[tau][v] & 0xFFFF0000u)));
+          w[tau][v] = pack_bf16x2(__fmul2_rn(__fmul2_rn(bf16_pair(w[tau][v]), make_float2(rr, rr)), bf16_pair(g_w[tau][v])));
       if (NORM == 2) {
         if (active) {
           uint32_t* drow = reinterpret_cast<uint32_t*>(reinterpret_cast<__nv_bfloat16*>(xq) + row * n_cand + col0 + e_thr);
