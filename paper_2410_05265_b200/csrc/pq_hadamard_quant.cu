@@ -383,6 +383,39 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float2 v) {
 }
 __device__ __forceinline__ float2 bf16_pair(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
 
+// The offset code u = clamp(rne(y / s) + 2^(BITS-1), 0, 2^BITS - 1) is taken in two fused multiply-adds:
+// f = sat(y * (inv / U) + 2^(BITS-1) / U) with U = 2^BITS - 1 is (y / s + 2^(BITS-1)) / U clamped to [0, 1] (the
+// clamp of the code range, applied before the rounding, which gives the same code), and f * U + 1.5 * 2^23
+// leaves rne(f * U) in the low mantissa bits. f carries one more rounding (2^-25 of the code range, i.e.
+// 5e-7 of a step for 4 bits, 8e-6 for 8 bits), far inside the distance from a tie within which a code may
+// differ from a double-precision evaluation. u ^ 2^(BITS-1) is the two's-complement code.
+// With a zero point (odd z would move ties) the rounding comes first: y * inv + (1.5 * 2^23 + 8), the integer
+// z - 8 added to the bit pattern, and an integer clamp.
+// Byte stores with a narrower code range (4-bit codes, one per byte): the caller's largest code in n_cand.
+template <int BITS, bool ZP>
+struct CodeRule {
+  float inv, U, invU, offU;
+  int zp, qmax;
+  __device__ __forceinline__ CodeRule(float inv_, int zp_, int n_cand) : inv(inv_), zp(zp_) {
+    qmax = (BITS == 8 && n_cand > 0) ? n_cand : (BITS == 4 ? 7 : 127);
+    U = static_cast<float>(2 * qmax + 1);
+    invU = __fdiv_rn(inv, U), offU = __fdiv_rn(static_cast<float>(qmax + 1), U);
+  }
+  __device__ __forceinline__ uint2 operator()(float2 y) const {  // bit patterns whose low BITS bits are the two offset codes
+    constexpr int BASE = 0x4B400000;
+    if (ZP) {
+      const float2 tq = __ffma2_rn(y, make_float2(inv, inv), make_float2(12582920.0f, 12582920.0f));
+      return make_uint2(static_cast<uint32_t>(max(min(__float_as_int(tq.x) + zp, BASE + 15), BASE)),
+                        static_cast<uint32_t>(max(min(__float_as_int(tq.y) + zp, BASE + 15), BASE)));
+    }
+    float fx, fy;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(fx) : "f"(y.x), "f"(invU), "f"(offU));
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(fy) : "f"(y.y), "f"(invU), "f"(offU));
+    const float2 tq = __ffma2_rn(make_float2(fx, fy), make_float2(U, U), make_float2(12582912.0f, 12582912.0f));
+    return make_uint2(__float_as_uint(tq.x), __float_as_uint(tq.y));
+  }
+};
+
 //
 // ROW (the one-call dynamic quantizer of rows of several 2048-element blocks): a CTA has a warp for every block of a row, up to 16, so
 // that the row's maximum is formed across its warps and the codes come from the registers that hold the rotated row: one pass and
@@ -668,31 +701,8 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
       }
     } else {
       // ---- quantize and pack ---------------------------------------------------------------------------
-      // The offset code u = clamp(rne(y / s) + 2^(BITS-1), 0, 2^BITS - 1) is taken in two fused multiply-adds:
-      // f = sat(y * (inv / U) + 2^(BITS-1) / U) with U = 2^BITS - 1 is (y / s + 2^(BITS-1)) / U clamped to [0, 1] (the
-      // clamp of the code range, applied before the rounding, which gives the same code), and f * U + 1.5 * 2^23
-      // leaves rne(f * U) in the low mantissa bits. f carries one more rounding (2^-25 of the code range, i.e.
-      // 5e-7 of a step for 4 bits, 8e-6 for 8 bits), far inside the distance from a tie within which a code may
-      // differ from a double-precision evaluation. u ^ 2^(BITS-1) is the two's-complement code.
-      // With a zero point (odd z would move ties) the rounding comes first: y * inv + (1.5 * 2^23 + 8), the integer
-      // z - 8 added to the bit pattern, and an integer clamp.
-      constexpr int BASE = 0x4B400000;
-      // byte stores with a narrower code range (4-bit codes, one per byte): the caller's largest code in n_cand
-      const int qmax = (BITS == 8 && n_cand > 0) ? n_cand : QMAX;
-      const float U = static_cast<float>(2 * qmax + 1);
-      const float invU = __fdiv_rn(inv, U), offU = __fdiv_rn(static_cast<float>(qmax + 1), U);
-      auto codes = [&](float2 y) -> uint2 {  // bit patterns whose low BITS bits are the two offset codes
-        if (ZP) {
-          const float2 tq = __ffma2_rn(y, make_float2(inv, inv), make_float2(12582920.0f, 12582920.0f));
-          return make_uint2(static_cast<uint32_t>(max(min(__float_as_int(tq.x) + zp, BASE + 15), BASE)),
-                            static_cast<uint32_t>(max(min(__float_as_int(tq.y) + zp, BASE + 15), BASE)));
-        }
-        float fx, fy;
-        asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(fx) : "f"(y.x), "f"(invU), "f"(offU));
-        asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(fy) : "f"(y.y), "f"(invU), "f"(offU));
-        const float2 tq = __ffma2_rn(make_float2(fx, fy), make_float2(U, U), make_float2(12582912.0f, 12582912.0f));
-        return make_uint2(__float_as_uint(tq.x), __float_as_uint(tq.y));
-      };
+      const CodeRule<BITS, ZP> codes(inv, zp, n_cand);
+      [[maybe_unused]] const int qmax = codes.qmax;
       // a thread's 32 bytes leave as one sector when the output is 32-byte aligned (rows are whole kilobytes)
       auto store32 = [&](uint8_t* dst, const uint32_t* v) {
         if (out32) {
@@ -750,6 +760,180 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
   }
 }
 
+// ---- wide blocks, few of them ---------------------------------------------------------------------------
+// The kernel above keeps 64 elements per thread, so a call of few blocks is one warp's chain of some 650 instructions on a mostly idle chip. Here a
+// thread has 16 elements and a block B / 16 threads, one block to a CTA: the same loads, MMAs and stages in the same order, so the codes are the
+// same bit for bit, spread over four times the warps. A warp (wide-kernel warp wv, tau bits 1 and 2) transforms bits {0, k1, k2, k3} by MMA,
+// then m3 and tau bit 0 in registers; after the one exchange a thread holds the pair of bit 0 for the eight values of tau, the lane is
+// bits 1..5 and the warp the bits between: tau bits 1 and 2 in registers, the rest by shuffles. Each thread stores the byte (4-bit codes)
+// of each of its pairs, a warp 32 consecutive ones. Latency bounds either kernel; us per call of M rows in a graph, wide kernel / this one:
+//   4096 (one block a row)   M = 1 2.08 / 1.84, 33 2.25 / 1.98, 148 2.39 / 2.16, 256 2.89 / 3.36; with RMSNorm 2.50 / 2.25, 2.75 / 2.35, 2.84 / 2.46, 3.70 / 4.51
+//   14336 (seven blocks)     M = 1 2.02 / 1.58, 33 2.21 / 1.95, 96 3.36 / 3.42; with SwiGLU 2.72 / 1.82, 2.98 / 2.39, 96 5.02 / 3.75, 148 4.77 / 4.64
+// so the line lies at one block of 4096 to an SM, two of 2048, five with SwiGLU. Blocks of 8192 (16 warps, five shuffle stages) stay with the
+// wide kernel: 2.28 / 2.85. Decode layer at 1021 tokens 53.8 -> 51.5.
+constexpr int hq_small_blocks_per_sm(int logb, bool swiglu) { return logb == 11 ? (swiglu ? 5 : 2) : (logb == 12 ? 1 : 0); }
+
+template <int LOGB, int BITS, bool PER_TOKEN, bool ZP, bool SWIGLU, int NORM>
+__global__ void __launch_bounds__(1 << (LOGB - 4))
+    hadamard_quant_small_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, int64_t K, const float* __restrict__ s_a_in,
+                                uint8_t* __restrict__ xq, float* __restrict__ s_a_out, float clip, const int32_t* __restrict__ zp_in,
+                                const __nv_bfloat16* __restrict__ x2, int n_cand) {
+  constexpr int QMAX = BITS == 4 ? 7 : 127;
+  static_assert(LOGB == 11 || LOGB == 12, "block width");
+  constexpr int B = 1 << LOGB, J = 13 - LOGB, WARPS = B / 512;
+  constexpr int T0S = 1, T1S = J == 2 ? 2 : 6, GS = J + 1, WS = J + 4;  // the index bits' roles are those of the wide kernel
+  constexpr int M3S = 8 - J, K3S = 9 - J, TAUS = 10 - J;
+  constexpr int PADK = J == 2 ? 4 : 20, BLKF = J == 2 ? 2176 : 4736;
+  __shared__ __align__(16) float my[NORM == 2 ? 1 : BLKF];
+  __shared__ float red[WARPS];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3, wv = warp >> 2, tp = warp & 3;
+  const int64_t blocks_per_row = K / B;
+  const int64_t row = blockIdx.x / blocks_per_row, col0 = blockIdx.x % blocks_per_row * B;
+  const int e_thr = ((t & 1) << T0S) | ((t >> 1) << T1S) | (g << GS) | (wv << WS);
+  auto load_words = [&](const __nv_bfloat16* base, uint32_t (&w)[2][4]) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(base + e_thr);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) w[i][v] = pq::ld_dep(src + (((2 * tp + i) << TAUS) | ((v & 1) << M3S) | ((v >> 1) << K3S)) / 2);
+  };
+  uint32_t w[2][4];
+  load_words(x + row * ldx + col0, w);
+  [[maybe_unused]] uint32_t u[2][4];
+  if (SWIGLU) load_words(x2 + row * ldx + col0, u);
+  if (NORM) load_words(x2 + col0, u);
+  const float norm = __fdiv_rn(1.0f, __fsqrt_rn(static_cast<float>(B)));
+  float inv = norm;
+  if (!PER_TOKEN && NORM != 2) inv = __fdiv_rn(norm, pq::ld_dep(s_a_in));
+  if (PER_TOKEN && s_a_out == nullptr) {
+    const float s_row = pq::ld_dep(s_a_in + row);
+    inv = __fdiv_rn(norm, s_row == 0.0f ? 1.0f : s_row);
+  }
+  const int zp = ZP ? pq::ld_dep(zp_in) - 8 : 0;
+
+  if (SWIGLU) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) w[i][v] = pack_bf16x2(pq::silu_mul_f32(bf16_pair(w[i][v]), bf16_pair(u[i][v])));
+  } else if (NORM) {
+    float ss = 0.0f;  // in an order of its own, shared by the stand-alone RMSNorm, which takes this kernel for the same calls
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const float2 a = bf16_pair(w[i][v]);
+        ss = __fmaf_rn(a.x, a.x, __fmaf_rn(a.y, a.y, ss));
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) red[warp] = ss;
+    __syncthreads();
+    ss = 0.0f;
+#pragma unroll
+    for (int i = 0; i < WARPS; ++i) ss += red[i];
+    const float rr = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(ss, static_cast<float>(B)), clip)));
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) w[i][v] = pack_bf16x2(__fmul2_rn(__fmul2_rn(bf16_pair(w[i][v]), make_float2(rr, rr)), bf16_pair(u[i][v])));
+    if (NORM == 2) {
+      uint32_t* drow = reinterpret_cast<uint32_t*>(reinterpret_cast<__nv_bfloat16*>(xq) + row * n_cand + col0 + e_thr);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) drow[(((2 * tp + i) << TAUS) | ((v & 1) << M3S) | ((v >> 1) << K3S)) / 2] = w[i][v];
+      return;
+    }
+  }
+
+  // ---- MMA stage, then m3 and tau bit 0 -------------------------------------------------------------------
+  float2 V[4][2];  // [m3 | tau bit 0 << 1][k3]
+#pragma unroll
+  for (int nb = 0; nb < 2; ++nb) {
+    uint32_t hb[2];  // H_16[k][n] for the columns n = lane / 4 + 8 nb
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = 2 * t + 8 * h, n = g + 8 * nb;
+      hb[h] = ((__popc(k & n) & 1) ? 0xBF80u : 0x3F80u) | ((__popc((k + 1) & n) & 1) ? 0xBF800000u : 0x3F800000u);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      float d[4];
+      mma_bf16_m16n8k16(d, w[i], hb[0], hb[1]);
+      V[2 * i][nb] = make_float2(d[0], d[1]);
+      V[2 * i + 1][nb] = make_float2(d[2], d[3]);
+    }
+  }
+  auto butterfly = [](float2& a, float2& b) {
+    const float2 lo = a, hi = b;
+    a = __fadd2_rn(lo, hi);
+    b = __ffma2_rn(hi, make_float2(-1.0f, -1.0f), lo);
+  };
+#pragma unroll
+  for (int nb = 0; nb < 2; ++nb) butterfly(V[0][nb], V[1][nb]), butterfly(V[2][nb], V[3][nb]);
+#pragma unroll
+  for (int nb = 0; nb < 2; ++nb) butterfly(V[0][nb], V[2][nb]), butterfly(V[1][nb], V[3][nb]);
+  // ---- exchange, in the wide kernel's padded layout ---------------------------------------------------------
+  const int wthr = e_thr + (J == 1 ? 16 * (t >> 1) : 0);
+#pragma unroll
+  for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int m3 = c & 1, tau = 2 * tp + (c >> 1);
+      *reinterpret_cast<float2*>(my + wthr + ((m3 << M3S) | (nb << K3S) | (tau << TAUS)) + PADK * (m3 | (nb << 1) | (tau << 2))) = V[c][nb];
+    }
+  __syncthreads();
+  const int rbase = 2 * lane + 64 * warp + PADK * (warp >> (M3S - 6)) + (J == 1 ? 16 * (warp & 1) : 0);
+  float2 P[8];
+#pragma unroll
+  for (int tau = 0; tau < 8; ++tau) P[tau] = *reinterpret_cast<const float2*>(my + rbase + (tau << TAUS) + PADK * (tau << 2));
+#pragma unroll
+  for (int s = 2; s < 8; s <<= 1)
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if ((c & s) == 0) butterfly(P[c], P[c | s]);
+#pragma unroll
+  for (int b = J; b < 5; ++b) {  // element bit b + 1 is bit b of the lane
+    const float sgn = (lane >> b) & 1 ? -1.0f : 1.0f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, P[c].x, 1 << b), __shfl_xor_sync(0xffffffffu, P[c].y, 1 << b));
+      P[c] = __ffma2_rn(P[c], make_float2(sgn, sgn), o);
+    }
+  }
+  if (PER_TOKEN && s_a_out != nullptr) {  // the row is this block: its step from its own maximum, in the operations of the wide kernel
+    float it_max = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) it_max = fmaxf(it_max, fmaxf(fabsf(P[c].x * norm), fabsf(P[c].y * norm)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) it_max = fmaxf(it_max, __shfl_xor_sync(0xffffffffu, it_max, o));
+    if (lane == 0) red[warp] = it_max;
+    __syncthreads();
+    it_max = 0.0f;
+#pragma unroll
+    for (int i = 0; i < WARPS; ++i) it_max = fmaxf(it_max, red[i]);
+    const float s_row = it_max > 0.0f ? __fdiv_rn(it_max * clip, static_cast<float>(QMAX)) : 0.0f;
+    if (tid == 0) s_a_out[row] = s_row;
+    inv = __fdiv_rn(norm, s_row == 0.0f ? 1.0f : s_row);
+  }
+  const CodeRule<BITS, ZP> rule(inv, zp, n_cand);
+  const int64_t e0 = col0 + 2 * lane + 64 * warp;
+#pragma unroll
+  for (int tau = 0; tau < 8; ++tau) {
+    const uint2 c = rule(P[tau]);
+    if (BITS == 4) {
+      xq[row * (K / 2) + (e0 + (tau << TAUS)) / 2] = static_cast<uint8_t>((c.x + (c.y << 4)) ^ 0x88u);
+    } else {
+      const uint32_t two = __vsub4(__byte_perm(c.x, c.y, 0x0040), static_cast<uint32_t>(rule.qmax + 1) * 0x01010101u);
+      *reinterpret_cast<uint16_t*>(xq + row * K + e0 + (tau << TAUS)) = static_cast<uint16_t>(two);
+    }
+  }
+}
 template <int LOGB, bool ROTATE, bool CALIB, int BITS, bool PER_TOKEN, bool ZP, bool SWIGLU, bool GRID, int NORM = 0>
 pq_status launch(pq_ctx* ctx, const void* x, int64_t ldx, int64_t n_rows, int64_t K, const float* s_a_in, uint8_t* xq,
                  float* s_a_out, float clip, const int32_t* zp_in, const void* x2, cudaStream_t st, int n_cand) {
@@ -768,6 +952,12 @@ pq_status launch(pq_ctx* ctx, const void* x, int64_t ldx, int64_t n_rows, int64_
     ctas_per_sm = HQW_CTAS_PER_SM;
   } else {
     kern = hadamard_quant_kernel<LOGB, ROTATE, CALIB, BITS, PER_TOKEN, ZP, SWIGLU, GRID, NORM>;
+  }
+  if constexpr (WIDE && !CALIB && !GRID && hq_small_blocks_per_sm(LOGB, SWIGLU) > 0) {
+    const int64_t blocks = n_rows * (K / B);
+    if (blocks <= static_cast<int64_t>(hq_small_blocks_per_sm(LOGB, SWIGLU)) * ctx->sm_count)
+      return pq_launch_pdl(hadamard_quant_small_kernel<LOGB, BITS, PER_TOKEN, ZP, SWIGLU, NORM>, dim3(static_cast<unsigned>(blocks)), B / 16, 0, st,
+                           static_cast<const __nv_bfloat16*>(x), ldx, K, s_a_in, xq, s_a_out, clip, zp_in, static_cast<const __nv_bfloat16*>(x2), n_cand);
   }
   // the shared-memory attribute is set once per device and instantiation (the call costs several microseconds of
   // host time, a visible share of a decode-sized launch)

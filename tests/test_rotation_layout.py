@@ -83,3 +83,27 @@ def test_a_warp_load_covers_whole_sectors_of_few_lines(logb, max_lines):
                         sectors.setdefault(b // 32, set()).update(range(b % 32, b % 32 + 4))
                     assert all(len(v) == 32 for v in sectors.values()), "every touched sector is used in full"
                     assert len({s // 4 for s in sectors}) <= max_lines
+
+
+@pytest.mark.parametrize("logb", [11, 12])
+def test_few_blocks_kernel_reads_back_what_its_warps_wrote(logb):
+    """hadamard_quant_small_kernel: warp 4 wv + tp writes the tiles 2 tp and 2 tp + 1 of the wide kernel's warp wv; after the exchange lane and warp
+    are index bits 1 and up, a thread's eight pairs the values of tau."""
+    r = roles(logb)
+    n, warps, j = 1 << logb, (1 << logb) // 512, r["J"]
+    where = {}
+    for warp in range(warps):
+        for lane in range(32):
+            for c in range(4):
+                for nb in range(2):
+                    i = writer_index(r, warp >> 2, lane, c & 1, nb, 2 * (warp & 3) + (c >> 1))
+                    assert i not in where
+                    where[i] = i + pad(i, r)
+    assert len(where) == n // 2 and max(where.values()) + 1 < r["BLKF"]
+    for warp in range(warps):
+        for lane in range(32):
+            base = 2 * lane + 64 * warp + r["PADK"] * (warp >> (r["M3"] - 6)) + (16 * (warp & 1) if j == 1 else 0)
+            for tau in range(8):
+                i = 2 * lane | (warp << 6) | (tau << r["TAU"])
+                assert where.pop(i) == base + (tau << r["TAU"]) + r["PADK"] * (tau << 2)
+    assert not where
