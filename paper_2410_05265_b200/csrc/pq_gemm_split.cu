@@ -69,6 +69,12 @@ struct __align__(8) SplitBarriers {
 
 static_assert(sizeof(SplitBarriers) <= SPLIT_BAR_BYTES, "shared memory budget");
 
+// When the next kernel of the stream may be placed (see pq_launch_pdl). Up to 32 tokens, when it is as small, at once. From 33 to 128 in a captured
+// graph, as a decode loop keeps one, when a cluster begins its reduction: us per pass, never / then, 8B linear set at 33 tokens 52.8 / 50.6, at 64
+// 60.0 / 57.9, W4A8 at 96 63.0 / 61.6, 70B at 40 113.9 / 112.0 (behind the K loop 51.3, 62.8, 63.7, 113.7). The same calls issued into a stream lose
+// by it (48 tokens 51.0 / 51.6, 120 74.5 / 75.8), as do larger ones (256 x 4096 x 4096 13.0 / 14.5).
+enum Early { NEVER, AT_ENTRY, AT_REDUCTION };
+
 struct SplitParams {
   const int32_t* zp;
   const int32_t* wsum;
@@ -80,7 +86,7 @@ struct SplitParams {
   int32_t* status;
   int64_t ldo;
   int M, N, K, n_kb;
-  int t_tiles, splits;
+  int t_tiles, splits, early;
   int vec_out;  // rows of out take 8-byte stores
   long long wait_clocks;
 };
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__(Cfg<NT, A8, WHOLE>::THREADS, Cfg<NT, A8, WHOLE
   const int kb0 = static_cast<int>(static_cast<int64_t>(p.n_kb) * rank / p.splits);
   const int total = static_cast<int>(static_cast<int64_t>(p.n_kb) * (rank + 1) / p.splits) - kb0;  // K blocks of this CTA
 
-  if (p.M <= 32) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next kernel is small, too (see pq_launch_pdl)
+  if (p.early == AT_ENTRY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const bool leader = pq::elect_one();  // the lane that issues copies and MMAs (each role's loop is warp-uniform)
   const int first = total < C::STAGES ? total : C::STAGES;
   if (warp == 0) {
@@ -509,6 +515,7 @@ __global__ void __launch_bounds__(Cfg<NT, A8, WHOLE>::THREADS, Cfg<NT, A8, WHOLE
     __syncthreads();
   }
   cluster_sync_all();  // every CTA's partial tile is in place
+  if (p.early == AT_REDUCTION) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (warp == 1) {
     pq::tc_fence_after();
     pq::tmem_dealloc(tmem_base, C::TMEM_COLS);
@@ -606,6 +613,9 @@ pq_status pq_gemm_split_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq
   p.M = static_cast<int>(M);
   p.N = static_cast<int>(N);
   p.K = static_cast<int>(K);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (M > 32 && M <= 128 && cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();  // (the launch says what is wrong with the stream)
+  p.early = M <= 32 ? AT_ENTRY : (capture == cudaStreamCaptureStatusActive ? AT_REDUCTION : NEVER);
   p.vec_out = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0;
   p.wait_clocks = ctx->wait_clocks;
   if (a8) return launch_tokens<true, false>(ctx, xq, wq, p, K, st);
