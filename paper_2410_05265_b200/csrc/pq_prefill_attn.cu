@@ -18,6 +18,11 @@
 // Inside every group of eight head dims the expansion leaves the order 0,4,1,5,2,6,3,7 (two codes per
 // instruction); Q and the prefix rows are stored in the same order (the contraction does not care) and the
 // output columns are put back when they are written. Every wait is bounded.
+//
+// KSPLIT (short prompts, whose 256-row CTAs fill less than half of the chip): a CTA has one 128-row tile, and S_0, O_0 and the first softmax
+// group take the even key tiles, S_1, O_1 and the second group the odd ones, each with a reference exponent of its own; at the end the two
+// groups put the halves together, 64 head dims each. K and V tiles are handed back separately, K as soon as its scores are done, so that
+// the expansion of the next K runs under the softmax. Bound by the chain of one key tile's softmax either way: half as many in sequence.
 #include <math.h>
 
 #include "pq_common.cuh"
@@ -39,7 +44,8 @@ constexpr float PA_LAZY = 8.0f;       // log2 units a score may exceed the runni
 
 struct PaBarriers {
   uint64_t land_full[PA_STAGES], land_empty[PA_STAGES];
-  uint64_t kv_full[PA_STAGES], kv_empty[PA_STAGES];
+  uint64_t kv_full[PA_STAGES], kv_empty[PA_STAGES];  // KSPLIT: of the V tiles
+  uint64_t k_full[PA_STAGES], k_empty[PA_STAGES];    // KSPLIT: of the K tiles
   uint64_t s_full[2], p_full[2], o_final[2];
   uint64_t q_ready, drain;
   uint32_t tmem_base;
@@ -193,7 +199,7 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // DYN (group-wise dynamic KV, Table 1 O1): every key's score and value row take the key's own step, read by the
 // softmax warps (all lanes the same address); the reference exponent is then the exact running maximum, so that
 // P * step stays inside fp16 for any step, and O is accumulated in value units.
-template <bool DYN>
+template <bool DYN, bool KSPLIT>
 __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const PrefillParams p) {
   extern __shared__ uint8_t pa_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pa_raw) + 1023) & ~uintptr_t(1023));
@@ -204,7 +210,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
 
   const int warp = pq::warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y, G = p.G;
-  const int R = 256 / G;                                   // query tokens of this CTA
+  const int R = (KSPLIT ? 128 : 256) / G;                  // query tokens of this CTA
   const int t0 = (static_cast<int>(gridDim.x) - 1 - static_cast<int>(blockIdx.x)) * R;  // long tiles first
   const int n_ctx = min(p.T, t0 + R);                      // cached keys any row of this CTA may see
   const int n_kt = (n_ctx + PA_KEYS - 1) / PA_KEYS;
@@ -218,6 +224,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
       pq::mbar_init(&bars->land_empty[i], PA_EXPAND_WARPS);
       pq::mbar_init(&bars->kv_full[i], PA_EXPAND_WARPS);
       pq::mbar_init(&bars->kv_empty[i], 1);
+      pq::mbar_init(&bars->k_full[i], PA_EXPAND_WARPS);
+      pq::mbar_init(&bars->k_empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
       pq::mbar_init(&bars->s_full[i], 1);
@@ -262,18 +270,19 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
   if (warp < PA_SOFTMAX_WARPS) {
     // ================================================================== softmax warps: one thread per query row
     const int i = warp >> 2, row = (warp & 3) * 32 + lane;      // Q tile and row inside it
-    const int r_cta = i * PA_ROWS + row;
+    const int r_cta = (KSPLIT ? 0 : i * PA_ROWS) + row;
     const int tok_raw = t0 + r_cta / G, head = h * G + r_cta % G;
     const int tok = min(tok_raw, p.T - 1);
     {
       // Q staging: the warp brings its 32 rows in, two rows (512 contiguous bytes) per load instruction; a thread per
       // row with 16-byte loads 256 bytes apart costs 32 tag look-ups per instruction and ~8000 clocks before the first MMA.
-      const uint32_t dst = pq::smem_u32(q_buf + i * PA_TILE);
-      const int c16 = lane & 15, lg = __ffs(G) - 1;
-      uint4 qv[16];
+      constexpr int LOADS = KSPLIT ? 8 : 16;  // KSPLIT: half of the warp's rows, the other group brings the other half
+      const uint32_t dst = pq::smem_u32(q_buf + (KSPLIT ? 0 : i * PA_TILE));
+      const int c16 = lane & 15, lg = __ffs(G) - 1, row0 = (warp & 3) * 32 + (KSPLIT ? i * 16 : 0);
+      uint4 qv[LOADS];
 #pragma unroll
-      for (int it = 0; it < 16; ++it) {
-        const int rq = i * PA_ROWS + (warp & 3) * 32 + it * 2 + (lane >> 4);
+      for (int it = 0; it < LOADS; ++it) {
+        const int rq = (KSPLIT ? 0 : i * PA_ROWS) + row0 + it * 2 + (lane >> 4);
         const int tq = min(t0 + (rq >> lg), p.T - 1), hq = h * G + (rq & (G - 1));  // G is a power of two
         const uint4* src = reinterpret_cast<const uint4*>(p.q + static_cast<int64_t>(tq) * p.ldq + hq * 128) + c16;  // eight bf16: dims 8 c16 .. +7
         asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];"  // volatile: the sixteen requests go out before the first use
@@ -281,12 +290,12 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
                      : "l"(src));
       }
 #pragma unroll
-      for (int it = 0; it < 16; ++it) {
+      for (int it = 0; it < LOADS; ++it) {
         const uint32_t w[4] = {qv[it].x, qv[it].y, qv[it].z, qv[it].w};
         float f[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float((e & 1) ? (w[e >> 1] & 0xFFFF0000u) : (w[e >> 1] << 16));
-        sts128(dst + tile_off((warp & 3) * 32 + it * 2 + (lane >> 4), c16),
+        sts128(dst + tile_off(row0 + it * 2 + (lane >> 4), c16),
                make_uint4(pack_h2(f[0], f[4]), pack_h2(f[1], f[5]), pack_h2(f[2], f[6]), pack_h2(f[3], f[7])));
       }
       pq::fence_proxy_async_smem();
@@ -300,13 +309,13 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
     constexpr float LAZY = DYN ? 0.0f : PA_LAZY;
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t s_addr = tmem_base + lane_base + i * 128, o_addr = tmem_base + lane_base + 256 + i * 128;
-    const int tile_min_tok = t0 + (i * PA_ROWS) / G;
+    const int tile_min_tok = t0 + (KSPLIT ? 0 : (i * PA_ROWS) / G);
     float m_ref = -INFINITY, l = 0.0f;
     bool ok = true;
-    for (int jt = 0; jt < n_tiles; ++jt) {
+    for (int jt = KSPLIT ? i : 0; jt < n_tiles; jt += KSPLIT ? 2 : 1) {
       const bool is_pre = has_prefix && jt == 0;
-      const int key0 = (jt - has_prefix) * PA_KEYS;
-      if (__any_sync(0xffffffffu, !wait(&bars->s_full[i], jt & 1))) {
+      const int key0 = (jt - has_prefix) * PA_KEYS, nth = KSPLIT ? jt >> 1 : jt;  // of this group's tiles
+      if (__any_sync(0xffffffffu, !wait(&bars->s_full[i], nth & 1))) {
         ok = false;
         break;
       }
@@ -350,7 +359,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
         const float m_new = grow ? mx_s : m_ref;
         const float alpha = grow ? ex2f(m_ref - m_new) : 1.0f;  // 2^(-inf) = 0 for a row that had seen nothing
         l *= alpha;
-        if (jt > 0) {  // S_i of this tile is complete, so O_i += P V of the tile before is, too
+        if (nth > 0) {  // S_i of this tile is complete, so O_i += P V of the tile before is, too
           for (int c = 0; c < 4; ++c) {
             uint32_t r[32];
             pq::tmem_ld_32x32(o_addr + c * 32, r);
@@ -406,15 +415,48 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
       __syncwarp();
       if (lane == 0) pq::mbar_arrive(&bars->p_full[i]);
     }
-    if (ok && __any_sync(0xffffffffu, !wait(&bars->o_final[i], 0))) ok = false;
+    float w_own = 1.0f, w_other = 0.0f;  // KSPLIT: this group's weight and the other's
+    bool other = false;
+    if (KSPLIT) {
+      float2* ml = reinterpret_cast<float2*>(q_buf + PA_TILE);  // [group][row]: the second Q tile is not used
+      ml[i * PA_ROWS + row] = make_float2(m_ref, l);
+      asm volatile("bar.sync 1, 256;" ::: "memory");  // the softmax warps, those that gave up among them
+      other = n_tiles > 1 || i == 1;  // with a single key tile the second group has nothing, not even zeros
+      const float2 o_ml = ml[(i ^ 1) * PA_ROWS + row];
+      const float m = fmaxf(m_ref, o_ml.x);
+      w_own = m_ref == -INFINITY ? 0.0f : ex2f(m_ref - m);
+      w_other = o_ml.x == -INFINITY ? 0.0f : ex2f(o_ml.x - m);
+      l = l * w_own + o_ml.y * w_other;
+      const bool mine_late = (i == 0 || n_tiles > 1) && __any_sync(0xffffffffu, !wait(&bars->o_final[i], 0));
+      const bool other_late = other && __any_sync(0xffffffffu, !wait(&bars->o_final[i ^ 1], 0));
+      if (mine_late || other_late) ok = false;
+    } else if (ok && __any_sync(0xffffffffu, !wait(&bars->o_final[i], 0))) {
+      ok = false;
+    }
     if (ok) {
       pq::tc_fence_after();
       const float norm = l > 0.0f ? sv / l : 0.0f;
+      const bool own = !KSPLIT || i == 0 || n_tiles > 1;
+      const uint32_t o_other = tmem_base + lane_base + 256 + (i ^ 1) * 128;
       __nv_bfloat16* dst = p.out + (static_cast<int64_t>(tok) * p.Hq + head) * 128;
-      for (int c = 0; c < 4; ++c) {
+      for (int c = KSPLIT ? 2 * i : 0; c < (KSPLIT ? 2 * i + 2 : 4); ++c) {
         uint32_t r[32];
-        pq::tmem_ld_32x32(o_addr + c * 32, r);
-        pq::tmem_ld_wait();
+        if (own) {
+          pq::tmem_ld_32x32(o_addr + c * 32, r);
+          pq::tmem_ld_wait();
+        }
+        if (KSPLIT) {
+          uint32_t r2[32];
+          if (other) {
+            pq::tmem_ld_32x32(o_other + c * 32, r2);
+            pq::tmem_ld_wait();
+          }
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            const float a = own ? __uint_as_float(r[e]) * w_own : 0.0f;
+            r[e] = __float_as_uint(other ? fmaf(__uint_as_float(r2[e]), w_other, a) : a);
+          }
+        }
         if (tok_raw < p.T) {
 #pragma unroll
           for (int a = 0; a < 4; ++a) {  // columns 8a .. 8a+7 hold dims 0,4,1,5,2,6,3,7 of the group
@@ -439,6 +481,48 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
     for (int jt = 0; jt < n_tiles && ok; ++jt) {
       const int stage = jt % PA_STAGES;
       const bool is_pre = has_prefix && jt == 0;
+      if constexpr (KSPLIT) {
+        const uint32_t k_tile = pq::smem_u32(kv_buf + stage * 2 * PA_TILE);
+        const int kt = jt - has_prefix, slot = kt & (PA_STAGES - 1);
+        const uint32_t src = pq::smem_u32(land + slot * PA_LAND);
+        if (!is_pre && __any_sync(0xffffffffu, !wait(&bars->land_full[slot], (kt / PA_STAGES) & 1))) {
+          ok = false;
+          break;
+        }
+#pragma unroll
+        for (int kv = 0; kv < 2 && ok; ++kv) {  // the K tile, then the V tile
+          if (__any_sync(0xffffffffu, !wait(kv ? &bars->kv_empty[stage] : &bars->k_empty[stage], ((jt / PA_STAGES) & 1) ^ 1))) {
+            ok = false;
+            break;
+          }
+          const uint32_t tile = k_tile + kv * PA_TILE;
+          if (is_pre) {
+            for (int unit = tid_e; unit < PA_MAX_PREFIX * 16; unit += PA_EXPAND_WARPS * 32) {
+              const int row = unit >> 4, c16 = unit & 15;
+              uint4 v = make_uint4(0, 0, 0, 0);
+              if (row < p.n_prefix)
+                v = permute8_h(__ldg(reinterpret_cast<const uint4*>((kv ? p.prefix_v : p.prefix_k) + (static_cast<int64_t>(h) * p.n_prefix + row) * 128 + c16 * 8)));
+              sts128(tile + tile_off(row, c16), v);
+            }
+          } else {
+#pragma unroll 2
+            for (int it = 0; it < PA_KEYS * 4 / (PA_EXPAND_WARPS * 32); ++it) {
+              const int unit = it * (PA_EXPAND_WARPS * 32) + tid_e, row = unit >> 2, part = unit & 3;
+              const uint4 w4 = lds128(src + kv * (PA_KEYS * 64) + unit * 16);
+              const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+              for (int w = 0; w < 4; ++w) sts128(tile + tile_off(row, 4 * part + w), expand8(ww[w]));
+            }
+          }
+          pq::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            pq::mbar_arrive(kv ? &bars->kv_full[stage] : &bars->k_full[stage]);
+            if (kv && !is_pre) pq::mbar_arrive(&bars->land_empty[slot]);
+          }
+        }
+        continue;
+      }
       if (__any_sync(0xffffffffu, !wait(&bars->kv_empty[stage], ((jt / PA_STAGES) & 1) ^ 1))) {
         ok = false;
         break;
@@ -517,7 +601,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
     const uint64_t v_desc0 = desc_sw128(pq::smem_u32(kv_buf + PA_TILE), PA_HALF);
     auto issue_s = [&](int i, int jt) {  // by the elected lane
       const uint32_t idesc = has_prefix && jt == 0 ? IDESC_S_PRE : IDESC_S;
-      const uint64_t q_desc = q_desc0 + i * (PA_TILE >> 4), k_desc = k_desc0 + (jt % PA_STAGES) * (2 * PA_TILE >> 4);
+      const uint64_t q_desc = q_desc0 + (KSPLIT ? 0 : i * (PA_TILE >> 4)), k_desc = k_desc0 + (jt % PA_STAGES) * (2 * PA_TILE >> 4);
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) {  // 16 head dims per instruction
         const uint32_t off = ((kk >> 2) * PA_HALF + (kk & 3) * 32) >> 4;
@@ -530,45 +614,75 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const Prefi
       const uint64_t v_desc = v_desc0 + (jt % PA_STAGES) * (2 * PA_TILE >> 4);
 #pragma unroll
       for (int kk = 0; kk < PA_MAX_PREFIX / 16; ++kk)  // 16 keys per instruction
-        mma_f16_ts(o_tm, p_tm + kk * 8, v_desc + kk * (2048 >> 4), IDESC_O, (jt > 0 || kk > 0) ? 1u : 0u);
+        mma_f16_ts(o_tm, p_tm + kk * 8, v_desc + kk * (2048 >> 4), IDESC_O, (jt > (KSPLIT ? 1 : 0) || kk > 0) ? 1u : 0u);
       if (!(has_prefix && jt == 0))
 #pragma unroll
         for (int kk = PA_MAX_PREFIX / 16; kk < PA_KEYS / 16; ++kk) mma_f16_ts(o_tm, p_tm + kk * 8, v_desc + kk * (2048 >> 4), IDESC_O, 1u);
     };
-    bool ok = wait_warp(&bars->q_ready, 0) && wait_warp(&bars->kv_full[0], 0);
-    if (ok) {
-      pq::tc_fence_after();
-      if (leader) {
-        issue_s(0, 0);
-        issue_s(1, 0);
-      }
-      __syncwarp();
-    }
-    for (int jt = 0; jt < n_tiles && ok; ++jt) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        if (!ok) break;
-        if (!wait_warp(&bars->p_full[i], jt & 1)) {
+    bool ok = wait_warp(&bars->q_ready, 0);
+    if constexpr (KSPLIT) {
+      auto scores = [&](int jt) {  // key tile jt into the columns of group jt & 1, once its K is there
+        if (!wait_warp(&bars->k_full[jt & 1], (jt >> 1) & 1)) return false;
+        pq::tc_fence_after();
+        if (leader) {
+          issue_s(jt & 1, jt);
+          pq::mma_commit(&bars->k_empty[jt & 1]);
+        }
+        __syncwarp();
+        return true;
+      };
+      ok = ok && scores(0) && (n_tiles < 2 || scores(1));
+      for (int jt = 0; jt < n_tiles && ok; ++jt) {
+        const int i = jt & 1, ph = (jt >> 1) & 1;
+        if (!wait_warp(&bars->p_full[i], ph) || !wait_warp(&bars->kv_full[i], ph)) {
           ok = false;
           break;
         }
         pq::tc_fence_after();
         if (leader) {
           issue_pv(i, jt);
-          if (i == 1) pq::mma_commit(&bars->kv_empty[jt % PA_STAGES]);  // both tiles' S and P V of this stage are issued
+          pq::mma_commit(&bars->kv_empty[i]);
+          if (jt + 2 >= n_tiles) pq::mma_commit(&bars->o_final[i]);
         }
         __syncwarp();
-        if (jt + 1 < n_tiles) {
-          if (i == 0 && !wait_warp(&bars->kv_full[(jt + 1) % PA_STAGES], ((jt + 1) / PA_STAGES) & 1)) {
+        if (jt + 2 < n_tiles) ok = scores(jt + 2);
+      }
+    } else {
+      ok = ok && wait_warp(&bars->kv_full[0], 0);
+      if (ok) {
+        pq::tc_fence_after();
+        if (leader) {
+          issue_s(0, 0);
+          issue_s(1, 0);
+        }
+        __syncwarp();
+      }
+      for (int jt = 0; jt < n_tiles && ok; ++jt) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (!ok) break;
+          if (!wait_warp(&bars->p_full[i], jt & 1)) {
             ok = false;
             break;
           }
           pq::tc_fence_after();
-          if (leader) issue_s(i, jt + 1);
-        } else if (leader) {
-          pq::mma_commit(&bars->o_final[i]);
+          if (leader) {
+            issue_pv(i, jt);
+            if (i == 1) pq::mma_commit(&bars->kv_empty[jt % PA_STAGES]);  // both tiles' S and P V of this stage are issued
+          }
+          __syncwarp();
+          if (jt + 1 < n_tiles) {
+            if (i == 0 && !wait_warp(&bars->kv_full[(jt + 1) % PA_STAGES], ((jt + 1) / PA_STAGES) & 1)) {
+              ok = false;
+              break;
+            }
+            pq::tc_fence_after();
+            if (leader) issue_s(i, jt + 1);
+          } else if (leader) {
+            pq::mma_commit(&bars->o_final[i]);
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
     }
     if (leader) {
@@ -629,16 +743,20 @@ extern "C" pq_status pq_prefill_attn_kv4_prefix(pq_ctx* ctx, const pq_kv4_cache*
   p.wait_clocks = ctx->wait_clocks;
   p.sm_scale = sm_scale;
   p.T = T, p.Hq = c->Hq, p.Hkv = c->Hkv, p.G = G, p.n_prefix = c->n_prefix, p.Tmax = c->Tmax;
-  static bool attr_set[64] = {};
+  // One 128-row tile per CTA while those CTAs still have an SM each. us, two row tiles / one, 32 query heads (8 KV heads): 17 tokens 8.3 / 7.6, 128 11.0 / 8.9,
+  // 256 13.0 / 10.3, 515 18.6 / 13.4, 700 (176 CTAs) 23.3 / 23.7, 1100 31.2 / 35.5; 64 heads: 256 13.4 / 11.0, 300 (152 CTAs) 16.2 / 17.1, 515 19.0 / 24.2.
+  // 8B block at 515 tokens 167.2 -> 162.5.
+  const bool ksplit = static_cast<int64_t>((T + 128 / G - 1) / (128 / G)) * c->Hkv <= ctx->sm_count;
+  const int form = (dyn ? 1 : 0) + (ksplit ? 2 : 0);
+  void (*const kerns[4])(const PrefillParams) = {prefill_attn_kernel<false, false>, prefill_attn_kernel<true, false>, prefill_attn_kernel<false, true>,
+                                                 prefill_attn_kernel<true, true>};
+  static bool attr_set[64][4] = {};
   if (ctx->device < 0 || ctx->device >= 64) return PQ_ERR_UNSUPPORTED;
-  if (!attr_set[ctx->device]) {
-    if (cudaFuncSetAttribute(prefill_attn_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(PA_SMEM_BYTES)) != cudaSuccess ||
-        cudaFuncSetAttribute(prefill_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(PA_SMEM_BYTES)) != cudaSuccess)
-      return PQ_ERR_CUDA;
-    attr_set[ctx->device] = true;
+  if (!attr_set[ctx->device][form]) {
+    if (cudaFuncSetAttribute(kerns[form], cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(PA_SMEM_BYTES)) != cudaSuccess) return PQ_ERR_CUDA;
+    attr_set[ctx->device][form] = true;
   }
-  const int R = 256 / G;
+  const int R = (ksplit ? 128 : 256) / G;
   dim3 grid((T + R - 1) / R, c->Hkv);
-  return pq_launch_pdl(dyn ? prefill_attn_kernel<true> : prefill_attn_kernel<false>, grid, PA_THREADS, PA_SMEM_BYTES,
-                       static_cast<cudaStream_t>(stream), p);
+  return pq_launch_pdl(kerns[form], grid, PA_THREADS, PA_SMEM_BYTES, static_cast<cudaStream_t>(stream), p);
 }
