@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(Cfg<NT, A8, WHOLE>::THREADS, Cfg<NT, A8, WHOLE
     }
     __syncthreads();
   }
-  cluster_sync_all();  // every CTA's partial tile is in place
+  if (p.splits > 1) cluster_sync_all();  // every CTA's partial tile is in place (28672 x 4096, one split: 0.5 us)
   if (p.early == AT_REDUCTION) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (warp == 1) {
     pq::tc_fence_after();
@@ -528,9 +528,11 @@ __global__ void __launch_bounds__(Cfg<NT, A8, WHOLE>::THREADS, Cfg<NT, A8, WHOLE
   else reduce_tile<MAX_SPLIT, 1, ZP>(p, smem, t0, n0, tokens, rank + p.splits * warp, p.splits * (C::THREADS / 32), lane, sw, zw);
   // no CTA leaves while a peer may still read its partial tile; relaxed: the reads are done, and the output stores need not
   // have reached memory
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (p.splits > 1) {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  }
 }
 
 template <int NT, bool A8, bool ZP, bool WHOLE>
