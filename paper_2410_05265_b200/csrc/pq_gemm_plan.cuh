@@ -231,6 +231,19 @@ inline int split_count(int tiles, int K, int slots) {
   return splits < 1 ? 1 : splits;
 }
 
+// The forms of which two CTAs share an SM. Above 64 tokens the partial tiles are large, and an SM's two CTAs exchange theirs at the same
+// time: one CTA to an SM and fewer splits, of at least 1280 elements of K, win with a short K, and with 8-bit tokens above 88 while that leaves four
+// splits. us with the rotation, two to an SM / one: W4A8 at 96 tokens 6144 x 4096 five splits 11.9 / two 10.0, 4096 x 4096 six 11.2 / three 9.6, 4096 x 14336
+// eight 16.6 / four 14.4 (at 80 15.5 / 16.3), but 8192 x 8192 four 15.7 / two 16.3, 8192 x 28672 four 30.6 / two 36.4; 4-bit 4096 x 4096 at 96 11.9 / 10.6,
+// at 128 six 13.4 / three 11.9 (four 13.7), 6144 x 4096 at 96 12.9 / 13.3, at 128 15.2 / 13.8, 4096 x 14336 at 80 18.0 / 20.2; at 64 tokens 4096 x 14336
+// eight 15.3 / four 17.6.
+inline int split_count_pairs(int tiles, int K, int sm_count, int M, bool a8) {
+  const int two = split_count(tiles, K, 2 * sm_count), one = sm_count * 9 / 10 / tiles, most = K / (10 * BK);
+  const bool short_k = K <= 16 * BK * one;
+  const bool fewer = M > 64 && two * tiles > sm_count && one >= 2 && (short_k ? a8 || M > 96 || one >= 4 : a8 && M > 88 && one >= 4);
+  return fewer && most >= 1 ? (one < most ? one : most) : two;
+}
+
 // The width of the token tiles up to 128 tokens.
 inline int split_width(int M) { return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 48 ? 48 : (M <= 64 ? 64 : (M <= 96 ? 96 : 128)))); }
 

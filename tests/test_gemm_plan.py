@@ -193,3 +193,21 @@ def test_narrow_forms_that_take_an_sm_alone_share_it_with_no_other():
 ])
 def test_width_above_128_tokens(M, N, K, a8, want):
     assert gp.width_whole(M, N, K, a8) == want
+
+
+@pytest.mark.parametrize("tiles,K,M,a8,want", [
+    (32, 4096, 64, False, 6), (32, 4096, 65, False, 3), (32, 14336, 128, False, 8), (32, 14336, 88, True, 8), (32, 14336, 89, True, 4),
+    (48, 4096, 96, False, 5), (48, 4096, 97, False, 2), (48, 4096, 66, True, 2), (64, 8192, 96, True, 4), (80, 8192, 128, True, 3), (8, 8192, 128, True, 8),
+    (1, 32, 100, True, 1), (224, 4096, 100, True, 1), (3, 640, 128, False, 1), (20, 1408, 100, True, 2),
+])
+def test_k_splits_of_two_ctas_to_an_sm(tiles, K, M, a8, want):
+    assert gp.splits_pairs(tiles, K, M, a8) == want
+
+
+def test_every_split_has_k_blocks_and_a_place():
+    for tiles in list(range(1, 40)) + [48, 64, 80, 131, 148, 149, 224, 296, 448]:
+        for K in (32, 96, 640, 1280, 1408, 4096, 8192, 14336, 28672):
+            for M in (17, 64, 65, 88, 89, 96, 97, 128):
+                for a8 in (False, True):
+                    s = gp.splits_pairs(tiles, K, M, a8)
+                    assert 1 <= s <= 8 and (s == 1 or (K >= 640 * s and tiles * s <= 2 * 148 * 7 // 8))
