@@ -771,7 +771,13 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
 //   14336 (seven blocks)     M = 1 2.02 / 1.58, 33 2.21 / 1.95, 96 3.36 / 3.42; with SwiGLU 2.72 / 1.82, 2.98 / 2.39, 96 5.02 / 3.75, 148 4.77 / 4.64
 // so the line lies at one block of 4096 to an SM, two of 2048, five with SwiGLU. Blocks of 8192 (16 warps, five shuffle stages) stay with the
 // wide kernel: 2.28 / 2.85. Decode layer at 1021 tokens 53.8 -> 51.5.
-constexpr int hq_small_blocks_per_sm(int logb, bool swiglu) { return logb == 11 ? (swiglu ? 5 : 2) : (logb == 12 ? 1 : 0); }
+// One step per token and blocks of 4096: up to four of them. Behind a split-K GEMM of up to 32 tokens, which triggers at once, this kernel fits beside
+// that GEMM's CTAs and lets the next ones in among them; us with the GEMM, wide kernel / this one: 6144 x 4096 at 4 rows 5.8 / 5.6, 14 7.6 / 8.2, 24
+// 7.9 / 8.8, 32 8.3 / 9.3, 64 11.1 / 11.1, 4096 x 4096 at 1 row 5.3 / 4.9, 8 6.0 / 6.2, 32 7.9 / 8.9, but 28672 x 4096 at 24 16.2 / 15.8. 8B linear set at 24
+// tokens 47.2 / 48.9.
+constexpr int hq_small_blocks(int logb, bool swiglu, bool per_token, int sm_count) {
+  return logb == 11 ? (swiglu ? 5 : 2) * sm_count : (logb == 12 ? (per_token ? 4 : sm_count) : 0);
+}
 
 template <int LOGB, int BITS, bool PER_TOKEN, bool ZP, bool SWIGLU, int NORM>
 __global__ void __launch_bounds__(1 << (LOGB - 4))
@@ -953,9 +959,9 @@ pq_status launch(pq_ctx* ctx, const void* x, int64_t ldx, int64_t n_rows, int64_
   } else {
     kern = hadamard_quant_kernel<LOGB, ROTATE, CALIB, BITS, PER_TOKEN, ZP, SWIGLU, GRID, NORM>;
   }
-  if constexpr (WIDE && !CALIB && !GRID && hq_small_blocks_per_sm(LOGB, SWIGLU) > 0) {
+  if constexpr (WIDE && !CALIB && !GRID && LOGB <= 12) {
     const int64_t blocks = n_rows * (K / B);
-    if (blocks <= static_cast<int64_t>(hq_small_blocks_per_sm(LOGB, SWIGLU)) * ctx->sm_count)
+    if (blocks <= hq_small_blocks(LOGB, SWIGLU, PER_TOKEN, ctx->sm_count))
       return pq_launch_pdl(hadamard_quant_small_kernel<LOGB, BITS, PER_TOKEN, ZP, SWIGLU, NORM>, dim3(static_cast<unsigned>(blocks)), B / 16, 0, st,
                            static_cast<const __nv_bfloat16*>(x), ldx, K, s_a_in, xq, s_a_out, clip, zp_in, static_cast<const __nv_bfloat16*>(x2), n_cand);
   }

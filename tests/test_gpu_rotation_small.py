@@ -1,5 +1,6 @@
 """Rotation kernel of calls with few wide blocks (16 elements to a thread, a block to a CTA): the codes, steps and normalised rows of the kernel for
-many blocks bit for bit, at the borders of the rule between the two (one block of 4096 to an SM, two of 2048, five with SwiGLU), for every form."""
+many blocks bit for bit, at the borders of the rule between the two (one block of 4096 to an SM, four in all with a step per token, two of 2048 to an SM,
+five with SwiGLU), for every form."""
 import pytest
 import torch
 
@@ -34,7 +35,8 @@ def test_same_codes_as_the_kernel_for_many_blocks(ctx, form, K, block, per_sm, w
     if form == "dynamic" and K != block:
         pytest.skip("rows of several blocks have a kernel of their own")
     per_row = K // block
-    M = row_begin + {"one": 1, "last": per_sm * sms() // per_row, "beyond": per_sm * sms() // per_row + 1}[where]
+    most = 4 if block == 4096 and form in ("rows", "dynamic") else per_sm * sms()
+    M = row_begin + {"one": 1, "last": most // per_row, "beyond": most // per_row + 1}[where]
     x = rows(row_begin + per_sm * sms() // per_row + 40, K, pitch)  # enough rows for the other kernel
     s, z = torch.full((1,), 0.37, device="cuda"), torch.full((1,), 6, dtype=torch.int32, device="cuda")
     s_tok = torch.rand(x.shape[0], device="cuda") + 0.1
