@@ -790,7 +790,7 @@ __global__ void __launch_bounds__(1 << (LOGB - 4))
   constexpr int T0S = 1, T1S = J == 2 ? 2 : 6, GS = J + 1, WS = J + 4;  // the index bits' roles are those of the wide kernel
   constexpr int M3S = 8 - J, K3S = 9 - J, TAUS = 10 - J;
   constexpr int PADK = J == 2 ? 4 : 20, BLKF = J == 2 ? 2176 : 4736;
-  __shared__ __align__(16) float my[NORM == 2 ? 1 : BLKF];
+  __shared__ __align__(16) float my[NORM == 2 ? B / 2 : BLKF];
   __shared__ float red[WARPS];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -827,21 +827,28 @@ __global__ void __launch_bounds__(1 << (LOGB - 4))
 #pragma unroll
       for (int v = 0; v < 4; ++v) w[i][v] = pack_bf16x2(pq::silu_mul_f32(bf16_pair(w[i][v]), bf16_pair(u[i][v])));
   } else if (NORM) {
-    float ss = 0.0f;  // in an order of its own, shared by the stand-alone RMSNorm, which takes this kernel for the same calls
+    // The sum of squares in the wide kernel's order, so that a row's values depend neither on the number of rows nor on which call forms them:
+    // the four warps that share a wide-kernel warp's words put them together, and each adds up all of them.
+    uint4* words = reinterpret_cast<uint4*>(my) + (wv * 8) * 32 + lane;  // [wv][tau][lane]
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 2; ++i) words[(2 * tp + i) * 32] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+    __syncthreads();
+    float ss = 0.0f;
+#pragma unroll
+    for (int tau = 0; tau < 8; ++tau) {
+      const uint4 q = words[tau * 32];
+      const uint32_t all[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        const float2 a = bf16_pair(w[i][v]);
+        const float2 a = bf16_pair(all[v]);
         ss = __fmaf_rn(a.x, a.x, __fmaf_rn(a.y, a.y, ss));
       }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) red[warp] = ss;
-    __syncthreads();
-    ss = 0.0f;
-#pragma unroll
-    for (int i = 0; i < WARPS; ++i) ss += red[i];
+    if (J == 1 && lane == 0 && tp == 0) red[wv] = ss;
+    if (J == 1 || NORM != 2) __syncthreads();  // (the exchange below writes where the words are)
+    if (J == 1) ss = 0.0f + red[0] + red[1];
     const float rr = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(ss, static_cast<float>(B)), clip)));
 #pragma unroll
     for (int i = 0; i < 2; ++i)

@@ -86,3 +86,21 @@ def test_rmsnorm_fused_and_alone_agree_on_both_sides_of_the_rule(ctx, K, per_sm,
     want = xd / torch.sqrt((xd * xd).mean(1, keepdim=True) + 1e-5) * g.double()
     # one bf16 rounding of a value that fp32 sums of K squares give within K/512 * 2^-24: half an ulp and a little
     assert bool(((h.double() - want).abs() <= want.abs() * (2.0**-8 + 2.0**-16) + 1e-30).all())
+
+
+@pytest.mark.parametrize("K,per_sm", [(4096, 1), (2048, 2)])
+@pytest.mark.parametrize("row_begin", [0, 4])
+def test_a_normalised_row_does_not_depend_on_the_rows_beside_it(ctx, K, per_sm, row_begin):
+    """Few rows, as many as the kernel of few blocks takes, and two more: the same values, and the fused call the codes of the two
+    calls also where row_begin leaves it on one side of the rule and the stand-alone call, which has none, on the other."""
+    most = per_sm * sms()
+    g = rows(1, K, seed=1)[0].contiguous()
+    s = torch.full((1,), 0.5, device="cuda")
+    for seed in range(8):  # two orders of the sum differ in some five of a million bf16 values
+        x = rows(most + 2, K, seed=seed)
+        many = ctx.rmsnorm(x, g, 1e-5)
+        for M in (3, most):
+            assert torch.equal(ctx.rmsnorm(x[:M], g, 1e-5), many[:M])
+        fused, two = ctx.rmsnorm_hadamard_quant_act(x, g, 1e-5, s, row_begin), ctx.hadamard_quant_act(many, K, s, row_begin)
+        assert torch.equal(fused[row_begin:], two[row_begin:])
+    ctx.check()
