@@ -87,6 +87,11 @@ __device__ __forceinline__ uint32_t ld_dep(const uint32_t* p) {
 }
 __device__ __forceinline__ float ld_dep(const float* p) { return __uint_as_float(ld_dep(reinterpret_cast<const uint32_t*>(p))); }
 __device__ __forceinline__ int32_t ld_dep(const int32_t* p) { return static_cast<int32_t>(ld_dep(reinterpret_cast<const uint32_t*>(p))); }
+__device__ __forceinline__ uint2 ld_dep(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.global.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
 __device__ __forceinline__ uint4 ld_dep(const uint4* p) {
   uint4 v;
   asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));

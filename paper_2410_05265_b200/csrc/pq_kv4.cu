@@ -315,17 +315,19 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
 #pragma unroll
     for (int w = 0; w < 4; ++w) q_raw[w] = row_ok ? pq::ld_dep(q4 + w) : make_uint4(0, 0, 0, 0);
   };
+  // What the one-launch step reads ahead of the wait, through the read-only path; the plain call behind it, in order (see ld_dep).
+  auto ld_cache = [](auto* ptr) { return FUSED ? __ldg(ptr) : pq::ld_dep(ptr); };
   if (!FUSED) load_q();
   // the fused kernel writes the lengths at its end: it reads them past the read-only path
-  int len_b = FUSED ? __ldcg(p.len + b) : __ldg(p.len + b);
-  const float s_k_h = DYN ? 1.0f : __ldg(p.s_k + h), s_v_h = DYN ? 1.0f : __ldg(p.s_v + h);
+  int len_b = FUSED ? __ldcg(p.len + b) : pq::ld_dep(p.len + b);
+  const float s_k_h = DYN ? 1.0f : ld_cache(p.s_k + h), s_v_h = DYN ? 1.0f : ld_cache(p.s_v + h);
   // prefix values of the four head dims this thread merges after the key loop, so that the merge does
   // not wait for them (keys past the fourth are read there)
   uint2 pv_early[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j)
     pv_early[j] = (has_prefix && j < p.n_prefix)
-                      ? __ldg(reinterpret_cast<const uint2*>(p.prefix_v + (static_cast<int64_t>(h) * p.n_prefix + j) * 128) + lane)
+                      ? ld_cache(reinterpret_cast<const uint2*>(p.prefix_v + (static_cast<int64_t>(h) * p.n_prefix + j) * 128) + lane)
                       : make_uint2(0u, 0u);
 
   const bool has_extra = FUSED && split == S - 1;
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
     const uint4* qr = reinterpret_cast<const uint4*>(p.q + (static_cast<int64_t>(b) * p.Hq + h * G + r) * 128 + 16 * sub);
     const uint4* kr = reinterpret_cast<const uint4*>(p.prefix_k + (static_cast<int64_t>(h) * p.n_prefix + j) * 128 + 16 * sub);
     if (want_q) pre_q[0] = pq::ld_dep(qr), pre_q[1] = pq::ld_dep(qr + 1);
-    if (want_k) pre_k[0] = __ldg(kr), pre_k[1] = __ldg(kr + 1);
+    if (want_k) pre_k[0] = ld_cache(kr), pre_k[1] = ld_cache(kr + 1);
   };
   load_pre(!FUSED, true);
 
@@ -435,7 +437,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
       const uint4* kr = reinterpret_cast<const uint4*>(p.prefix_k + (static_cast<int64_t>(h) * p.n_prefix + j) * 128 + 16 * sub);
       const bool early = pair0 == 0;
       const uint4 qv[2] = {early ? pre_q[0] : pq::ld_dep(qr), early ? pre_q[1] : pq::ld_dep(qr + 1)};
-      const uint4 kv[2] = {early ? pre_k[0] : __ldg(kr), early ? pre_k[1] : __ldg(kr + 1)};
+      const uint4 kv[2] = {early ? pre_k[0] : ld_cache(kr), early ? pre_k[1] : ld_cache(kr + 1)};
       float acc = 0.0f;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -543,8 +545,8 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
   auto load_steps = [&](int r) {  // lane i: key i % 16 of block i / 16 of the two blocks this warp takes of round r
     const int j = round_key0(r) + (lane >> 4) * DA_CHUNK + 16 * warp + (lane & 15);
     const bool in = r < n_rounds && j < t1;
-    sk_next = in ? __ldg(skb + j) : 0.0f;
-    sv_next = in ? __ldg(svb + j) : 0.0f;
+    sk_next = in ? pq::ld_dep(skb + j) : 0.0f;
+    sv_next = in ? pq::ld_dep(svb + j) : 0.0f;
   };
   if (DYN) load_steps(0);
 
@@ -793,7 +795,7 @@ __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(co
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj)
           if (j == jj) pv = pv_early[jj];
-        if (j >= 4) pv = __ldg(reinterpret_cast<const uint2*>(p.prefix_v + (static_cast<int64_t>(h) * p.n_prefix + j) * 128) + c4);
+        if (j >= 4) pv = ld_cache(reinterpret_cast<const uint2*>(p.prefix_v + (static_cast<int64_t>(h) * p.n_prefix + j) * 128) + c4);
         const float2 v01 = __half22float2(*reinterpret_cast<const __half2*>(&pv.x));
         const float2 v23 = __half22float2(*reinterpret_cast<const __half2*>(&pv.y));
         acc.x = fmaf(e, v01.x, acc.x), acc.y = fmaf(e, v01.y, acc.y), acc.z = fmaf(e, v23.x, acc.z), acc.w = fmaf(e, v23.y, acc.w);

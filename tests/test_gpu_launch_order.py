@@ -245,3 +245,60 @@ def test_query_and_token_written_just_before_reach_the_decode_step(ctx, T):
         for w, r in zip(want, run(call)):
             assert all(torch.equal(p, q) for p, q in zip(w, r))
     ctx.check()
+
+
+@pytest.mark.parametrize("dyn", [False, True])
+@pytest.mark.parametrize("B,Tmax", [(1, 256), (8, 256), (1, 9000)])
+def test_plain_decode_attention_straight_behind_the_append(ctx, dyn, B, Tmax):
+    """residual add (writes the step's k and v) -> append -> plain decode attention -> residual add over its output, in a graph and called
+    back to back, against the calls apart: lengths, cache rows and (with steps per vector) the steps are the ones just written. One
+    cluster per (sequence, head) pair and, in the long cache, several."""
+    from paper_2410_05265_b200 import binding
+
+    Hq, Hkv, P, T0 = 8, 2, 4, 130
+    g = torch.Generator(device="cuda").manual_seed(B + Tmax)
+    rand = lambda *sh: torch.randn(sh, generator=g, device="cuda").to(torch.bfloat16)
+    pk, pv = rand(Hkv, P, D).half(), rand(Hkv, P, D).half()
+    codes = torch.randint(0, 256, (2, B, Hkv, Tmax, D // 2), dtype=torch.uint8, device="cuda", generator=g)
+    s = torch.full((Hkv,), 0.3, device="cuda")
+    steps = dict(sk_tok=torch.full((B, Hkv, Tmax), 0.3, device="cuda"), sv_tok=torch.full((B, Hkv, Tmax), 0.2, device="cuda")) if dyn else {}
+    cache = binding.KV4Cache(pk, pv, codes[0], codes[1], None if dyn else s, None if dyn else s, torch.zeros(B, dtype=torch.int32, device="cuda"), Hq, **steps)
+    ws = ctx.decode_attn_workspace(cache)
+    n = B * Hkv * D
+    base, kv, new = rand(2 * n), torch.zeros(2 * n, dtype=torch.bfloat16, device="cuda"), torch.zeros(2 * n, dtype=torch.bfloat16, device="cuda")
+    q, out, after = rand(B, Hq, D), rand(B, Hq, D), rand(B, Hq, D)
+    inputs_ = [rand(2 * n) * 2.0**i for i in range(4)]
+
+    def chain(step):
+        for _ in range(3):
+            ctx.residual_add(kv, base, out=new)
+            step()
+            ctx.kv4_append(cache, new[:n].view(B, 1, Hkv, D), new[n:].view(B, 1, Hkv, D))
+            step()
+            ctx.decode_attn(cache, q, 1 / math.sqrt(D), ws, out=out)
+            step()
+            ctx.residual_add(out, q, out=after)
+            step()
+            ctx.residual_add(new, base, out=kv)
+            step()
+
+    def run(call):
+        res = []
+        for v in inputs_:
+            kv.copy_(v)
+            cache.length.fill_(T0)
+            torch.cuda.synchronize()
+            call()
+            torch.cuda.synchronize()
+            res.append([t.clone() for t in (out, after, cache.kq, cache.vq, cache.length, *steps.values())])
+        return res
+
+    want = run(lambda: chain(torch.cuda.synchronize))
+    assert int(want[0][4][0]) == T0 + 3
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(lambda: None)
+    for call in (graph.replay, lambda: chain(lambda: None)):
+        for w, r in zip(want, run(call)):
+            assert all(torch.equal(a, b) for a, b in zip(w, r))
+    ctx.check()

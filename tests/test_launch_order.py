@@ -65,11 +65,22 @@ def test_what_a_predecessor_may_write_is_not_read_through_the_read_only_path(sou
             text = f.read()
         body += block_from(text, text.index("void reduce_tile("))
     static = re.compile(r"s_w|wsum|gsrc|\bgr\b|s_k|s_v|p\.len|prefix_|\bkr\b|skb|svb")
+    if name == "decode_attn_kernel":  # one helper, which reads so in the one-launch step only
+        static = re.compile(r"^ptr$")
     read_only = re.findall(r"__ldg\(((?:[^()]|\([^()]*\))*)\)", body) + re.findall(r'"ld\.global\.nc[^"]*"[^;]*"l"\((\w+)\)', body)
     wrong = [a for a in read_only if not static.search(a)]
     assert not wrong, wrong
     if name.startswith("hadamard"):  # its parameters are const __restrict__: no plain load through them either
         assert not re.search(r"\b(?:x|x2|s_a_in|zp_in)\[", body)
+
+
+def test_the_plain_decode_attention_reads_nothing_through_the_read_only_path():
+    """The header promises that it waits before it reads anything: a read-only load may be moved ahead of the wait. The one-launch step may."""
+    body = kernel_body("pq_kv4.cu", "decode_attn_kernel")
+    assert re.findall(r"(FUSED \? )?__ldg\(", body) == ["FUSED ? "]
+    for step in ("skb", "svb"):  # (the one-launch step has no steps per vector)
+        assert len(re.findall(r"%s \+" % step, body)) == len(re.findall(r"ld_dep\(%s \+" % step, body)) == 1
+    assert "FUSED ? __ldcg(p.len + b) : pq::ld_dep(p.len + b)" in body
 
 
 @pytest.mark.parametrize("source,name", [("pq_gemm_tc2.cu", "gemm_w4a4_pair_kernel"), ("pq_gemm_tc3.cu", "gemm_w4a4_pair_ts_kernel")])
