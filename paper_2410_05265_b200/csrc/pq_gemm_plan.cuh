@@ -188,7 +188,7 @@ struct SplitCfg {
   static constexpr int GROUPS = WHOLE ? 4 : 2;
   static constexpr int SLOTS = !WHOLE && (KB == 256 || (NT == 128 && !A8)) ? 2 : 4;
   static constexpr int W_STAGE = CH * ROWB;
-  static constexpr int STAGES = WHOLE ? (NT <= 128 ? 8 : 4) : KB == 128 ? 4 : (NT <= (A8 ? 32 : 16) ? 6 : (NT <= (A8 ? 96 : 48) ? 4 : 3));  // landing ring, weights
+  static constexpr int STAGES = WHOLE ? (NT <= 128 ? 8 : 4) : KB == 128 ? 4 : (NT <= 16 ? 6 : (NT <= (A8 ? 96 : 48) ? 4 : 3));  // landing ring, weights
   static constexpr int X_STAGES = !WHOLE && KB == 256 && NT > 48 ? 3 : 4;                                               // landing ring, tokens
   static constexpr bool TOGETHER = KB == 256;  // weights and tokens of a K block are waited for together
   static constexpr bool SLOT_FIRST = STAGES % GROUPS != 0 || (!A8 && X_STAGES % GROUPS != 0);
@@ -213,9 +213,14 @@ struct SplitCfg {
 // At least 80 KB for 256 columns of tensor memory and 160 KB for 512, so that no more CTAs share an SM (228 KB) than its tensor memory
 // serves, those of other launches included: a CTA that waited for columns which another cluster's CTA gives back only behind its
 // cluster barrier could wait for itself. (8-bit tokens 192 wide need 130 KB, which leave room for a CTA of a narrow form.)
+// From 33 to 96 tokens half of an SM's shared memory, also where the rings need less: otherwise CTAs of the next rotation find room beside two of these,
+// and let the launch behind them in among the running ones, on whichever SMs have room. us, rotation and GEMM in a graph, rings alone / half: 8-bit
+// tokens 56 x 6120 x 3456 13.2 / 10.6, 50 x 9248 x 1280 9.3 / 8.0, 59 x 6320 x 3712 13.3 / 11.5, 62 x 4584 x 2944 11.4 / 10.3; linear sets equal. Up to
+// 32 tokens it is a toss-up (4-bit 24 x 2816 x 14720 13.5 / 12.0, 28 x 4440 x 7680 10.3 / 12.6) and at 128 a loss (97 to 128 tokens 1.5 % in the mean of 58 shapes).
+// Nor more than the rings of 8-bit tokens 32 wide hold now, 80 KB: with six weight stages, 112 KB, 24 x 4608 x 6912 went 10.6 -> 12.8 us, and no shape gained.
 template <int NT, bool A8, bool WHOLE = (NT > 128)>
 constexpr size_t split_smem() {
-  const size_t need = SplitCfg<NT, A8, WHOLE>::RING + SPLIT_BAR_BYTES, least = SplitCfg<NT, A8, WHOLE>::TMEM_COLS / 256 * (80 * 1024);
+  const size_t need = SplitCfg<NT, A8, WHOLE>::RING + SPLIT_BAR_BYTES, least = WHOLE ? 160 * 1024 : (NT > 32 && NT < 128 ? 113 : 80) * 1024;
   return need < least ? least : need;
 }
 

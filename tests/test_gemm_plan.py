@@ -181,6 +181,13 @@ def test_ctas_that_fit_one_sm_find_their_tensor_memory():
                     assert sum(cols for _, _, cols, _ in group) <= 512, group
 
 
+def test_two_ctas_of_33_to_96_tokens_leave_no_room_for_a_rotation():
+    """16 elements to a thread keep 2176 floats of shared memory at the least."""
+    for nt, _, _, smem in gp.split_shapes():
+        if 32 < nt < 128:
+            assert 0 <= 228 * 1024 - 2 * (smem + 1024) < 2176 * 4
+
+
 def test_narrow_forms_that_take_an_sm_alone_share_it_with_no_other():
     for a in gp.whole_shapes():
         for b in gp.whole_shapes() + gp.split_shapes():
