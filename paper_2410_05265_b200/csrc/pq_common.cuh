@@ -38,7 +38,7 @@ static inline pq_status pq_launch_status() { return cudaGetLastError() == cudaSu
 // Who lets its successor be placed EARLY is decided by the successor's size. CTAs placed while the predecessor still runs land on
 // the SMs that happen to have room, four to an SM, instead of being spread over the chip; that costs more than the hidden
 // launch. So the rotation kernels (the GEMM behind them takes whole SMs, or prefetches its weights), the decode kernels and the
-// small kernels of small grids trigger early; the CTA-pair GEMMs, the split-K GEMM above 32 tokens (in a captured graph above 128) and the
+// small kernels of small grids trigger early; the CTA-pair GEMMs, the split-K GEMM above 32 tokens (in a captured graph above 96) and the
 // kernels of larger grids do not, and their successor starts when they end without a launch gap. Measured on whole passes (us, before the rule,
 // when the GEMMs always triggered and the element-wise kernels were launched plainly / with it): 8B linear set at 2044 tokens
 // 395 / 376, per-token set at 1000 253 / 243, W4A8 set at 300 137 / 129; 8B block at 515 tokens 243 / 228, at 1500 418 / 398,

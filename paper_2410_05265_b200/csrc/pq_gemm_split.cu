@@ -69,10 +69,15 @@ struct __align__(8) SplitBarriers {
 
 static_assert(sizeof(SplitBarriers) <= SPLIT_BAR_BYTES, "shared memory budget");
 
-// When the next kernel of the stream may be placed (see pq_launch_pdl). Up to 32 tokens, when it is as small, at once. From 33 to 128 in a captured
-// graph, as a decode loop keeps one, when a cluster begins its reduction: us per pass, never / then, 8B linear set at 33 tokens 52.8 / 50.6, at 64
-// 60.0 / 57.9, W4A8 at 96 63.0 / 61.6, 70B at 40 113.9 / 112.0 (behind the K loop 51.3, 62.8, 63.7, 113.7). The same calls issued into a stream lose
-// by it (48 tokens 51.0 / 51.6, 120 74.5 / 75.8), as do larger ones (256 x 4096 x 4096 13.0 / 14.5).
+// When the next kernel of the stream may be placed (see pq_launch_pdl). Up to 32 tokens, when it is as small, at once. From 33 to 96 in a captured
+// graph, as a decode loop keeps one, when a cluster begins its reduction, and up to 128 with a step per token. us per pass, never / then, 8B linear set:
+//   4-bit    33 tokens 52.6 / 50.3, 48 54.2 / 51.9, 64 59.9 / 58.0, 96 72.8 / 70.9, 112 76.5 / 77.7, 128 77.6 / 79.2
+//   8-bit    33 50.0 / 48.3, 64 56.2 / 53.3, 80 60.5 / 57.9, 112 64.6 / 66.2, 128 65.5 / 67.7
+//   per token 33 57.4 / 55.1, 64 61.9 / 60.1, 112 81.2 / 79.7, 128 82.4 / 81.5;    70B set, 4-bit, 33 111.3 / 109.1, 96 158.2 / 156.5, 128 161.7 / 162.1
+// (behind the K loop 51.3 at 33, 62.8 at 64.) A chain of one shape does not always gain: of 163 shapes of 33 to 96 tokens the mean is 0.989, but 4096 x 14336 with steps
+// per token, whose quantizer takes a CTA a row, goes 20.5 / 16.8 at 49 tokens, 15.5 / 17.4 at 53 to 64 and 18.3 / 19.6 at 80. Above 96 tokens
+// 127 x 2816 x 14720 goes 20.0 / 22.3. Calls issued into a stream lose by it (8B set with steps per token at 33 tokens 54.5 / 56.4, 70B set at 33
+// 106.8 / 109.3), as do larger ones (256 x 4096 x 4096 13.0 / 14.5): so they ask whether the stream is being captured.
 enum Early { NEVER, AT_ENTRY, AT_REDUCTION };
 
 struct SplitParams {
@@ -615,9 +620,12 @@ pq_status pq_gemm_split_launch(pq_ctx* ctx, const uint8_t* xq, const uint8_t* wq
   p.M = static_cast<int>(M);
   p.N = static_cast<int>(N);
   p.K = static_cast<int>(K);
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (M > 32 && M <= 128 && cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();  // (the launch says what is wrong with the stream)
-  p.early = M <= 32 ? AT_ENTRY : (capture == cudaStreamCaptureStatusActive ? AT_REDUCTION : NEVER);
+  p.early = M <= 32 ? AT_ENTRY : NEVER;
+  if (M > 32 && M <= (s_row ? 128 : 96)) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();  // (the launch says what is wrong with the stream)
+    if (capture == cudaStreamCaptureStatusActive) p.early = AT_REDUCTION;
+  }
   p.vec_out = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0;
   p.wait_clocks = ctx->wait_clocks;
   if (a8) return launch_tokens<true, false>(ctx, xq, wq, p, K, st);

@@ -302,3 +302,75 @@ def test_plain_decode_attention_straight_behind_the_append(ctx, dyn, B, Tmax):
         for w, r in zip(want, run(call)):
             assert all(torch.equal(a, b) for a, b in zip(w, r))
     ctx.check()
+
+
+@pytest.mark.parametrize("mode", ["w4a4", "w4a8", "rows", "asym"])
+@pytest.mark.parametrize("M", [33, 64, 96, 97, 128])
+@pytest.mark.parametrize("N", [4096, 28672])
+def test_what_follows_a_captured_gemm_reads_its_output_and_overwrites_its_tokens(ctx, mode, M, N):
+    """rotate + quantize -> GEMM -> residual add -> rotate + quantize over the sum, into the buffer the GEMM took its tokens from -> GEMM back
+    to the width of the start -> residual add, twice, replayed as one graph with other inputs, against the calls apart. In a graph the split-K GEMM of 33 to
+    96 rows (to 128 with a step per token) lets its successor be placed while it still adds and stores; 4096 channels are split along K, 28672 are not."""
+    K = 4096
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    rand = lambda *sh: torch.randn(sh, generator=g, device="cuda").to(torch.bfloat16)
+    wq = [torch.randint(0, 256, sh, dtype=torch.uint8, device="cuda", generator=g) for sh in ((N, K // 2), (K, N // 2))]
+    s_w = [torch.full((n,), 4e-3, device="cuda") for n in (N, K)]
+    wsum = [ctx.weight_code_sums(w) for w in wq]
+    s_a, s_tok = torch.full((1,), 0.02 if mode == "w4a8" else 0.3, device="cuda"), torch.full((M,), 0.3, device="cuda")
+    z = torch.full((1,), 6, dtype=torch.int32, device="cuda")
+    flat = torch.zeros(M * max(N, K), dtype=torch.int8 if mode == "w4a8" else torch.uint8, device="cuda")
+    x, base, out, mid = rand(M, K), rand(M, N), torch.zeros((M, N), dtype=torch.bfloat16, device="cuda"), torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    back = torch.zeros((M, K), dtype=torch.bfloat16, device="cuda")
+    xs = [rand(M, K) * 2.0**i for i in range(4)]
+
+    def linear(src, i, dst, step):
+        k = src.shape[1]
+        xq = flat[: M * (k if mode == "w4a8" else k // 2)].view(M, -1)
+        if mode == "w4a8":
+            ctx.hadamard_quant_act8(src, 4096, s_a, out=xq)
+        elif mode == "rows":
+            ctx.hadamard_quant_act_rows(src, 4096, s_tok, out=xq)
+        elif mode == "asym":
+            ctx.hadamard_quant_act_asym(src, 4096, s_a, z, out=xq)
+        else:
+            ctx.hadamard_quant_act(src, 4096, s_a, out=xq)
+        step()
+        if mode == "w4a8":
+            ctx.w4a8_gemm(xq, wq[i], s_a, s_w[i], out=dst)
+        elif mode == "rows":
+            ctx.w4a4_gemm_rows(xq, wq[i], s_tok, s_w[i], out=dst)
+        elif mode == "asym":
+            ctx.w4a4_gemm_asym(xq, wq[i], s_a, z, s_w[i], wsum[i], out=dst)
+        else:
+            ctx.w4a4_gemm(xq, wq[i], s_a, s_w[i], out=dst)
+        step()
+
+    def chain(step):
+        for _ in range(2):
+            linear(x, 0, out, step)
+            ctx.residual_add(out, base, out=mid)
+            step()
+            linear(mid, 1, back, step)
+            ctx.residual_add(back, x, out=x)
+            step()
+
+    def run(call):
+        res = []
+        for v in xs:
+            x.copy_(v)
+            torch.cuda.synchronize()
+            call()
+            torch.cuda.synchronize()
+            res.append([t.clone() for t in (x, out, mid, back, flat)])
+        return res
+
+    want = run(lambda: chain(torch.cuda.synchronize))
+    assert all(len(torch.unique(t)) > 12 for t in want[0]) and bool(torch.isfinite(want[-1][0].float()).all())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(lambda: None)
+    for call in (graph.replay, lambda: chain(lambda: None), graph.replay):
+        for i, (w, r) in enumerate(zip(want, run(call))):
+            assert all(torch.equal(a, b) for a, b in zip(w, r)), f"input {i}"
+    ctx.check()
