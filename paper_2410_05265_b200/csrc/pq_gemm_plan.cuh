@@ -249,6 +249,17 @@ inline int split_count_pairs(int tiles, int K, int sm_count, int M, bool a8) {
   return fewer && most >= 1 ? (one < most ? one : most) : two;
 }
 
+// Is a launch of those forms kept to one CTA to an SM? Above 64 tokens, when the CTAs have an SM each (7/8 of the SMs, clusters of four at most: a
+// cluster of eight does not find eight free ones everywhere) and are more than half of the SMs. It then asks for more than half of an SM's shared
+// memory. Otherwise its CTAs, placed while the rotation kernel before them still holds a part of the SMs, shared the others by twos. us, rotation and GEMM issued
+// into a stream, by twos / alone: 100 x 4096 x 4096 14.3 / 11.9 (before one CTA to an SM was the rule 13.4), 112 x 6144 x 4096 16.5 / 13.9, W4A8 100 x 4096 x 4096
+// 12.6 / 11.0, 96 x 4096 x 14336 15.3 / 14.7; linear set in a graph, 4-bit at 112 tokens 78.1 / 73.1, W4A8 at 96 57.1 / 55.0, per token at 128 81.3 / 77.0.
+// Without the three conditions: 20 x 2048 x 8192 (clusters of eight) 7.7 / 11.5, 48 x 4096 x 2048 7.1 / 7.6, W4A8 96 x 2048 x 4096 (48 CTAs) 8.6 / 10.0.
+constexpr int SPLIT_ALONE_SMEM = 120 * 1024;
+inline bool split_alone(int M, int ctas, int splits, int sm_count) {
+  return M > 64 && 2 * ctas > sm_count && ctas <= sm_count * 7 / 8 && splits <= 4;
+}
+
 // The width of the token tiles up to 128 tokens.
 inline int split_width(int M) { return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 48 ? 48 : (M <= 64 ? 64 : (M <= 96 ? 96 : 128)))); }
 

@@ -544,10 +544,12 @@ template <int NT, bool A8, bool ZP, bool WHOLE>
 pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw, SplitParams& p, cudaStream_t st) {
   using C = Cfg<NT, A8, WHOLE>;
   constexpr size_t smem = split_smem<NT, A8, WHOLE>();
+  static_assert(WHOLE || smem <= SPLIT_ALONE_SMEM, "half of an SM at most");
   static bool attr_set[64] = {};  // the attribute belongs to the device's copy of the kernel: once per device
   if (ctx->device < 0 || ctx->device >= 64) return PQ_ERR_UNSUPPORTED;
   if (!attr_set[ctx->device]) {
-    if (cudaFuncSetAttribute(gemm_w4_split_kernel<NT, A8, ZP, WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (cudaFuncSetAttribute(gemm_w4_split_kernel<NT, A8, ZP, WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(WHOLE ? smem : SPLIT_ALONE_SMEM)) != cudaSuccess)
       return PQ_ERR_CUDA;
     attr_set[ctx->device] = true;
   }
@@ -558,7 +560,7 @@ pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(tiles) * p.splits);
   cfg.blockDim = dim3(C::THREADS);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = !WHOLE && split_alone(p.M, tiles * p.splits, p.splits, ctx->sm_count) ? SPLIT_ALONE_SMEM : smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;

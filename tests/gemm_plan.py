@@ -32,6 +32,8 @@ void acc_slots(const PairPlan* p, int h, int first, int step, int count, int* ou
 }
 int width(int m) { return split_width(m); }
 int splits_pairs(int tiles, int k, int m, int a8) { return split_count_pairs(tiles, k, 148, m, a8 != 0); }
+int alone(int m, int ctas, int splits) { return split_alone(m, ctas, splits, 148); }
+int alone_smem() { return SPLIT_ALONE_SMEM; }
 int width_whole(int m, int n, int k, int a8) { return split_width_whole(m, n, k, a8 != 0, 148); }
 #define ROW(NT, A8) {NT, A8, SplitCfg<NT, A8>::TMEM_COLS, (int)split_smem<NT, A8>()}
 int split_rows(int (*out)[4]) {
@@ -126,3 +128,12 @@ def width_whole(M, N, K, a8):
 def splits_pairs(tiles, K, M, a8):
     """K splits of a launch of the split-K kernel's forms of two CTAs to an SM."""
     return lib().splits_pairs(tiles, K, M, int(a8))
+
+
+def alone(M, ctas, splits):
+    """Is such a launch kept to one CTA to an SM?"""
+    return bool(lib().alone(M, ctas, splits))
+
+
+def alone_smem():
+    return lib().alone_smem()

@@ -181,11 +181,30 @@ def test_ctas_that_fit_one_sm_find_their_tensor_memory():
                     assert sum(cols for _, _, cols, _ in group) <= 512, group
 
 
+def test_ctas_kept_to_one_an_sm_find_their_tensor_memory_too():
+    """The same where one of the CTAs is of a launch kept to one to an SM; two of those never share one."""
+    one = (64, 0, 256, gp.alone_smem())
+    assert 2 * (one[3] + 1024) > 228 * 1024
+    for b in gp.split_shapes() + gp.whole_shapes():
+        for c in gp.split_shapes() + [(0, 0, 0, 0)]:
+            group = [f for f in (one, b, c) if f[0]]
+            if sum(smem + 1024 for *_, smem in group) <= 228 * 1024:
+                assert sum(cols for _, _, cols, _ in group) <= 512, group
+
+
 def test_two_ctas_of_33_to_96_tokens_leave_no_room_for_a_rotation():
     """16 elements to a thread keep 2176 floats of shared memory at the least."""
     for nt, _, _, smem in gp.split_shapes():
         if 32 < nt < 128:
             assert 0 <= 228 * 1024 - 2 * (smem + 1024) < 2176 * 4
+
+
+@pytest.mark.parametrize("M,ctas,splits,want", [
+    (96, 96, 3, True), (64, 96, 3, False), (65, 75, 1, True), (65, 74, 2, False), (128, 129, 3, True), (128, 130, 2, False), (128, 128, 4, True),
+    (100, 120, 5, False), (100, 128, 8, False), (96, 240, 5, False),
+])
+def test_launches_kept_to_one_cta_an_sm(M, ctas, splits, want):
+    assert gp.alone(M, ctas, splits) == want
 
 
 def test_narrow_forms_that_take_an_sm_alone_share_it_with_no_other():
