@@ -1,5 +1,5 @@
 """Rotation kernel of calls with few wide blocks (16 elements to a thread, a block to a CTA): the codes, steps and normalised rows of the kernel for
-many blocks bit for bit, at the borders of the rule between the two (one block of 4096 to an SM, four in all with a step per token, two of 2048 to an SM,
+many blocks bit for bit, at the borders of the rule between the two (7/16 of a block of 4096 to an SM, four in all with a step per token, two of 2048 to an SM,
 five with SwiGLU), for every form."""
 import pytest
 import torch
@@ -28,16 +28,16 @@ def sms():
 
 
 @pytest.mark.parametrize("form", ["static", "bytes", "nibbles_in_bytes", "zero_point", "rows", "dynamic"])
-@pytest.mark.parametrize("K,block,per_sm", [(4096, 4096, 1), (2048, 2048, 2), (14336, 2048, 2), (8192, 4096, 1)])
+@pytest.mark.parametrize("K,block,per_sm", [(4096, 4096, 7 / 16), (4096, 4096, 1), (2048, 2048, 2), (14336, 2048, 2), (8192, 4096, 7 / 16), (8192, 4096, 1)])
 @pytest.mark.parametrize("where", ["one", "last", "beyond"])
 @pytest.mark.parametrize("pitch,row_begin", [(0, 0), (34, 3)])
 def test_same_codes_as_the_kernel_for_many_blocks(ctx, form, K, block, per_sm, where, pitch, row_begin):
     if form == "dynamic" and K != block:
         pytest.skip("rows of several blocks have a kernel of their own")
     per_row = K // block
-    most = 4 if block == 4096 and form in ("rows", "dynamic") else per_sm * sms()
+    most = 4 if block == 4096 and form in ("rows", "dynamic") else int(per_sm * sms())
     M = row_begin + {"one": 1, "last": most // per_row, "beyond": most // per_row + 1}[where]
-    x = rows(row_begin + per_sm * sms() // per_row + 40, K, pitch)  # enough rows for the other kernel
+    x = rows(row_begin + int(per_sm * sms()) // per_row + 40, K, pitch)  # enough rows for the other kernel
     s, z = torch.full((1,), 0.37, device="cuda"), torch.full((1,), 6, dtype=torch.int32, device="cuda")
     s_tok = torch.rand(x.shape[0], device="cuda") + 0.1
 
@@ -72,10 +72,10 @@ def test_swiglu_same_codes_as_the_two_launches(ctx, extra):
     assert torch.equal(fused, two) and len(torch.unique(fused)) > 12
 
 
-@pytest.mark.parametrize("K,per_sm", [(4096, 1), (2048, 2)])
+@pytest.mark.parametrize("K,per_sm", [(4096, 7 / 16), (4096, 1), (2048, 2)])
 @pytest.mark.parametrize("extra", [0, 1])
 def test_rmsnorm_fused_and_alone_agree_on_both_sides_of_the_rule(ctx, K, per_sm, extra):
-    M = per_sm * sms() + extra
+    M = int(per_sm * sms()) + extra
     x, g = rows(M, K), rows(1, K, seed=1)[0].contiguous()
     s = torch.full((1,), 0.5, device="cuda")
     h = ctx.rmsnorm(x, g, 1e-5)
@@ -88,12 +88,12 @@ def test_rmsnorm_fused_and_alone_agree_on_both_sides_of_the_rule(ctx, K, per_sm,
     assert bool(((h.double() - want).abs() <= want.abs() * (2.0**-8 + 2.0**-16) + 1e-30).all())
 
 
-@pytest.mark.parametrize("K,per_sm", [(4096, 1), (2048, 2)])
+@pytest.mark.parametrize("K,per_sm", [(4096, 7 / 16), (4096, 1), (2048, 2)])
 @pytest.mark.parametrize("row_begin", [0, 4])
 def test_a_normalised_row_does_not_depend_on_the_rows_beside_it(ctx, K, per_sm, row_begin):
     """Few rows, as many as the kernel of few blocks takes, and two more: the same values, and the fused call the codes of the two
     calls also where row_begin leaves it on one side of the rule and the stand-alone call, which has none, on the other."""
-    most = per_sm * sms()
+    most = int(per_sm * sms())
     g = rows(1, K, seed=1)[0].contiguous()
     s = torch.full((1,), 0.5, device="cuda")
     for seed in range(8):  # two orders of the sum differ in some five of a million bf16 values
