@@ -88,6 +88,8 @@ constexpr int DA_TICKET0 = 16;
 // more splits pay for their second merge through the workspace. us, one cluster / more splits, plain call in a graph: 1 x 1021 keys (8 pairs)
 // 5.4 / 9.1, 1 x 2000 6.2 / 8.5, 1 x 4092 8.0 / 8.9, 3 x 3000 7.8 / 13.6, steps per vector 2 x 4000 10.4 / 15.5; the one-launch step inside a
 // decode layer: 1021 keys 55.4 / 55.7, 4000 keys 58.5 / 58.0 (its first rounds are on their way before it starts).
+// The rounds are those of the capacity, since the lengths are on the device: 1 x 1021 keys in a cache of 1085 or 4096 take 4.9 us, in one of 8192, where 24 of
+// the 32 splits have no round and the merge goes through the workspace, 8.4 (before one cluster was an option 7.8 and 8.6).
 constexpr int DA_ONE_CLUSTER_ROUNDS = 32, DA_ONE_CLUSTER_ROUNDS_FUSED = 24;
 constexpr float DA_HEADROOM = 15.0f;  // log2 units a score may exceed the reference exponent before it is moved
 constexpr float DA_HEADROOM_DYN = 4.0f;  // DYN: P * step * code stays within 2^7 of the largest cached value
@@ -249,13 +251,14 @@ struct AttnParams {
 //            denominator.
 // The CTA of the last split also scores the full-precision prefix keys and folds them into its partial.
 // CLUSTER: the splits of a (sequence, head) form one thread-block cluster and merge their partials
-// through distributed shared memory (no workspace, no ticket); otherwise the partials go through the
-// caller's workspace and the last CTA to finish merges them.
+// through distributed shared memory (no workspace, no ticket); otherwise, in the allocation-free call only, the partials go
+// through the workspace and the last CTA to finish merges them.
 // FUSED: the call also appends one token per sequence (what pq_kv4_append does for T_new = 1). The attention
 // streams the cache as it was; the CTA of the last split quantizes the new k and v of its head, writes their codes
 // to row len[b] and folds the new key into its partial like one more full-precision key whose key and value are
-// the dequantized codes. The last CTA of the grid to finish (every CTA has read the lengths by then) advances
-// every len[b]. As with the two calls, nothing is appended anywhere when any sequence is full.
+// the dequantized codes. Every CTA draws a ticket once it has read the lengths, and the CTA that drew the last one advances every len[b] when it
+// is done: the lengths are not read behind the ticket, and an advanced length does not say that the other CTAs have stored
+// their rows; both are seen by others at the end of the kernel only. As with the two calls, nothing is appended anywhere when any sequence is full.
 // MULTI (with CLUSTER): a (sequence, head) has several clusters of eight splits.
 // DYN (group-wise dynamic KV, Table 1 O1): every cached vector has its own step. The setting's arithmetic is that of fp32:
 //   scores   codes as exact bf16 integers (one more operation per word pair, no offset to cancel) times the query as it is
@@ -270,6 +273,7 @@ struct AttnParams {
 // sequences of up to 3000 keys, 64 heads: 50 / 55 now), but lost bits, up to all of them, where one step of the cache was far above the rest.
 template <bool CLUSTER, bool FUSED, bool MULTI = false, bool DYN = false>
 __global__ void __launch_bounds__(DA_THREADS, DYN ? 3 : 4) decode_attn_kernel(const AttnParams p) {
+  static_assert(CLUSTER || !(FUSED || MULTI || DYN), "without clusters only the plain static form");
   extern __shared__ __align__(128) uint8_t da_stage[];  // DA_SLOTS slots of [K rows | V rows] of one round
   // the per-warp partial outputs reuse the staging area once the key loop is over
   // [warp][head][DA_SO_STRIDE]; head dim d = 16a + 2b + c sits at 16b + 2a + c and the rows are padded so
@@ -952,15 +956,11 @@ bool set_attn_smem() {
             cudaSuccess ||
         cudaFuncSetAttribute(decode_attn_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DA_SMEM_BYTES) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(decode_attn_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DA_SMEM_BYTES) !=
-            cudaSuccess ||
         cudaFuncSetAttribute(decode_attn_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DA_SMEM_BYTES) !=
             cudaSuccess ||
         cudaFuncSetAttribute(decode_attn_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              DA_SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(decode_attn_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             DA_SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(decode_attn_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              DA_SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(decode_attn_kernel<true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              DA_SMEM_BYTES) != cudaSuccess ||
@@ -1054,23 +1054,17 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   }
   int S = choose_splits(ctx, cache);
   const int rounds = (cache->Tmax + DA_ROUND - 1) / DA_ROUND;  // a split without a round would only take part in the merge
-  // With enough (sequence, head) pairs, eight splits already fill the GPU: the splits then form one
+  // With enough (sequence, head) pairs eight splits fill the GPU, and a short cache has no work for more: the splits of a pair then form one
   // cluster and merge through distributed shared memory (the workspace and the tickets stay unused).
-  bool cluster = static_cast<int64_t>(cache->B) * cache->Hkv * 8 >= 2LL * ctx->sm_count;
-  if (cluster && S > 8) S = 8;
+  const bool one_cluster = static_cast<int64_t>(cache->B) * cache->Hkv * 8 >= 2LL * ctx->sm_count ||
+                           rounds <= (k_new ? DA_ONE_CLUSTER_ROUNDS_FUSED : DA_ONE_CLUSTER_ROUNDS);
+  if (one_cluster && S > 8) S = 8;
   if (S > rounds && rounds > 0) S = rounds;
-  // Few (sequence, head) pairs with long caches: several clusters of eight splits per pair; each merges its eight
+  // Few pairs with long caches: several clusters of eight splits per pair (such a call has at least sixteen); each merges its eight
   // partials on chip, the workspace sees one partial per cluster.
-  if (!cluster && rounds <= (k_new ? DA_ONE_CLUSTER_ROUNDS_FUSED : DA_ONE_CLUSTER_ROUNDS)) {
-    if (S > 8) S = 8;
-    cluster = true;
-  }
-  if (!cluster && S >= 16) {
-    S = S / 8 * 8;
-    cluster = true;
-  }
-  const int n_parts = cluster ? (S < 8 ? 1 : S / 8) : S;
-  const bool multi = cluster && n_parts > 1;
+  if (!one_cluster) S = S / 8 * 8;
+  const int n_parts = S < 8 ? 1 : S / 8;
+  const bool multi = n_parts > 1;
   const int G = cache->Hq / cache->Hkv;
   AttnParams p{};
   p.q = static_cast<const __nv_bfloat16*>(q);
@@ -1098,48 +1092,31 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
   p.len_tickets = ctx->d_tickets + DA_LEN_TICKET0;
   dim3 grid(S, cache->Hkv, cache->B);
   if (!set_attn_smem()) return PQ_ERR_CUDA;
-  if (cluster) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(DA_THREADS);
-    cfg.dynamicSmemBytes = DA_SMEM_BYTES;
-    cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = S < 8 ? S : 8;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    cudaError_t e;
-    if (dyn)
-      e = multi ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true, true>, p)
-                : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, false, true>, p);
-    else if (multi)
-      e = fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, true, true>, p)
-                : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true>, p);
-    else
-      e = fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, true, false>, p)
-                : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, false>, p);
-    if (e != cudaSuccess) return PQ_ERR_CUDA;
-    return pq_launch_status();
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(DA_THREADS);
   cfg.dynamicSmemBytes = DA_SMEM_BYTES;
   cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = S < 8 ? S : 8;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if ((dyn     ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false, true>, p)
-       : fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, true, false>, p)
-               : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false, false, false>, p)) != cudaSuccess)
-    return PQ_ERR_CUDA;
+  cfg.numAttrs = 2;
+  cudaError_t e;
+  if (dyn)
+    e = multi ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true, true>, p)
+              : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, false, true>, p);
+  else if (multi)
+    e = fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, true, true>, p)
+              : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, true>, p);
+  else
+    e = fused ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, true, false>, p)
+              : cudaLaunchKernelEx(&cfg, decode_attn_kernel<true, false, false>, p);
+  if (e != cudaSuccess) return PQ_ERR_CUDA;
   return pq_launch_status();
 }
 }  // namespace
