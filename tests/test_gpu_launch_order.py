@@ -374,3 +374,41 @@ def test_what_follows_a_captured_gemm_reads_its_output_and_overwrites_its_tokens
         for i, (w, r) in enumerate(zip(want, run(call))):
             assert all(torch.equal(a, b) for a, b in zip(w, r)), f"input {i}"
     ctx.check()
+
+
+@pytest.mark.parametrize("M", [1, 24, 64, 96, 300, 1030])
+@pytest.mark.parametrize("N,K", [(4096, 4096), (8448, 1024)])
+def test_weights_are_not_overwritten_under_the_gemm_that_reads_them(ctx, M, N, K):
+    """GEMM -> weight quantizer into the codes and steps that GEMM reads -> GEMM on the new ones, and on, in a graph and called back to back:
+    the quantizer is placed while the GEMM drains and writes only when it has ended. Sums and outputs as by the calls apart."""
+    g = torch.Generator(device="cuda").manual_seed(M)
+    W = [inputs.weights(N, K, seed=2 + s).cuda() * 2.0**s for s in range(3)]
+    wq, s_w = torch.zeros((N, K // 2), dtype=torch.uint8, device="cuda"), torch.zeros(N, device="cuda")
+    xq = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+    s_a = torch.full((1,), 0.3, device="cuda")
+    out = torch.zeros((4, M, N), dtype=torch.bfloat16, device="cuda")
+    acc = torch.zeros((4, M, N), dtype=torch.int32, device="cuda")
+
+    def chain(step):
+        for i in range(4):
+            ctx.quant_weights(W[i % 3], out=(wq, s_w))
+            step()
+            ctx.w4a4_gemm(xq, wq, s_a, s_w, out=out[i], acc_dbg=acc[i])
+            step()
+
+    def run(call):
+        out.zero_(), acc.zero_()
+        torch.cuda.synchronize()
+        call()
+        torch.cuda.synchronize()
+        return out.clone(), acc.clone()
+
+    want = run(lambda: chain(torch.cuda.synchronize))
+    assert not torch.equal(want[1][0], want[1][1])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(lambda: None)
+    for call in (graph.replay, lambda: chain(lambda: None)) * 3:
+        for a, b in zip(want, run(call)):
+            assert torch.equal(a, b)
+    ctx.check()

@@ -51,7 +51,8 @@ def test_the_one_launch_decode_step_never_triggers():
 @pytest.mark.parametrize("source,name", [
     ("pq_gemm_stream.cu", "gemm_w4a4_stream_kernel"), ("pq_gemm_split.cu", "gemm_w4_split_kernel"), ("pq_gemm_tc2.cu", "gemm_w4a4_pair_kernel"),
     ("pq_gemm_tc3.cu", "gemm_w4a4_pair_ts_kernel"), ("pq_hadamard_quant.cu", "hadamard_quant_kernel"),
-    ("pq_hadamard_quant.cu", "hadamard_quant_wide_kernel"), ("pq_kv4.cu", "decode_attn_kernel"), ("pq_prefill_attn.cu", "prefill_attn_kernel"),
+    ("pq_hadamard_quant.cu", "hadamard_quant_wide_kernel"), ("pq_hadamard_quant.cu", "hadamard_quant_small_kernel"),
+    ("pq_quant_weights.cu", "quant_weights_once_kernel"), ("pq_kv4.cu", "decode_attn_kernel"), ("pq_prefill_attn.cu", "prefill_attn_kernel"),
     ("pq_block.cu", "rmsnorm_kernel"), ("pq_block.cu", "rope_kernel"), ("pq_block.cu", "rope_rotate_kernel"), ("pq_block.cu", "silu_mul_kernel"),
     ("pq_block.cu", "add_kernel"), ("pq_block.cu", "rope_kv4_append_kernel"),
 ])
@@ -72,6 +73,8 @@ def test_what_a_predecessor_may_write_is_not_read_through_the_read_only_path(sou
     assert not wrong, wrong
     if name.startswith("hadamard"):  # its parameters are const __restrict__: no plain load through them either
         assert not re.search(r"\b(?:x|x2|s_a_in|zp_in)\[", body)
+    if name.startswith("quant_weights"):
+        assert body.count("row + j") == 1 and not re.search(r"\b(?:W|row)\[|\*row|\*W\b", body) and body.index("pdl_wait") < body.index("row + j")
 
 
 def test_the_plain_decode_attention_reads_nothing_through_the_read_only_path():
