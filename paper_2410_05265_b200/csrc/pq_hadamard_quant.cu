@@ -522,8 +522,10 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
 #pragma unroll
       for (int tau = 0; tau < 8; ++tau)
 #pragma unroll
-        for (int v = 0; v < 4; ++v)
-          w[tau][v] = pack_bf16x2(pq::silu_mul_f32(bf16_pair(w[tau][v]), bf16_pair(u[tau][v])));
+        for (int v = 0; v < 4; ++v) {  // packed pairs spill at blocks of 4096 and 8192 (28672 wide, blocks of 4096: 1000 rows 33.2 us, element by element 31.6); the same bits
+          const float2 ga = bf16_pair(w[tau][v]), up = bf16_pair(u[tau][v]);
+          w[tau][v] = pack_bf16x2(LOGB == 11 ? pq::silu_mul_f32(ga, up) : make_float2(pq::silu_mul_f32(ga.x, up.x), pq::silu_mul_f32(ga.y, up.y)));
+        }
     } else if (NORM) {
       uint32_t g_w[8][4];  // requested ahead of the sum: behind it their trip stood in the chain of every row
       load_words(x2 + col0, true, g_w);
@@ -769,18 +771,19 @@ __global__ void __launch_bounds__(ROW ? 32 * HQ_ROW_WARPS : HQ_THREADS, ROW ? 1 
 // of each of its pairs, a warp 32 consecutive ones. Latency bounds either kernel; us per call of M rows in a graph, wide kernel / this one:
 //   4096 (one block a row)   M = 1 1.84 / 1.61, 33 2.17 / 1.88, 64 2.22 / 2.09, 100 2.39 / 2.38; with RMSNorm 2.29 / 2.18, 2.69 / 2.43, 2.71 / 2.57, 2.83 / 3.22
 //   14336 (seven blocks)     M = 1 1.83 / 1.49, 33 2.27 / 2.13, 42 2.14 / 2.18, 96 3.42 / 3.81; with SwiGLU 2.57 / 1.71, 3.15 / 2.75, 2.80 / 2.74, 96 5.36 / 3.72
-// so the line lies at 7/16 of a block of 4096 to an SM (64), two of 2048, five with SwiGLU. Blocks of 8192 (16 warps, five shuffle stages) stay with the
+// so the line lies at 7/16 of a block of 4096 to an SM (64; with SwiGLU one, 100 x 4096 3.13 / 2.50), two of 2048, five with SwiGLU. Blocks of 8192 (16 warps, five shuffle stages) stay with the
 // wide kernel: 2.28 / 2.85. Decode layer at 1021 tokens 53.8 -> 50.3.
 // What stands behind it counts as much: with a CTA on every SM the next GEMM's CTAs, which take an SM each above 64 rows, are not spread evenly. us with the
 // GEMM, static step, wide / this: 28672 x 4096 at 100 rows 23.7 / 24.2, at 148 25.3 / 26.2; 8B linear set at 80 tokens 66.7 / 67.5, 128 74.5 / 76.3, W4A8 at
 // 128 63.1 / 64.6; only GEMMs of few channels lose (W4A8 96 x 512 x 4096 8.0 / 7.6). Up to 64 rows: 6144 x 4096 at 24 rows 8.0 / 8.3, 28672 x 4096 16.3 / 16.0,
+// (the streaming GEMM of 4096 x 14336 loses a little behind it: 8B set at 8 tokens, blocks of 2048 by the wide kernel, 40.1, with a zero point 41.3 / 41.9)
 // 8B set at 8 tokens 40.9 / 40.8, at 24 46.4 / 47.4, at 64 57.6 / 58.0, W4A8 at 8 51.3 / 49.1, at 33 49.6 / 48.7, at 64 54.6 / 53.8, with a zero point at 24 47.6 / 47.2.
 // One step per token and blocks of 4096: up to four of them. Behind a split-K GEMM of up to 32 tokens, which triggers at once, this kernel fits beside
 // that GEMM's CTAs and lets the next ones in among them; us with the GEMM, wide kernel / this one: 6144 x 4096 at 4 rows 5.8 / 5.6, 14 7.6 / 8.2, 24
 // 7.9 / 8.8, 32 8.3 / 9.3, 64 11.1 / 11.1, 4096 x 4096 at 1 row 5.3 / 4.9, 8 6.0 / 6.2, 32 7.9 / 8.9, but 28672 x 4096 at 24 16.2 / 15.8. 8B linear set at 24
 // tokens 47.2 / 48.9.
 constexpr int hq_small_blocks(int logb, bool swiglu, bool per_token, int sm_count) {
-  return logb == 11 ? (swiglu ? 5 : 2) * sm_count : (logb == 12 ? (per_token ? 4 : sm_count * 7 / 16) : 0);
+  return logb == 11 ? (swiglu ? 5 : 2) * sm_count : (logb == 12 ? (per_token ? 4 : swiglu ? sm_count : sm_count * 7 / 16) : 0);
 }
 
 template <int LOGB, int BITS, bool PER_TOKEN, bool ZP, bool SWIGLU, int NORM>

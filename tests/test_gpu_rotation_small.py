@@ -62,12 +62,13 @@ def test_same_codes_as_the_kernel_for_many_blocks(ctx, form, K, block, per_sm, w
 
 
 @pytest.mark.parametrize("extra", [0, 1])
-def test_swiglu_same_codes_as_the_two_launches(ctx, extra):
-    M, F = 5 * sms() // 7 + extra, 14336
+@pytest.mark.parametrize("F,block,per_sm", [(14336, 2048, 5), (8192, 4096, 1), (8192, 8192, 1)])
+def test_swiglu_same_codes_as_the_two_launches(ctx, F, block, per_sm, extra):
+    M = per_sm * sms() // (F // block) + extra
     gu = rows(M, 2 * F)
     s = torch.full((1,), 0.2, device="cuda")
-    fused = ctx.swiglu_hadamard_quant_act(gu[:, :F], gu[:, F:], 2048, s)
-    two = ctx.hadamard_quant_act(ctx.silu_mul(gu[:, :F], gu[:, F:]), 2048, s)
+    fused = ctx.swiglu_hadamard_quant_act(gu[:, :F], gu[:, F:], block, s)
+    two = ctx.hadamard_quant_act(ctx.silu_mul(gu[:, :F], gu[:, F:]), block, s)
     ctx.check()
     assert torch.equal(fused, two) and len(torch.unique(fused)) > 12
 
