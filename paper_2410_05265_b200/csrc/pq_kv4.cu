@@ -1056,13 +1056,17 @@ pq_status decode_attn_launch(pq_ctx* ctx, const pq_kv4_cache* cache, const void*
     if (k_new) return PQ_ERR_UNSUPPORTED;  // the one-launch decode step serves the static setting
   }
   int S = choose_splits(ctx, cache);
-  const int rounds = (cache->Tmax + DA_ROUND - 1) / DA_ROUND;  // a split without a round would only take part in the merge
+  const int rounds = (cache->Tmax + DA_ROUND - 1) / DA_ROUND;
   // With enough (sequence, head) pairs eight splits fill the GPU, and a short cache has no work for more: the splits of a pair then form one
   // cluster and merge through distributed shared memory (the workspace and the tickets stay unused).
   const bool one_cluster = static_cast<int64_t>(cache->B) * cache->Hkv * 8 >= 2LL * ctx->sm_count ||
                            rounds <= (k_new ? DA_ONE_CLUSTER_ROUNDS_FUSED : DA_ONE_CLUSTER_ROUNDS);
   if (one_cluster && S > 8) S = 8;
-  if (S > rounds && rounds > 0) S = rounds;
+  // A split without a round only takes part in the merge, but for the last one, which has the prefix and the appended key: it may have nothing else
+  // while the CTAs are two to an SM (8 x 300 keys, three splits / four, 5.9 / 5.5 us; 16 x 300 6.8 / 7.1, with steps per vector 7.3 / 10.7).
+  const int64_t pairs = static_cast<int64_t>(cache->B) * cache->Hkv;
+  const int useful = rounds + ((cache->n_prefix > 0 || k_new) && pairs * (rounds + 1) <= 2LL * ctx->sm_count ? 1 : 0);
+  if (rounds > 0 && S > useful) S = useful;
   // Few pairs with long caches: several clusters of eight splits per pair (such a call has at least sixteen); each merges its eight
   // partials on chip, the workspace sees one partial per cluster.
   if (!one_cluster) S = S / 8 * 8;
