@@ -229,9 +229,13 @@ constexpr int MAX_SPLIT = 8;  // portable cluster size
 // As many K splits as leave every CTA resident at once with room for the clusters to be placed (7/8 of the slots: 48 tiles
 // x 6 = 288 CTAs ran in two waves, 10.7 us against 7.0 with 96), and at least 640 elements of K per CTA (below that the two
 // cluster barriers cost more than the shorter loop saves: 4096 x 4096 at 32 tokens 6.1 us with six splits, 6.6 with eight).
-inline int split_count(int tiles, int K, int slots) {
-  int splits = slots * 7 / 8 / tiles;
+// A cluster's CTAs lie in one GPC: of clusters of seven or eight with a CTA to an SM only fifteen find a place (cudaOccupancyMaxActiveClusters; 22, 26, 33, 45
+// of six, five, four, three, so that 7/8 of the SMs is the lower line there). The sixteenth ran behind the others: 345 x 768 x 14336, eighteen tiles, seven splits / six,
+// 24.3 / 15.8 us, W4A8 160 x 1152 x 14336 20.3 / 13.4, 200 x 2176 x 8192 24.7 / 15.1. Two CTAs to an SM find 37 of seven and 33 of eight.
+inline int split_count(int tiles, int K, int sm_count, int per_sm) {
+  int splits = sm_count * per_sm * 7 / 8 / tiles;
   if (splits > MAX_SPLIT) splits = MAX_SPLIT;
+  if (per_sm == 1 && splits > 6 && tiles > 15 * sm_count / 148) splits = 6;
   if (splits > K / (5 * BK)) splits = K / (5 * BK);
   return splits < 1 ? 1 : splits;
 }
@@ -243,7 +247,7 @@ inline int split_count(int tiles, int K, int slots) {
 // at 128 six 13.4 / three 11.9 (four 13.7), 6144 x 4096 at 96 12.9 / 13.3, at 128 15.2 / 13.8, 4096 x 14336 at 80 18.0 / 20.2; at 64 tokens 4096 x 14336
 // eight 15.3 / four 17.6.
 inline int split_count_pairs(int tiles, int K, int sm_count, int M, bool a8) {
-  const int two = split_count(tiles, K, 2 * sm_count), one = sm_count * 9 / 10 / tiles, most = K / (10 * BK);
+  const int two = split_count(tiles, K, sm_count, 2), one = sm_count * 9 / 10 / tiles, most = K / (10 * BK);
   const bool short_k = K <= 16 * BK * one;
   const bool fewer = M > 64 && two * tiles > sm_count && one >= 2 && (short_k ? a8 || M > 96 || one >= 4 : a8 && M > 88 && one >= 4);
   return fewer && most >= 1 ? (one < most ? one : most) : two;
@@ -275,7 +279,7 @@ inline int split_width_whole(int M, int N, int K, bool a8, int sm_count) {
   int best = 0;
   double best_us = 0.0;
   for (int i = 0; i < 4; ++i) {
-    const int t_tiles = (M + widths[i] - 1) / widths[i], tiles = t_tiles * ((N + CH - 1) / CH), splits = split_count(tiles, K, sm_count);
+    const int t_tiles = (M + widths[i] - 1) / widths[i], tiles = t_tiles * ((N + CH - 1) / CH), splits = split_count(tiles, K, sm_count, 1);
     const int rounds = (tiles * splits + sm_count - 1) / sm_count, blocks = ((K + BK - 1) / BK + splits - 1) / splits;
     const double tokens = (M + t_tiles - 1) / t_tiles;
     const double us = rounds * blocks * (a8 ? us8 : us4)[i] + tokens * tokens * (splits - 1) / splits * (4.5 / 65536);

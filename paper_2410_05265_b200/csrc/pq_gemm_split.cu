@@ -556,7 +556,7 @@ pq_status launch_split(pq_ctx* ctx, const CUtensorMap& tx, const CUtensorMap& tw
   p.t_tiles = (p.M + NT - 1) / NT;
   p.n_kb = (p.K + C::KB - 1) / C::KB;
   const int tiles = p.t_tiles * ((p.N + CH - 1) / CH);
-  p.splits = WHOLE ? split_count(tiles, p.K, ctx->sm_count) : split_count_pairs(tiles, p.K, ctx->sm_count, p.M, A8);
+  p.splits = WHOLE ? split_count(tiles, p.K, ctx->sm_count, 1) : split_count_pairs(tiles, p.K, ctx->sm_count, p.M, A8);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(tiles) * p.splits);
   cfg.blockDim = dim3(C::THREADS);

@@ -34,6 +34,7 @@ int width(int m) { return split_width(m); }
 int splits_pairs(int tiles, int k, int m, int a8) { return split_count_pairs(tiles, k, 148, m, a8 != 0); }
 int alone(int m, int ctas, int splits) { return split_alone(m, ctas, splits, 148); }
 int alone_smem() { return SPLIT_ALONE_SMEM; }
+int splits_whole(int tiles, int k) { return split_count(tiles, k, 148, 1); }
 int width_whole(int m, int n, int k, int a8) { return split_width_whole(m, n, k, a8 != 0, 148); }
 #define ROW(NT, A8) {NT, A8, SplitCfg<NT, A8>::TMEM_COLS, (int)split_smem<NT, A8>()}
 int split_rows(int (*out)[4]) {
@@ -137,3 +138,8 @@ def alone(M, ctas, splits):
 
 def alone_smem():
     return lib().alone_smem()
+
+
+def splits_whole(tiles, K):
+    """K splits of a launch of the split-K kernel's forms that take an SM alone."""
+    return lib().splits_whole(tiles, K)

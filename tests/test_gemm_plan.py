@@ -237,3 +237,13 @@ def test_every_split_has_k_blocks_and_a_place():
                 for a8 in (False, True):
                     s = gp.splits_pairs(tiles, K, M, a8)
                     assert 1 <= s <= 8 and (s == 1 or (K >= 640 * s and tiles * s <= 2 * 148 * 7 // 8))
+
+
+def test_clusters_of_one_cta_an_sm_all_find_a_place():
+    """Whole clusters that a 148-SM GPU places at once with a CTA to an SM, as its driver reports them."""
+    places = {1: 148, 2: 74, 3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15}
+    for tiles in range(1, 149):
+        for K in (640, 1280, 4096, 8832, 14336, 28672):
+            s = gp.splits_whole(tiles, K)
+            assert s == 1 or tiles <= places[s], (tiles, K, s)
+    assert [gp.splits_whole(t, 14336) for t in (15, 16, 18, 21, 22)] == [8, 6, 6, 6, 5]
