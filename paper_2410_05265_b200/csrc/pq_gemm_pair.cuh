@@ -214,9 +214,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor map over a dense packed matrix [rows, kbytes] of bytes; box = [box_rows, box_bytes]. The kernel that reads
-// the landing buffer one row per thread asks for the 64-byte swizzle (16-byte chunk index XOR (row >> 1) & 3) so that
-// those reads hit distinct banks; the other reads it chunk by chunk and takes it unswizzled.
+// Tensor map over a dense packed matrix [rows, kbytes] of bytes; box = [box_rows, box_bytes]. Kernels that read
+// the landing buffer one row per thread ask for the swizzle of their row, so that those reads hit distinct banks: 64 bytes (16-byte chunk index
+// XOR (row >> 1) & 3) or, in the split-K kernel's K blocks of 256 elements, 128 bytes (XOR row & 7). What is read chunk by chunk is unswizzled.
 inline bool make_packed_map(pq_ctx* ctx, CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t kbytes, int box_rows,
                             CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE, int box_bytes = PK_ROW) {
   cuuint64_t gdim[2] = {static_cast<cuuint64_t>(kbytes), static_cast<cuuint64_t>(rows)};

@@ -229,6 +229,8 @@ constexpr int MAX_SPLIT = 8;  // portable cluster size
 // As many K splits as leave every CTA resident at once with room for the clusters to be placed (7/8 of the slots: 48 tiles
 // x 6 = 288 CTAs ran in two waves, 10.7 us against 7.0 with 96), and at least 640 elements of K per CTA (below that the two
 // cluster barriers cost more than the shorter loop saves: 4096 x 4096 at 32 tokens 6.1 us with six splits, 6.6 with eight).
+// The splits share whole K blocks, so that their shares can differ by one (16 blocks over five CTAs); the fewest splits with the same longest share
+// lose all the same, because fewer CTAs read: 48 x 6144 x 4096, five / four splits, 9.6 / 10.2, per token at 32 8.0 / 9.3, 8B linear set at 32 47.9 / 48.8.
 // A cluster's CTAs lie in one GPC: of clusters of seven or eight with a CTA to an SM only fifteen find a place (cudaOccupancyMaxActiveClusters; 22, 26, 33, 45
 // of six, five, four, three, so that 7/8 of the SMs is the lower line there). The sixteenth ran behind the others: 345 x 768 x 14336, eighteen tiles, seven splits / six,
 // 24.3 / 15.8 us, W4A8 160 x 1152 x 14336 20.3 / 13.4, 200 x 2176 x 8192 24.7 / 15.1. Two CTAs to an SM find 37 of seven and 33 of eight.
@@ -242,7 +244,7 @@ inline int split_count(int tiles, int K, int sm_count, int per_sm) {
 
 // The forms of which two CTAs share an SM. Above 64 tokens the partial tiles are large, and an SM's two CTAs exchange theirs at the same
 // time: one CTA to an SM and fewer splits, of at least 1280 elements of K, win with a short K, and with 8-bit tokens above 88 while that leaves four
-// splits. us with the rotation, two to an SM / one: W4A8 at 96 tokens 6144 x 4096 five splits 11.9 / two 10.0, 4096 x 4096 six 11.2 / three 9.6, 4096 x 14336
+// splits. us with the rotation, two to an SM / one (before such launches were kept to one, see split_alone): W4A8 at 96 tokens 6144 x 4096 five splits 11.9 / two 10.0, 4096 x 4096 six 11.2 / three 9.6, 4096 x 14336
 // eight 16.6 / four 14.4 (at 80 15.5 / 16.3), but 8192 x 8192 four 15.7 / two 16.3, 8192 x 28672 four 30.6 / two 36.4; 4-bit 4096 x 4096 at 96 11.9 / 10.6,
 // at 128 six 13.4 / three 11.9 (four 13.7), 6144 x 4096 at 96 12.9 / 13.3, at 128 15.2 / 13.8, 4096 x 14336 at 80 18.0 / 20.2; at 64 tokens 4096 x 14336
 // eight 15.3 / four 17.6.

@@ -51,7 +51,6 @@ using namespace pq_pair;
 using namespace pq_plan;
 
 constexpr int EXPAND_WARP0 = 4;
-constexpr int MAX_SPLIT = 8;               // portable cluster size
 
 template <int NT, bool A8, bool WHOLE>
 struct Cfg : SplitCfg<NT, A8, WHOLE> {
